@@ -11,6 +11,7 @@
 
 #include <nvtx3/nvToolsExt.h>
 
+#include "sinkhorn_class.h"
 #include "taot_internal.cuh"
 
 namespace {
@@ -278,9 +279,16 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
             }
         }
     }
-    // first Sinkhorn row update with v = 1 on every rank: log-sum-exp of -C_ij/eps over all j
+    taot_class_plan classes;
+    taot_build_classes(&classes, h_C, R);
+    h->cls_kind = classes.kind;
+    h->cls_nc = classes.nc; h->cls_gpl = classes.gpl; h->cls_npg = classes.npg;
+    for (int i = 0; i < 3; ++i) h->cls_tier[i] = classes.tier[i];
+    // first Sinkhorn row update with v = 1 on every rank: log-sum-exp of -C_ij/eps over all j (beyond 256 ranks once per
+    // class, whose ranks have the same terms in another order)
     std::vector<double> lse0(R);
     for (int i = 0; i < R; ++i) {
+        if (R > 256 && classes.rep[i] != i) { lse0[i] = lse0[classes.rep[i]]; continue; }
         double mx = -INFINITY;
         for (int j = 0; j < R; ++j) {
             const double x = -(double)h_C[(size_t)i * R + j] / (double)params->eps;
@@ -294,7 +302,7 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
     // M and its transpose, each split into two TF32-exact parts (high: low 13 mantissa bits cleared; low: the rest,
     // again with 13 bits cleared)
     std::vector<float> gibbs;
-    if (R > 256 && R % 128 == 0 && !h->tier_ok && !std::getenv("TAOT_NO_TENSOR_CORES")) {
+    if (R > 256 && R % 128 == 0 && !classes.kind && !std::getenv("TAOT_NO_TENSOR_CORES")) {
         double worst = 0.0;
         for (size_t q = 0; q < (size_t)R * R; ++q) worst = std::max(worst, (double)h_C[q] / (double)params->eps);
         if (worst <= 20.0) {
@@ -334,6 +342,27 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
     if (rc == TAOT_OK) rc = upload(&h->d_C, h_C, (size_t)R * R);
     if (rc == TAOT_OK) rc = upload(&h->d_B, B.data(), (size_t)R * R);
     if (rc == TAOT_OK) rc = upload(&h->d_rowlse0, lse0.data(), (size_t)R);
+    if (rc == TAOT_OK && h->cls_kind) {
+        std::vector<double> cl(classes.slot_rep.size(), 0.0);
+        for (size_t q = 0; q < cl.size(); ++q)
+            if (classes.slot_rep[q] >= 0) cl[q] = lse0[classes.slot_rep[q]];
+        // one block for the five arrays, the widest elements first
+        const size_t nl = cl.size() * sizeof(double), nc = classes.cost.size() * sizeof(float),
+                     no = classes.off.size() * sizeof(int32_t), nr = (size_t)R * sizeof(uint16_t);
+        std::vector<unsigned char> blob(nl + nc + no + 2 * nr);
+        std::memcpy(blob.data(), cl.data(), nl);
+        std::memcpy(blob.data() + nl, classes.cost.data(), nc);
+        std::memcpy(blob.data() + nl + nc, classes.off.data(), no);
+        std::memcpy(blob.data() + nl + nc + no, classes.cls.data(), nr);
+        std::memcpy(blob.data() + nl + nc + no + nr, classes.list.data(), nr);
+        unsigned char* d = nullptr;
+        rc = upload(&d, blob.data(), blob.size());
+        h->d_cls_lse0 = reinterpret_cast<double*>(d);
+        h->d_cls_cost = reinterpret_cast<float*>(d + nl);
+        h->d_cls_off = reinterpret_cast<int32_t*>(d + nl + nc);
+        h->d_cls = reinterpret_cast<uint16_t*>(d + nl + nc + no);
+        h->d_cls_list = reinterpret_cast<uint16_t*>(d + nl + nc + no + nr);
+    }
     if (rc == TAOT_OK && !gibbs.empty()) rc = upload(&h->d_gibbs, gibbs.data(), gibbs.size());
     if (rc == TAOT_OK) rc = upload(&h->d_rank_off, off.data(), (size_t)R + 1);
     if (rc == TAOT_OK) rc = upload(&h->d_rank_list, list.data(), (size_t)E);
@@ -451,6 +480,7 @@ int taot_destroy(taot_handle_t h)
     cudaFree(h->d_rank_off); cudaFree(h->d_rank_list); cudaFree(h->d_tierval); cudaFree(h->d_tiermask);
     cudaFree(h->d_tpos); cudaFree(h->d_torder); cudaFree(h->d_tdest); cudaFree(h->d_bidlist);
     cudaFree(h->d_merge_part); cudaFree(h->d_merge_cnt);
+    cudaFree(h->d_cls_lse0);                       // and the other four arrays of the block
     for (int i = 0; i < 6; ++i)
         if (h->ev[i]) cudaEventDestroy(h->ev[i]);
     delete h;
@@ -560,7 +590,8 @@ int taot_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, int32_t B
                                  ws ? reinterpret_cast<float*>(at(ws, h->off_tc)) : nullptr);
     if (a < 0) return a;
     // s and d are the caller's here: problems with a NaN or an infinity in them are closed out after the solve
-    int g = taot_launch_sinkhorn_guard(h, d_s, d_d, B, d_plan, d_iters, d_row_err, d_info, static_cast<cudaStream_t>(stream));
+    // (the class kernels look for them themselves)
+    int g = taot_sinkhorn_takes_classes(h, false) ? 0 : taot_launch_sinkhorn_guard(h, d_s, d_d, B, d_plan, d_iters, d_row_err, d_info, static_cast<cudaStream_t>(stream));
     if (g < 0) return g;
     h->last_launches = a + g;
     return TAOT_OK;
@@ -686,7 +717,7 @@ int plan_stages(taot_handle_t h, const int32_t* d_topk, const taot_outputs* o, v
         TAOT_CUDA_OK(cudaMemsetAsync(o->row_err, 0, sizeof(float) * p.L, st));
         a = 0;
     } else if ((a = taot_launch_sinkhorn(h, fs, fd, p.L, o->plan, o->sinkhorn_iters, o->row_err, o->info,
-                                         reinterpret_cast<float*>(at(ws, h->off_kt)), st)) < 0) {
+                                         reinterpret_cast<float*>(at(ws, h->off_kt)), st, nullptr, true)) < 0) {
         nvtxRangePop();
         return a;
     }

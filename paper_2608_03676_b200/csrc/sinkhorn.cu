@@ -336,6 +336,7 @@ __global__ void __launch_bounds__(1024) sinkhorn_kernel(SinkArgs a)
 int taot_launch_sinkhorn_tile(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st);
 int taot_launch_sinkhorn_cluster(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st);
 int taot_launch_sinkhorn_tiered(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st);
+int taot_launch_sinkhorn_class(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st);
 int taot_launch_sinkhorn_dense_tc(taot_handle_t h, const SinkArgs& a, int32_t B, float* ws_tc, cudaStream_t st);
 
 // Caller-supplied supply / demand vectors (the stand-alone entry point; inside taot_plan they come from integer
@@ -370,8 +371,18 @@ int taot_launch_sinkhorn_guard(taot_handle_t h, const float* d_s, const float* d
     return 1;
 }
 
+// Costs with classes of interchangeable ranks: the class kernels beyond 256 ranks and, up to there, for a caller's own
+// batch with a fixed iteration count (R > 32: below, the register tiles are as fast).  Inside taot_plan, and in tolerance mode,
+// Phase 1 stays on the tile and tier-sum kernels: the placement that follows decides exact ties (experts of one node's
+// ranks on one cold rank) by the last bits of the hint, so its kernel is part of the result.
+bool taot_sinkhorn_takes_classes(taot_handle_t h, bool from_loads)
+{
+    const taot_params& p = h->p;
+    return h->cls_kind && (p.R > 256 || (!from_loads && p.tol <= 0.0f && p.R > 32));
+}
+
 int taot_launch_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, int32_t B, float* d_plan,
-                         int32_t* d_iters, float* d_row_err, int32_t* d_info, float* d_kt, cudaStream_t st, float* d_tc)
+                         int32_t* d_iters, float* d_row_err, int32_t* d_info, float* d_kt, cudaStream_t st, float* d_tc, bool from_loads)
 {
     const taot_params& p = h->p;
     SinkArgs a;
@@ -394,10 +405,11 @@ int taot_launch_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, in
         a.s = d_s + (int64_t)b0 * p.R; a.d = d_d + (int64_t)b0 * p.R;
         a.plan = d_plan + (int64_t)b0 * p.R * p.R; a.iters = d_iters + b0; a.row_err = d_row_err + b0;
         a.info = d_info + b0;
-        const int nt = taot_launch_sinkhorn_tiered(h, a, nb, st);
+        const bool classes = taot_sinkhorn_takes_classes(h, from_loads);
+        const int nt = classes ? taot_launch_sinkhorn_class(h, a, nb, st) : taot_launch_sinkhorn_tiered(h, a, nb, st);
         if (nt < 0) return nt;
         if (nt > 0) {
-            // tiered cost: O(R) sums per half-step, one warp per problem; what it hands back goes to the kernel below
+            // complete, except for problems handed back: with classes those that have a rank with both supply and demand
             launched += nt;
             a.only_marked = 1;
         } else if (p.R <= 256) {

@@ -607,8 +607,6 @@ int launch_mw(const SinkArgs& a, const TierCosts& tc, int32_t B, cudaStream_t st
 // Warps per problem by batch size (measured, 500 fixed iterations, B = 1 / 64 / 1024 / 4096, ms):
 //   256 ranks:  8 warps 0.175 / 0.177 / 0.478 / 1.77,  4 warps 0.174 / 0.175 / 0.285 / 0.981,  2 warps 0.216 / 0.218 / 0.287 / 0.843
 //               (one warp with 8 ranks per lane, a kernel of its own until then: - / - / 0.414 / 0.988)
-//   512 ranks:  8 warps 0.214 / 0.218 / 0.779 / 2.63,  4 warps 0.236 / 0.240 / 0.619 / 1.88,   2 warps 0.318 / 0.324 / 0.811 / 2.09
-//   1024 ranks: 8 warps 0.343 / 0.359 / 1.68 / 5.92,   4 warps 0.384 / 0.412 / 1.61 / 5.11
 // A problem that has an SM to itself is one dependent chain and wants the fewest instructions per warp (8 warps; with a
 // tolerance also at 256 ranks, 0.381 against 0.391 ms at config 4); a batch that fills the GPU wants the fewest
 // instructions per problem that still leave enough warps to hide each other's latency (4 warps, 2 for the largest
@@ -621,33 +619,16 @@ int launch_mw_ranks(const SinkArgs& a, const TierCosts& tc, int32_t B, cudaStrea
     TAOT_CUDA_OK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     const bool alone = 2 * B <= sms;               // every problem gets an SM to itself
     const bool huge = B >= 16 * sms;
-    switch (a.R) {
-        case 256:
-            if constexpr (kNode >= 4) {
-                if (huge) return launch_mw<kNode, kGroup, 2, 4>(a, tc, B, st);
-            }
-            if constexpr (kNode >= 2) {
-                if (!alone) return launch_mw<kNode, kGroup, 4, 2>(a, tc, B, st);
-            }
-            return launch_mw<kNode, kGroup, 8, 1>(a, tc, B, st);
-        case 512:
-            if constexpr (kNode >= 4) {
-                if (!alone) return launch_mw<kNode, kGroup, 4, 4>(a, tc, B, st);
-            }
-            if constexpr (kNode >= 2) return launch_mw<kNode, kGroup, 8, 2>(a, tc, B, st); else return 0;
-        case 1024:
-            if constexpr (kNode >= 8) {
-                if (!alone) return launch_mw<kNode, kGroup, 4, 8>(a, tc, B, st);
-            }
-            if constexpr (kNode >= 4) return launch_mw<kNode, kGroup, 8, 4>(a, tc, B, st); else return 0;
-        default: return 0;
-    }
+    if (a.R != 256) return 0;
+    if (huge) return launch_mw<kNode, kGroup, 2, 4>(a, tc, B, st);
+    if (!alone) return launch_mw<kNode, kGroup, 4, 2>(a, tc, B, st);
+    return launch_mw<kNode, kGroup, 8, 1>(a, tc, B, st);
 }
 
 }  // namespace
 
 // Launches the tiered-cost kernel if the handle's cost matrix has the node / rail-group structure (checked at
-// taot_create, which also requires 256, 512 or 1024 ranks); returns the number of kernels launched (0: not
+// taot_create) and 256 ranks; returns the number of kernels launched (0: not
 // applicable or a hierarchy that is not built, the caller takes the general kernels).
 int taot_launch_sinkhorn_tiered(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st)
 {

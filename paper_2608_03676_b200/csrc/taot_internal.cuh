@@ -40,9 +40,18 @@ struct taot_handle_s {
     int32_t nbid;            // 0: no list (no tiers, or price step <= 0): the auction scans densely
     int32_t* d_merge_part;   // [L][TAOT_MERGE_PARTS][E] expert loads of the parts of a layer's merge, or null (one CTA per layer)
     int32_t* d_merge_cnt;    // [L] parts of a layer's merge that are done; zero between calls
-    int32_t tier_ok;         // 1: C has a node / rail-group structure one of the tier-by-tier kernels is built for and R is 256, 512 or 1024
-    int32_t tier_node, tier_group;   // ranks per node and per rail group of that structure (8 / 32, 4 / 16, 4 / 32 or 16 / 32)
+    // Classes of interchangeable ranks of the cost matrix, for the class kernels of Phase 1 (sinkhorn_class.cu)
+    int32_t cls_kind;        // 0 none, 1 dense (at most 32 classes), 2 tree (three tiers between the classes)
+    int32_t cls_nc, cls_gpl, cls_npg;
+    float cls_tier[3];
+    uint16_t* d_cls;         // [R] slot of each rank's class
+    int32_t* d_cls_off;      // [slots + 1] CSR of ranks by slot
+    uint16_t* d_cls_list;    // [R]
+    double* d_cls_lse0;      // [slots]
+    float* d_cls_cost;       // [nc][nc] (dense)
+    int32_t tier_ok;         // 1: C has a node / rail-group structure the tier-by-tier kernels are built for and R is 256, 512 or 1024
     float tier_cost[3];      // its three costs off the diagonal: same node, same rail group, otherwise
+    int32_t tier_node, tier_group;   // ranks per node and per rail group of that structure (8 / 32, 4 / 16, 4 / 32 or 16 / 32)
     // derived sizes
     int64_t seg;             // elements per (layer, rank) segment
     int32_t nc;              // chunks per segment
@@ -90,7 +99,8 @@ int taot_launch_excess_spare(taot_handle_t h, const int32_t* d_rank_load, int32_
                              int32_t* d_spare, float* d_s, float* d_d, cudaStream_t st);
 int taot_launch_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, int32_t B, float* d_plan,
                          int32_t* d_iters, float* d_row_err, int32_t* d_info, float* d_kt, cudaStream_t st,
-                         float* d_tc = nullptr);
+                         float* d_tc = nullptr, bool from_loads = false);   // from_loads: called by taot_plan
+bool taot_sinkhorn_takes_classes(taot_handle_t h, bool from_loads);
 size_t taot_sinkhorn_tc_ws_floats(int32_t R, int32_t B);
 int taot_launch_sinkhorn_guard(taot_handle_t h, const float* d_s, const float* d_d, int32_t B, float* d_plan,
                                int32_t* d_iters, float* d_row_err, int32_t* d_info, cudaStream_t st);
