@@ -45,13 +45,11 @@ int taot_get_group_trace(taot_handle_t h, int32_t* groups, float* h_ms /* [6][6]
  * With profiling level 2 (taot_set_profiling), taot_match / taot_plan make the kernel count SM clock cycles, as thread 0 of each layer's
  * CTA sees them, into `ws`; this call copies them to the host (it synchronises the device).
  *   h_cycles [L][16]: 0 set-up (loads, spill, round-invariant score terms), 1 Phase 2 (Algorithm 2),
- *   2 set-up of Phase 3, 3 Phase-3 bids (round start to the barrier after arbitration, summed over rounds),
- *   4 Phase-3 updates (to the barrier that ends the round), 5 the whole kernel, 6 / 7 the probe and the
- *   arbitration time of the thread that spent most on each (its own time, no waiting at barriers),
+ *   2 set-up of Phase 3, 3 Phase-3 rounds with more than 32 classes of slots (several warps), 4 Phase-3 rounds with at
+ *   most 32 (one warp), 5 the whole kernel, 6 classes, 7 the round the one warp went on with,
  *   8-11 Phase 2 split: rank scans + arbitration, winners, re-forming the served experts' keys, forming all keys
- *   once per slot index; 12 the Phase-3 loop as a whole (3 and 4 are what thread 0 sees between its own clock reads:
- *   loads of the next round that the compiler starts before the round's first clock read fall outside them, and the
- *   counting build itself is slower than the timed one, so 12 / rounds is an upper bound per round); 13-15 zero.
+ *   once per slot index; 12 the Phase-3 loop as a whole (the counting build itself is slower than the timed one, so
+ *   12 / rounds is an upper bound per round); 13-15 zero.
  * `ws` is the workspace of the profiled call.  Errors: TAOT_ERR_NULL, TAOT_ERR_UNSUPPORTED (R > 256).
  */
 int taot_get_match_cycles(taot_handle_t h, const void* ws, int64_t* h_cycles /* [L][16] */);

@@ -228,8 +228,8 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
     // Every score a bid of the tiered auction can take is  tierval[t] - price_step * w  for a tier t and a win count
     // w in [0, S].  All (t, w) pairs are listed once, best score first (evaluated with the same two fp32 operations
     // the kernel uses), so that a slot walks the list instead of comparing tiers; pairs with the same score form a
-    // group (bit 31 = "the next entry has the same score").  Entry: w << 8 | t.
-    std::vector<uint32_t> bidlist;
+    // group (bit 31 = "the next entry has the same score").  Entry: w << 8 | t.  bident has them by pair (auction.cuh).
+    std::vector<uint32_t> bidlist, bident;
     if (h->ntiers > 0 && params->price_step > 0.0f && R <= 256) {
         const int S = R * params->K;
         struct Pair { float sc; int t, w; };
@@ -243,9 +243,19 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
             }
         std::stable_sort(pairs.begin(), pairs.end(), [](const Pair& x, const Pair& y) { return x.sc > y.sc; });
         bidlist.resize(pairs.size());
+        bident.resize(pairs.size());
         for (size_t i = 0; i < pairs.size(); ++i) {
             const bool tie_next = i + 1 < pairs.size() && pairs[i + 1].sc == pairs[i].sc;
+            if (tie_next) h->bid_ties = 1;
+            uint32_t above = 0;                                               // tiers that score strictly higher at this win count
+            float last = INFINITY;
+            for (int t = 0; t < pairs[i].t; ++t) {                            // (tier values descend)
+                volatile float price = params->price_step * (float)pairs[i].w;
+                volatile float sc = tierval[t] - price;
+                if (sc > pairs[i].sc && sc < last) { ++above; last = sc; }
+            }
             bidlist[i] = ((uint32_t)pairs[i].w << 8) | (uint32_t)pairs[i].t | (tie_next ? 0x80000000u : 0u);
+            bident[(size_t)pairs[i].t * (S + 1) + pairs[i].w] = ((uint32_t)i << 16) | (tie_next ? 1u << 14 : 0u) | (above << 11) | (uint32_t)pairs[i].w;
         }
     }
     h->nbid = (int32_t)bidlist.size();
@@ -382,7 +392,22 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
         if (rc == TAOT_OK) rc = upload(&h->d_tdest, tdest.data(), tdest.size());
     }
     if (rc == TAOT_OK && h->ntiers > 0) rc = upload(&h->d_tiermask, tiermask.data(), tiermask.size());
-    if (rc == TAOT_OK && h->nbid > 0) rc = upload(&h->d_bidlist, bidlist.data(), bidlist.size());
+    if (rc == TAOT_OK && h->nbid > 0) {
+        std::vector<int32_t> hostcls(R);
+        const int TW = h->ntiers * ((R + 31) / 32);
+        for (int x = 0; x < R; ++x) {
+            hostcls[x] = x;
+            for (int y = 0; y < x && hostcls[x] == x; ++y) {
+                if (hostcls[y] != y) continue;
+                bool same = true;
+                for (int q = 0; q < TW && same; ++q) same = tiermask[(size_t)q * R + x] == tiermask[(size_t)q * R + y];
+                if (same) hostcls[x] = y;
+            }
+        }
+        rc = upload(&h->d_bidlist, bidlist.data(), bidlist.size());
+        if (rc == TAOT_OK) rc = upload(&h->d_bident, bident.data(), bident.size());
+        if (rc == TAOT_OK) rc = upload(&h->d_hostcls, hostcls.data(), hostcls.size());
+    }
     // the merge of a layer's chunk counts is shared by several CTAs where a layer has enough of them (the kernel sits in
     // the chain of latency-bound stages): their partial expert loads and a counter of finished parts per layer
     if (rc == TAOT_OK && R % (32 * TAOT_MERGE_PARTS) == 0) {
@@ -478,7 +503,7 @@ int taot_destroy(taot_handle_t h)
     if (h->bstream) cudaStreamDestroy(h->bstream);
     cudaFree(h->d_e2r); cudaFree(h->d_C); cudaFree(h->d_B); cudaFree(h->d_rowlse0); cudaFree(h->d_gibbs);
     cudaFree(h->d_rank_off); cudaFree(h->d_rank_list); cudaFree(h->d_tierval); cudaFree(h->d_tiermask);
-    cudaFree(h->d_tpos); cudaFree(h->d_torder); cudaFree(h->d_tdest); cudaFree(h->d_bidlist);
+    cudaFree(h->d_tpos); cudaFree(h->d_torder); cudaFree(h->d_tdest); cudaFree(h->d_bidlist); cudaFree(h->d_bident); cudaFree(h->d_hostcls);
     cudaFree(h->d_merge_part); cudaFree(h->d_merge_cnt);
     cudaFree(h->d_cls_lse0);                       // and the other four arrays of the block
     for (int i = 0; i < 6; ++i)

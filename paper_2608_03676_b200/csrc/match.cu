@@ -13,20 +13,12 @@
 // are computed once per layer for the experts that spill; a round is then one thread per rank
 // scanning those experts with coalesced reads.
 //
-// Phase 3: the bonus matrix of a real topology has a handful of distinct values (tiers).  Within
-// a tier a slot's score  B3 - step*wins[r]  depends on r only through wins[r], so every score a bid
-// can take is one of (tier, win count) pairs, and those are listed once per handle in order of
-// decreasing fp32 score (equal scores grouped).  Ranks are kept as bit sets (per tier and host, per
-// win count, per expert availability); a slot walks the list with a cursor that never moves back
-// and a probe is a few word-wide ANDs instead of a scan over all R ranks.  The exact fp32 score is
-// what orders the list, so win counts or tiers whose scores round to the same float compete on the
-// rank index alone, as in a dense scan.  A bonus matrix with more than kMaxTiers distinct values (or
-// a price step that is not positive) takes the dense scan instead.
-// A round of the bit-set auction is a chain of a few dozen dependent instructions between two plain barriers, so its
-// cost is the instructions on that chain: every lane, whatever its slot's state, runs the same straight code (a slot
-// that is done has an empty mask and sends its key to a word nobody reads), shared memory is addressed by 32-bit
-// shared addresses, the end of the auction is read from a counter of live slots instead of a reducing barrier, and
-// only the two rare events -- a cursor that has to move, a win -- branch off.
+// Phase 3: the bonus matrix of a real topology has a handful of distinct values (tiers): the auction of auction.cuh.  A bonus
+// matrix with more than TAOT_MAX_TIERS distinct values, a price step that is not positive or more than 1024 slots take a
+// dense scan instead.
+#include <type_traits>
+
+#include "auction.cuh"
 #include "taot_internal.cuh"
 
 namespace {
@@ -44,7 +36,9 @@ struct MatchArgs {
     const int32_t* rank_list;    // [E]
     const uint32_t* tiermask;    // [ntiers][W][R hosts] bit r of word w: B3[32w + r][host] == tierval[t]
     const float* tierval;        // [ntiers] descending
-    const uint32_t* bidlist;     // [nbid] (tier, win count) pairs by decreasing score: w << 8 | t, bit 31: next has the same score
+    const uint32_t* bidlist;     // [nbid] (tier, win count) pairs by decreasing score: tier | win count << 8, bit 31: next has the same score
+    const uint32_t* bident;      // [nbid] the same by tier and win count (see auction.cuh)
+    const int32_t* hostcls;      // [R] hosts that see every rank at the same bonus share a number
     int32_t* slot_expert;        // [L,R,K]
     int32_t* slot_tokens;        // [L,R,K]
     int32_t* X;                  // [L,R,S]
@@ -60,11 +54,9 @@ struct MatchArgs {
     int32_t tm_in_smem;
     int32_t big_floats;          // 4-byte words of the shared block that holds the Phase-2 score rows, then nrem
     long long* cyc;              // [L][16] SM cycles per part of the kernel as thread 0 sees them, or null (profiling aid):
-                                 // 0 set-up, 1 Phase 2, 2 Phase-3 set-up, 3 Phase-3 bids (to the first barrier of a round),
-                                 // 4 Phase-3 updates (to the second barrier), 5 whole kernel, 6 / 7 the busiest thread's own
-                                 // probe and arbitration time in Phase 3, 8-11 Phase-2 split, 12 the Phase-3 loop as a whole.
-                                 // A barrier does not hold a warp up until its next shared-memory access, so the wait at
-                                 // the first barrier is counted under 4 and the wait at the second under 3 of the next round.
+                                 // 0 set-up, 1 Phase 2, 2 Phase-3 set-up, 3 Phase-3 rounds of more than 32 classes, 4 of at most
+                                 // 32 (one warp), 5 whole kernel, 6 classes, 7 the round the one warp went on with, 8-11 Phase-2
+                                 // split, 12 the Phase-3 loop as a whole
 };
 
 __device__ __forceinline__ uint32_t ordered_bits(float f)
@@ -82,50 +74,8 @@ __device__ __forceinline__ u64 warp_max_u64(u64 k)
     return k;
 }
 
-// Barrier over the first `nthreads` threads of the CTA only (a multiple of 32), on hardware barrier 1: the auction's
-// rounds involve the warps that hold slots, the others wait at the CTA-wide barrier that follows the auction.  The
-// aligned form: every lane of a warp that takes part reaches it together (the loop's conditions are the same for all
-// lanes of a warp and the branches inside a round close before it).
-__device__ __forceinline__ void bar_part(int nthreads)
-{
-    asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
-}
-
-// Shared-memory accesses of the auction's rounds by 32-bit shared address: one instruction each, no 64-bit address
-// arithmetic and no address-space conversion on the chain of a round.
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ uint32_t lds_u32(uint32_t addr)
-{
-    uint32_t v;
-    asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ void sts_u32(uint32_t addr, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
-__device__ __forceinline__ void red_max_u32(uint32_t addr, uint32_t v) { asm volatile("red.shared.max.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
-__device__ __forceinline__ void red_and_u32(uint32_t addr, uint32_t v) { asm volatile("red.shared.and.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
-__device__ __forceinline__ void red_add_u32(uint32_t addr, uint32_t v) { asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
-__device__ __forceinline__ void red_or_u32(uint32_t addr, uint32_t v) { asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(addr), "r"(v) : "memory"); }
-
 constexpr int kMaxW = 8;          // words of a rank bit set: R <= 256
 constexpr size_t kSmemBudget = 224 * 1024;   // dynamic shared memory the kernel plans with (227 KB per CTA less the static part)
-
-// Lowest set bit over kMaxW words (bit index = 32*w + bit), or -1: independent ANDs and a select tree
-// instead of a word-by-word scan, so that a lone warp is not held up by a long dependency chain.
-__device__ __forceinline__ int first_hit(const uint32_t (&cand)[8], const uint32_t* lv, int stride, int W)
-{
-    uint32_t h[8];
-#pragma unroll
-    for (int w = 0; w < 8; ++w) h[w] = (w < W) ? (cand[w] & lv[w * stride]) : 0u;
-    // pairwise: keep the lower word if it is nonzero
-    const uint32_t a0 = h[0] ? h[0] : h[1]; const int i0 = h[0] ? 0 : 1;
-    const uint32_t a1 = h[2] ? h[2] : h[3]; const int i1 = h[2] ? 2 : 3;
-    const uint32_t a2 = h[4] ? h[4] : h[5]; const int i2 = h[4] ? 4 : 5;
-    const uint32_t a3 = h[6] ? h[6] : h[7]; const int i3 = h[6] ? 6 : 7;
-    const uint32_t b0 = a0 ? a0 : a1; const int j0 = a0 ? i0 : i1;
-    const uint32_t b1 = a2 ? a2 : a3; const int j1 = a2 ? i2 : i3;
-    const uint32_t c = b0 ? b0 : b1; const int k = b0 ? j0 : j1;
-    return c ? (k << 5) + __ffs(c) - 1 : -1;
-}
 
 // Arbitration "best bidder per target" for one warp's worth of bids.  Many bidders often pick the
 // same target (all slots of a tier chase the cheapest rank), so the lanes that bid for the same
@@ -149,8 +99,9 @@ __device__ __forceinline__ void arbitrate(u64* arb, int target, u64 key)
     }
 }
 
-template <bool TIMED>
-__global__ void __launch_bounds__(1024)
+// LEAN: the auction's build for handles with at most four tiers and no equal scores; NSM: what the ranks hold is in shared memory
+template <bool TIMED, int MAXT, bool LEAN, bool NSM>
+__global__ void __launch_bounds__(MAXT, 1)
 match_kernel(MatchArgs a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -177,12 +128,17 @@ match_kernel(MatchArgs a)
     uint32_t* lvl = avail + a.dmax * W;                        // [W][S+1]   ranks by win count (word-major)
     uint32_t* tm_s = lvl + (S + 1) * W;                                // [ntiers][W][S] tier masks by slot, if they fit
     uint32_t* bid_s = tm_s + (a.tm_in_smem ? a.ntiers * W * S : 0);    // [nbid] (tier, win count) pairs, best score first
-    int32_t* tw_word = reinterpret_cast<int32_t*>(bid_s + a.nbid);     // [ntiers][S] word holding the whole tier for the slot's host, or -1
+    int32_t* tw_word = reinterpret_cast<int32_t*>(bid_s + a.nbid);     // [ntiers][S] word holding the whole tier for the class, or -1
     uint32_t* tw_mask = reinterpret_cast<uint32_t*>(tw_word + (a.nbid ? a.ntiers * S : 0));   // [ntiers][S] that word's mask
-    int32_t* nrem_s = reinterpret_cast<int32_t*>(tw_mask + (a.nbid ? a.ntiers * S : 0));      // [dmax*R] if it fits
+    uint32_t* ent_s = tw_mask + (a.nbid ? a.ntiers * S : 0);           // [nbid] the pairs by tier and win count
+    int32_t* key_s = reinterpret_cast<int32_t*>(ent_s + a.nbid);       // [S] class keys, then the classes' lists
+    uint16_t* nxt_s = reinterpret_cast<uint16_t*>(key_s + (a.nbid ? S : 0));            // [S] next slot of the class
+    uint16_t* lead_s = nxt_s + (a.nbid ? S : 0);                       // [S] first slot of each class
+    int32_t* nrem_s = reinterpret_cast<int32_t*>(lead_s + (a.nbid ? S : 0));            // [dmax*R] if it fits
     __shared__ long long s_tot;
     __shared__ int s_cnt, s_any, s_ns;
-    __shared__ uint32_t s_live3, s_lastwin;      // Phase 3: slots that can still bid; 1 + the last round somebody won
+    __shared__ taot_auction::Control ctl;
+    __shared__ uint32_t idle_s[32];
     __shared__ int s_wcnt[32];
 
     const int32_t* n = a.n + l * (int64_t)R * E;
@@ -194,7 +150,7 @@ match_kernel(MatchArgs a)
 
     const bool timed = TIMED && tid == 0;
     const long long c_start = timed ? clock64() : 0;
-    long long c_bid = 0, c_upd = 0, c_probe = 0, c_atom = 0, c_scan = 0, c_win = 0, c_row = 0, c_build = 0;
+    long long c_scan = 0, c_win = 0, c_row = 0, c_build = 0;
     // ---- integer mean, excess, spare (Appendix A.1)
     if (tid == 0) { s_tot = 0; s_cnt = 0; }
     __syncthreads();
@@ -452,7 +408,7 @@ match_kernel(MatchArgs a)
 
     // =========================================================== Phase 3
     const long long c_p3 = timed ? clock64() : 0;
-    long long c_p3loop = c_p3, c_p3end = c_p3;
+    long long c_p3loop = c_p3, c_p3warp = c_p3, c_p3end = c_p3, c_classes = 0, c_handed = 0;
     // compact the experts that sit in some slot; keep their per-rank remaining counts transposed [col][r]
     for (int e = tid; e < E; e += NT) dcol[e] = -1;
     if (tid == 0) s_cnt = 0;
@@ -487,198 +443,100 @@ match_kernel(MatchArgs a)
     const long long cap = (long long)R * S + S;
     const bool tiered = a.nbid > 0 && S <= NT;
     if (tiered && D > 0) {
-        // ---- bit-set auction: thread s is slot s for the whole auction and keeps the slot's state in registers.
-        // A bid walks the list of all (tier, win count) pairs in order of decreasing score: the first pair that still
-        // has a candidate rank (in the tier for this slot's host, holding tokens of the slot's expert, with that win
-        // count) is the bid; pairs of equal score are scanned together and the lowest rank wins.  Win counts only grow
-        // and holdings only shrink, so no pair before the cursor can ever regain a candidate: the cursor never moves
-        // back and a round costs one or two probes per slot.
+        // ---- bit-set auction (auction.cuh): bidders are classes of slots that make the same bids
+        namespace au = taot_auction;
+        uint32_t* const arb = reinterpret_cast<uint32_t*>(arb_r);       // [2][R]
+        for (int q = tid; q < 2 * R; q += NT) arb[q] = 0u;
+        for (int q = tid; q < a.nbid; q += NT) { bid_s[q] = a.bidlist[q]; ent_s[q] = a.bident[q]; }
+        // a live slot's class: expert and the way its host sees the ranks; the lowest slot leads, the others queue behind it
         const int s = tid;
-        bool live = s < S && slot_e[s] >= 0 && slot_a[s] > 0;
-        const int e = live ? slot_e[s] : 0;
-        const int col = live ? dcol[e] : 0;
-        const int host = s < S ? s / K : 0;
-        int32_t A = live ? slot_a[s] : 0;
-        const uint32_t* av = avail + col;                          // word w at av[w * dmax]
-        // this slot's tier masks: tier t, word w at tm[(t * W + w) * tms]; a shared-memory copy when it fits
-        const uint32_t* tm = a.tiermask + host;
-        int tms = R;
-        if (a.tm_in_smem) {
-            for (int q = tid; q < a.ntiers * W * S; q += NT) {
-                const int ss = q % S, tw = q / S;
-                tm_s[q] = a.tiermask[(int64_t)tw * R + ss / K];
-            }
-            tm = tm_s + (s < S ? s : 0);
-            tms = S;
-        }
-        for (int q = tid; q < a.nbid; q += NT) bid_s[q] = a.bidlist[q];
-        for (int q = tid; q < 2 * R; q += NT) reinterpret_cast<uint32_t*>(arb_r)[q] = 0u;     // the two arbiter sets
-        __syncthreads();
-        const int LS = S + 1;                                      // lvl: word w of level wl at lvl[w * LS + wl]
-        // a tier whose ranks (for this slot's host) all sit in one 32-bit word is probed with that word alone
+        const bool slive = s < S && slot_e[s] >= 0 && slot_a[s] > 0;
         if (s < S) {
-            for (int t = 0; t < a.ntiers; ++t) {
-                int nz = 0, wd = 0;
-                uint32_t val = 0u;
-                for (int w = 0; w < W; ++w) {
-                    const uint32_t mk = tm[(t * W + w) * tms];
-                    if (mk) { ++nz; wd = w; val = mk; }
-                }
-                tw_word[t * S + s] = nz <= 1 ? wd : -1;
-                tw_mask[t * S + s] = nz <= 1 ? val : tm[(t * W) * tms];      // several words: the mask of word 0
+            key_s[s] = slive ? slot_e[s] * R + a.hostcls[s / K] : -1 - s;
+            nxt_s[s] = (uint16_t)au::kNoSlot;
+        }
+        if (tid == 0) { ctl.event[0] = ctl.event[1] = ctl.dead[0] = ctl.dead[1] = ctl.last = ctl.handed = 0u; }
+        __syncthreads();
+        bool lead = slive;
+        if (slive) {
+            const int32_t mine = key_s[s];
+            int prev = -1;
+#pragma unroll 8
+            for (int q = 0; q < s; ++q) prev = key_s[q] == mine ? q : prev;
+            if (prev >= 0) { nxt_s[prev] = (uint16_t)s; lead = false; }
+        }
+        const unsigned lb = __ballot_sync(0xffffffffu, lead);
+        if (lane == 0) s_wcnt[warp] = __popc(lb);
+        __syncthreads();
+        int C = 0;
+        {
+            int off = 0;
+            for (int w = 0; w < NW; ++w) { const int cnt = s_wcnt[w]; if (w < warp) off += cnt; C += cnt; }
+            if (lead) lead_s[off + __popc(lb & ((1u << lane) - 1u))] = (uint16_t)s;
+        }
+        __syncthreads();
+        // tier masks by class, and for each tier the word that holds all of it
+        if (a.tm_in_smem) {
+            for (int q = tid; q < a.ntiers * W * C; q += NT) {
+                const int tw = q / C, c = q - tw * C;
+                tm_s[tw * S + c] = a.tiermask[(int64_t)tw * R + lead_s[c] / K];
             }
         }
-        // Per-slot state of the walk, all in registers: the cursor, and the entry under it decoded once per cursor
-        // position into exactly what a probe needs -- this slot's tier mask for the word it looks at, the addresses of
-        // that word in the expert's availability set and in the win-count set, and the arbitration key of the entry.
-        int cur = 0;                             // list entry (start of a group of equal scores) that may still hit
-        int pw = 0;                              // word the probe looks at
-        uint32_t e_pr = 0u;                      // the list word under the cursor
-        uint32_t e_mk = 0u;                      // tier mask for word pw; 0 for a group of tied entries (generic probe)
-        int e_wd = -1;                           // the tier's only word, or -1 if it spans several
-        const uint32_t* p_av = av;               // &avail[pw][col]
-        uint32_t* p_lv = lvl;                    // &lvl[pw][win count of the entry]
-        uint32_t keyb = 0u;                      // (list position, slot) packed for the arbiter
-        auto load_entry = [&]() {
-            if (cur >= a.nbid) { live = false; e_mk = 0u; return; }     // nothing left this slot could ever bid for
-            e_pr = bid_s[cur];
-            const int t = (int)(e_pr & 0xFFu), wl = (int)((e_pr >> 8) & 0xFFFFu);
-            e_wd = tw_word[t * S + s];
-            pw = e_wd >= 0 ? e_wd : 0;
-            e_mk = (e_pr & 0x80000000u) ? 0u : tw_mask[t * S + s];      // several words: the mask of word 0
-            p_av = av + pw * a.dmax;
-            p_lv = lvl + pw * LS + wl;
-            keyb = ((uint32_t)(a.nbid - cur) << 16) | (uint32_t)(0xFFFF - s);
-        };
-        if (live) load_entry();
-        // The rounds end when no slot can bid any more.  A count of the slots that still can, kept in shared memory,
-        // tells: it is only ever changed between the two barriers of a round and only read between the second barrier
-        // of one round and the first of the next, so every thread sees the same value and no round needs a barrier that
-        // also reduces a predicate (about 150 cycles more than a plain one after a shared-memory atomic).
-        if (tid == 0) { s_live3 = 0u; s_lastwin = 0u; }
+        const uint32_t* tm = a.tm_in_smem ? tm_s : a.tiermask;
+        const int tms = a.tm_in_smem ? S : R;
         __syncthreads();
-        if (live) atomicAdd(&s_live3, 1u);
+        for (int q = tid; q < a.ntiers * C; q += NT) {
+            const int t = q / C, c = q - t * C;
+            int nz = 0, wd = 0;
+            uint32_t val = 0u;
+            for (int w = 0; w < W; ++w) {
+                const uint32_t mk = tm[(t * W + w) * tms + (a.tm_in_smem ? c : lead_s[c] / K)];
+                if (mk) { ++nz; wd = w; val = mk; }
+            }
+            tw_word[t * S + c] = nz <= 1 ? wd : -1;
+            tw_mask[t * S + c] = val;
+        }
         __syncthreads();
-        uint32_t* const arb = reinterpret_cast<uint32_t*>(arb_r);     // [R] best bid per rank; the winner clears its entry
         long long limit = cap;
         if (a.auction_max_rounds > 0 && a.auction_max_rounds < limit) limit = a.auction_max_rounds;
-        const int round_limit = (int)(limit < 0x7fffffffLL ? limit : 0x7fffffffLL);
+        const uint32_t round_limit = (uint32_t)limit;                   // at most R * S + S < 2^19
         if (timed) c_p3loop = clock64();
-        const int NP = ((S + 31) >> 5) << 5;      // threads that take part in the rounds: the warps holding slots
-        const uint32_t a_arb = smem_u32(arb), a_avc = smem_u32(av);
-        const uint32_t a_live = smem_u32(&s_live3), a_lastwin = smem_u32(&s_lastwin);
-        // a slot that does not bid sends its key to a word of its own behind the R arbiters (the block holds 4R words):
-        // the bid is one instruction for every lane, whatever the slot's state
-        const uint32_t a_idle = a_arb + 4u * (uint32_t)(R + tid % (3 * R));
-        const uint32_t dmax4 = (uint32_t)a.dmax * 4u;
-        uint32_t a_av = smem_u32(p_av), a_lv = smem_u32(p_lv);       // the two words a probe reads
-        const bool nrem_smem = a.nrem_in_smem != 0;
-        int32_t* const nrem_col = nrem + col * R;                    // this slot's expert: what each rank still holds
-        const uint32_t a_cell0 = nrem_smem ? smem_u32(nrem_col) : 0u;
-        int32_t* const Xs = Xl + s;                                   // column s of the plan
-        bool dying = false;                       // the cursor ran off the list: leave the count after the next barrier
-        while (tid < NP && rounds3 < round_limit) {
-            const long long c_r0 = TIMED ? clock64() : 0;
-            // Step 1: bid for the source rank with the best bonus minus price.
-            // An entry whose score no other entry shares: while the cursor rests on it its candidate set (tier for this
-            // host AND holding the expert AND this win count) can only shrink -- a rank enters this win count from the
-            // one below, and the entry of the same tier with that lower count comes earlier in the list, so it was found
-            // empty for good before the cursor got here.  Words found empty therefore stay empty: the probe is one word
-            // (the tier's only word, or the word of the last hit), two loads and two ANDs, the same for every lane; a
-            // slot that is done keeps a zero mask.  Only a probe that comes back empty leaves this path.
-            const uint32_t nlive = lds_u32(a_live);
-            uint32_t hit = e_mk & lds_u32(a_av) & lds_u32(a_lv);
-            uint32_t a_sel = a_lv;               // win-count word of the rank bid for (the tied groups set their own)
-            int r_best = (pw << 5) + __ffs(hit) - 1;
-            bool bids = hit != 0u;
-            if (hit == 0u && live) {
-                uint32_t* p_sel = p_lv;
-                r_best = -1;
-                for (;;) {
-                    hit = e_mk & *p_av & *p_lv;
-                    if (hit) { r_best = (pw << 5) + __ffs(hit) - 1; p_sel = p_lv; break; }
-                    if (!(e_pr & 0x80000000u)) { // an empty word: the tier's next word, or the next entry
-                        if (e_wd < 0 && pw + 1 < W) {
-                            ++pw;
-                            e_mk = tm[((int)(e_pr & 0xFFu) * W + pw) * tms];
-                            p_av += a.dmax;
-                            p_lv += LS;
-                        } else {
-                            ++cur;
-                            load_entry();
-                        }
-                    } else {
-                        // a group of entries with one and the same fp32 score: probe every entry, the lowest rank wins
-                        int g = cur;
-                        uint32_t pr;
-                        do {
-                            pr = bid_s[g++];
-                            const int t = (int)(pr & 0xFFu), wl = (int)((pr >> 8) & 0xFFFFu);
-                            const int wd = tw_word[t * S + s];
-                            int r;
-                            if (wd >= 0) {
-                                const uint32_t h1 = tw_mask[t * S + s] & av[wd * a.dmax] & lvl[wd * LS + wl];
-                                r = h1 ? (wd << 5) + __ffs(h1) - 1 : -1;
-                            } else {
-                                uint32_t cand[kMaxW];
-#pragma unroll
-                                for (int w = 0; w < kMaxW; ++w) cand[w] = (w < W) ? (tm[(t * W + w) * tms] & av[w * a.dmax]) : 0u;
-                                r = first_hit(cand, lvl + wl, LS, W);
-                            }
-                            if (r >= 0 && (r_best < 0 || r < r_best)) { r_best = r; p_sel = lvl + (r >> 5) * LS + wl; }
-                        } while (pr & 0x80000000u);
-                        if (r_best >= 0) break;
-                        cur = g;                 // the whole group is empty for good
-                        load_entry();
-                    }
-                    if (!live) break;
+        const au::Tables tab{arb, avail, lvl, bid_s, ent_s, tm, tw_word, tw_mask, slot_e, slot_a, nxt_s, dcol, nrem, Xl,
+                             R, S, K, W, a.dmax, a.ntiers, tms, au::smem_u32(idle_s + lane),
+                             reinterpret_cast<int32_t*>(a.t12 + l * (int64_t)E * 2 * R)};       // (Phase 2's scratch)
+        const int NP = ((C + 31) >> 5) << 5;
+        auto run = [&](auto bidder) {
+            using B = decltype(bidder);
+            uint32_t rd = 1u;
+            if (C > 32) {
+                if (tid < NP) {
+                    B b(tab);
+                    if (tid < C) b.start(tid, lead_s[tid]);
+                    __syncwarp();
+                    rd = au::run_block(b, NP, C, round_limit, &ctl);
                 }
-                a_av = smem_u32(p_av);
-                a_lv = smem_u32(p_lv);
-                a_sel = smem_u32(p_sel);
-                bids = r_best >= 0;
-                dying = !live;
+                __syncthreads();
             }
-            // Step 2: the rank keeps its best bidder (ties: lowest slot).  The position of a score in the list orders
-            // scores exactly as their fp32 values do, so (list position, slot) packs into one 32-bit key and a single
-            // native shared-memory max arbitrates: smaller position = higher score, then the lower slot.
-            const uint32_t a_mine = bids ? a_arb + ((uint32_t)r_best << 2) : a_idle;
-            const long long c_rp = TIMED ? clock64() : 0;
-            red_max_u32(a_mine, keyb);
-            if (TIMED) { const long long c_ra = clock64(); c_probe += c_rp - c_r0; c_atom += c_ra - c_rp; }
-            bar_part(NP);
-            const long long c_r1 = TIMED ? clock64() : 0;
-            // Steps 3-4: the winning slot of each rank collects x = min(n, A); holdings, plan and price follow.  The
-            // rank bid for holds tokens of the expert (its availability bit was set) and the slot still wants some, so
-            // x > 0 and the rank's win count goes from the entry's to the next: its bit moves one word up in lvl.
-            const bool won = (lds_u32(a_mine) == keyb) & bids;
-            if (dying) { red_add_u32(a_live, 0xFFFFFFFFu); dying = false; }
-            if (won) {
-                const uint32_t bit = 1u << (r_best & 31);
-                red_and_u32(a_sel, ~bit);
-                red_or_u32(a_sel + 4u, bit);
-                sts_u32(a_mine, 0u);             // losers of this round compare against their own key: 0 is nobody's
-                sts_u32(a_lastwin, (uint32_t)rounds3 + 1u);
-                int32_t have;
-                if (nrem_smem) have = (int32_t)lds_u32(a_cell0 + ((uint32_t)r_best << 2));
-                else have = nrem_col[r_best];
-                const int32_t x = have < A ? have : A;
-                if (nrem_smem) sts_u32(a_cell0 + ((uint32_t)r_best << 2), (uint32_t)(have - x));
-                else nrem_col[r_best] = have - x;
-                A -= x;
-                if (have == x) red_and_u32(a_avc + (uint32_t)(r_best >> 5) * dmax4, ~bit);
-                if (A <= 0) { live = false; e_mk = 0u; red_add_u32(a_live, 0xFFFFFFFFu); }
-                Xs[(int64_t)r_best * S] = x;     // a (rank, slot) pair is served at most once
+            if (timed) { c_p3warp = clock64(); c_classes = C; c_handed = (long long)rd; }
+            if (warp == 0) {
+                B b(tab);
+                if (C > 32) {
+                    if (lane < (int)ctl.handed) b.start((int)(ctl.hand[lane] >> 16), (int)(ctl.hand[lane] & 0xFFFFu));
+                } else if (lane < C) {
+                    b.start(lane, lead_s[lane]);
+                }
+                __syncwarp();
+                const uint32_t last = au::run_warp(b, rd, round_limit, ctl.last);
+                __syncwarp();
+                if (lane == 0) ctl.last = last;
             }
-            // nobody was left before this round (the same answer in every thread): one more round, empty, ends the loop
-            rounds3 = nlive ? rounds3 + 1 : round_limit;
-            bar_part(NP);
-            if (TIMED && timed) { const long long c_r2 = clock64(); c_bid += c_r1 - c_r0; c_upd += c_r2 - c_r1; }
-        }
+        };
+        if constexpr (!LEAN) run(au::Bidder<TAOT_MAX_TIERS, true, false, kMaxW>(tab));
+        else if (W <= 2) run(au::Bidder<4, false, NSM, 2>(tab));
+        else run(au::Bidder<4, false, NSM, kMaxW>(tab));
         if (timed) c_p3end = clock64();
-        if (s < S) slot_a[s] = A;
         __syncthreads();
-        rounds3 = (int)s_lastwin;                 // rounds in which somebody bid
+        rounds3 = (int)ctl.last;                  // rounds in which somebody bid
     } else {
         for (;;) {
             if (a.auction_max_rounds > 0 && rounds3 >= a.auction_max_rounds) break;
@@ -738,27 +596,14 @@ match_kernel(MatchArgs a)
         if (slot_e[s] >= 0 && slot_a[s] > 0) residual = 1;
     }
     residual = __syncthreads_or(residual);
-    if (TIMED) {                                  // the busiest thread's own probe and arbitration time
-        __shared__ unsigned long long s_mx[2];
-        if (tid == 0) { s_mx[0] = 0; s_mx[1] = 0; }
-        __syncthreads();
-        unsigned long long mp = (unsigned long long)c_probe, ma = (unsigned long long)c_atom;
-        for (int o = 16; o > 0; o >>= 1) {        // one atomic per warp: 64-bit shared-memory atomics from every thread
-            const unsigned long long op = __shfl_xor_sync(0xffffffffu, mp, o), oa = __shfl_xor_sync(0xffffffffu, ma, o);
-            mp = op > mp ? op : mp;               // would cost more than the rounds they report on
-            ma = oa > ma ? oa : ma;
-        }
-        if ((tid & 31) == 0) { atomicMax(&s_mx[0], mp); atomicMax(&s_mx[1], ma); }
-        __syncthreads();
-        c_probe = (long long)s_mx[0]; c_atom = (long long)s_mx[1];
-    }
     if (tid == 0) {
         if (a.rounds) { a.rounds[l * 2] = rounds2; a.rounds[l * 2 + 1] = rounds3; }
         if (residual) atomicOr(a.info + l, TAOT_INFO_AUCTION_RESIDUAL);
         if (timed) {
             long long* c = a.cyc + l * 16;
-            c[0] = c_p2 - c_start; c[1] = c_p3 - c_p2; c[2] = c_p3loop - c_p3; c[3] = c_bid; c[4] = c_upd;
-            c[5] = clock64() - c_start; c[6] = c_probe; c[7] = c_atom;
+            c[0] = c_p2 - c_start; c[1] = c_p3 - c_p2; c[2] = c_p3loop - c_p3;
+            c[3] = c_p3warp - c_p3loop; c[4] = c_p3end - c_p3warp;
+            c[5] = clock64() - c_start; c[6] = c_classes; c[7] = c_handed;
             c[8] = c_scan; c[9] = c_win; c[10] = c_row; c[11] = c_build;
             c[12] = c_p3end - c_p3loop;
             for (int i = 13; i < 16; ++i) c[i] = 0;
@@ -786,6 +631,7 @@ int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expe
     a.n = d_n; a.expert_load = d_expert_load; a.rank_load = d_rank_load; a.plan = d_plan;
     a.e2r = h->d_e2r; a.B = h->d_B; a.rank_off = h->d_rank_off; a.rank_list = h->d_rank_list;
     a.tiermask = h->d_tiermask; a.tierval = h->d_tierval; a.bidlist = h->d_bidlist;
+    a.bident = h->d_bident; a.hostcls = h->d_hostcls;
     a.slot_expert = d_slot_expert; a.slot_tokens = d_slot_tokens; a.X = d_X; a.rounds = d_rounds;
     a.info = d_info; a.nrem_g = d_nrem; a.t12 = d_t12;
     a.R = p.R; a.E = p.E; a.K = p.K;
@@ -796,7 +642,9 @@ int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expe
     a.eps0 = p.eps0; a.price_step = p.price_step; a.auction_max_rounds = p.auction_max_rounds;
     a.ablation = p.ablation;
     size_t smem = match_smem_fixed(p.R, p.E, p.K, a.dmax, a.W, a.ntiers);
-    if (a.nbid > 0) smem += sizeof(uint32_t) * ((size_t)a.nbid + 2 * (size_t)a.ntiers * p.R * p.K);
+    const size_t lists = sizeof(uint32_t) * (2 * (size_t)h->nbid + 2 * (size_t)h->ntiers * p.R * p.K + 2 * (size_t)p.R * p.K);
+    if (a.nbid > 0 && smem + lists > kSmemBudget) { a.nbid = 0; a.ntiers = 0; }      // (no room for the lists: the dense scan)
+    if (a.nbid > 0) smem += lists;
     const size_t nrem_bytes = sizeof(int32_t) * (size_t)a.dmax * p.R;
     const size_t tm_bytes = sizeof(uint32_t) * (size_t)a.ntiers * a.W * p.R * p.K;
     a.tm_in_smem = (a.ntiers > 0 && smem + tm_bytes <= 96 * 1024) ? 1 : 0;
@@ -812,15 +660,25 @@ int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expe
     a.big_floats = (int32_t)(big / 4);
     smem += big;
     if (smem > 227 * 1024) return TAOT_ERR_UNSUPPORTED;
-    TAOT_CUDA_OK(cudaFuncSetAttribute(match_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    if (d_cyc) TAOT_CUDA_OK(cudaFuncSetAttribute(match_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    int need = p.R * p.K > p.R ? p.R * p.K : p.R;
-    // two threads per slot (or rank): Phase 2 splits each rank's scan over more lanes, and the extra warps cost the
-    // auction's barriers less than that saves (measured: 256 threads for 16 and 64 ranks, 512 for 256 ranks x 1 slot)
+    const int need = p.R * p.K;
+    // two threads per slot: Phase 2 splits each rank's scan over more lanes, and the extra warps cost less than that saves
+    // (measured: 256 threads for 16 and 64 ranks, 512 for 256 ranks x 1 slot); more than 512 only if there are more slots,
+    // since the registers of the auction's builds are cut in half there
     int NT = 2 * (((need + 31) / 32) * 32);
-    NT = NT < 256 ? 256 : (NT > 1024 ? 1024 : NT);
-    if (d_cyc) match_kernel<true><<<p.L, NT, smem, st>>>(a);
-    else match_kernel<false><<<p.L, NT, smem, st>>>(a);
-    TAOT_CUDA_OK(cudaGetLastError());
-    return 1;
+    NT = NT < 256 ? 256 : (NT > 512 && need <= 512 ? 512 : (NT > 1024 ? 1024 : NT));
+    auto launch = [&](auto kernel) -> int {
+        TAOT_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        kernel<<<p.L, NT, smem, st>>>(a);
+        TAOT_CUDA_OK(cudaGetLastError());
+        return 1;
+    };
+    const bool lean = a.nbid > 0 && a.ntiers <= 4 && !h->bid_ties, nsm = a.nrem_in_smem != 0;
+    auto build = [&](auto timed, auto maxt) -> int {
+        constexpr bool TIMED = decltype(timed)::value;
+        constexpr int MAXT = decltype(maxt)::value;
+        if (!lean) return launch(match_kernel<TIMED, MAXT, false, false>);
+        return nsm ? launch(match_kernel<TIMED, MAXT, true, true>) : launch(match_kernel<TIMED, MAXT, true, false>);
+    };
+    if (d_cyc) return build(std::true_type{}, std::integral_constant<int, 1024>{});
+    return NT <= 512 ? build(std::false_type{}, std::integral_constant<int, 512>{}) : build(std::false_type{}, std::integral_constant<int, 1024>{});
 }

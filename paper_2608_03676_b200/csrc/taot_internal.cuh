@@ -37,6 +37,9 @@ struct taot_handle_s {
     float* d_tierval;        // [ntiers] distinct values of the auction bonus matrix, descending
     int32_t ntiers;          // 0: too many distinct values, the auction scans densely
     uint32_t* d_bidlist;     // [nbid] every (tier, win count) pair, best score first: w << 8 | t, bit 31 = next has the same score
+    uint32_t* d_bident;      // [ntiers][S+1] the same by pair: position << 16 | tie << 14 | tiers that score higher << 11 | w
+    int32_t* d_hostcls;      // [R] hosts that see every rank at the same bonus share a number
+    int32_t bid_ties;        // some pairs have equal scores
     int32_t nbid;            // 0: no list (no tiers, or price step <= 0): the auction scans densely
     int32_t* d_merge_part;   // [L][TAOT_MERGE_PARTS][E] expert loads of the parts of a layer's merge, or null (one CTA per layer)
     int32_t* d_merge_cnt;    // [L] parts of a layer's merge that are done; zero between calls

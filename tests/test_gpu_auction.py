@@ -1,0 +1,39 @@
+"""Phase 3 on classes of slots: one warp and several, the hand-over between them, word edges of the rank sets, remaining counts
+in and out of shared memory, and pairs of equal score, against the oracle."""
+import pytest
+
+import oracle as O
+import workloads as W
+from helpers import cpu, make_planner, oracle_schedule_layer, topology
+
+pytestmark = pytest.mark.gpu
+
+BASE = W.get_config("cfg3").replace(L=2, max_iters=60, tol=0.0)
+SHAPES = {
+    "one_word": BASE.replace(R=32, E=128, T=32 * 512),
+    "two_words_first_rank_of_the_second": BASE.replace(R=33, E=99, T=33 * 512),
+    "three_words": BASE.replace(R=72, E=144, K=3, T=72 * 300),
+    "many_classes": BASE.replace(R=120, E=480, K=3, T=120 * 700, gpus_per_node=4),       # more than 128 classes
+    "counts_in_global_memory": BASE.replace(R=200, E=400, K=2, T=200 * 400),
+    "eight_words_four_tiers": BASE.replace(R=256, E=256, K=2, T=256 * 300, tiers=(0.0, 1.0, 3.0, 9.0), nodes_per_group=4),
+    "equal_scores": BASE.replace(R=48, E=192, K=2, T=48 * 600, tiers=(0.0, 1.0, 2.0)),   # bonus 1 and 0.5, step 0.125
+}
+
+
+@pytest.mark.parametrize("name", sorted(SHAPES))
+@pytest.mark.parametrize("step,cap", [(0.1, 0), (0.125, 0), (0.1, 17), (1e-9, 0)])
+def test_auction_bit_exact(name, step, cap):
+    cfg = SHAPES[name]
+    e2r, C = topology(cfg)
+    topk = W.routing_topk(cfg, device="cuda")
+    pl = make_planner(cfg, price_step=step, auction_max_rounds=cap)
+    out = {k: cpu(v) for k, v in pl.plan(topk).items()}
+    B = O.default_preference(C.numpy())
+    for l in range(cfg.L):
+        m, a = oracle_schedule_layer(cfg, e2r.numpy(), B, out["n"][l], out["expert_load"][l], out["rank_load"][l], out["plan"][l],
+                                     price_step=step, auction_max_rounds=cap)
+        assert (out["slot_expert"][l].ravel() == m["slot_expert"]).all()
+        assert (out["X"][l] == a["X"]).all()
+        assert out["rounds"][l].tolist() == [m["inner_rounds"], a["rounds"]]
+        assert bool(out["info"][l] & 8) == (a["residual"] > 0)
+    pl.close()
