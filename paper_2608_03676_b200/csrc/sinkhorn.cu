@@ -336,6 +336,7 @@ __global__ void __launch_bounds__(1024) sinkhorn_kernel(SinkArgs a)
 int taot_launch_sinkhorn_tile(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st);
 int taot_launch_sinkhorn_cluster(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st);
 int taot_launch_sinkhorn_tiered(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st);
+int taot_launch_sinkhorn_wide(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st);
 int taot_launch_sinkhorn_class(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st);
 int taot_launch_sinkhorn_dense_tc(taot_handle_t h, const SinkArgs& a, int32_t B, float* ws_tc, cudaStream_t st);
 
@@ -375,6 +376,8 @@ int taot_launch_sinkhorn_guard(taot_handle_t h, const float* d_s, const float* d
 // batch with a fixed iteration count (R > 32: below, the register tiles are as fast).  Inside taot_plan, and in tolerance mode,
 // Phase 1 stays on the tile and tier-sum kernels: the placement that follows decides exact ties (experts of one node's
 // ranks on one cold rank) by the last bits of the hint, so its kernel is part of the result.
+constexpr int kWideMinIters = 64;     // see taot_launch_sinkhorn_wide
+
 bool taot_sinkhorn_takes_classes(taot_handle_t h, bool from_loads)
 {
     const taot_params& p = h->p;
@@ -420,17 +423,24 @@ int taot_launch_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, in
             if (n < 0) return n;
             launched += n;
         } else {
-            // beyond 256 ranks, a large batch with a fixed iteration count and a Gibbs kernel inside fp32: the whole
-            // batch as dense products on the tensor cores (complete: nothing is handed on)
-            const int ntc = taot_launch_sinkhorn_dense_tc(h, a, nb, d_tc, st);
-            if (ntc < 0) return ntc;
-            if (ntc > 0) { launched += ntc; continue; }
-            // otherwise four-CTA clusters hold the kernel matrix in distributed shared memory; what they hand
-            // back (or everything, if no slice fits) goes to the kernel below with the matrix in workspace
+            // beyond 256 ranks.  A large batch with a short fixed count and a Gibbs kernel inside fp32 (or more than 512
+            // ranks): the whole batch as dense products on the tensor cores (complete: nothing is handed on)
+            if (p.R > 512 || p.max_iters < kWideMinIters) {
+                const int ntc = taot_launch_sinkhorn_dense_tc(h, a, nb, d_tc, st);
+                if (ntc < 0) return ntc;
+                if (ntc > 0) { launched += ntc; continue; }
+            }
+            // otherwise up to 512 ranks one CTA holds the compacted matrix in registers; what it hands back, and larger
+            // problems, go to four-CTA clusters that hold it in distributed shared memory; what those hand back (or
+            // everything, if no slice fits) to the kernel below with the matrix in workspace
+            a.skip_solved = 0;
+            const int nw = taot_launch_sinkhorn_wide(h, a, nb, st);
+            if (nw < 0) return nw;
+            a.skip_solved = nw;
             const int n = taot_launch_sinkhorn_cluster(h, a, nb, st);
             if (n < 0) return n;
-            launched += n;
-            a.only_marked = n > 0 ? 1 : 0;
+            launched += nw + n;
+            a.only_marked = nw + n > 0 ? 1 : 0;
         }
         sinkhorn_kernel<<<nb, NT, smem, st>>>(a);
         TAOT_CUDA_OK(cudaGetLastError());

@@ -109,6 +109,9 @@ sinkhorn_cluster_kernel(SinkArgs a, int32_t kcap)
     const int64_t b = blockIdx.x / kCluster;
     __shared__ double s_sum[2];
     const int XS = R + kXTail;                               // floats per exchange buffer
+    // chained launch: only what an earlier kernel left (a problem left over has supply and demand, so none of the four
+    // CTAs writes iters[b] before all of them have met at the barrier below, or writes the mark that is there)
+    if (a.skip_solved && a.iters[b] != kHandBack) return;
 
     // ---- supply scaling gamma = min(1, sum d / max(sum s, eps0)), compaction (every CTA, identically)
     {
