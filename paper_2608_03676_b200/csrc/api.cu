@@ -75,7 +75,7 @@ void layout(taot_handle_t h)
     h->off_tc = take((p.R > 256 && p.R % 128 == 0) ? sizeof(float) * taot_sinkhorn_tc_ws_floats(p.R, p.L) : 0);
     h->tb_ok = (path && p.E <= 256 && h->seg % 16 == 0) ? 1 : 0;
     h->off_tb = take(h->tb_ok ? (size_t)p.L * (size_t)p.T * p.k : 0);
-    h->off_tbflag = take(h->tb_ok ? sizeof(int32_t) * LR * h->nc : 0);
+    h->off_tbflag = take(path * sizeof(int32_t) * LR * h->nc);
     h->ws_bytes = off;
 
     const size_t S = (size_t)p.R * p.K;
@@ -712,7 +712,6 @@ int plan_stages(taot_handle_t h, const int32_t* d_topk, const taot_outputs* o, v
     int32_t* spare = o->spare ? o->spare : reinterpret_cast<int32_t*>(at(ws, h->off_spare));
     float* fs = reinterpret_cast<float*>(at(ws, h->off_s));
     float* fd = reinterpret_cast<float*>(at(ws, h->off_d));
-    TAOT_CUDA_OK(cudaMemsetAsync(o->info, 0, sizeof(int32_t) * p.L, st));
     int total = 0, a;
 #define TAOT_MARK(i) if (marks) TAOT_CUDA_OK(cudaEventRecord(h->ev[i], st))
     // NVTX ranges around the enqueue of each stage (header-only NVTX: free unless a profiler is attached)
@@ -724,14 +723,15 @@ int plan_stages(taot_handle_t h, const int32_t* d_topk, const taot_outputs* o, v
     if (hist_after) TAOT_CUDA_OK(cudaStreamWaitEvent(st, hist_after, 0));
     {
         Range r("taot:histogram");
-        if ((a = taot_launch_histogram(h, d_topk, cc, o->info, st, ws, !bytes_later)) < 0) return a;
+        if ((a = taot_launch_histogram(h, d_topk, cc, nullptr, st, ws, !bytes_later)) < 0) return a;
     }
     total += a;
     if (hist_done) TAOT_CUDA_OK(cudaEventRecord(hist_done, st));
     TAOT_MARK(1);
     {
         Range r("taot:merge+excess_spare");
-        if ((a = taot_launch_merge(h, cc, o->n, o->expert_load, o->rank_load, excess, spare, fs, fd, st)) < 0) return a;
+        if ((a = taot_launch_merge(h, cc, o->n, o->expert_load, o->rank_load, excess, spare, fs, fd, st, nullptr,
+                                   reinterpret_cast<const int32_t*>(at(ws, h->off_tbflag)), o->info)) < 0) return a;
     }
     total += a;
     TAOT_MARK(2);
@@ -869,7 +869,7 @@ int taot_plan(taot_handle_t h, const int32_t* d_topk, const taot_outputs* o, voi
 }
 
 // H2D copy of the routing table, the whole path on device staging buffers; `d` receives the device pointers
-static int plan_on_staging(taot_handle_t h, const int32_t* h_topk, void* d_ws, void* stream, taot_outputs* d)
+static int plan_on_staging(taot_handle_t h, const int32_t* h_topk, int32_t* h_new, void* d_ws, void* stream, taot_outputs* d)
 {
     const taot_params& p = h->p;
     if (p.R > 256) return TAOT_ERR_UNSUPPORTED;      // what taot_plan would refuse is refused before the copy is queued
@@ -890,8 +890,13 @@ static int plan_on_staging(taot_handle_t h, const int32_t* h_topk, void* d_ws, v
     d->new_idx = reinterpret_cast<int32_t*>(at(d_ws, h->hoff_new));
     d->info = reinterpret_cast<int32_t*>(at(d_ws, h->hoff_info));
     int32_t* d_topk = reinterpret_cast<int32_t*>(at(d_ws, h->hoff_topk));
-    TAOT_CUDA_OK(cudaMemcpyAsync(d_topk, h_topk, sizeof(int32_t) * NE, cudaMemcpyHostToDevice, st));
-    return taot_plan(h, d_topk, d, at(d_ws, h->hoff_ws), stream);
+    {
+        TAOT_CUDA_OK(cudaMemcpyAsync(d_topk, h_topk, sizeof(int32_t) * NE, cudaMemcpyHostToDevice, st));
+        const int rc = taot_plan(h, d_topk, d, at(d_ws, h->hoff_ws), stream);
+        if (rc != TAOT_OK || !h_new) return rc;
+        TAOT_CUDA_OK(cudaMemcpyAsync(h_new, d->new_idx, sizeof(int32_t) * NE, cudaMemcpyDeviceToHost, st));
+        return TAOT_OK;
+    }
 }
 
 int taot_plan_host(taot_handle_t h, const int32_t* h_topk, const taot_outputs* o, void* d_ws, void* stream)
@@ -900,9 +905,9 @@ int taot_plan_host(taot_handle_t h, const int32_t* h_topk, const taot_outputs* o
     if (reinterpret_cast<uintptr_t>(d_ws) & 255) return TAOT_ERR_ALIGN;
     const taot_params& p = h->p;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const size_t LR = (size_t)p.L * p.R, S = (size_t)p.R * p.K, NE = (size_t)p.L * p.T * p.k;
+    const size_t LR = (size_t)p.L * p.R, S = (size_t)p.R * p.K;
     taot_outputs d;
-    const int rc = plan_on_staging(h, h_topk, d_ws, stream, &d);
+    const int rc = plan_on_staging(h, h_topk, o->new_idx, d_ws, stream, &d);
     if (rc != TAOT_OK) return rc;
 #define TAOT_BACK(member, count, type)                                                                       \
     if (o->member)                                                                                           \
@@ -919,7 +924,6 @@ int taot_plan_host(taot_handle_t h, const int32_t* h_topk, const taot_outputs* o
     TAOT_BACK(slot_tokens, p.L * S, int32_t);
     TAOT_BACK(X, LR * S, int32_t);
     TAOT_BACK(rounds, (size_t)p.L * 2, int32_t);
-    TAOT_BACK(new_idx, NE, int32_t);
     TAOT_BACK(info, (size_t)p.L, int32_t);
 #undef TAOT_BACK
     return TAOT_OK;
@@ -943,13 +947,11 @@ int taot_plan_host_block(taot_handle_t h, const int32_t* h_topk, int32_t* h_new_
     if (reinterpret_cast<uintptr_t>(d_ws) & 255) return TAOT_ERR_ALIGN;
     const taot_params& p = h->p;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    const size_t NE = (size_t)p.L * p.T * p.k;
     taot_outputs d;
-    const int rc = plan_on_staging(h, h_topk, d_ws, stream, &d);
+    const int rc = plan_on_staging(h, h_topk, h_new_idx, d_ws, stream, &d);
     if (rc != TAOT_OK) return rc;
     // the staging buffers of all outputs but the routing table are one contiguous range: one copy
     TAOT_CUDA_OK(cudaMemcpyAsync(h_block, at(d_ws, h->hoff_n), h->hoff_ws - h->hoff_n, cudaMemcpyDeviceToHost, st));
-    TAOT_CUDA_OK(cudaMemcpyAsync(h_new_idx, d.new_idx, sizeof(int32_t) * NE, cudaMemcpyDeviceToHost, st));
     return TAOT_OK;
 }
 

@@ -391,6 +391,7 @@ assign_chunk_kernel(AssignArgs a)
     const int c = (int)(id % a.nc);
     int64_t goff; int32_t len;
     chunk_geometry(a, id, goff, len);
+    taot_await();
     const void* buf = a.topk + goff;
     if (STAGE) {
         if (tid == 0) {
@@ -467,15 +468,15 @@ int taot_launch_assign(taot_handle_t h, const int32_t* d_topk, void* ws, const i
         a.tbflag = reinterpret_cast<const int32_t*>(w + h->off_tbflag);
         const size_t smem = (size_t)TAOT_CHUNK + sizeof(int32_t) * words;
         TAOT_CUDA_OK(cudaFuncSetAttribute(assign_chunk_kernel<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        assign_chunk_kernel<true, true, true><<<blocks, kThreads, smem, st>>>(a);
+        TAOT_CUDA_OK(taot_launch_chained(assign_chunk_kernel<true, true, true>, blocks, kThreads, smem, st, a));
     } else if (vec_ok) {
         const size_t smem = (size_t)TAOT_CHUNK * 4 + sizeof(int32_t) * words;
         TAOT_CUDA_OK(cudaFuncSetAttribute(assign_chunk_kernel<true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        assign_chunk_kernel<true, true, false><<<blocks, kThreads, smem, st>>>(a);
+        TAOT_CUDA_OK(taot_launch_chained(assign_chunk_kernel<true, true, false>, blocks, kThreads, smem, st, a));
     } else {
         const size_t smem = sizeof(int32_t) * words;
         TAOT_CUDA_OK(cudaFuncSetAttribute(assign_chunk_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        assign_chunk_kernel<false, false, false><<<blocks, kThreads, smem, st>>>(a);
+        TAOT_CUDA_OK(taot_launch_chained(assign_chunk_kernel<false, false, false>, blocks, kThreads, smem, st, a));
     }
     TAOT_CUDA_OK(cudaGetLastError());
     return 1;

@@ -59,6 +59,8 @@ dispatch_offsets_kernel(DispatchArgs a)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t lr = blockIdx.x;
     int32_t* dc = a.dc + lr * NC * (int64_t)NB;
+    taot_await();
+    taot_release();
     for (int r = tid; r <= R; r += kThreads) sc[r] = 0;
     for (int b = tid; b < NB; b += kThreads) {
         int32_t t = 0;
@@ -118,6 +120,7 @@ dispatch_scatter_kernel(DispatchArgs a)
     int32_t* dst = a.perm + goff;
     for (int q = tid; q < (ALT ? 3 : 2) * kWarps * NB; q += kThreads) wh[q] = 0;
     __syncthreads();
+    taot_await();
     const int s0 = warp * kWarpSpan, s1 = min(len, s0 + kWarpSpan);
     int32_t* mine = wh + warp * NB;
     unsigned* mask = reinterpret_cast<unsigned*>(wh + (kWarps + warp) * NB);
@@ -195,10 +198,8 @@ int taot_launch_dispatch(taot_handle_t h, const int32_t* d_new_idx, int32_t* d_s
     else TAOT_CUDA_OK(cudaFuncSetAttribute(dispatch_scatter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3));
     const int rc = taot_launch_chunk_counts(h, d_new_idx, a.dc, d_info, a.NB - 1, st);
     if (rc < 0) return rc;
-    dispatch_offsets_kernel<<<(unsigned)((int64_t)p.L * p.R), kThreads, sm2, st>>>(a);
-    TAOT_CUDA_OK(cudaGetLastError());
-    if (alt) dispatch_scatter_kernel<true><<<chunks, kThreads, sm3, st>>>(a);
-    else dispatch_scatter_kernel<false><<<chunks, kThreads, sm3, st>>>(a);
-    TAOT_CUDA_OK(cudaGetLastError());
+    TAOT_CUDA_OK(taot_launch_chained(dispatch_offsets_kernel, (unsigned)((int64_t)p.L * p.R), kThreads, sm2, st, a));
+    if (alt) TAOT_CUDA_OK(taot_launch_chained(dispatch_scatter_kernel<true>, chunks, kThreads, sm3, st, a));
+    else TAOT_CUDA_OK(taot_launch_chained(dispatch_scatter_kernel<false>, chunks, kThreads, sm3, st, a));
     return 3;
 }

@@ -66,6 +66,8 @@ hist_chunk_kernel(const int32_t* __restrict__ topk, int32_t* __restrict__ cc, in
 
     for (int i = tid; i < kWarps * nb; i += kThreads) sh_hist[i] = 0;
     __syncthreads();
+    taot_await();
+    taot_release();
     int32_t* hist = sh_hist + warp * nb;
     int bad = 0;
 
@@ -106,7 +108,7 @@ hist_chunk_kernel(const int32_t* __restrict__ topk, int32_t* __restrict__ cc, in
         for (int w = 0; w < kWarps; ++w) tot += sh_hist[w * nb + e];
         out[e] = tot;
     }
-    if (any_bad && tid == 0) atomicOr(info + l, TAOT_INFO_BAD_INDEX);
+    if (info && any_bad && tid == 0) atomicOr(info + l, TAOT_INFO_BAD_INDEX);
     if (!EXTRA && tbflag && tid == 0) tbflag[id] = any_bad;
 }
 
@@ -141,7 +143,7 @@ __global__ void __launch_bounds__(1024)
 merge_kernel(const int32_t* __restrict__ cc, const int32_t* __restrict__ e2r, int32_t* __restrict__ n,
              int32_t* __restrict__ expert_load, int32_t* __restrict__ rank_load, int32_t* excess,
              int32_t* spare, float* fs, float* fd, int32_t R, int32_t E, int32_t nc, int32_t* info,
-             int32_t parts, int32_t* part_el, int32_t* part_cnt)
+             int32_t parts, int32_t* part_el, int32_t* part_cnt, const int32_t* __restrict__ chunk_bad, int32_t* info_out)
 {
     extern __shared__ int32_t sh[];                      // el[E], rl[R]
     __shared__ long long s_tot;
@@ -151,6 +153,8 @@ merge_kernel(const int32_t* __restrict__ cc, const int32_t* __restrict__ e2r, in
     const int l = blockIdx.x / parts, part = blockIdx.x - l * parts, tid = threadIdx.x;
     for (int i = tid; i < E + R; i += blockDim.x) sh[i] = 0;
     __syncthreads();
+    taot_await();
+    taot_release();
     const int32_t RE = R * E;                            // at most 256 x 1024
     const int32_t* ccl = cc + (int64_t)l * RE * nc;
     int32_t* nl = n + (int64_t)l * RE;
@@ -183,6 +187,12 @@ merge_kernel(const int32_t* __restrict__ cc, const int32_t* __restrict__ e2r, in
         }
         if (tid == 0) part_cnt[l] = 0;                   // as the next call expects it
         __syncthreads();
+    }
+    if (info_out) {
+        int bad = 0;
+        for (int q = tid; q < R * nc; q += blockDim.x) bad |= chunk_bad[(int64_t)l * R * nc + q];
+        bad = __syncthreads_or(bad);
+        if (tid == 0) info_out[l] = bad ? TAOT_INFO_BAD_INDEX : 0;
     }
     for (int e = tid; e < E; e += blockDim.x) {
         const int32_t v = s_el[e];
@@ -267,10 +277,9 @@ int taot_launch_histogram(taot_handle_t h, const int32_t* d_topk, int32_t* d_cc,
     // with a workspace (and 16-byte accesses) the pass also leaves the table as one byte per entry for the reassignment
     const bool bytes = ws && h->tb_ok && vec_ok;
     uint8_t* tb = (bytes && write_bytes) ? reinterpret_cast<uint8_t*>(static_cast<char*>(ws) + h->off_tb) : nullptr;
-    int32_t* tbflag = bytes ? reinterpret_cast<int32_t*>(static_cast<char*>(ws) + h->off_tbflag) : nullptr;
-    hist_chunk_kernel<false><<<(unsigned)blocks, kThreads, smem, st>>>(d_topk, d_cc, d_info, layer_elems, h->seg,
-                                                                        h->nc, p.R, p.E, vec_ok, tb, tbflag);
-    TAOT_CUDA_OK(cudaGetLastError());
+    int32_t* tbflag = ws ? reinterpret_cast<int32_t*>(static_cast<char*>(ws) + h->off_tbflag) : nullptr;
+    TAOT_CUDA_OK(taot_launch_chained(hist_chunk_kernel<false>, (unsigned)blocks, kThreads, smem, st, d_topk, d_cc, d_info, layer_elems,
+                                     h->seg, h->nc, p.R, p.E, vec_ok, tb, tbflag));
     return 1;
 }
 
@@ -286,23 +295,21 @@ int taot_launch_chunk_counts(taot_handle_t h, const int32_t* d_idx, int32_t* d_c
     // the default limit is 48 KB
     if (smem > 48 * 1024)
         TAOT_CUDA_OK(cudaFuncSetAttribute(hist_chunk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    hist_chunk_kernel<true><<<(unsigned)blocks, kThreads, smem, st>>>(d_idx, d_counts, d_info, p.T * p.k, h->seg, h->nc,
-                                                                       p.R, bins, vec_ok, nullptr, nullptr);
-    TAOT_CUDA_OK(cudaGetLastError());
+    TAOT_CUDA_OK(taot_launch_chained(hist_chunk_kernel<true>, (unsigned)blocks, kThreads, smem, st, d_idx, d_counts, d_info,
+                                     (int64_t)p.T * p.k, h->seg, h->nc, p.R, bins, vec_ok, nullptr, nullptr));
     return 1;
 }
 
 int taot_launch_merge(taot_handle_t h, const int32_t* d_cc, int32_t* d_n, int32_t* d_expert_load,
                       int32_t* d_rank_load, int32_t* d_excess, int32_t* d_spare, float* d_s, float* d_d,
-                      cudaStream_t st, int32_t* d_info)
+                      cudaStream_t st, int32_t* d_info, const int32_t* d_chunk_bad, int32_t* d_info_out)
 {
     const taot_params& p = h->p;
     const size_t smem = sizeof(int32_t) * (p.E + p.R);
     const int parts = (h->d_merge_part && h->d_merge_cnt) ? TAOT_MERGE_PARTS : 1;
-    merge_kernel<<<p.L * parts, 1024, smem, st>>>(d_cc, h->d_e2r, d_n, d_expert_load, d_rank_load, d_excess, d_spare,
-                                                  d_s, d_d, p.R, p.E, h->nc, d_info, parts, h->d_merge_part,
-                                                  h->d_merge_cnt);
-    TAOT_CUDA_OK(cudaGetLastError());
+    TAOT_CUDA_OK(taot_launch_chained(merge_kernel, p.L * parts, 1024, smem, st, d_cc, h->d_e2r, d_n, d_expert_load, d_rank_load,
+                                     d_excess, d_spare, d_s, d_d, p.R, p.E, h->nc, d_info, parts, h->d_merge_part, h->d_merge_cnt,
+                                     d_chunk_bad, d_info_out));
     return 1;
 }
 

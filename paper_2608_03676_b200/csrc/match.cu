@@ -148,6 +148,7 @@ match_kernel(MatchArgs a)
     int32_t* nrem = a.nrem_in_smem ? nrem_s : a.nrem_g + l * (int64_t)a.dmax * R;
     float* t12 = a.t12 + l * (int64_t)E * 2 * R;      // global scratch; replaced by shared memory below if the rows fit
 
+    taot_await();
     const bool timed = TIMED && tid == 0;
     const long long c_start = timed ? clock64() : 0;
     long long c_scan = 0, c_win = 0, c_row = 0, c_build = 0;
@@ -588,6 +589,7 @@ match_kernel(MatchArgs a)
         }
     }
 
+    taot_release();
     // ---- outputs
     int residual = 0;
     for (int s = tid; s < S; s += NT) {
@@ -668,8 +670,7 @@ int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expe
     NT = NT < 256 ? 256 : (NT > 512 && need <= 512 ? 512 : (NT > 1024 ? 1024 : NT));
     auto launch = [&](auto kernel) -> int {
         TAOT_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        kernel<<<p.L, NT, smem, st>>>(a);
-        TAOT_CUDA_OK(cudaGetLastError());
+        TAOT_CUDA_OK(taot_launch_chained(kernel, p.L, NT, smem, st, a));
         return 1;
     };
     const bool lean = a.nbid > 0 && a.ntiers <= 4 && !h->bid_ties, nsm = a.nrem_in_smem != 0;

@@ -142,6 +142,8 @@ __global__ void __launch_bounds__(1024) sinkhorn_kernel(SinkArgs a)
     Smem m = carve(smem_raw, R, NT);
     const int64_t b = blockIdx.x;
     __shared__ double s_sum[2];
+    taot_await();
+    taot_release();
     if (a.only_marked && a.iters[b] != kHandBack) return;
 
     // ---- supply scaling gamma = min(1, sum d / max(sum s, eps0)), compaction
@@ -351,6 +353,7 @@ sinkhorn_input_guard_kernel(const float* __restrict__ s, const float* __restrict
 {
     const int lane = threadIdx.x & 31;
     const int64_t b = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    taot_await();
     if (b >= B) return;
     bool bad = false;
     for (int r = lane; r < R; r += 32) bad |= !isfinite(s[b * R + r]) || !isfinite(d[b * R + r]);
@@ -367,8 +370,7 @@ sinkhorn_input_guard_kernel(const float* __restrict__ s, const float* __restrict
 int taot_launch_sinkhorn_guard(taot_handle_t h, const float* d_s, const float* d_d, int32_t B, float* d_plan,
                                int32_t* d_iters, float* d_row_err, int32_t* d_info, cudaStream_t st)
 {
-    sinkhorn_input_guard_kernel<<<(B + 3) / 4, 128, 0, st>>>(d_s, d_d, B, h->p.R, d_plan, d_iters, d_row_err, d_info);
-    TAOT_CUDA_OK(cudaGetLastError());
+    TAOT_CUDA_OK(taot_launch_chained(sinkhorn_input_guard_kernel, (B + 3) / 4, 128, 0, st, d_s, d_d, B, h->p.R, d_plan, d_iters, d_row_err, d_info));
     return 1;
 }
 
@@ -442,8 +444,7 @@ int taot_launch_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, in
             launched += nw + n;
             a.only_marked = nw + n > 0 ? 1 : 0;
         }
-        sinkhorn_kernel<<<nb, NT, smem, st>>>(a);
-        TAOT_CUDA_OK(cudaGetLastError());
+        TAOT_CUDA_OK(taot_launch_chained(sinkhorn_kernel, nb, NT, smem, st, a));
         launched += 1;
     }
     return launched;

@@ -396,6 +396,7 @@ sinkhorn_class_kernel(ClassArgs k, int64_t nprob)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int R = a.R, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t b0 = (int64_t)blockIdx.x * PPC;
+    taot_await();
     if (blockIdx.x >= k.solvers) {
         zero_rows_of_batch(a, nprob, k.wide, (int64_t)(blockIdx.x - k.solvers) * (kThreads / 32) + warp,
                            (int64_t)(gridDim.x - k.solvers) * (kThreads / 32));
@@ -665,6 +666,7 @@ sinkhorn_class_tree_kernel(ClassArgs k, int64_t nprob)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int R = a.R, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t b0 = (int64_t)blockIdx.x * PPC;
+    taot_await();
     if (blockIdx.x >= k.solvers) {
         zero_rows_of_batch(a, nprob, k.wide, (int64_t)(blockIdx.x - k.solvers) * (kThreads / 32) + warp,
                            (int64_t)(gridDim.x - k.solvers) * (kThreads / 32));
@@ -947,8 +949,7 @@ int launch_dense(const ClassArgs& k, int32_t B, int32_t zeroers, cudaStream_t st
 {
     const size_t smem = (size_t)k.a.R * (PPC * 2 * sizeof(float) + 2 * sizeof(uint16_t));
     TAOT_CUDA_OK(cudaFuncSetAttribute(sinkhorn_class_kernel<NC, VPL, TOL, PPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    sinkhorn_class_kernel<NC, VPL, TOL, PPC><<<(unsigned)(k.solvers + zeroers), kThreads, smem, st>>>(k, (int64_t)B);
-    TAOT_CUDA_OK(cudaGetLastError());
+    TAOT_CUDA_OK(taot_launch_chained(sinkhorn_class_kernel<NC, VPL, TOL, PPC>, (unsigned)(k.solvers + zeroers), kThreads, smem, st, k, (int64_t)B));
     return 1;
 }
 
@@ -957,8 +958,7 @@ int launch_tree(const ClassArgs& k, int32_t B, int32_t zeroers, cudaStream_t st)
 {
     const size_t smem = PPC * (sizeof(TreeSmem<32 * GPL * NPG>) + 2 * sizeof(double) * 32 * GPL * NPG) + (size_t)k.a.R * (PPC * 4 * sizeof(float) + 2 * sizeof(uint16_t));
     TAOT_CUDA_OK(cudaFuncSetAttribute(sinkhorn_class_tree_kernel<GPL, NPG, TOL, PPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    sinkhorn_class_tree_kernel<GPL, NPG, TOL, PPC><<<(unsigned)(k.solvers + zeroers), kThreads, smem, st>>>(k, (int64_t)B);
-    TAOT_CUDA_OK(cudaGetLastError());
+    TAOT_CUDA_OK(taot_launch_chained(sinkhorn_class_tree_kernel<GPL, NPG, TOL, PPC>, (unsigned)(k.solvers + zeroers), kThreads, smem, st, k, (int64_t)B));
     return 1;
 }
 

@@ -98,21 +98,13 @@ __device__ int compact_list(const float* val, int R, int32_t* list, int32_t* wcn
     return total;
 }
 
-__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kNT, 1)
-sinkhorn_cluster_kernel(SinkArgs a, int32_t kcap)
+__device__ void cluster_problem(const SinkArgs& a, int32_t kcap, const int64_t b, unsigned char* smem_raw, cg::cluster_group& cluster)
 {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    cg::cluster_group cluster = cg::this_cluster();
     const int rank = (int)cluster.block_rank();
     const int R = a.R, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     CSmem m = ccarve(smem_raw, R);
-    const int64_t b = blockIdx.x / kCluster;
     __shared__ double s_sum[2];
     const int XS = R + kXTail;                               // floats per exchange buffer
-    // chained launch: only what an earlier kernel left (a problem left over has supply and demand, so none of the four
-    // CTAs writes iters[b] before all of them have met at the barrier below, or writes the mark that is there)
-    if (a.skip_solved && a.iters[b] != kHandBack) return;
-
     // ---- supply scaling gamma = min(1, sum d / max(sum s, eps0)), compaction (every CTA, identically)
     {
         double ps = 0.0, pd = 0.0;
@@ -374,6 +366,24 @@ sinkhorn_cluster_kernel(SinkArgs a, int32_t kcap)
     }
 }
 
+constexpr int32_t kChained = 32;      // about as many as are resident at a time
+
+// One problem per cluster; in a chained launch few clusters walk the batch and solve what an earlier kernel left (a problem
+// left over has supply and demand, so none of the four CTAs writes iters[b] before all of them have met at a barrier, or
+// writes the mark that is there: the four always agree on what to skip).
+__global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kNT, 1)
+sinkhorn_cluster_kernel(SinkArgs a, int32_t kcap, int32_t nprob)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    cg::cluster_group cluster = cg::this_cluster();
+    taot_await();
+    for (int64_t b = blockIdx.x / kCluster; b < nprob; b += gridDim.x / kCluster) {
+        if (a.skip_solved && a.iters[b] != kHandBack) continue;
+        cluster_problem(a, kcap, b, smem_raw, cluster);
+        cluster.sync();
+    }
+}
+
 }  // namespace
 
 int taot_launch_sinkhorn_cluster(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st)
@@ -385,7 +395,8 @@ int taot_launch_sinkhorn_cluster(taot_handle_t h, const SinkArgs& a, int32_t B, 
     const int32_t kcap = (int32_t)((budget - state) / sizeof(float));
     const size_t smem = state + sizeof(float) * (size_t)kcap;
     TAOT_CUDA_OK(cudaFuncSetAttribute(sinkhorn_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    sinkhorn_cluster_kernel<<<(unsigned)B * kCluster, kNT, smem, st>>>(a, kcap);
+    const int32_t clusters = a.skip_solved && B > kChained ? kChained : B;
+    sinkhorn_cluster_kernel<<<(unsigned)clusters * kCluster, kNT, smem, st>>>(a, kcap, B);
     TAOT_CUDA_OK(cudaGetLastError());
     return 1;
 }

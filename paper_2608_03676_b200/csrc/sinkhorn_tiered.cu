@@ -137,6 +137,7 @@ sinkhorn_tiered_mw_kernel(SinkArgs a, TierCosts tc, int64_t nprob)
     const int R = a.R, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const bool mainw = warp < kWarps;             // this warp owns ranks
     const int64_t b = blockIdx.x;
+    taot_await();
     if (b >= nprob) return;
     double* alpha = reinterpret_cast<double*>(smem_raw);          // [R] potentials by rank (supply ranks; -inf elsewhere)
     double* beta = alpha + R;                                      // [R] (demand ranks)
@@ -528,6 +529,7 @@ sinkhorn_tiered_mw_kernel(SinkArgs a, TierCosts tc, int64_t nprob)
     // group), a3_i F_g(j) f_n(j) w_j (neither), times the cap of column j; a factor that underflows belongs to an
     // entry e^-87 below the largest of its row.  The factors go to shared memory (over the potentials, which are no
     // longer needed) and a row costs one multiplication per entry.
+    taot_release();
     fold(true);
     float cap[RPL];
     {
@@ -595,10 +597,10 @@ int launch_mw(const SinkArgs& a, const TierCosts& tc, int32_t B, cudaStream_t st
     if (2 * B <= sms && smem < kExclusiveSmem) smem = kExclusiveSmem;
     if (a.tol > 0.0f) {
         TAOT_CUDA_OK(cudaFuncSetAttribute(sinkhorn_tiered_mw_kernel<kNode, kGroup, KW, RPL, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        sinkhorn_tiered_mw_kernel<kNode, kGroup, KW, RPL, true><<<B, kThreads + 32, smem, st>>>(a, tc, (int64_t)B);
+        TAOT_CUDA_OK(taot_launch_chained(sinkhorn_tiered_mw_kernel<kNode, kGroup, KW, RPL, true>, B, kThreads + 32, smem, st, a, tc, (int64_t)B));
     } else {
         TAOT_CUDA_OK(cudaFuncSetAttribute(sinkhorn_tiered_mw_kernel<kNode, kGroup, KW, RPL, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        sinkhorn_tiered_mw_kernel<kNode, kGroup, KW, RPL, false><<<B, kThreads, smem, st>>>(a, tc, (int64_t)B);
+        TAOT_CUDA_OK(taot_launch_chained(sinkhorn_tiered_mw_kernel<kNode, kGroup, KW, RPL, false>, B, kThreads, smem, st, a, tc, (int64_t)B));
     }
     TAOT_CUDA_OK(cudaGetLastError());
     return 1;

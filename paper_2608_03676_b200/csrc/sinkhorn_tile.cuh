@@ -243,6 +243,7 @@ __device__ __forceinline__ bool tile_solve(const SinkArgs& a, TileSmem<NW, CG>& 
         }
     }
 
+    taot_release();
     // ---- T = diag(u) M diag(v) from the total potentials, then the column cap
     if (NW > 1) __syncthreads();
     if (row_owner) sm.alpha[rowl] += log((double)uo);
@@ -570,6 +571,7 @@ __device__ __forceinline__ bool grid_solve(const SinkArgs& a, TileSmem<1, CG>& s
         ++t;
     }
 
+    taot_release();
     // ---- T = diag(u) M diag(v) from the total potentials, then the column cap
 #pragma unroll
     for (int ra = 0; ra < NRA; ++ra)
@@ -749,6 +751,7 @@ sinkhorn_tile_kernel(SinkArgs a, int64_t nprob)
     __shared__ TileSmem<NW, CG> sm;
     // one problem per CTA (a stride loop over the problems with a grid sized to the SMs was measured slower: the
     // set-up and write-out of one problem no longer overlap the iterations of the CTAs next to it)
+    taot_await();
     if ((int64_t)blockIdx.x < nprob) tile_problem<NW, CG, RP0, RP1, RP2, TOLK>(a, sm, (int64_t)blockIdx.x);
 }
 

@@ -6,7 +6,7 @@
 
 int taot_launch_sinkhorn_tile_r256_batch(const SinkArgs& a, int32_t B, cudaStream_t st)
 {
-    sinkhorn_tile_kernel<4, 8, 4, 8, 8, 1><<<B, 128, 0, st>>>(a, (int64_t)B);
+    TAOT_CUDA_OK(taot_launch_chained(sinkhorn_tile_kernel<4, 8, 4, 8, 8, 1>, B, 128, 0, st, a, (int64_t)B));
     TAOT_CUDA_OK(cudaGetLastError());
     return 1;
 }

@@ -54,7 +54,8 @@ __device__ __forceinline__ bool in_range(float x) { return x > kSumLo && x < kSu
 struct WideSmem {
     double alpha[kMaxRows], beta[kMaxR], red[2][kMaxWarps + 1];
     float st[kMaxRows], dd[kMaxR];
-    __align__(16) float u[2][kMaxRows * 2];        // u~ by parity of the iteration, each twice (a packed operand)
+    __align__(16) float u[2][kMaxRows / 8 * 20 + 16 * 8];   // u~ by parity of the iteration, each twice (a packed operand), by row lane
+                                                   // with a stride of 2 RT + 4 (no bank conflicts between the row lanes)
     __align__(16) float v[kMaxR];                  // v~
     __align__(16) float part[kMaxWarps][80];       // row sums by warp (stride: the two readers of a row meet no bank conflict)
     float err[kMaxRows];
@@ -80,12 +81,13 @@ __device__ __forceinline__ bool wide_solve(const SinkArgs& a, WideSmem& sm, floa
     u64 v2[4];                                     // v~ of those columns
     float vo = 1.0f, vprev = 1.0f;                 // v~ of column `col`: iterate t, iterate t - 1
 
-    auto build = [&]() {                           // block-wide: the tile from the potentials
+    auto build = [&](const bool staged) {          // block-wide: the tile from the potentials (staged: it holds the costs)
         __syncthreads();
+#pragma unroll 4
         for (int q = tid; q < NR * NC; q += NT) {
             const int i = q / NC, j = q - i * NC;
             const bool ok = i < Hn && j < Cn;
-            const double c = (double)a.C[(int64_t)sm.hot[ok ? i : 0] * R + sm.cold[ok ? j : 0]] * a.inv_eps;
+            const double c = (double)(staged ? tile[q] : a.C[(int64_t)sm.hot[ok ? i : 0] * R + sm.cold[ok ? j : 0]]) * a.inv_eps;
             const float e = exp_split(sm.alpha[ok ? i : 0] + sm.beta[ok ? j : 0] - c);
             tile[q] = ok ? e : 0.0f;
         }
@@ -152,14 +154,48 @@ __device__ __forceinline__ bool wide_solve(const SinkArgs& a, WideSmem& sm, floa
         }
         return s + __shfl_xor_sync(kFull, s, 1);
     };
+    const int uq = (tid >> 1) / RT * (2 * RT + 4) + (tid >> 1) % RT * 2 + (tid & 1);      // this thread's place in u
     const bool totals = tid < 2 * NR;              // whole warps: NR is a multiple of 16
     const int row = tid >> 1;
     const bool row_ok = totals && row < Hn;
     const float st = row_ok ? sm.st[row] : 1.0f;
 
-    build();
+    // the rows of the plan without supply, a row per warp and iteration, while the iterations run
+    const bool wide4 = R % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0;
+    int zero_row = mainw ? warp : R;
+    auto write_zero_row = [&]() {
+        if (sm.hpos[zero_row] < 0) {
+            float* o = out + (int64_t)zero_row * R;
+            if (wide4) {
+                for (int j = lane * 4; j < R; j += 128) *reinterpret_cast<float4*>(o + j) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            } else {
+                for (int j = lane; j < R; j += 32) o[j] = 0.0f;
+            }
+        }
+        zero_row += NW;
+    };
+
+    // ---- the costs into the staging, and iteration 1 in the log domain (v = 1 on every rank): phi = log s~ -
+    //      LSE_j(-C_ij/eps) over all j (the caller's), psi_j = log d_j - LSE_i(phi_i - C_ij/eps)
+#pragma unroll 8
+    for (int q = tid; q < NR * NC; q += NT) {
+        const int i = q / NC, j = q - i * NC;
+        const bool ok = i < Hn && j < Cn;
+        tile[q] = a.C[(int64_t)sm.hot[ok ? i : 0] * R + sm.cold[ok ? j : 0]];
+    }
+    __syncthreads();
+    for (int j = tid; j < Cn; j += NT) {
+        double mx = -INFINITY;
+#pragma unroll 4
+        for (int i = 0; i < Hn; ++i) mx = fmax(mx, sm.alpha[i] - (double)tile[i * NC + j] * a.inv_eps);
+        double acc = 0.0;
+#pragma unroll 4
+        for (int i = 0; i < Hn; ++i) acc += (double)exp_split(sm.alpha[i] - (double)tile[i * NC + j] * a.inv_eps - mx);
+        sm.beta[j] = log((double)sm.dd[j]) - (mx + log(acc));
+    }
+    build(true);
     load_tile();
-    if (totals) sm.u[1][tid] = 1.0f;               // iterate 1
+    if (totals) sm.u[1][uq] = 1.0f;               // iterate 1
     if (tid == 0) { sm.event[0] = -1; sm.event[1] = -1; sm.bad = 0; }
     if (mainw) share_v(1.0f);
     __syncthreads();
@@ -178,18 +214,18 @@ __device__ __forceinline__ bool wide_solve(const SinkArgs& a, WideSmem& sm, floa
             } else if (ev_drift == t) {
                 // u~ or v~ of iterate t left the window: fold it into the potentials, or hand the problem back if a sum left
                 // the range in which fp32 products are trustworthy
-                const float un = row_ok ? sm.u[t & 1][tid] : 1.0f;
+                const float un = row_ok ? sm.u[t & 1][uq] : 1.0f;
                 if (!in_range(un) || !in_range(vo)) sm.bad = 1;
                 __syncthreads();
                 if (sm.bad) return false;
                 if (row_ok && !(tid & 1)) sm.alpha[row] += log((double)un);
                 if (col_ok) sm.beta[col] += log((double)vo);
                 __syncthreads();
-                if (totals) sm.u[t & 1][tid] = 1.0f;
+                if (totals) sm.u[t & 1][uq] = 1.0f;
                 if (tid == 0) sm.event[0] = -1;
                 vo = 1.0f;
                 if (mainw) share_v(1.0f);
-                build();
+                build(false);
                 load_tile();
                 continue;
             }
@@ -203,7 +239,7 @@ __device__ __forceinline__ bool wide_solve(const SinkArgs& a, WideSmem& sm, floa
                 const float r = row_total();
                 if (row_ok) {
                     if (!in_range(r)) sm.bad = 1;
-                    if (!(tid & 1)) e = (double)fabsf(fmaf(sm.u[t & 1][tid], r, -st));
+                    if (!(tid & 1)) e = (double)fabsf(fmaf(sm.u[t & 1][uq], r, -st));
                 }
             }
 #pragma unroll
@@ -225,8 +261,8 @@ __device__ __forceinline__ bool wide_solve(const SinkArgs& a, WideSmem& sm, floa
         if (totals) {
             const float r = row_total();
             const float un = row_ok ? st * rcp_fast(r) : 1.0f;
-            if (TOL && check_now && !(tid & 1)) sm.err[row] = row_ok ? fabsf(fmaf(sm.u[t & 1][tid], r, -st)) : 0.0f;
-            sm.u[(t + 1) & 1][tid] = un;
+            if (TOL && check_now && !(tid & 1)) sm.err[row] = row_ok ? fabsf(fmaf(sm.u[t & 1][uq], r, -st)) : 0.0f;
+            sm.u[(t + 1) & 1][uq] = un;
             if (!in_window(un)) sm.event[0] = t + 1;
         }
         __syncthreads();
@@ -235,7 +271,7 @@ __device__ __forceinline__ bool wide_solve(const SinkArgs& a, WideSmem& sm, floa
             float q[8];
             {
                 u64 q2[4];
-                const ulonglong2* up = reinterpret_cast<const ulonglong2*>(&sm.u[(t + 1) & 1][2 * rl * RT]);
+                const ulonglong2* up = reinterpret_cast<const ulonglong2*>(&sm.u[(t + 1) & 1][rl * (2 * RT + 4)]);
 #pragma unroll
                 for (int r = 0; r < RT; r += 2) {
                     const ulonglong2 uu = up[r / 2];
@@ -262,6 +298,7 @@ __device__ __forceinline__ bool wide_solve(const SinkArgs& a, WideSmem& sm, floa
             vo = col_ok ? dd * rcp_fast(q[0]) : 1.0f;
             if (!in_window(vo)) sm.event[0] = t + 1;
             share_v(vo);
+            if (zero_row < R) write_zero_row();
         } else if (TOL && check_now) {             // the error warp: the 64 terms of iterate t
             float e = 0.0f;
             for (int i = lane; i < NR; i += 32) e += sm.err[i];
@@ -273,9 +310,10 @@ __device__ __forceinline__ bool wide_solve(const SinkArgs& a, WideSmem& sm, floa
     }
 
     // ---- T = diag(u) M diag(v) from the total potentials, then the column cap
-    if (row_ok && !(tid & 1)) sm.alpha[row] += log((double)sm.u[t & 1][tid]);
+    if (row_ok && !(tid & 1)) sm.alpha[row] += log((double)sm.u[t & 1][uq]);
     if (col_ok) sm.beta[col] += log((double)vo);
-    build();
+    while (zero_row < R) write_zero_row();
+    build(false);
     for (int j = tid; j < NC; j += NT) {
         float acc = 0.0f;
         for (int i = 0; i < Hn; ++i) acc += tile[i * NC + j];
@@ -286,10 +324,8 @@ __device__ __forceinline__ bool wide_solve(const SinkArgs& a, WideSmem& sm, floa
     for (int i = warp; i < R; i += NT >> 5) {
         const int h = sm.hpos[i];
         float* o = out + (int64_t)i * R;
-        if (h < 0) {
-            for (int j = lane; j < R; j += 32) o[j] = 0.0f;
-            continue;
-        }
+        if (h < 0) continue;
+#pragma unroll 4
         for (int j = lane; j < R; j += 32) {
             const int c = sm.cpos[j];
             const float w = c >= 0 ? tile[h * NC + c] * sm.v[c] : 0.0f;
@@ -315,6 +351,7 @@ sinkhorn_wide_kernel(SinkArgs a, int64_t nprob)
     float* tile = reinterpret_cast<float*>(smem_raw + ((sizeof(WideSmem) + 15) & ~(size_t)15));
     const int R = a.R, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NT = blockDim.x, NW = (R + 31) >> 5;
     const int64_t b = blockIdx.x;
+    taot_await();
     if (b >= nprob) return;
 
     // ---- supply scaling gamma = min(1, sum d / max(sum s, eps0)), compaction of the ranks with supply / demand
@@ -365,20 +402,8 @@ sinkhorn_wide_kernel(SinkArgs a, int64_t nprob)
     double sum_st = 0.0;
     for (int i = 0; i < Hn; ++i) sum_st += (double)sm.st[i];          // same order in every thread
 
-    // ---- iteration 1 in the log domain (v = 1 on every rank): phi = log s~ - LSE_j(-C_ij/eps) over all j,
-    //      psi_j = log d_j - LSE_i(phi_i - C_ij/eps)
     for (int i = tid; i < Hn; i += NT) sm.alpha[i] = log((double)sm.st[i]) - a.rowlse0[sm.hot[i]];
     __syncthreads();
-    for (int j = tid; j < Cn; j += NT) {
-        const float* cj = a.C + sm.cold[j];
-        double mx = -INFINITY;
-#pragma unroll 4
-        for (int i = 0; i < Hn; ++i) mx = fmax(mx, sm.alpha[i] - (double)cj[(int64_t)sm.hot[i] * R] * a.inv_eps);
-        double acc = 0.0;
-#pragma unroll 4
-        for (int i = 0; i < Hn; ++i) acc += (double)exp_split(sm.alpha[i] - (double)cj[(int64_t)sm.hot[i] * R] * a.inv_eps - mx);
-        sm.beta[j] = log((double)sm.dd[j]) - (mx + log(acc));
-    }
     bool done;
     if (Hn <= 16) done = wide_solve<2, TOL>(a, sm, tile, NW, Hn, Cn, sum_st, info, out, b);
     else if (Hn <= 32) done = wide_solve<4, TOL>(a, sm, tile, NW, Hn, Cn, sum_st, info, out, b);
@@ -400,10 +425,10 @@ int taot_launch_sinkhorn_wide(taot_handle_t h, const SinkArgs& a, int32_t B, cud
     const size_t smem = ((sizeof(WideSmem) + 15) & ~(size_t)15) + sizeof(float) * kMaxRows * 32 * NW;
     if (a.tol > 0.0f) {
         TAOT_CUDA_OK(cudaFuncSetAttribute(sinkhorn_wide_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        sinkhorn_wide_kernel<true><<<B, NW * 32 + 32, smem, st>>>(a, (int64_t)B);
+        TAOT_CUDA_OK(taot_launch_chained(sinkhorn_wide_kernel<true>, B, NW * 32 + 32, smem, st, a, (int64_t)B));
     } else {
         TAOT_CUDA_OK(cudaFuncSetAttribute(sinkhorn_wide_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        sinkhorn_wide_kernel<false><<<B, NW * 32, smem, st>>>(a, (int64_t)B);
+        TAOT_CUDA_OK(taot_launch_chained(sinkhorn_wide_kernel<false>, B, NW * 32, smem, st, a, (int64_t)B));
     }
     TAOT_CUDA_OK(cudaGetLastError());
     return 1;

@@ -62,7 +62,7 @@ struct taot_handle_s {
     int64_t kcap_global;     // same, global-memory scratch per problem (R > 256 only), else 0
     // workspace layout (byte offsets)
     size_t off_cc, off_excess, off_spare, off_s, off_d, off_nrem, off_t12, off_kt, off_dc, off_cyc, off_tc;
-    size_t off_tb, off_tbflag;   // one-byte copy of the routing table and one flag per chunk (see tb_ok)
+    size_t off_tb, off_tbflag;   // one-byte copy of the routing table (see tb_ok) and one flag per chunk (a value that is no expert)
     int32_t tb_ok;               // 1: the histogram pass also leaves the table as one byte per entry (E <= 256 experts,
                                  // segments of a multiple of 16 entries) for the reassignment to read instead of the table
     size_t ws_bytes;
@@ -91,13 +91,15 @@ struct taot_handle_s {
 static inline size_t taot_align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 // kernel launchers (each returns the number of kernels it enqueued, or a negative taot_status)
+// d_info == nullptr: the flags of the chunks are all that is left of values that are no expert
 int taot_launch_histogram(taot_handle_t h, const int32_t* d_topk, int32_t* d_cc, int32_t* d_info, cudaStream_t st,
                           void* ws = nullptr, bool write_bytes = true);
 // the table as one byte per entry, by a few CTAs that leave the other SMs alone (returns 0 if this handle keeps no such copy)
 int taot_launch_table_bytes(taot_handle_t h, const int32_t* d_topk, void* ws, cudaStream_t st);
 int taot_launch_merge(taot_handle_t h, const int32_t* d_cc, int32_t* d_n, int32_t* d_expert_load,
                       int32_t* d_rank_load, int32_t* d_excess, int32_t* d_spare, float* d_s, float* d_d,
-                      cudaStream_t st, int32_t* d_info = nullptr);
+                      cudaStream_t st, int32_t* d_info = nullptr, const int32_t* d_chunk_bad = nullptr,
+                      int32_t* d_info_out = nullptr);   // d_info_out: starts the call's status words from the chunks' flags
 int taot_launch_excess_spare(taot_handle_t h, const int32_t* d_rank_load, int32_t B, int32_t* d_excess,
                              int32_t* d_spare, float* d_s, float* d_d, cudaStream_t st);
 int taot_launch_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, int32_t B, float* d_plan,
@@ -123,6 +125,29 @@ int taot_launch_chunk_counts(taot_handle_t h, const int32_t* d_idx, int32_t* d_c
                              cudaStream_t st);
 int taot_launch_dispatch(taot_handle_t h, const int32_t* d_new_idx, int32_t* d_send_counts, int32_t* d_target_counts,
                          int32_t* d_perm, int32_t* d_info, void* ws, cudaStream_t st);
+
+// Launch of a kernel that may be set up while the kernel before it on the stream still runs (programmatic dependent launch):
+// its blocks are placed once every block of that kernel has called taot_release() or ended, and wait in taot_await() until that
+// kernel has ended and its writes are visible.  Every kernel of a chain calls taot_await() before it reads or writes anything
+// of the call; launched the ordinary way both are no-ops.
+__device__ __forceinline__ void taot_await() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void taot_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... P, typename... A>
+cudaError_t taot_launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
 
 #define TAOT_CUDA_OK(expr)                              \
     do {                                                \

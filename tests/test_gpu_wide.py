@@ -1,0 +1,34 @@
+"""Phase 1 with a cost without structure at 257 to 512 ranks (the kernel matrix in the registers of one CTA): the edges of its
+row builds (16, 32 and 64 supply ranks, and one more, which goes to the kernels behind it), ragged rank counts, a fixed count
+and the stopping rule, against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+from helpers import check_sinkhorn_problem, cpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("R,rows", [(257, (1, 16, 17, 32)), (288, (33, 64, 65, 2)), (300, (31, 63, 66, 15)), (512, (54, 64, 16, 200))])
+@pytest.mark.parametrize("iters,tol,check_every", [(70, 0.0, 1), (300, 1e-5, 1), (300, 1e-5, 7)])
+def test_wide_kernel_by_supply_ranks(R, rows, iters, tol, check_every):
+    import paper_2608_03676_b200 as P
+    g = torch.Generator().manual_seed(R)
+    C = 1.0 + 15.0 * torch.rand((R, R), generator=g)
+    C.fill_diagonal_(0.0)
+    B, eps = len(rows), 2.0
+    s = torch.zeros((B, R)); d = torch.zeros((B, R))
+    for b, h in enumerate(rows):
+        p = torch.randperm(R, generator=g)
+        s[b, p[:h]] = torch.randint(1, 40000, (h,), generator=g).float()
+        d[b, p[h:]] = torch.randint(1, 9000, (R - h,), generator=g).float()
+        d[b] *= float(s[b].sum() / d[b].sum()) * (1.0 if b % 2 else 0.97)      # odd: enough room, even: the supply is scaled
+    pl = P.Planner(L=B, R=R, E=R, K=1, k=1, T=R, e2r=torch.arange(R, dtype=torch.int32), C=C, eps=eps, max_iters=iters, tol=tol,
+                   check_every=check_every)
+    out = pl.sinkhorn(s.cuda(), d.cuda())
+    torch.cuda.synchronize()
+    for b in range(B):
+        check_sinkhorn_problem(s[b].numpy(), d[b].numpy(), C.numpy(), eps, cpu(out["plan"])[b], cpu(out["iters"])[b],
+                               cpu(out["row_err"])[b], iters, tol, check_every)
+    pl.close()
