@@ -15,6 +15,7 @@
 #define TAOT_STREAM_THREADS 256            // threads of the streaming kernels: 64 elements each
 #define TAOT_MAX_TIERS 8                   // distinct bonus values the bit-set auction handles
 #define TAOT_MERGE_PARTS 8                 // CTAs that share the merge of one layer's chunk counts (256-rank tables)
+#define TAOT_HOST_GROUP_BYTES (2 << 20)    // routing table from which a host call is split into layer groups
 #define TAOT_MAX_GROUPS 6                  // layer groups taot_plan overlaps on internal streams
 
 struct taot_handle_s {
@@ -84,6 +85,11 @@ struct taot_handle_s {
     int32_t group_len[TAOT_MAX_GROUPS];
     cudaStream_t gstream[TAOT_MAX_GROUPS];     // [0] unused: group 0 runs on the caller's stream
     cudaEvent_t ev_fork, ev_hist[TAOT_MAX_GROUPS], ev_join[TAOT_MAX_GROUPS];
+    // Layer groups of the host calls (tables of at least TAOT_HOST_GROUP_BYTES): views like the ones above, each on a stream
+    // of its own (gstream), so that copies in, kernels and copies out of different groups run side by side.
+    int32_t hgroups;
+    taot_handle_s* hgroup[TAOT_MAX_GROUPS];
+    int32_t hgroup_l0[TAOT_MAX_GROUPS];
     cudaStream_t bstream;                      // the one-byte copies of the groups' tables are made here, after all histograms
     cudaEvent_t ev_bytes[TAOT_MAX_GROUPS];     // group g's copy is there
 };
