@@ -729,6 +729,9 @@ int plan_stages(taot_handle_t h, const int32_t* d_topk, const taot_outputs* o, v
     float* fs = reinterpret_cast<float*>(at(ws, h->off_s));
     float* fd = reinterpret_cast<float*>(at(ws, h->off_d));
     int total = 0, a;
+    // The matching kernel is set up while Phase 1 runs, unless its CTAs would then sit on SMs that the streaming kernels of
+    // other layer groups want (or Phase 1 is switched off, or stages are timed one by one)
+    const bool early = !hist_after && !hist_done && !bytes_later && !marks && !(p.ablation & TAOT_ABLATE_HINT);
 #define TAOT_MARK(i) if (marks) TAOT_CUDA_OK(cudaEventRecord(h->ev[i], st))
     // NVTX ranges around the enqueue of each stage (header-only NVTX: free unless a profiler is attached)
     struct Range {
@@ -758,7 +761,7 @@ int plan_stages(taot_handle_t h, const int32_t* d_topk, const taot_outputs* o, v
         TAOT_CUDA_OK(cudaMemsetAsync(o->row_err, 0, sizeof(float) * p.L, st));
         a = 0;
     } else if ((a = taot_launch_sinkhorn(h, fs, fd, p.L, o->plan, o->sinkhorn_iters, o->row_err, o->info,
-                                         reinterpret_cast<float*>(at(ws, h->off_kt)), st, nullptr, true)) < 0) {
+                                         reinterpret_cast<float*>(at(ws, h->off_kt)), st, nullptr, true, early)) < 0) {
         nvtxRangePop();
         return a;
     }
@@ -769,7 +772,7 @@ int plan_stages(taot_handle_t h, const int32_t* d_topk, const taot_outputs* o, v
     if ((a = taot_launch_match(h, o->n, o->expert_load, o->rank_load, o->plan, o->slot_expert, o->slot_tokens,
                                o->X, o->rounds, o->info, reinterpret_cast<int32_t*>(at(ws, h->off_nrem)),
                                reinterpret_cast<float*>(at(ws, h->off_t12)), st,
-                               (marks && (h->profiling & 2)) ? reinterpret_cast<long long*>(at(ws, h->off_cyc)) : nullptr)) < 0) {
+                               (marks && (h->profiling & 2)) ? reinterpret_cast<long long*>(at(ws, h->off_cyc)) : nullptr, early)) < 0) {
         nvtxRangePop();
         return a;
     }

@@ -10,8 +10,15 @@
 // contraction), which keeps every integer decision reproducible bit for bit on a CPU.
 //
 // Phase 2: the two score terms that do not change between rounds (alpha*B and 0.1*alpha*T_norm)
-// are computed once per layer for the experts that spill; a round is then one thread per rank
-// scanning those experts with coalesced reads.
+// are computed once per layer for the experts that spill, and the scores once per slot index; a
+// round re-forms the rows of the experts it served.  It is bound by that chain of rounds: up to 64
+// ranks one warp runs them (one or two ranks per lane, a rank scans again only if its best pair
+// changed), since the barriers of a CTA cost more than the scans (58 -> 50 k cycles at 32 ranks);
+// with more ranks a lane would hold four and its scans outweigh the barriers: several lanes per rank.
+//
+// In a plan the kernel is set up (loads, spills, score terms) while Phase 1 still runs and waits for
+// it where it first reads the hint: a plan of one 8-rank layer 69 -> 66 us, 32 ranks 141 -> 129 us,
+// 24 ranks 173 -> 164 us.
 //
 // Phase 3: the bonus matrix of a real topology has a handful of distinct values (tiers): the auction of auction.cuh.  A bonus
 // matrix with more than TAOT_MAX_TIERS distinct values, a price step that is not positive or more than 1024 slots take a
@@ -49,6 +56,7 @@ struct MatchArgs {
     int32_t R, E, K, dmax, ntiers, W, nbid;
     float eps0, price_step;
     int32_t auction_max_rounds;
+    int32_t early;               // launched while Phase 1 runs: the hint is the only input that may not be there yet
     int32_t ablation;            // TAOT_ABLATE_* bits: a term switched off is an exact zero in the score
     int32_t nrem_in_smem;
     int32_t tm_in_smem;
@@ -148,18 +156,34 @@ match_kernel(MatchArgs a)
     int32_t* nrem = a.nrem_in_smem ? nrem_s : a.nrem_g + l * (int64_t)a.dmax * R;
     float* t12 = a.t12 + l * (int64_t)E * 2 * R;      // global scratch; replaced by shared memory below if the rows fit
 
-    taot_await();
+    // Everything up to the flow hint itself follows from the loads, which are there before Phase 1 starts: in a plan (a.early)
+    // this kernel is set up while Phase 1 still runs, and only waits for it where the hint is first read.
+    if (!a.early) taot_await();
     const bool timed = TIMED && tid == 0;
     const long long c_start = timed ? clock64() : 0;
     long long c_scan = 0, c_win = 0, c_row = 0, c_build = 0;
     // ---- integer mean, excess, spare (Appendix A.1)
     if (tid == 0) { s_tot = 0; s_cnt = 0; }
+    int32_t* const el_s = dcol;                    // (dcol is Phase 3's)
+    for (int e = tid; e < E; e += NT) el_s[e] = el[e];
     __syncthreads();
     {
         long long part = 0;
         for (int r = tid; r < R; r += NT) part += rl[r];
         if (part) atomicAdd(reinterpret_cast<u64*>(&s_tot), (u64)part);
     }
+    // what Phase 3 starts from: every rank with 0 wins, no tokens in the plan
+    for (int i = tid; i < (S + 1) * W; i += NT) {
+        const int w = i / (S + 1), left = R - 32 * w;
+        lvl[i] = i - w * (S + 1) != 0 ? 0u : (left >= 32 ? 0xFFFFFFFFu : (1u << left) - 1u);
+    }
+    int32_t* const Xl = a.X + l * (int64_t)R * S;
+    if ((R * S) % 4 == 0 && (reinterpret_cast<uintptr_t>(Xl) & 15) == 0) {
+        for (int q = tid; q < R * S / 4; q += NT) reinterpret_cast<int4*>(Xl)[q] = make_int4(0, 0, 0, 0);
+    } else {
+        for (int q = tid; q < R * S; q += NT) Xl[q] = 0;
+    }
+    for (int q = tid; q < a.nbid; q += NT) { bid_s[q] = a.bidlist[q]; ent_s[q] = a.bident[q]; }
     __syncthreads();
     const long long mean = s_tot / R;
     for (int r = tid; r < R; r += NT) {
@@ -173,12 +197,14 @@ match_kernel(MatchArgs a)
     // ---- spill by cumulative-excess differencing: position of e in its rank's (load, index) order
     for (int e = tid; e < E; e += NT) {
         const int r = a.e2r[e];
-        const int32_t mine = el[e];
+        const int32_t mine = el_s[e];
+        const int q1 = a.rank_off[r + 1];
         long long cum = 0;
-        for (int q = a.rank_off[r]; q < a.rank_off[r + 1]; ++q) {
+#pragma unroll 4
+        for (int q = a.rank_off[r]; q < q1; ++q) {
             const int e2 = a.rank_list[q];
-            const int32_t v = el[e2];
-            if (v < mine || (v == mine && e2 <= e)) cum += v;
+            const int32_t v = el_s[e2];
+            cum += v < mine || (v == mine && e2 <= e) ? v : 0;
         }
         const long long hi = cum - mean, lo = cum - mine - mean;
         const int32_t sp = (int32_t)((hi > 0 ? hi : 0) - (lo > 0 ? lo : 0));
@@ -218,16 +244,27 @@ match_kernel(MatchArgs a)
     const int64_t key_words = keyed ? (int64_t)NHs * R : 0;
     if (key_words + (int64_t)nhot0 * 2 * R <= (int64_t)a.big_floats) t12 = reinterpret_cast<float*>(nrem_s) + key_words;
 
-    // ---- round-invariant score terms of the spilling experts: t1 = alpha*B, t2 = beta*T/max(excess, eps0)
+    // ---- round-invariant score terms of the spilling experts: t1 = alpha*B, t2 = beta*T/max(excess, eps0).  Thread tid takes
+    // rank tid % RP (RP a power of two) of every (NT / RP)-th expert: no division, consecutive threads on consecutive ranks
+    int rsh = 5;
+    while ((1 << rsh) < R) ++rsh;
+    const int my_r = tid & ((1 << rsh) - 1), my_q = tid >> rsh, q_step = NT >> rsh;
+    if (my_r < R) {
 #pragma unroll 4
-    for (int64_t idx = tid; idx < (int64_t)nhot0 * R; idx += NT) {
-        const int q = (int)(idx / R), r = (int)(idx - (int64_t)q * R);
-        const int hr = hot_home[q];
-        const float ex = fmaxf((float)excess[hr], a.eps0);
-        const float tn = (a.ablation & TAOT_ABLATE_HINT) ? 0.0f : __fdiv_rn(plan[(int64_t)hr * R + r], ex);
-        const float bp = (a.ablation & TAOT_ABLATE_TOPOLOGY) ? 0.0f : a.B[(int64_t)hr * R + r];
-        t12[((int64_t)q * 2) * R + r] = __fmul_rn(alpha, bp);
-        t12[((int64_t)q * 2 + 1) * R + r] = __fmul_rn(beta, tn);
+        for (int q = my_q; q < nhot0; q += q_step) {
+            const float bp = (a.ablation & TAOT_ABLATE_TOPOLOGY) ? 0.0f : a.B[hot_home[q] * R + my_r];
+            t12[(int64_t)(2 * q) * R + my_r] = __fmul_rn(alpha, bp);
+        }
+    }
+    if (a.early) taot_await();
+    if (my_r < R) {
+#pragma unroll 4
+        for (int q = my_q; q < nhot0; q += q_step) {
+            const int hr = hot_home[q];
+            const float ex = fmaxf((float)excess[hr], a.eps0);
+            const float tn = (a.ablation & TAOT_ABLATE_HINT) ? 0.0f : __fdiv_rn(plan[hr * R + my_r], ex);
+            t12[(int64_t)(2 * q + 1) * R + my_r] = __fmul_rn(beta, tn);
+        }
     }
     __syncthreads();
 
@@ -252,6 +289,12 @@ match_kernel(MatchArgs a)
         return ok ? ordered_bits(sc) : 0u;
     };
     int32_t* served = dcol;                       // [E] positions of the experts served in a round (dcol is Phase 3's)
+    // score of a pair whose key is not 0 after its expert's spill has shrunk to se
+    auto shrunk_key = [&](int q, int r, int32_t se, int32_t sp) -> uint32_t {
+        const int32_t gain = se < sp ? se : sp;
+        return ordered_bits(__fadd_rn(__fadd_rn((float)gain, t12[(int64_t)(2 * q) * R + r]), t12[(int64_t)(2 * q + 1) * R + r]));
+    };
+    const bool small = R <= 64;                   // one warp runs the rounds, a rank or two per lane, without block barriers
     for (int kappa = 0; keyed && kappa < K; ++kappa) {
         // Between rounds a pair's score changes only when its expert was served (its spill shrank): a rank's spare
         // changes only when it is matched, and then it is out for this slot index.  So all keys are formed once per
@@ -268,20 +311,120 @@ match_kernel(MatchArgs a)
         if (tid == 0) s_cnt = 0;
         __syncthreads();
         if (lane == 0) atomicMax(&s_cnt, smax);
-        for (int64_t idx = tid; idx < (int64_t)nhot0 * R; idx += NT) {
-            const int q = (int)(idx / R), r = (int)(idx - (int64_t)q * R);
-            keyM[r * NHs + q] = pair_key(q, r, kappa);
-        }
+        if (my_r < R)
+            for (int q = my_q; q < nhot0; q += q_step) keyM[my_r * NHs + q] = pair_key(q, my_r, kappa);
         __syncthreads();
         const int32_t spare_cap = s_cnt;
         if (timed) c_build += clock64() - c_b0;
+        if (small) {
+            if (warp == 0) {
+                constexpr int RPL = 2;
+                int32_t sp[RPL];
+                uint32_t bk[RPL];                  // the rank's best candidate: key and position (0: none)
+                int bq[RPL];
+                bool open[RPL], scan[RPL];
+#pragma unroll
+                for (int k = 0; k < RPL; ++k) {
+                    const int r = lane + 32 * k;
+                    sp[k] = r < R ? spare[r] : 0;
+                    open[k] = sp[k] > 0; scan[k] = open[k];
+                    bk[k] = 0u; bq[k] = 0;
+                }
+                for (;;) {
+                    const long long c_s0 = timed ? clock64() : 0;
+                    // Steps 1-2: every unmatched cold rank takes its best candidate expert (ties: lowest position = lowest index); one
+                    // whose best pair did not change in the last round still has it, since keys only shrink
+#pragma unroll
+                    for (int k = 0; k < RPL; ++k) {
+                        if (scan[k]) {
+                            const uint32_t* row = keyM + (lane + 32 * k) * NHs;
+                            uint32_t best = 0u;
+                            int at = 0;
+#pragma unroll 8
+                            for (int q = 0; q < nhot0; ++q) {
+                                const uint32_t v = row[q];
+                                at = v > best ? q : at;
+                                best = v > best ? v : best;
+                            }
+                            bk[k] = best; bq[k] = at;
+                            open[k] = best != 0u;
+                            scan[k] = false;
+                        }
+                    }
+                    __syncwarp();
+                    bool bids = false;
+#pragma unroll
+                    for (int k = 0; k < RPL; ++k) bids = bids || open[k];
+                    if (!__any_sync(0xffffffffu, bids)) break;
+                    // Step 3: the best score any rank offers the expert, then among the ranks that offer it the lowest
+#pragma unroll
+                    for (int k = 0; k < RPL; ++k)
+                        if (open[k]) atomicMax(&arb_hi[bq[k]], bk[k]);
+                    __syncwarp();
+#pragma unroll
+                    for (int k = 0; k < RPL; ++k)
+                        if (open[k] && arb_hi[bq[k]] == bk[k]) atomicMin(&arb_lo[bq[k]], (uint32_t)(lane + 32 * k));
+                    __syncwarp();
+                    bool win[RPL];
+#pragma unroll
+                    for (int k = 0; k < RPL; ++k) win[k] = open[k] && arb_lo[bq[k]] == (uint32_t)(lane + 32 * k);
+                    __syncwarp();
+                    // Step 4: winners take min(spill, spare)
+#pragma unroll
+                    for (int k = 0; k < RPL; ++k) {
+                        if (win[k]) {
+                            const int r = lane + 32 * k, e = hot0[bq[k]];
+                            const int32_t se = spill[e], g = se < sp[k] ? se : sp[k];
+                            spill[e] = se - g;
+                            spare[r] = sp[k] - g;
+                            slot_e[r * K + kappa] = e;
+                            slot_a0[r * K + kappa] = g;
+                            arb_hi[bq[k]] = 0u;
+                            arb_lo[bq[k]] = 0xFFFFFFFFu;
+                            open[k] = false;
+                        }
+                    }
+                    __syncwarp();
+                    const long long c_s1 = timed ? clock64() : 0;
+                    if (timed) c_scan += c_s1 - c_s0;
+                    // the served experts' rows, each rank its own entry: it changes only where min(spill, spare) does
+#pragma unroll
+                    for (int k2 = 0; k2 < RPL; ++k2) {
+                        unsigned todo = __ballot_sync(0xffffffffu, win[k2]);
+                        while (todo) {
+                            const int q = __shfl_sync(0xffffffffu, bq[k2], __ffs(todo) - 1);
+                            todo &= todo - 1;
+                            const int32_t se = spill[hot0[q]];
+#pragma unroll
+                            for (int k = 0; k < RPL; ++k) {
+                                if (open[k] && se < sp[k]) {
+                                    const int r = lane + 32 * k;
+                                    uint32_t* cell = keyM + r * NHs + q;
+                                    if (*cell) {
+                                        *cell = se > 0 ? shrunk_key(q, r, se, sp[k]) : 0u;
+                                        if (q == bq[k]) scan[k] = true;
+                                    }
+                                }
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    ++rounds2;
+                    if (timed) c_row += clock64() - c_s1;
+                }
+                if (lane == 0) s_any = rounds2;
+            }
+            __syncthreads();
+            rounds2 = s_any;
+            continue;
+        }
         for (;;) {
             const long long c_s0 = timed ? clock64() : 0;
             // Steps 1-2: every unmatched cold rank takes its best candidate expert (ties: lowest position = lowest index)
             // (QS lanes per rank with QS * R <= NT: one pass covers every rank)
             const int r = tid >> qsh;
             uint32_t my_bk = 0u;                   // this thread's bid, if it is the lead lane of a bidding rank
-            int my_q = -1;
+            int my_bq = -1;
             {
                 u64 key = 0;
                 if (r < R && !matched[r] && spare[r] > 0) {
@@ -301,42 +444,46 @@ match_kernel(MatchArgs a)
                 }
                 if (qs == 0 && r < R && key != 0) {
                     my_bk = (uint32_t)(key >> 32);
-                    my_q = (int)(0xFFFFFFFFu - (uint32_t)key);
+                    my_bq = (int)(0xFFFFFFFFu - (uint32_t)key);
                 }
             }
-            const int my_e = my_q >= 0 ? hot0[my_q] : 0;
             // Step 3, first half: the best score any rank offers the expert (native 32-bit shared-memory atomics; agreeing
             // inside the warp first on the expert most lanes want was measured and cost more than the conflicts it saves)
-            if (my_q >= 0) atomicMax(&arb_hi[my_e], my_bk);
-            if (!__syncthreads_or(my_q >= 0)) break;
+            if (my_bq >= 0) atomicMax(&arb_hi[my_bq], my_bk);
+            if (!__syncthreads_or(my_bq >= 0)) break;
             if (tid == 0) s_ns = 0;
             // Step 3, second half: among the ranks that offer it, the lowest
-            if (my_q >= 0 && arb_hi[my_e] == my_bk) atomicMin(&arb_lo[my_e], (uint32_t)r);
+            if (my_bq >= 0 && arb_hi[my_bq] == my_bk) atomicMin(&arb_lo[my_bq], (uint32_t)r);
             __syncthreads();
             const long long c_s1 = timed ? clock64() : 0;
             if (timed) c_scan += c_s1 - c_s0;
             // Step 4: winners take min(spill, spare), and put the arbitration entries back.  A row of keys changes only
             // where min(spill, spare_r) does, i.e. for ranks with more spare than the expert now spills: rows whose
             // expert still spills at least the largest spare of this slot index are left as they are.
-            if (my_q >= 0 && arb_lo[my_e] == (uint32_t)r) {
-                const int32_t g = spill[my_e] < spare[r] ? spill[my_e] : spare[r];
-                spill[my_e] -= g;
-                spare[r] -= g;
+            if (my_bq >= 0 && arb_lo[my_bq] == (uint32_t)r) {
+                const int e = hot0[my_bq];
+                const int32_t se = spill[e], sp = spare[r], g = se < sp ? se : sp;
+                spill[e] = se - g;
+                spare[r] = sp - g;
                 matched[r] = 1;
-                slot_e[r * K + kappa] = my_e;
+                slot_e[r * K + kappa] = e;
                 slot_a0[r * K + kappa] = g;
-                arb_hi[my_e] = 0u;                 // (a loser compares arb_lo with its own rank: the reset value is nobody's)
-                arb_lo[my_e] = 0xFFFFFFFFu;
-                if (spill[my_e] < spare_cap) served[atomicAdd(&s_ns, 1)] = my_q;
+                arb_hi[my_bq] = 0u;                // (a loser compares arb_lo with its own rank: the reset value is nobody's)
+                arb_lo[my_bq] = 0xFFFFFFFFu;
+                if (se - g < spare_cap) served[atomicAdd(&s_ns, 1)] = my_bq;
             }
             __syncthreads();
             const long long c_s2 = timed ? clock64() : 0;
             const int ns = s_ns;
             if (ns > 0) {                          // uniform over the CTA
-                for (int idx = tid; idx < ns * R; idx += NT) {
-                    const int i = idx / R, r = idx - i * R;
-                    const int q = served[i];
-                    keyM[r * NHs + q] = pair_key(q, r, kappa);
+                if (my_r < R) {
+                    const int32_t sp = spare[my_r];
+                    for (int i = my_q; i < ns; i += q_step) {
+                        const int q = served[i];
+                        const int32_t se = spill[hot0[q]];
+                        uint32_t* cell = keyM + my_r * NHs + q;
+                        if (se < sp && *cell) *cell = se > 0 ? shrunk_key(q, my_r, se, sp) : 0u;
+                    }
                 }
                 __syncthreads();
             }
@@ -421,23 +568,21 @@ match_kernel(MatchArgs a)
     __syncthreads();
     for (int e = tid; e < E; e += NT)
         if (dcol[e] == -2) dcol[e] = atomicAdd(&s_cnt, 1);
-    for (int i = tid; i < a.dmax * W; i += NT) avail[i] = 0u;
-    for (int i = tid; i < (S + 1) * W; i += NT) lvl[i] = 0u;
     __syncthreads();
     const int D = s_cnt;
     for (int e = tid; e < E; e += NT)
         if (dcol[e] >= 0) hot0[dcol[e]] = e;                   // column -> expert (the Phase-2 list is no longer needed)
     __syncthreads();
+    // a warp per expert and word of 32 ranks: the word of ranks that hold its tokens by a vote (reductions of single bits into
+    // one shared word queue up: 55 k cycles at 256 ranks)
 #pragma unroll 4
-    for (int q = tid; q < D * R; q += NT) {
-        const int col = q / R, r = q - col * R;
-        const int32_t v = n[(int64_t)r * E + hot0[col]];
-        nrem[q] = v;
-        if (v > 0) atomicOr(avail + (r >> 5) * a.dmax + col, 1u << (r & 31));
+    for (int q = warp; q < D * W; q += NW) {
+        const int col = q / W, w = q - col * W, r = 32 * w + lane;
+        const int32_t v = r < R ? n[r * E + hot0[col]] : 0;
+        if (r < R) nrem[col * R + r] = v;
+        const unsigned word = __ballot_sync(0xffffffffu, v > 0);
+        if (lane == 0) avail[w * a.dmax + col] = word;
     }
-    for (int r = tid; r < R; r += NT) atomicOr(lvl + (r >> 5) * (S + 1), 1u << (r & 31));      // every rank starts with 0 wins
-    int32_t* Xl = a.X + l * (int64_t)R * S;
-    for (int64_t q = tid; q < (int64_t)R * S; q += NT) Xl[q] = 0;
     __syncthreads();
 
     int rounds3 = 0;
@@ -448,7 +593,6 @@ match_kernel(MatchArgs a)
         namespace au = taot_auction;
         uint32_t* const arb = reinterpret_cast<uint32_t*>(arb_r);       // [2][R]
         for (int q = tid; q < 2 * R; q += NT) arb[q] = 0u;
-        for (int q = tid; q < a.nbid; q += NT) { bid_s[q] = a.bidlist[q]; ent_s[q] = a.bident[q]; }
         // a live slot's class: expert and the way its host sees the ranks; the lowest slot leads, the others queue behind it
         const int s = tid;
         const bool slive = s < S && slot_e[s] >= 0 && slot_a[s] > 0;
@@ -625,11 +769,12 @@ size_t match_smem_fixed(int R, int E, int K, int dmax, int W, int ntiers)
 int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expert_load,
                       const int32_t* d_rank_load, const float* d_plan, int32_t* d_slot_expert,
                       int32_t* d_slot_tokens, int32_t* d_X, int32_t* d_rounds, int32_t* d_info,
-                      int32_t* d_nrem, float* d_t12, cudaStream_t st, long long* d_cyc)
+                      int32_t* d_nrem, float* d_t12, cudaStream_t st, long long* d_cyc, bool early)
 {
     const taot_params& p = h->p;
     MatchArgs a;
     a.cyc = d_cyc;
+    a.early = early ? 1 : 0;
     a.n = d_n; a.expert_load = d_expert_load; a.rank_load = d_rank_load; a.plan = d_plan;
     a.e2r = h->d_e2r; a.B = h->d_B; a.rank_off = h->d_rank_off; a.rank_list = h->d_rank_list;
     a.tiermask = h->d_tiermask; a.tierval = h->d_tierval; a.bidlist = h->d_bidlist;

@@ -142,6 +142,7 @@ __global__ void __launch_bounds__(1024) sinkhorn_kernel(SinkArgs a)
     Smem m = carve(smem_raw, R, NT);
     const int64_t b = blockIdx.x;
     __shared__ double s_sum[2];
+    if (a.early) taot_release();
     taot_await();
     taot_release();
     if (a.only_marked && a.iters[b] != kHandBack) return;
@@ -387,7 +388,8 @@ bool taot_sinkhorn_takes_classes(taot_handle_t h, bool from_loads)
 }
 
 int taot_launch_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, int32_t B, float* d_plan,
-                         int32_t* d_iters, float* d_row_err, int32_t* d_info, float* d_kt, cudaStream_t st, float* d_tc, bool from_loads)
+                         int32_t* d_iters, float* d_row_err, int32_t* d_info, float* d_kt, cudaStream_t st, float* d_tc, bool from_loads,
+                         bool early)
 {
     const taot_params& p = h->p;
     SinkArgs a;
@@ -397,6 +399,7 @@ int taot_launch_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, in
     a.eps0 = p.eps0; a.max_iters = p.max_iters; a.tol = p.tol;
     a.check_every = p.check_every < 1 ? 1 : p.check_every;
     a.skip_solved = 0;
+    a.early = early ? 1 : 0;
     a.kt_global = h->kcap_global > 0 ? d_kt : nullptr;
     a.kcap_global = h->kcap_global;
     const int NT = p.R <= 32 ? 32 : (p.R <= 64 ? 128 : (p.R <= 128 ? 256 : (p.R <= 256 ? 512 : 1024)));

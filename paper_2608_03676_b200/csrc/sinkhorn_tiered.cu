@@ -138,6 +138,7 @@ sinkhorn_tiered_mw_kernel(SinkArgs a, TierCosts tc, int64_t nprob)
     const bool mainw = warp < kWarps;             // this warp owns ranks
     const int64_t b = blockIdx.x;
     taot_await();
+    if (a.early) taot_release();
     if (b >= nprob) return;
     double* alpha = reinterpret_cast<double*>(smem_raw);          // [R] potentials by rank (supply ranks; -inf elsewhere)
     double* beta = alpha + R;                                      // [R] (demand ranks)

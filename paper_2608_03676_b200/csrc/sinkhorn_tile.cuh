@@ -752,6 +752,7 @@ sinkhorn_tile_kernel(SinkArgs a, int64_t nprob)
     // one problem per CTA (a stride loop over the problems with a grid sized to the SMs was measured slower: the
     // set-up and write-out of one problem no longer overlap the iterations of the CTAs next to it)
     taot_await();
+    if (a.early) taot_release();
     if ((int64_t)blockIdx.x < nprob) tile_problem<NW, CG, RP0, RP1, RP2, TOLK>(a, sm, (int64_t)blockIdx.x);
 }
 

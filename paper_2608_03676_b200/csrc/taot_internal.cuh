@@ -110,7 +110,8 @@ int taot_launch_excess_spare(taot_handle_t h, const int32_t* d_rank_load, int32_
                              int32_t* d_spare, float* d_s, float* d_d, cudaStream_t st);
 int taot_launch_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, int32_t B, float* d_plan,
                          int32_t* d_iters, float* d_row_err, int32_t* d_info, float* d_kt, cudaStream_t st,
-                         float* d_tc = nullptr, bool from_loads = false);   // from_loads: called by taot_plan
+                         float* d_tc = nullptr, bool from_loads = false, bool early = false);   // from_loads: called by taot_plan; early: its kernels
+                                                                                       // let the matching kernel be set up beside them
 bool taot_sinkhorn_takes_classes(taot_handle_t h, bool from_loads);
 size_t taot_sinkhorn_tc_ws_floats(int32_t R, int32_t B);
 int taot_launch_sinkhorn_guard(taot_handle_t h, const float* d_s, const float* d_d, int32_t B, float* d_plan,
@@ -118,7 +119,8 @@ int taot_launch_sinkhorn_guard(taot_handle_t h, const float* d_s, const float* d
 int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expert_load,
                       const int32_t* d_rank_load, const float* d_plan, int32_t* d_slot_expert,
                       int32_t* d_slot_tokens, int32_t* d_X, int32_t* d_rounds, int32_t* d_info,
-                      int32_t* d_nrem, float* d_t12, cudaStream_t st, long long* d_cyc = nullptr);
+                      int32_t* d_nrem, float* d_t12, cudaStream_t st, long long* d_cyc = nullptr,
+                      bool early = false);   // early: behind a Phase 1 launched with `early`, see match_kernel
 int taot_launch_assign(taot_handle_t h, const int32_t* d_topk, void* ws, const int32_t* d_slot_expert,
                        const int32_t* d_X, int32_t* d_new_idx, int32_t* d_info, cudaStream_t st);
 
