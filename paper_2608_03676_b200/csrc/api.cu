@@ -71,6 +71,7 @@ void layout(taot_handle_t h)
     h->off_t12 = take(path * sizeof(float) * (size_t)p.L * p.E * 2 * p.R);
     h->off_kt = take(sizeof(float) * (size_t)p.L * (size_t)h->kcap_global);
     h->off_dc = take(path * sizeof(int32_t) * LR * h->nc * ((size_t)p.E + (size_t)p.R * p.K + 1));
+    h->off_wp = take(path * sizeof(uint16_t) * LR * h->nc * (TAOT_STREAM_THREADS / 32) * ((size_t)p.E + (size_t)p.R * p.K + 1));
     h->off_cyc = take(path * sizeof(long long) * (size_t)p.L * 16);
     h->off_tc = take((p.R > 256 && p.R % 128 == 0) ? sizeof(float) * taot_sinkhorn_tc_ws_floats(p.R, p.L) : 0);
     h->tb_ok = (path && p.E <= 256 && h->seg % 16 == 0) ? 1 : 0;
@@ -119,6 +120,7 @@ taot_handle_s* make_view(const taot_handle_s* h, int g, int l0, int Lg)
     v->off_nrem += 4 * l * dmax * R;
     v->off_t12 += 4 * l * E * 2 * R;
     v->off_dc += 4 * l * R * nc * (E + S + 1);
+    v->off_wp += 2 * l * R * nc * (TAOT_STREAM_THREADS / 32) * (E + S + 1);
     v->off_cyc += 8 * l * 16;
     v->off_tb += l * (size_t)p.T * p.k;
     v->off_tbflag += 4 * l * R * nc;
@@ -380,15 +382,14 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
     if (rc == TAOT_OK && R <= 256) {
         // targets (experts, then guest slots) in the order of the send buffer: by destination rank, then by index
         const int K = params->K, NT = E + R * K;
-        std::vector<int32_t> tdest(NT + 1), torder(NT + 1), tpos(NT + 1), fill(R + 1, 0);
+        std::vector<int32_t> tdest(NT + 1), torder(NT + 1), fill(R + 1, 0);
         for (int t = 0; t < NT; ++t) tdest[t] = t < E ? h_e2r[t] : (t - E) / K;
         tdest[NT] = R;
         for (int t = 0; t <= NT; ++t) fill[tdest[t]]++;
         int32_t run = 0;
         for (int q = 0; q <= R; ++q) { const int32_t c = fill[q]; fill[q] = run; run += c; }
-        for (int t = 0; t <= NT; ++t) { tpos[t] = fill[tdest[t]]++; torder[tpos[t]] = t; }   // ascending t inside a rank
-        rc = upload(&h->d_tpos, tpos.data(), tpos.size());
-        if (rc == TAOT_OK) rc = upload(&h->d_torder, torder.data(), torder.size());
+        for (int t = 0; t <= NT; ++t) torder[fill[tdest[t]]++] = t;   // ascending t inside a rank
+        rc = upload(&h->d_torder, torder.data(), torder.size());
         if (rc == TAOT_OK) rc = upload(&h->d_tdest, tdest.data(), tdest.size());
     }
     if (rc == TAOT_OK && h->ntiers > 0) rc = upload(&h->d_tiermask, tiermask.data(), tiermask.size());
@@ -519,7 +520,7 @@ int taot_destroy(taot_handle_t h)
     if (h->bstream) cudaStreamDestroy(h->bstream);
     cudaFree(h->d_e2r); cudaFree(h->d_C); cudaFree(h->d_B); cudaFree(h->d_rowlse0); cudaFree(h->d_gibbs);
     cudaFree(h->d_rank_off); cudaFree(h->d_rank_list); cudaFree(h->d_tierval); cudaFree(h->d_tiermask);
-    cudaFree(h->d_tpos); cudaFree(h->d_torder); cudaFree(h->d_tdest); cudaFree(h->d_bidlist); cudaFree(h->d_bident); cudaFree(h->d_hostcls);
+    cudaFree(h->d_torder); cudaFree(h->d_tdest); cudaFree(h->d_bidlist); cudaFree(h->d_bident); cudaFree(h->d_hostcls);
     cudaFree(h->d_merge_part); cudaFree(h->d_merge_cnt);
     cudaFree(h->d_cls_lse0);                       // and the other four arrays of the block
     for (int i = 0; i < 6; ++i)

@@ -3,17 +3,18 @@
 // entries execute on each rank, how many go to each target (expert or guest slot), and the position of every
 // entry in the rank's send buffer ordered by (destination rank, target, original order) -- a stable counting
 // sort with E + S keys, done as three passes over chunks of <= 16384 entries:
-//   hist_chunk_kernel        (histogram.cu) one CTA per chunk: histogram of the chunk over the E + S targets,
-//                            with one more bin for values that are no target
+//   dispatch_count_kernel    one CTA per chunk, every warp over its own contiguous span: counts over the E + S targets, with
+//                            one more bin for values that are no target, and their sums over the spans before
 //   dispatch_offsets_kernel  one CTA per (layer, source rank): totals, exclusive scan in destination order,
 //                            per-chunk bases (in place), send counts per destination rank
-//   dispatch_scatter_kernel  one CTA per chunk: per-warp histograms of the warp's contiguous span, bases per
-//                            warp, then each warp walks its span in order, 32 entries at a time; the lanes with
+//   dispatch_scatter_kernel  one CTA per chunk: each warp walks its span in order, 32 entries at a time; the lanes with
 //                            the same target inside a step are found by OR-ing lane bits into a shared-memory
-//                            word per target and ranked by lane, so the order stays stable; the lowest lane of
-//                            a group hands the group's running position to the others by a shuffle (one warp
-//                            barrier per step; the mask words of consecutive steps sit in alternating rows)
-// 12 bytes of HBM traffic per entry (two reads of the table, one write of the positions).
+//                            word per target and ranked by lane, so the order stays stable
+// 12 bytes of HBM traffic per entry (two reads of the table, one write of the positions), but what bounds it is random access
+// to shared memory: 32 lanes on 385 targets meet in the same bank 3.3 deep, and a step makes five such accesses beside the
+// count's one.  The count is made by warp, so that the scatter need not count its spans again: 64 ranks x 58 layers (1 GB)
+// 877 -> 757 us.  (One cluster per segment that reads the table once was built and made the same accesses in the same time:
+// 0.83 to 1.05 ms at 64 ranks x 58 layers; finding the lanes by votes 1.05, by match 1.8 ms.)
 #include "taot_internal.cuh"
 
 namespace {
@@ -25,7 +26,7 @@ constexpr int kWarpSpan = TAOT_CHUNK / kWarps;
 struct DispatchArgs {
     const int32_t* idx;        // [L,T,k] rewritten routing table
     int32_t* dc;               // [L,R,NC,NB] chunk counts, then chunk bases
-    const int32_t* tpos;       // [NB] sorted position of each bin
+    uint16_t* wp;              // [L,R,NC,kWarps,NB] entries of the bin in the spans of the chunk before this warp's
     const int32_t* torder;     // [NB] bin at each sorted position
     const int32_t* tdest;      // [NB] destination rank of each bin (R for the undeliverable bin)
     int32_t* send_counts;      // [L,R,R]
@@ -33,7 +34,8 @@ struct DispatchArgs {
     int32_t* perm;             // [L,T,k]
     int32_t* info;
     int64_t layer_elems, seg;
-    int32_t nc, R, NB, nbits;  // nbits: bits needed for a bin index in [0, NB)
+    int32_t nc, R, NB;
+    int32_t vec_ok;            // the table's chunks start on 16-byte boundaries
 };
 
 __device__ __forceinline__ void chunk_span(const DispatchArgs& a, int64_t id, int64_t& goff, int32_t& len)
@@ -46,6 +48,58 @@ __device__ __forceinline__ void chunk_span(const DispatchArgs& a, int64_t id, in
 }
 
 __device__ __forceinline__ int bin_of(int32_t v, int NB) { return (unsigned)v < (unsigned)(NB - 1) ? v : NB - 1; }
+
+__device__ __forceinline__ void count_add(uint32_t addr) { asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory"); }
+
+// Counts of a chunk by warp, each over its contiguous span, and from them the chunk's counts and the sums over the spans
+// before each warp's.  (At most 16384 entries before a span: 16 bits.)
+__global__ void __launch_bounds__(kThreads)
+dispatch_count_kernel(DispatchArgs a)
+{
+    extern __shared__ int32_t wh[];            // [kWarps][NB]
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NB = a.NB;
+    const int64_t id = blockIdx.x;
+    int64_t goff; int32_t len;
+    chunk_span(a, id, goff, len);
+    for (int q = tid; q < kWarps * NB; q += kThreads) wh[q] = 0;
+    __syncthreads();
+    taot_await();
+    taot_release();
+    const int s0 = warp * kWarpSpan, n = min(len - s0, kWarpSpan);
+    const int32_t* src = a.idx + goff + s0;
+    const uint32_t mine = (uint32_t)__cvta_generic_to_shared(wh + warp * NB);
+    int i = 0;
+    if (a.vec_ok && n == kWarpSpan) {
+        const int4* src4 = reinterpret_cast<const int4*>(src) + lane;
+#pragma unroll 1
+        for (int h = 0; h < kWarpSpan / 128; h += 8) {
+            int4 x[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) x[u] = __ldcs(src4 + (h + u) * 32);
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                count_add(mine + 4u * (uint32_t)bin_of(x[u].x, NB));
+                count_add(mine + 4u * (uint32_t)bin_of(x[u].y, NB));
+                count_add(mine + 4u * (uint32_t)bin_of(x[u].z, NB));
+                count_add(mine + 4u * (uint32_t)bin_of(x[u].w, NB));
+            }
+        }
+        i = kWarpSpan;
+    }
+    for (i += lane; i < n; i += 32) count_add(mine + 4u * (uint32_t)bin_of(__ldcs(src + i), NB));
+    __syncthreads();
+    int32_t* out = a.dc + id * NB;
+    uint16_t* wp = a.wp + id * kWarps * NB;
+    for (int b = tid; b < NB; b += kThreads) {
+        int32_t run = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) {
+            wp[w * NB + b] = (uint16_t)run;
+            run += wh[w * NB + b];
+        }
+        out[b] = run;
+    }
+}
 
 __global__ void __launch_bounds__(kThreads)
 dispatch_offsets_kernel(DispatchArgs a)
@@ -104,75 +158,81 @@ dispatch_offsets_kernel(DispatchArgs a)
     if (tid == 0 && sc[R] != 0) atomicOr(a.info + (int32_t)(lr / R), TAOT_INFO_BAD_INDEX);
 }
 
-// ALT: the mask words of consecutive ranking steps sit in alternating rows (one warp barrier per step); otherwise one
-// row and a second barrier per step, for target counts whose three rows would not fit in shared memory.
+// ALT: the mask words of consecutive ranking steps sit in alternating rows (one warp barrier fewer per step); otherwise one
+// row, for target counts whose three rows would not fit in shared memory.
 template <bool ALT>
 __global__ void __launch_bounds__(kThreads)
 dispatch_scatter_kernel(DispatchArgs a)
 {
-    extern __shared__ int32_t wh[];            // [kWarps][NB]: counts of the warp's span, then running positions;
+    extern __shared__ int32_t wh[];            // [kWarps][NB]: running positions;
                                                // then (ALT: 2 x) [kWarps][NB] lane masks of the steps being ranked
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NB = a.NB;
     const int64_t id = blockIdx.x;
     int64_t goff; int32_t len;
     chunk_span(a, id, goff, len);
-    const int32_t* src = a.idx + goff;
-    int32_t* dst = a.perm + goff;
-    for (int q = tid; q < (ALT ? 3 : 2) * kWarps * NB; q += kThreads) wh[q] = 0;
-    __syncthreads();
+    const int s0 = warp * kWarpSpan, n = min(len - s0, kWarpSpan);
+    const int32_t* src = a.idx + goff + s0;
+    int32_t* dst = a.perm + goff + s0;
+    for (int q = kWarps * NB + tid; q < (ALT ? 3 : 2) * kWarps * NB; q += kThreads) wh[q] = 0;
     taot_await();
-    const int s0 = warp * kWarpSpan, s1 = min(len, s0 + kWarpSpan);
-    int32_t* mine = wh + warp * NB;
-    unsigned* mask = reinterpret_cast<unsigned*>(wh + (kWarps + warp) * NB);
-#pragma unroll 8
-    for (int i = s0 + lane; i < s1; i += 32) atomicAdd(&mine[bin_of(__ldg(src + i), NB)], 1);
-    __syncthreads();
-    const int32_t* base = a.dc + id * (int64_t)NB;
-    for (int b = tid; b < NB; b += kThreads) {
-        int32_t run = base[b];
+    {
+        const int32_t* base = a.dc + id * (int64_t)NB;
+        const uint16_t* wp = a.wp + id * kWarps * (int64_t)NB;
+        for (int b = tid; b < NB; b += kThreads) {
+            const int32_t first = base[b];
+            uint32_t before[kWarps];
 #pragma unroll
-        for (int w = 0; w < kWarps; ++w) {
-            const int32_t t = wh[w * NB + b];
-            wh[w * NB + b] = run;
-            run += t;
+            for (int w = 0; w < kWarps; ++w) before[w] = wp[w * NB + b];
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) wh[w * NB + b] = first + (int32_t)before[w];
         }
     }
     __syncthreads();
-    const unsigned lt = (1u << lane) - 1u;
-    constexpr int U = 4;
-    unsigned* mask2 = ALT ? mask + kWarps * NB : mask;      // the second set of mask rows: steps alternate between the two
-    for (int i0 = s0; i0 < s1; i0 += 32 * U) {
-        int32_t v[U];
+    const unsigned bit = 1u << lane, lt = bit - 1u;
+    int32_t* const mine = wh + warp * NB;
+    const uint32_t a_pos = (uint32_t)__cvta_generic_to_shared(mine);
+    const uint32_t a_mask = a_pos + 4u * (uint32_t)(kWarps * NB), a_alt = ALT ? 4u * (uint32_t)(kWarps * NB) : 0u;
+    constexpr int U = 8;
+    int i0 = 0;
+    // Whole steps of 32 entries, every lane the same instructions: OR my bit into the target's word (a set: the order does not
+    // matter), read the word and the target's running position, then all of a target's lanes store the same new position and
+    // clear the word.  The word is next written two steps later (ALT), the position next read behind the next barrier.
+    for (; i0 + 32 * U <= n; i0 += 32 * U) {
+        uint32_t b4[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) b4[u] = 4u * (uint32_t)bin_of(__ldcs(src + i0 + u * 32 + lane), NB);
 #pragma unroll
         for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * 32 + lane;
-            v[u] = i < s1 ? __ldg(src + i) : 0;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-            const int i = i0 + u * 32 + lane;
-            const bool ok = i < s1;
-            const int b = ok ? bin_of(v[u], NB) : 0;
-            unsigned* mrow = (u & 1) ? mask2 : mask;
-            // the lanes of this step that share my target: every lane ORs its bit into the target's word of the
-            // warp's mask row (a set, so the result does not depend on the order of the atomics)
-            if (ok) atomicOr(&mrow[b], 1u << lane);
+            const uint32_t am = a_mask + ((u & 1) ? a_alt : 0u) + b4[u], ap = a_pos + b4[u];
+            asm volatile("red.shared.or.b32 [%0], %1;" ::"r"(am), "r"(bit) : "memory");
             __syncwarp();
-            const unsigned peers = ok ? mrow[b] : (1u << lane);
-            // the lowest lane of a group reads the group's running position and hands it to the others by a shuffle,
-            // which every lane reaches with its copy of the word read; only then does that lane move the position on
-            // and clear the word.  The word is next written two steps later (the rows alternate) and the running
-            // position is next read after the next step's barrier.
-            const bool lead = ok && (peers & lt) == 0;
-            int32_t first = lead ? mine[b] : 0;
-            first = __shfl_sync(0xffffffffu, first, __ffs(peers) - 1);
-            if (lead) {
-                mine[b] = first + __popc(peers);
-                mrow[b] = 0u;
-            }
-            if (ok) dst[i] = first + __popc(peers & lt);
-            if (!ALT) __syncwarp();              // the cleared word is written again in the very next step
+            uint32_t peers, first;
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(peers) : "r"(am) : "memory");
+            asm volatile("ld.shared.u32 %0, [%1];" : "=r"(first) : "r"(ap) : "memory");
+            __syncwarp();
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(am), "r"(0u) : "memory");
+            asm volatile("st.shared.u32 [%0], %1;" ::"r"(ap), "r"(first + (uint32_t)__popc(peers)) : "memory");
+            if (!ALT) __syncwarp();
+            __stcs(dst + i0 + u * 32 + lane, (int32_t)(first + (uint32_t)__popc(peers & lt)));
         }
+    }
+    __syncwarp();
+    for (; i0 < n; i0 += 32) {                 // what is left of a short span
+        const int i = i0 + lane;
+        const bool ok = i < n;
+        const int b = ok ? bin_of(__ldcs(src + i), NB) : 0;
+        unsigned* const word = reinterpret_cast<unsigned*>(mine + kWarps * NB) + b;
+        if (ok) atomicOr(word, bit);
+        __syncwarp();
+        const unsigned peers = ok ? *word : bit;
+        const int32_t first = mine[b];
+        __syncwarp();
+        if (ok) {
+            *word = 0u;
+            mine[b] = first + __popc(peers);
+            dst[i] = first + __popc(peers & lt);
+        }
+        __syncwarp();
     }
 }
 
@@ -185,19 +245,20 @@ int taot_launch_dispatch(taot_handle_t h, const int32_t* d_new_idx, int32_t* d_s
     DispatchArgs a;
     a.idx = d_new_idx;
     a.dc = reinterpret_cast<int32_t*>(static_cast<char*>(ws) + h->off_dc);
-    a.tpos = h->d_tpos; a.torder = h->d_torder; a.tdest = h->d_tdest;
+    a.wp = reinterpret_cast<uint16_t*>(static_cast<char*>(ws) + h->off_wp);
+    a.torder = h->d_torder; a.tdest = h->d_tdest;
     a.send_counts = d_send_counts; a.target_counts = d_target_counts; a.perm = d_perm; a.info = d_info;
     a.layer_elems = p.T * p.k; a.seg = h->seg; a.nc = h->nc; a.R = p.R; a.NB = p.E + p.R * p.K + 1;
     const unsigned chunks = (unsigned)((int64_t)p.L * p.R * h->nc);
-    a.nbits = 1;
-    while ((1 << a.nbits) < a.NB) ++a.nbits;
+    a.vec_ok = ((reinterpret_cast<uintptr_t>(d_new_idx) & 15) == 0 && h->seg % 4 == 0) ? 1 : 0;
+    const size_t sm1 = sizeof(int32_t) * (size_t)kWarps * a.NB;
     const size_t sm2 = sizeof(int32_t) * (2 * (size_t)a.NB + p.R + 1);
     const bool alt = sizeof(int32_t) * 3 * (size_t)kWarps * a.NB <= 64 * 1024;
     const size_t sm3 = sizeof(int32_t) * (alt ? 3 : 2) * (size_t)kWarps * a.NB;
     if (alt) TAOT_CUDA_OK(cudaFuncSetAttribute(dispatch_scatter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3));
     else TAOT_CUDA_OK(cudaFuncSetAttribute(dispatch_scatter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3));
-    const int rc = taot_launch_chunk_counts(h, d_new_idx, a.dc, d_info, a.NB - 1, st);
-    if (rc < 0) return rc;
+    TAOT_CUDA_OK(cudaFuncSetAttribute(dispatch_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
+    TAOT_CUDA_OK(taot_launch_chained(dispatch_count_kernel, chunks, kThreads, sm1, st, a));
     TAOT_CUDA_OK(taot_launch_chained(dispatch_offsets_kernel, (unsigned)((int64_t)p.L * p.R), kThreads, sm2, st, a));
     if (alt) TAOT_CUDA_OK(taot_launch_chained(dispatch_scatter_kernel<true>, chunks, kThreads, sm3, st, a));
     else TAOT_CUDA_OK(taot_launch_chained(dispatch_scatter_kernel<false>, chunks, kThreads, sm3, st, a));

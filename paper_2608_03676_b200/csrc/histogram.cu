@@ -28,12 +28,11 @@ __device__ __forceinline__ int4 ld_stream(const int4* p)
     return v;
 }
 
-// EXTRA == false: out-of-range values are only flagged; true: they are also counted, in bin E (rows of E + 1 bins)
-template <bool EXTRA>
+// (out-of-range values are only flagged)
 __device__ __forceinline__ void count_one(int32_t* hist, int32_t e, int32_t E, int& bad)
 {
     if ((uint32_t)e < (uint32_t)E) atomicAdd(hist + e, 1);
-    else { bad = 1; if (EXTRA) atomicAdd(hist + E, 1); }
+    else bad = 1;
 }
 
 // four entries as four bytes (E <= 256; a value that is no expert leaves a byte nobody reads: its chunk is flagged)
@@ -45,14 +44,12 @@ __device__ __forceinline__ uint32_t pack_bytes(const int4& x)
 // tb (may be null; only with vec_ok): the table again as one byte per entry, written beside the counts, and tbflag:
 // one word per chunk, nonzero if the chunk holds a value that is no expert.  The reassignment reads these 1-byte
 // entries instead of the table (a quarter of the bytes) wherever the chunk's flag is zero.
-template <bool EXTRA>
 __global__ void __launch_bounds__(kThreads)
 hist_chunk_kernel(const int32_t* __restrict__ topk, int32_t* __restrict__ cc, int32_t* __restrict__ info,
                   int64_t layer_elems, int64_t seg, int32_t nc, int32_t R, int32_t E, int vec_ok,
                   uint8_t* __restrict__ tb, int32_t* __restrict__ tbflag)
 {
-    const int32_t nb = EXTRA ? E + 1 : E;
-    extern __shared__ int32_t sh_hist[];                 // [kWarps][nb]
+    extern __shared__ int32_t sh_hist[];                 // [kWarps][E]
     const int tid = threadIdx.x, warp = tid >> 5;
     const int64_t id = blockIdx.x;
     const int32_t c = (int32_t)(id % nc);
@@ -62,13 +59,13 @@ hist_chunk_kernel(const int32_t* __restrict__ topk, int32_t* __restrict__ cc, in
     const int64_t start = (int64_t)c * TAOT_CHUNK;
     const int32_t len = (int32_t)((seg - start) < (int64_t)TAOT_CHUNK ? (seg - start) : (int64_t)TAOT_CHUNK);
     const int32_t* src = topk + (int64_t)l * layer_elems + (int64_t)r * seg + start;
-    uint32_t* tb4 = (!EXTRA && tb) ? reinterpret_cast<uint32_t*>(tb + (int64_t)l * layer_elems + (int64_t)r * seg + start) : nullptr;
+    uint32_t* tb4 = tb ? reinterpret_cast<uint32_t*>(tb + (int64_t)l * layer_elems + (int64_t)r * seg + start) : nullptr;
 
-    for (int i = tid; i < kWarps * nb; i += kThreads) sh_hist[i] = 0;
+    for (int i = tid; i < kWarps * E; i += kThreads) sh_hist[i] = 0;
     __syncthreads();
     taot_await();
     taot_release();
-    int32_t* hist = sh_hist + warp * nb;
+    int32_t* hist = sh_hist + warp * E;
     int bad = 0;
 
     if (vec_ok) {
@@ -80,36 +77,36 @@ hist_chunk_kernel(const int32_t* __restrict__ topk, int32_t* __restrict__ cc, in
             int4 x[8];
 #pragma unroll
             for (int u = 0; u < 8; ++u) x[u] = ld_stream(src4 + v + u * kThreads);
-            if (!EXTRA && tb4) {
+            if (tb4) {
 #pragma unroll
                 for (int u = 0; u < 8; ++u) tb4[v + u * kThreads] = pack_bytes(x[u]);
             }
 #pragma unroll
             for (int u = 0; u < 8; ++u) {
-                count_one<EXTRA>(hist, x[u].x, E, bad); count_one<EXTRA>(hist, x[u].y, E, bad);
-                count_one<EXTRA>(hist, x[u].z, E, bad); count_one<EXTRA>(hist, x[u].w, E, bad);
+                count_one(hist, x[u].x, E, bad); count_one(hist, x[u].y, E, bad);
+                count_one(hist, x[u].z, E, bad); count_one(hist, x[u].w, E, bad);
             }
         }
         for (; v < nvec; v += kThreads) {
             const int4 x = ld_stream(src4 + v);
-            if (!EXTRA && tb4) tb4[v] = pack_bytes(x);
-            count_one<EXTRA>(hist, x.x, E, bad); count_one<EXTRA>(hist, x.y, E, bad);
-            count_one<EXTRA>(hist, x.z, E, bad); count_one<EXTRA>(hist, x.w, E, bad);
+            if (tb4) tb4[v] = pack_bytes(x);
+            count_one(hist, x.x, E, bad); count_one(hist, x.y, E, bad);
+            count_one(hist, x.z, E, bad); count_one(hist, x.w, E, bad);
         }
-        for (int32_t i = (nvec << 2) + tid; i < len; i += kThreads) count_one<EXTRA>(hist, src[i], E, bad);
+        for (int32_t i = (nvec << 2) + tid; i < len; i += kThreads) count_one(hist, src[i], E, bad);
     } else {
-        for (int32_t i = tid; i < len; i += kThreads) count_one<EXTRA>(hist, src[i], E, bad);
+        for (int32_t i = tid; i < len; i += kThreads) count_one(hist, src[i], E, bad);
     }
     const int any_bad = __syncthreads_or(bad);
-    int32_t* out = cc + id * nb;
-    for (int e = tid; e < nb; e += kThreads) {
+    int32_t* out = cc + id * E;
+    for (int e = tid; e < E; e += kThreads) {
         int32_t tot = 0;
 #pragma unroll
-        for (int w = 0; w < kWarps; ++w) tot += sh_hist[w * nb + e];
+        for (int w = 0; w < kWarps; ++w) tot += sh_hist[w * E + e];
         out[e] = tot;
     }
     if (info && any_bad && tid == 0) atomicOr(info + l, TAOT_INFO_BAD_INDEX);
-    if (!EXTRA && tbflag && tid == 0) tbflag[id] = any_bad;
+    if (tbflag && tid == 0) tbflag[id] = any_bad;
 }
 
 // excess / spare of one row of rank loads held in shared memory (Appendix A.1, integer mean)
@@ -278,25 +275,8 @@ int taot_launch_histogram(taot_handle_t h, const int32_t* d_topk, int32_t* d_cc,
     const bool bytes = ws && h->tb_ok && vec_ok;
     uint8_t* tb = (bytes && write_bytes) ? reinterpret_cast<uint8_t*>(static_cast<char*>(ws) + h->off_tb) : nullptr;
     int32_t* tbflag = ws ? reinterpret_cast<int32_t*>(static_cast<char*>(ws) + h->off_tbflag) : nullptr;
-    TAOT_CUDA_OK(taot_launch_chained(hist_chunk_kernel<false>, (unsigned)blocks, kThreads, smem, st, d_topk, d_cc, d_info, layer_elems,
+    TAOT_CUDA_OK(taot_launch_chained(hist_chunk_kernel, (unsigned)blocks, kThreads, smem, st, d_topk, d_cc, d_info, layer_elems,
                                      h->seg, h->nc, p.R, p.E, vec_ok, tb, tbflag));
-    return 1;
-}
-
-// The same chunk histogram over `bins` values with one more bin for everything out of range (rows of bins + 1
-// counts): the counting pass of the dispatch metadata, where the table holds experts and guest slots.
-int taot_launch_chunk_counts(taot_handle_t h, const int32_t* d_idx, int32_t* d_counts, int32_t* d_info, int32_t bins,
-                             cudaStream_t st)
-{
-    const taot_params& p = h->p;
-    const int64_t blocks = (int64_t)p.L * p.R * h->nc;
-    const int vec_ok = ((reinterpret_cast<uintptr_t>(d_idx) & 15) == 0) && (h->seg % 4 == 0);
-    const size_t smem = sizeof(int32_t) * kWarps * (size_t)(bins + 1);
-    // the default limit is 48 KB
-    if (smem > 48 * 1024)
-        TAOT_CUDA_OK(cudaFuncSetAttribute(hist_chunk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    TAOT_CUDA_OK(taot_launch_chained(hist_chunk_kernel<true>, (unsigned)blocks, kThreads, smem, st, d_idx, d_counts, d_info,
-                                     (int64_t)p.T * p.k, h->seg, h->nc, p.R, bins, vec_ok, nullptr, nullptr));
     return 1;
 }
 

@@ -32,7 +32,6 @@ struct taot_handle_s {
     int32_t* d_rank_off;     // [R+1] CSR of experts by home rank
     int32_t* d_rank_list;    // [E]
     uint32_t* d_tiermask;    // [ntiers][W][R hosts] bit r of word w set iff bonus(32w + r -> host) == tierval[t]; null if ntiers == 0
-    int32_t* d_tpos;         // [E+S+1] position of each target in (destination rank, target) order; last = undeliverable
     int32_t* d_torder;       // [E+S+1] target at each position
     int32_t* d_tdest;        // [E+S+1] destination rank of each target (R for the undeliverable bin)
     float* d_tierval;        // [ntiers] distinct values of the auction bonus matrix, descending
@@ -62,7 +61,7 @@ struct taot_handle_s {
     int32_t kcap;            // Sinkhorn kernel-matrix capacity in floats per problem (shared memory)
     int64_t kcap_global;     // same, global-memory scratch per problem (R > 256 only), else 0
     // workspace layout (byte offsets)
-    size_t off_cc, off_excess, off_spare, off_s, off_d, off_nrem, off_t12, off_kt, off_dc, off_cyc, off_tc;
+    size_t off_cc, off_excess, off_spare, off_s, off_d, off_nrem, off_t12, off_kt, off_dc, off_wp, off_cyc, off_tc;
     size_t off_tb, off_tbflag;   // one-byte copy of the routing table (see tb_ok) and one flag per chunk (a value that is no expert)
     int32_t tb_ok;               // 1: the histogram pass also leaves the table as one byte per entry (E <= 256 experts,
                                  // segments of a multiple of 16 entries) for the reassignment to read instead of the table
@@ -129,8 +128,6 @@ int taot_launch_report(taot_handle_t h, const int32_t* d_expert_load, const int3
                        int32_t* d_spill, int32_t* d_load_after, int32_t* d_slot_moved, int32_t* d_slot_kind,
                        cudaStream_t st);
 
-int taot_launch_chunk_counts(taot_handle_t h, const int32_t* d_idx, int32_t* d_counts, int32_t* d_info, int32_t bins,
-                             cudaStream_t st);
 int taot_launch_dispatch(taot_handle_t h, const int32_t* d_new_idx, int32_t* d_send_counts, int32_t* d_target_counts,
                          int32_t* d_perm, int32_t* d_info, void* ws, cudaStream_t st);
 
