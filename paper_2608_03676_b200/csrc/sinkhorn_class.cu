@@ -20,10 +20,11 @@
 // window is taken again in the log domain in fp64, so no problem is handed on except one that has a rank with both
 // supply and demand.
 //
-// Measured (B200, 500 iterations, whole call): 64 ranks, one problem 124 -> 59 us (register tile before; 150 cycles per
-// iteration against 370); 256 ranks, 1024 problems 283 -> 139 us; 1024 ranks, 64 problems 375 -> 162 us (tier sums over
-// eight warps before; 360 cycles per iteration against 1400).  What is left at 1024 ranks: 90 us of iterations, 48 us to
-// write 268 MB of plan (hidden but for the supply rows), 15 us of fp64 set-up and folds.
+// Measured (B200, 500 iterations, whole call): 64 ranks, one problem 125 -> 56 us (register tile before; 150 cycles per
+// iteration against 370); 256 ranks, 1024 problems 283 -> 137 to 148 us; 1024 ranks, 64 problems 373 -> 160 us (tier sums over
+// eight warps before; 340 cycles per iteration against 1400; of the last 18 us, clusters that share the supply rows and
+// fp32 exponentials in the log-domain half-steps).  What is left at 1024 ranks: 87 us of iterations, the rest loading,
+// the log-domain half-steps and the supply rows, which only the SMs of the problem can write.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -89,7 +90,8 @@ struct ClassArgs {
     const float* cost;        // dense kernel: [NC][NC] cost between classes; tree kernel: unused
     double c1, c2, c3;        // tree kernel: cost / eps inside a class, inside a group, elsewhere
     int32_t wide;             // rows of the plan can be written 16 bytes at a time
-    int32_t solvers;          // CTAs that solve; any beyond them write the rows without supply
+    int32_t solvers;          // CTAs of the problems; any beyond them write the rows without supply
+    int32_t cluster;          // tree kernel: CTAs per problem
 };
 
 // what a problem's solve leaves in shared memory for the warps that write the plan
@@ -657,6 +659,18 @@ __device__ __forceinline__ double warp_max(double v)
 }
 __device__ __forceinline__ float exp_or_zero(double x) { return x == -INFINITY ? 0.0f : exp_split(x); }
 
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// the same word of the shared memory of the cluster's first CTA
+__device__ __forceinline__ float leader_f32(const float* p)
+{
+    uint32_t at;
+    float v;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(at) : "r"((uint32_t)__cvta_generic_to_shared(p)));
+    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(at) : "memory");
+    return v;
+}
+
 template <int GPL, int NPG, bool TOL, int PPC>
 __global__ void __launch_bounds__(kThreads)
 sinkhorn_class_tree_kernel(ClassArgs k, int64_t nprob)
@@ -665,7 +679,10 @@ sinkhorn_class_tree_kernel(ClassArgs k, int64_t nprob)
     const SinkArgs& a = k.a;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int R = a.R, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int64_t b0 = (int64_t)blockIdx.x * PPC;
+    // PPC == 1: the problem's CTA may lead a cluster (k.cluster CTAs): the others write the rows without supply meanwhile
+    // and, once it is solved, their share of the supply rows, from factors they fetch from the leader
+    const int crank = PPC == 1 ? (int)(blockIdx.x % k.cluster) : 0, csize = PPC == 1 ? (int)k.cluster : 1;
+    const int64_t b0 = (int64_t)blockIdx.x / csize * PPC;
     taot_await();
     if (blockIdx.x >= k.solvers) {
         zero_rows_of_batch(a, nprob, k.wide, (int64_t)(blockIdx.x - k.solvers) * (kThreads / 32) + warp,
@@ -682,7 +699,7 @@ sinkhorn_class_tree_kernel(ClassArgs k, int64_t nprob)
     __shared__ int32_t off[NS + 1];
     __shared__ Verdict ver[PPC];
 
-    if (tid < PPC) { ver[tid].flags = 0; ver[tid].state = 1; }
+    if (tid < PPC) { ver[tid].flags = 0; ver[tid].state = 1; ver[tid].info = 0; }
     __syncthreads();
 #pragma unroll
     for (int p = 0; p < PPC; ++p)
@@ -690,9 +707,11 @@ sinkhorn_class_tree_kernel(ClassArgs k, int64_t nprob)
     for (int i = tid; i < R; i += kThreads) { cls[i] = k.cls[i]; list[i] = k.list[i]; }
     for (int i = tid; i <= NS; i += kThreads) off[i] = k.off[i];
     __syncthreads();
-    class_masses<PPC>(k, off, list, st, dm, 3 * R, NS, mS, mD, nprob - b0, ver);
+    if (crank == 0) class_masses<PPC>(k, off, list, st, dm, 3 * R, NS, mS, mD, nprob - b0, ver);
 
-    if (warp < PPC) {
+    if (crank > 0) {
+        zero_rows(a.plan + b0 * (int64_t)R * R, st, R, k.wide, (crank - 1) * (kThreads / 32) + warp, (csize - 1) * (kThreads / 32));
+    } else if (warp < PPC) {
         if (b0 + warp < nprob) {
             TreeSmem<NS>& m = sm[warp];
             const int slot0 = lane * NPL;
@@ -722,45 +741,62 @@ sinkhorn_class_tree_kernel(ClassArgs k, int64_t nprob)
                 // one half-step in the log domain, by tiers (each lane only reads and writes its own slots)
                 auto exact_half = [&](const bool rows) {
                     const unsigned src = rows ? cold : hot, dst = rows ? hot : cold;
+                    // (exponentials as fp32 factors of an exact fp64 scale, and no branch around any of them: with fp64 exp
+                    // behind branches a half-step took 5 us)
                     double lt[NPL], gm[GPL], gs[GPL];       // log terms of the other side, their group maxima and sums
+                    float F[GPL];
                     double tm = -INFINITY;
 #pragma unroll
-                    for (int i = 0; i < NPL; ++i)
-                        lt[i] = ((src >> i) & 1u) ? log((double)(rows ? m.D[slot0 + i] : m.S[slot0 + i])) + (rows ? m.be[slot0 + i] : m.al[slot0 + i]) : -INFINITY;
+                    for (int i = 0; i < NPL; ++i) {
+                        const bool on = (src >> i) & 1u;
+                        const double l = log(on ? (double)(rows ? m.D[slot0 + i] : m.S[slot0 + i]) : 1.0) + (rows ? m.be[slot0 + i] : m.al[slot0 + i]);
+                        lt[i] = on ? l : -INFINITY;
+                    }
 #pragma unroll
                     for (int g = 0; g < GPL; ++g) {
                         gm[g] = -INFINITY; gs[g] = 0.0;
 #pragma unroll
                         for (int n = 0; n < NPG; ++n) gm[g] = fmax(gm[g], lt[g * NPG + n]);
+                        const double base = gm[g] > -INFINITY ? gm[g] : 0.0;
 #pragma unroll
-                        for (int n = 0; n < NPG; ++n)
-                            if (lt[g * NPG + n] > -INFINITY) gs[g] += exp(lt[g * NPG + n] - gm[g]);
+                        for (int n = 0; n < NPG; ++n) {
+                            const float w = exp_or_zero(lt[g * NPG + n] - base);
+                            m.e1[slot0 + g * NPG + n] = w;
+                            gs[g] += (double)w;
+                        }
                         tm = fmax(tm, gm[g]);
                     }
                     tm = warp_max(tm);
+                    const double tbase = tm > -INFINITY ? tm : 0.0;
                     double ts = 0.0;
 #pragma unroll
-                    for (int g = 0; g < GPL; ++g)
-                        if (gm[g] > -INFINITY) ts += exp(gm[g] - tm) * gs[g];
+                    for (int g = 0; g < GPL; ++g) {
+                        F[g] = exp_or_zero(gm[g] - tbase);
+                        ts += (double)F[g] * gs[g];
+                    }
                     ts = warp_sum(ts);
 #pragma unroll 1
                     for (int i = 0; i < NPL; ++i) {
-                        if (!((dst >> i) & 1u)) continue;
                         const int g = i / NPG;
-                        double own = -INFINITY, grp = 0.0, gmi = -INFINITY, gsi = 0.0;
-                        for (int j = 0; j < NPL; ++j) {
-                            if (j == i) own = lt[j];
-                            else if (j / NPG == g && lt[j] > -INFINITY) grp += exp(lt[j] - gm[g]);
-                        }
-                        gmi = gm[g]; gsi = gs[g];
-                        const double rest = ts - (gmi > -INFINITY ? exp(gmi - tm) * gsi : 0.0);
+                        double own = lt[0], gmi = gm[0], gsi = gs[0];
+                        float Fi = F[0];
+#pragma unroll
+                        for (int j = 1; j < NPL; ++j) own = j == i ? lt[j] : own;
+#pragma unroll
+                        for (int j = 1; j < GPL; ++j)
+                            if (j == g) { gmi = gm[j]; gsi = gs[j]; Fi = F[j]; }
+                        double grp = 0.0;
+#pragma unroll
+                        for (int n = 0; n < NPG; ++n) grp += g * NPG + n != i ? (double)m.e1[slot0 + g * NPG + n] : 0.0;
+                        const double rest = ts - (double)Fi * gsi;
                         const double l1 = own - k.c1;
-                        const double l2 = grp > 0.0 ? gmi + log(grp) - k.c2 : -INFINITY;
-                        const double l3 = rest > 0.0 ? tm + log(rest) - k.c3 : -INFINITY;
-                        const double mx = fmax(l1, fmax(l2, l3));
-                        const double sum = (l1 > -INFINITY ? exp(l1 - mx) : 0.0) + (l2 > -INFINITY ? exp(l2 - mx) : 0.0) +
-                                           (l3 > -INFINITY ? exp(l3 - mx) : 0.0);
-                        (rows ? m.al : m.be)[slot0 + i] = -(mx + log(sum));
+                        const double g2 = log(grp > 0.0 ? grp : 1.0), g3 = log(rest > 0.0 ? rest : 1.0);
+                        const double l2 = grp > 0.0 ? gmi + g2 - k.c2 : -INFINITY;
+                        const double l3 = rest > 0.0 ? tm + g3 - k.c3 : -INFINITY;
+                        const double mx = fmax(l1, fmax(l2, l3)), base = mx > -INFINITY ? mx : 0.0;
+                        const double sum = (double)exp_or_zero(l1 - base) + (double)exp_or_zero(l2 - base) + (double)exp_or_zero(l3 - base);
+                        const double res = -(mx + log(sum > 0.0 ? sum : 1.0));
+                        if ((dst >> i) & 1u) (rows ? m.al : m.be)[slot0 + i] = res;
                     }
                     __syncwarp();
                 };
@@ -867,7 +903,7 @@ sinkhorn_class_tree_kernel(ClassArgs k, int64_t nprob)
                 for (int i = 0; i < NPL; ++i) m.yc[slot0 + i] = x[i];
             }
         }
-    } else if (gridDim.x == k.solvers) {
+    } else if (gridDim.x == k.solvers && csize == 1) {
         for (int p = 0; p < PPC; ++p)
             if (b0 + p < nprob)
                 zero_rows(a.plan + (b0 + p) * (int64_t)R * R, st + p * R, R, k.wide, warp - PPC, kThreads / 32 - PPC);
@@ -875,7 +911,7 @@ sinkhorn_class_tree_kernel(ClassArgs k, int64_t nprob)
     __syncthreads();
 
     // ---- column cap, then the factors of a column by tier
-    for (int i = tid; i < PPC * R; i += kThreads) {
+    for (int i = tid; crank == 0 && i < PPC * R; i += kThreads) {
         const int p = i / R, j = i - p * R;
         if (b0 + p < nprob && ver[p].state == 0) {
             const int c = cls[j];
@@ -887,13 +923,23 @@ sinkhorn_class_tree_kernel(ClassArgs k, int64_t nprob)
         }
     }
     __syncthreads();
+    if (csize > 1) {
+        cluster_arrive(); cluster_wait();                               // the leader's factors are there
+        if (crank > 0) {
+            for (int i = tid; i < 4 * R; i += kThreads) st[i] = leader_f32(st + i);      // st, then dm
+            for (int i = tid; i < 3 * NS; i += kThreads) sm[0].e1[i] = leader_f32(sm[0].e1 + i);
+            if (tid == 0) ver[0].state = __float_as_int(leader_f32(reinterpret_cast<const float*>(&ver[0].state)));
+        }
+        __syncthreads();
+        cluster_arrive();                                               // (the leader must not go before they are read)
+    }
     int nonfinite = 0;
     for (int p = 0; p < PPC; ++p) {
         if (b0 + p >= nprob || ver[p].state == 2) continue;
         const bool solved = ver[p].state == 0;
         float* out = a.plan + (b0 + p) * (int64_t)R * R;
         const float* col = dm + 3 * p * R;
-        for (int row = warp; row < R; row += kThreads / 32) {
+        for (int row = crank * (kThreads / 32) + warp; row < R; row += csize * (kThreads / 32)) {
             const float sv = st[p * R + row];
             if (!(sv > 0.0f)) continue;
             float* o = out + (int64_t)row * R;
@@ -933,8 +979,11 @@ sinkhorn_class_tree_kernel(ClassArgs k, int64_t nprob)
         for (int p = 0; p < PPC; ++p)
             if ((nonfinite >> p) & 1) atomicOr(&ver[p].info, TAOT_INFO_NONFINITE);
     }
+    if (csize > 1) cluster_wait();
     __syncthreads();
-    if (tid < PPC && b0 + tid < nprob) {
+    if (crank > 0) {
+        if (tid == 0 && (ver[0].info & TAOT_INFO_NONFINITE)) atomicOr(a.info + b0, TAOT_INFO_NONFINITE);
+    } else if (tid < PPC && b0 + tid < nprob) {
         const Verdict& v = ver[tid];
         a.iters[b0 + tid] = v.state == 2 ? kHandBack : v.iters;
         if (v.state != 2) {
@@ -954,16 +1003,23 @@ int launch_dense(const ClassArgs& k, int32_t B, int32_t zeroers, cudaStream_t st
 }
 
 template <int GPL, int NPG, bool TOL, int PPC>
-int launch_tree(const ClassArgs& k, int32_t B, int32_t zeroers, cudaStream_t st)
+int launch_tree(ClassArgs& k, int32_t B, int32_t zeroers, int32_t cluster, cudaStream_t st)
 {
-    const size_t smem = PPC * (sizeof(TreeSmem<32 * GPL * NPG>) + 2 * sizeof(double) * 32 * GPL * NPG) + (size_t)k.a.R * (PPC * 4 * sizeof(float) + 2 * sizeof(uint16_t));
+    size_t smem = PPC * (sizeof(TreeSmem<32 * GPL * NPG>) + 2 * sizeof(double) * 32 * GPL * NPG) + (size_t)k.a.R * (PPC * 4 * sizeof(float) + 2 * sizeof(uint16_t));
+    k.cluster = PPC == 1 ? cluster : 1;
+    if (k.cluster > 1) {
+        k.solvers = B * k.cluster;
+        zeroers = 0;
+        if (smem < 120 * 1024) smem = 120 * 1024;              // one CTA per SM: a solving SM's stores slow its exchanges down
+    }
     TAOT_CUDA_OK(cudaFuncSetAttribute(sinkhorn_class_tree_kernel<GPL, NPG, TOL, PPC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    TAOT_CUDA_OK(taot_launch_chained(sinkhorn_class_tree_kernel<GPL, NPG, TOL, PPC>, (unsigned)(k.solvers + zeroers), kThreads, smem, st, k, (int64_t)B));
+    TAOT_CUDA_OK(taot_launch_chained_cluster(sinkhorn_class_tree_kernel<GPL, NPG, TOL, PPC>, (unsigned)(k.solvers + zeroers), kThreads,
+                                             (unsigned)k.cluster, smem, st, k, (int64_t)B));
     return 1;
 }
 
 template <bool TOL, int PPC>
-int launch_kind(const taot_handle_s* h, ClassArgs& k, int32_t B, int32_t zeroers, cudaStream_t st)
+int launch_kind(const taot_handle_s* h, ClassArgs& k, int32_t B, int32_t zeroers, int32_t cluster, cudaStream_t st)
 {
     k.solvers = (B + PPC - 1) / PPC;
     if (h->cls_kind == 1) {
@@ -975,11 +1031,11 @@ int launch_kind(const taot_handle_s* h, ClassArgs& k, int32_t B, int32_t zeroers
             default: return launch_dense<32, 1, TOL, PPC>(k, B, zeroers, st);
         }
     }
-    if (h->cls_npg == 8) return launch_tree<1, 8, TOL, PPC>(k, B, zeroers, st);
+    if (h->cls_npg == 8) return launch_tree<1, 8, TOL, PPC>(k, B, zeroers, cluster, st);
     switch (h->cls_gpl) {
-        case 1: return launch_tree<1, 4, TOL, PPC>(k, B, zeroers, st);
-        case 2: return launch_tree<2, 4, TOL, PPC>(k, B, zeroers, st);
-        default: return launch_tree<4, 4, TOL, PPC>(k, B, zeroers, st);
+        case 1: return launch_tree<1, 4, TOL, PPC>(k, B, zeroers, cluster, st);
+        case 2: return launch_tree<2, 4, TOL, PPC>(k, B, zeroers, cluster, st);
+        default: return launch_tree<4, 4, TOL, PPC>(k, B, zeroers, cluster, st);
     }
 }
 
@@ -1004,8 +1060,13 @@ int taot_launch_sinkhorn_class(taot_handle_t h, const SinkArgs& a, int32_t B, cu
     // otherwise the writing warps of the solving CTAs do
     const int32_t left = h->sm_count - B;
     const int32_t zeroers = left > 0 && (int64_t)B * a.R * a.R >= (1 << 20) ? 2 * left : 0;
-    if (a.tol > 0.0f) return share ? launch_kind<true, 4>(h, k, B, zeroers, st) : launch_kind<true, 1>(h, k, B, zeroers, st);
-    return share ? launch_kind<false, 4>(h, k, B, zeroers, st) : launch_kind<false, 1>(h, k, B, zeroers, st);
+    // The supply rows can only be written when their problem is solved, and one SM stores about 60 GB/s: from plans of 1 MB on
+    // (512 ranks: 5 us and more) a problem takes a cluster of as many SMs as there are for each, 2, 4 or 8 (some less than
+    // sm_count / B, since a cluster sits in one GPC)
+    const int32_t per = h->sm_count / (B > 0 ? B : 1);
+    const int32_t cluster = h->cls_kind == 2 && (int64_t)a.R * a.R >= (1 << 18) && per >= 2 ? (per >= 10 ? 8 : (per >= 5 ? 4 : 2)) : 1;
+    if (a.tol > 0.0f) return share ? launch_kind<true, 4>(h, k, B, zeroers, cluster, st) : launch_kind<true, 1>(h, k, B, zeroers, cluster, st);
+    return share ? launch_kind<false, 4>(h, k, B, zeroers, cluster, st) : launch_kind<false, 1>(h, k, B, zeroers, cluster, st);
 }
 
 namespace {

@@ -154,6 +154,26 @@ cudaError_t taot_launch_chained(void (*kernel)(P...), unsigned grid, unsigned bl
     return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// the same as clusters of `cluster` CTAs
+template <class... P, class... A>
+cudaError_t taot_launch_chained_cluster(void (*kernel)(P...), unsigned grid, unsigned block, unsigned cluster, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 #define TAOT_CUDA_OK(expr)                              \
     do {                                                \
         cudaError_t _e = (expr);                        \
