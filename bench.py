@@ -241,8 +241,8 @@ def cpu_model():
 
 
 def tiered_sums(C, B):
-    """Does the library take the tier-by-tier Sinkhorn kernel for this cost matrix?  Its rule, applied to the matrix
-    itself: 256, 512 or 1024 ranks and every off-diagonal cost equal to one of three values according to same node /
+    """Does a plan take the tier-by-tier Sinkhorn kernel (256 ranks), a batch of its own the class kernels (from 256 ranks up) for
+    this cost matrix?  The rule, applied to the matrix itself: 256, 512 or 1024 ranks and every off-diagonal cost equal to one of three values according to same node /
     same rail group / neither, with the block sizes read off the first row (ranks per node / per group 8 / 32, 4 / 16,
     4 / 32 or 16 / 32; a two-valued cost has no group tier)."""
     R = C.shape[0]
@@ -776,10 +776,11 @@ def run_sweep(args):
         hn = (ex > 0).sum(1).double(); cn = (sp > 0).sum(1).double()
         dense_fma = float((2 * hn * cn * (SWEEP_ITERS - 1)).sum())        # a solver that holds the kernel matrix
         tiered = tiered_sums(C, B)
+        # (classes: the multiply-adds the rank-by-rank tier sums would take, kept as the common yardstick)
         fma = float(B * tiered_fma_per_iteration(R) * (SWEEP_ITERS - 1)) if tiered else dense_fma
         t = float(np.median(ms)) * 1e-3
         # the library's rule for the dense products on the tensor cores, mirrored
-        tensor = (not tiered and R > 256 and R % 128 == 0 and B >= 256 and float(C.max()) / (eps_frac * max(SWEEP_TIERS)) <= 20.0
+        tensor = (not tiered and R > 512 and R % 128 == 0 and B >= 256 and float(C.max()) / (eps_frac * max(SWEEP_TIERS)) <= 20.0
                   and not os.environ.get("TAOT_NO_TENSOR_CORES"))
         if tensor:
             # executed: per iteration two products [R,R] x [R,B], each as three TF32 products
@@ -794,7 +795,7 @@ def run_sweep(args):
             torch.cuda.empty_cache()
             continue
         cells.append(dict(B=B, R=R, eps_frac=eps_frac, ms=t * 1e3, plans_per_s=B / t,
-                          kernel="tiered sums" if tiered else "kernel matrix",
+                          kernel="classes" if tiered or (R > 32 and not args.sweep_general_cost) else "kernel matrix",
                           tflops=2 * fma / t / 1e12, frac_fp32_peak=2 * fma / t / 1e12 / fp32_peak,
                           matrix_equiv_tflops=2 * dense_fma / t / 1e12,
                           hot_mean=float(hn.mean()), cold_mean=float(cn.mean()),
