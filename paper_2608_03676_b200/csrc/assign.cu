@@ -39,7 +39,7 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kWarpSpan = TAOT_CHUNK / kWarps;           // entries one warp owns, contiguous: 2048
 constexpr int kIters = kWarpSpan / 128;                  // 16-byte accesses per lane: 16
 constexpr int kFewSplits = 4;                            // splits of a chunk that are applied as predicated overrides from registers
-                                                         // (only up to 2: 16 ranks 158 -> 165 us a plan, 24 ranks 141 -> 149)
+                                                         // (only up to 2: 16 ranks 158 -> 165 us a plan, 24 ranks 141 -> 149; up to 6: 32 ranks 114 -> 117)
 
 struct AssignArgs {
     const int32_t* topk;
