@@ -29,7 +29,8 @@
  *   - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  Calls
  *     enqueue work and return; they never synchronise (except taot_create / taot_destroy).
  *   - Return value: TAOT_OK, or a negative taot_status found on the host before anything was
- *     launched.  Data-dependent conditions never fault or trap: they are OR-ed into d_info[l]
+ *     launched (TAOT_ERR_CUDA: possibly half way; everything that was queued then still comes before
+ *     what the caller queues next on `stream`).  Data-dependent conditions never fault or trap: they are OR-ed into d_info[l]
  *     (TAOT_INFO_* bits).  The caller zeroes d_info before the first stage it runs; taot_plan
  *     and taot_plan_host zero it themselves.
  *   - Same inputs give the same output bits on every call.

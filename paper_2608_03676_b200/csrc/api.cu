@@ -819,6 +819,62 @@ taot_outputs outputs_from_layer(const taot_params& p, const taot_outputs* o, int
     return g;
 }
 
+// Whatever groups 1 to G - 1 have queued on their streams comes before what the caller queues next.  Also on the way out of a
+// call that failed half way: copies to and from the caller's buffers may still be under way there.
+int join_groups(taot_handle_t h, int G, cudaStream_t st)
+{
+    int rc = TAOT_OK;
+    for (int g = 1; g < G; ++g)
+        if (cudaEventRecord(h->ev_join[g], h->gstream[g]) != cudaSuccess || cudaStreamWaitEvent(st, h->ev_join[g], 0) != cudaSuccess)
+            rc = TAOT_ERR_CUDA;
+    return rc;
+}
+
+// taot_plan in layer groups: group 0 on the caller's stream, the others on the handle's streams, forked from the caller's
+// stream by an event (*forked: how many of the groups have work on a stream; the caller of this function joins them).  No
+// allocation, no synchronisation, and the fork / join pattern is what stream capture expects.
+int plan_in_groups(taot_handle_t h, const int32_t* d_topk, const taot_outputs* o, void* ws, cudaStream_t st, int* forked, bool* bytes_begun,
+                   int* total)
+{
+    const taot_params& p = h->p;
+    TAOT_CUDA_OK(cudaEventRecord(h->ev_fork, st));
+    const bool side_bytes = h->bstream != nullptr && h->tb_ok && (reinterpret_cast<uintptr_t>(d_topk) & 15) == 0 &&
+                            (reinterpret_cast<uintptr_t>(o->new_idx) & 15) == 0;
+    for (int g = 0; g < h->ngroups; ++g) {
+        taot_handle_s* v = h->group[g];
+        const int l0 = h->group_l0[g];
+        cudaStream_t gs = g == 0 ? st : h->gstream[g];
+        if (g > 0) TAOT_CUDA_OK(cudaStreamWaitEvent(gs, h->ev_fork, 0));
+        *forked = g + 1;
+        const taot_outputs go = outputs_from_layer(p, o, l0);
+        const int rc = plan_stages(v, d_topk + (size_t)l0 * p.T * p.k, &go, ws, gs, h->profiling == 3,
+                                   g > 0 ? h->ev_hist[g - 1] : nullptr,
+                                   (g + 1 < h->ngroups || side_bytes) ? h->ev_hist[g] : nullptr, total, side_bytes);
+        if (rc != TAOT_OK) return rc;
+    }
+    if (!side_bytes) return TAOT_OK;
+    // The one-byte copies the reassignment reads are made on a stream of their own once every histogram is done (the
+    // memory system is idle from then until the first matching ends), by a grid too small to get in the way of the
+    // chains; each group's reassignment waits for its copy.
+    TAOT_CUDA_OK(cudaStreamWaitEvent(h->bstream, h->ev_hist[h->ngroups - 1], 0));
+    *bytes_begun = true;
+    for (int g = 0; g < h->ngroups; ++g) {
+        const int a = taot_launch_table_bytes(h->group[g], d_topk + (size_t)h->group_l0[g] * p.T * p.k, ws, h->bstream);
+        if (a < 0) return a;
+        *total += a;
+        TAOT_CUDA_OK(cudaEventRecord(h->ev_bytes[g], h->bstream));
+    }
+    for (int g = 0; g < h->ngroups; ++g) {
+        cudaStream_t gs = g == 0 ? st : h->gstream[g];
+        const taot_outputs go = outputs_from_layer(p, o, h->group_l0[g]);
+        TAOT_CUDA_OK(cudaStreamWaitEvent(gs, h->ev_bytes[g], 0));
+        const int rc = assign_stage(h->group[g], d_topk + (size_t)h->group_l0[g] * p.T * p.k, &go, ws, gs,
+                                    h->profiling == 3, total);
+        if (rc != TAOT_OK) return rc;
+    }
+    return TAOT_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -844,47 +900,45 @@ int taot_plan(taot_handle_t h, const int32_t* d_topk, const taot_outputs* o, voi
         h->last_launches = total;
         return TAOT_OK;
     }
-    // Layer groups: group 0 on the caller's stream, the others on the handle's streams, forked from the caller's
-    // stream by an event and joined back into it by one event each; no allocation, no synchronisation, and the fork /
-    // join pattern is what stream capture expects.
-    TAOT_CUDA_OK(cudaEventRecord(h->ev_fork, st));
-    const bool side_bytes = h->bstream != nullptr && h->tb_ok && (reinterpret_cast<uintptr_t>(d_topk) & 15) == 0 &&
-                            (reinterpret_cast<uintptr_t>(o->new_idx) & 15) == 0;
-    for (int g = 0; g < h->ngroups; ++g) {
-        taot_handle_s* v = h->group[g];
-        const int l0 = h->group_l0[g];
-        cudaStream_t gs = g == 0 ? st : h->gstream[g];
-        if (g > 0) TAOT_CUDA_OK(cudaStreamWaitEvent(gs, h->ev_fork, 0));
-        const taot_outputs go = outputs_from_layer(p, o, l0);
-        const int rc = plan_stages(v, d_topk + (size_t)l0 * p.T * p.k, &go, ws, gs, h->profiling == 3,
-                                   g > 0 ? h->ev_hist[g - 1] : nullptr,
-                                   (g + 1 < h->ngroups || side_bytes) ? h->ev_hist[g] : nullptr, &total, side_bytes);
-        if (rc != TAOT_OK) return rc;
-        if (g > 0 && !side_bytes) TAOT_CUDA_OK(cudaEventRecord(h->ev_join[g], gs));
+    int forked = 0;
+    bool bytes_begun = false;
+    const int rc = plan_in_groups(h, d_topk, o, ws, st, &forked, &bytes_begun, &total);
+    const int joined = join_groups(h, forked, st);
+    if (rc != TAOT_OK) {
+        // (after a whole call every group has waited for its copy)
+        if (bytes_begun && cudaEventRecord(h->ev_bytes[0], h->bstream) == cudaSuccess) cudaStreamWaitEvent(st, h->ev_bytes[0], 0);
+        return rc;
     }
-    if (side_bytes) {
-        // The one-byte copies the reassignment reads are made on a stream of their own once every histogram is done (the
-        // memory system is idle from then until the first matching ends), by a grid too small to get in the way of the
-        // chains; each group's reassignment waits for its copy.
-        TAOT_CUDA_OK(cudaStreamWaitEvent(h->bstream, h->ev_hist[h->ngroups - 1], 0));
-        for (int g = 0; g < h->ngroups; ++g) {
-            const int a = taot_launch_table_bytes(h->group[g], d_topk + (size_t)h->group_l0[g] * p.T * p.k, ws, h->bstream);
-            if (a < 0) return a;
-            total += a;
-            TAOT_CUDA_OK(cudaEventRecord(h->ev_bytes[g], h->bstream));
-        }
-        for (int g = 0; g < h->ngroups; ++g) {
-            cudaStream_t gs = g == 0 ? st : h->gstream[g];
-            const taot_outputs go = outputs_from_layer(p, o, h->group_l0[g]);
-            TAOT_CUDA_OK(cudaStreamWaitEvent(gs, h->ev_bytes[g], 0));
-            const int rc = assign_stage(h->group[g], d_topk + (size_t)h->group_l0[g] * p.T * p.k, &go, ws, gs,
-                                        h->profiling == 3, &total);
-            if (rc != TAOT_OK) return rc;
-            if (g > 0) TAOT_CUDA_OK(cudaEventRecord(h->ev_join[g], gs));
-        }
-    }
-    for (int g = 1; g < h->ngroups; ++g) TAOT_CUDA_OK(cudaStreamWaitEvent(st, h->ev_join[g], 0));
+    if (joined != TAOT_OK) return joined;
     h->last_launches = total;
+    return TAOT_OK;
+}
+
+// The layer groups of a host call, forked from the caller's stream (*forked: how many have work on a stream; the caller joins
+// them): the copies of one group run under the kernels of another, and both copy engines at once.
+static int plan_host_groups(taot_handle_t h, const int32_t* h_topk, int32_t* h_new, int32_t* d_topk, const taot_outputs* d, void* ws,
+                            cudaStream_t st, int* forked, int* total)
+{
+    const taot_params& p = h->p;
+    const int G = h->hgroups;
+    const size_t per_layer = (size_t)p.T * p.k;
+    auto stream_of = [&](int g) { return g == 0 ? st : h->gstream[g]; };
+    auto layers_of = [&](int g) { return (g + 1 < G ? h->hgroup_l0[g + 1] : p.L) - h->hgroup_l0[g]; };
+    TAOT_CUDA_OK(cudaEventRecord(h->ev_fork, st));
+    for (int g = 0; g < G; ++g) {
+        const size_t o0 = (size_t)h->hgroup_l0[g] * per_layer;
+        if (g > 0) TAOT_CUDA_OK(cudaStreamWaitEvent(stream_of(g), h->ev_fork, 0));
+        *forked = g + 1;
+        TAOT_CUDA_OK(cudaMemcpyAsync(d_topk + o0, h_topk + o0, sizeof(int32_t) * per_layer * layers_of(g), cudaMemcpyHostToDevice, stream_of(g)));
+    }
+    for (int g = 0; g < G; ++g) {
+        const size_t o0 = (size_t)h->hgroup_l0[g] * per_layer;
+        const taot_outputs go = outputs_from_layer(p, d, h->hgroup_l0[g]);
+        const int rc = plan_stages(h->hgroup[g], d_topk + o0, &go, ws, stream_of(g), false, nullptr, nullptr, total);
+        if (rc != TAOT_OK) return rc;
+        if (h_new)
+            TAOT_CUDA_OK(cudaMemcpyAsync(h_new + o0, d->new_idx + o0, sizeof(int32_t) * per_layer * layers_of(g), cudaMemcpyDeviceToHost, stream_of(g)));
+    }
     return TAOT_OK;
 }
 
@@ -920,27 +974,10 @@ static int plan_on_staging(taot_handle_t h, const int32_t* h_topk, int32_t* h_ne
         TAOT_CUDA_OK(cudaMemcpyAsync(h_new, d->new_idx, sizeof(int32_t) * NE, cudaMemcpyDeviceToHost, st));
         return TAOT_OK;
     }
-    const int G = h->hgroups;
-    const size_t per_layer = (size_t)p.T * p.k;
-    auto stream_of = [&](int g) { return g == 0 ? st : h->gstream[g]; };
-    auto layers_of = [&](int g) { return (g + 1 < G ? h->hgroup_l0[g + 1] : p.L) - h->hgroup_l0[g]; };
-    TAOT_CUDA_OK(cudaEventRecord(h->ev_fork, st));
-    for (int g = 0; g < G; ++g) {
-        const size_t o0 = (size_t)h->hgroup_l0[g] * per_layer;
-        if (g > 0) TAOT_CUDA_OK(cudaStreamWaitEvent(stream_of(g), h->ev_fork, 0));
-        TAOT_CUDA_OK(cudaMemcpyAsync(d_topk + o0, h_topk + o0, sizeof(int32_t) * per_layer * layers_of(g), cudaMemcpyHostToDevice, stream_of(g)));
-    }
-    int total = 0;
-    for (int g = 0; g < G; ++g) {
-        const size_t o0 = (size_t)h->hgroup_l0[g] * per_layer;
-        const taot_outputs go = outputs_from_layer(p, d, h->hgroup_l0[g]);
-        const int rc = plan_stages(h->hgroup[g], d_topk + o0, &go, at(d_ws, h->hoff_ws), stream_of(g), false, nullptr, nullptr, &total);
-        if (rc != TAOT_OK) return rc;
-        if (h_new)
-            TAOT_CUDA_OK(cudaMemcpyAsync(h_new + o0, d->new_idx + o0, sizeof(int32_t) * per_layer * layers_of(g), cudaMemcpyDeviceToHost, stream_of(g)));
-        if (g > 0) TAOT_CUDA_OK(cudaEventRecord(h->ev_join[g], stream_of(g)));
-    }
-    for (int g = 1; g < G; ++g) TAOT_CUDA_OK(cudaStreamWaitEvent(st, h->ev_join[g], 0));
+    int forked = 0, total = 0;
+    const int rc = plan_host_groups(h, h_topk, h_new, d_topk, d, at(d_ws, h->hoff_ws), st, &forked, &total);
+    const int joined = join_groups(h, forked, st);
+    if (rc != TAOT_OK || joined != TAOT_OK) return rc != TAOT_OK ? rc : joined;
     h->last_launches = total;
     return TAOT_OK;
 }

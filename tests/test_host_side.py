@@ -1,0 +1,41 @@
+"""What the host code queues, on a CPU with a fake runtime: streams, joins, errors, the kernels that a call takes."""
+import pytest
+
+import fake_cuda as F
+import workloads as W
+
+
+@pytest.fixture(scope="module")
+def so(tmp_path_factory):
+    return F.load(str(tmp_path_factory.mktemp("fake")))
+
+
+def _host_planner(so, L=24):
+    return F.FakePlanner(so, L, 16, 64, 2, 8, 16 * 1024, W.cost_matrix(16, 8, (0.0, 1.0, 10.0), None), tol=1e-6)
+
+
+def _large_planner(so, R=256, L=12):                 # tables that taot_plan splits into layer groups
+    return F.FakePlanner(so, L, R, 128, 1, 8, R * 2048, W.cost_matrix(R, 8, (0.0, 1.0, 6.0, 16.0), 4), tol=1e-6)
+
+
+@pytest.mark.parametrize("make,call,groups", [(_host_planner, "plan_host_block", 6), (_large_planner, "plan", 6),
+                                              (lambda so: _large_planner(so, 64, 24), "plan", 3)])
+def test_a_failing_launch_leaves_nothing_behind_on_internal_streams(so, make, call, groups):
+    """Whatever a call queued on streams of the handle is joined into the caller's stream, also when one of its launches or copies
+    fails: the caller may free or reuse its buffers in the order of its own stream."""
+    so.fake_reset()
+    pl = make(so)
+    assert getattr(pl, call)() == 0
+    so.fake_reset()
+    assert getattr(pl, call)() == 0
+    whole = F.log(so)
+    assert len({e.stream for e in whole if e.kind == F.LAUNCH}) >= groups and not F.not_joined(whole)
+    for kind in (F.LAUNCH, F.COPY):
+        for after in range(sum(e.kind == kind for e in whole)):
+            so.fake_reset()
+            so.fake_fail(kind, after)
+            assert getattr(pl, call)() == -4
+            assert not F.not_joined(F.log(so)), (kind, after)
+            so.fake_reset()
+            assert getattr(pl, call)() == 0 and [e.name for e in F.log(so)] == [e.name for e in whole]
+    pl.close()
