@@ -422,12 +422,13 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
         if (cudaEventCreate(&h->ev[i]) != cudaSuccess) rc = TAOT_ERR_CUDA;
     // Layer groups for taot_plan: only where every group's routing table still keeps the memory system busy (more
     // chunks than three waves of the per-chunk kernels), i.e. where there are bandwidth-bound stages to hide
+    int most_groups = TAOT_MAX_GROUPS;
+    if (const char* env = std::getenv("TAOT_PLAN_GROUPS")) {      // tuning knob: cap on the number of groups (1 = never split)
+        const int cap = std::atoi(env);
+        if (cap >= 1 && cap < most_groups) most_groups = cap;
+    }
     if (rc == TAOT_OK && R <= 256) {
-        int G = TAOT_MAX_GROUPS;
-        if (const char* env = std::getenv("TAOT_PLAN_GROUPS")) {      // tuning knob: cap on the number of groups (1 = never split)
-            const int cap = std::atoi(env);
-            if (cap >= 1 && cap < G) G = cap;
-        }
+        int G = most_groups;
         const int64_t chunks_per_layer = (int64_t)R * h->nc;
         while (G > 1 && (params->L < 2 * G || (params->L / G) * chunks_per_layer <= 3 * (int64_t)h->sm_count)) --G;
         if (G > 1) {
@@ -472,7 +473,7 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
     // Layer groups of the host calls.  A call's time is the copy in, one group's chain of kernels and the last group's copy
     // out: as many equal groups as there are streams (16 ranks, 24 layers, 12.6 MB each way: see plan_on_staging)
     if (rc == TAOT_OK && R <= 256 && params->L > 1 && (int64_t)params->L * params->T * params->k * 4 >= TAOT_HOST_GROUP_BYTES) {
-        h->hgroups = params->L < TAOT_MAX_GROUPS ? params->L : TAOT_MAX_GROUPS;
+        h->hgroups = params->L < most_groups ? params->L : most_groups;
         if (!h->ev_fork && cudaEventCreate(&h->ev_fork) != cudaSuccess) rc = TAOT_ERR_CUDA;
         for (int g = 0; g < h->hgroups && rc == TAOT_OK; ++g) {
             h->hgroup_l0[g] = (int32_t)((int64_t)params->L * g / h->hgroups);

@@ -39,3 +39,18 @@ def test_a_failing_launch_leaves_nothing_behind_on_internal_streams(so, make, ca
             so.fake_reset()
             assert getattr(pl, call)() == 0 and [e.name for e in F.log(so)] == [e.name for e in whole]
     pl.close()
+
+
+def _streams_of(so, pl):
+    assert pl.plan_host_block() == 0
+    return {e.stream for e in F.log(so) if e.kind in (F.LAUNCH, F.COPY)}
+
+
+@pytest.mark.parametrize("cap,L,want", [("1", 24, 1), ("3", 24, 3), (None, 24, 6), (None, 5, 5), ("9", 7, 6)])
+def test_the_cap_on_layer_groups_holds_for_host_calls(so, monkeypatch, cap, L, want):
+    so.fake_reset()
+    if cap:
+        monkeypatch.setenv("TAOT_PLAN_GROUPS", cap)
+    pl = _host_planner(so, L)
+    assert len(_streams_of(so, pl)) == want and not F.not_joined(F.log(so))
+    pl.close()
