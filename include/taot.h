@@ -270,8 +270,11 @@ int taot_plan(taot_handle_t h, const int32_t* d_topk, const taot_outputs* out, v
 
 /*
  * The whole path with HOST buffers: h_topk [L,T,k] is copied to the device, the path runs, and
- * every non-NULL member of `out` (HOST pointers) is copied back, all enqueued on `stream`.
+ * every non-NULL member of `out` (HOST pointers) is copied back, all in the order of `stream`.
  * Pinned host memory makes the copies asynchronous.  d_ws: taot_host_workspace_bytes bytes.
+ * A table of 2 MB or more goes in up to six groups of layers (TAOT_PLAN_GROUPS caps them too) on streams of the handle,
+ * forked from and joined back into `stream`; the results are the same bits.  taot_host_block_layout or the handle's first
+ * host call makes those streams; a call that is captured before either stays on `stream`.
  */
 int taot_plan_host(taot_handle_t h, const int32_t* h_topk, const taot_outputs* out, void* d_ws,
                    void* stream);

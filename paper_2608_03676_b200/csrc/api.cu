@@ -471,16 +471,9 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
         }
     }
     // Layer groups of the host calls.  A call's time is the copy in, one group's chain of kernels and the last group's copy
-    // out: as many equal groups as there are streams (16 ranks, 24 layers, 12.6 MB each way: see plan_on_staging)
-    if (rc == TAOT_OK && R <= 256 && params->L > 1 && (int64_t)params->L * params->T * params->k * 4 >= TAOT_HOST_GROUP_BYTES) {
+    // out: as many equal groups as there are streams.  Their streams and views are made when a host call is in sight (make_host_groups).
+    if (R <= 256 && (int64_t)params->L * params->T * params->k * 4 >= TAOT_HOST_GROUP_BYTES)
         h->hgroups = params->L < most_groups ? params->L : most_groups;
-        if (!h->ev_fork && cudaEventCreate(&h->ev_fork) != cudaSuccess) rc = TAOT_ERR_CUDA;
-        for (int g = 0; g < h->hgroups && rc == TAOT_OK; ++g) {
-            h->hgroup_l0[g] = (int32_t)((int64_t)params->L * g / h->hgroups);
-            if (g > 0 && !h->gstream[g] && cudaStreamCreateWithFlags(&h->gstream[g], cudaStreamNonBlocking) != cudaSuccess) rc = TAOT_ERR_CUDA;
-            if (rc == TAOT_OK && !h->ev_join[g] && cudaEventCreateWithFlags(&h->ev_join[g], cudaEventDisableTiming) != cudaSuccess) rc = TAOT_ERR_CUDA;
-        }
-    }
     if (rc == TAOT_OK && cudaDeviceSynchronize() != cudaSuccess) rc = TAOT_ERR_CUDA;
     if (rc != TAOT_OK) {
         taot_destroy(h);
@@ -493,10 +486,6 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
             h->group[g]->ev[i] = nullptr;
             if (cudaEventCreate(&h->group[g]->ev[i]) != cudaSuccess) { taot_destroy(h); return TAOT_ERR_CUDA; }
         }
-    }
-    for (int g = 0; g < h->hgroups; ++g) {
-        const int end = g + 1 < h->hgroups ? h->hgroup_l0[g + 1] : params->L;
-        h->hgroup[g] = make_view(h, g, h->hgroup_l0[g], end - h->hgroup_l0[g]);
     }
     *out = h;
     return TAOT_OK;
@@ -915,6 +904,24 @@ int taot_plan(taot_handle_t h, const int32_t* d_topk, const taot_outputs* o, voi
     return TAOT_OK;
 }
 
+static bool host_groups_made(const taot_handle_s* h) { return h->hgroups > 1 && h->hgroup[h->hgroups - 1]; }
+
+// Streams, events and views of a host call's layer groups.  Made by taot_host_block_layout or by the first host call (0.3 ms):
+// most handles plan tables that are on the device.
+static int make_host_groups(taot_handle_t h)
+{
+    if (h->hgroups <= 1 || host_groups_made(h)) return TAOT_OK;
+    if (!h->ev_fork) TAOT_CUDA_OK(cudaEventCreate(&h->ev_fork));
+    for (int g = 1; g < h->hgroups; ++g) {
+        if (!h->gstream[g]) TAOT_CUDA_OK(cudaStreamCreateWithFlags(&h->gstream[g], cudaStreamNonBlocking));
+        if (!h->ev_join[g]) TAOT_CUDA_OK(cudaEventCreateWithFlags(&h->ev_join[g], cudaEventDisableTiming));
+    }
+    for (int g = 0; g <= h->hgroups; ++g) h->hgroup_l0[g] = (int32_t)((int64_t)h->p.L * g / h->hgroups);
+    for (int g = 0; g < h->hgroups; ++g)
+        if (!h->hgroup[g]) h->hgroup[g] = make_view(h, g, h->hgroup_l0[g], h->hgroup_l0[g + 1] - h->hgroup_l0[g]);
+    return TAOT_OK;
+}
+
 // The layer groups of a host call, forked from the caller's stream (*forked: how many have work on a stream; the caller joins
 // them): the copies of one group run under the kernels of another, and both copy engines at once.
 static int plan_host_groups(taot_handle_t h, const int32_t* h_topk, int32_t* h_new, int32_t* d_topk, const taot_outputs* d, void* ws,
@@ -924,7 +931,7 @@ static int plan_host_groups(taot_handle_t h, const int32_t* h_topk, int32_t* h_n
     const int G = h->hgroups;
     const size_t per_layer = (size_t)p.T * p.k;
     auto stream_of = [&](int g) { return g == 0 ? st : h->gstream[g]; };
-    auto layers_of = [&](int g) { return (g + 1 < G ? h->hgroup_l0[g + 1] : p.L) - h->hgroup_l0[g]; };
+    auto layers_of = [&](int g) { return h->hgroup_l0[g + 1] - h->hgroup_l0[g]; };
     TAOT_CUDA_OK(cudaEventRecord(h->ev_fork, st));
     for (int g = 0; g < G; ++g) {
         const size_t o0 = (size_t)h->hgroup_l0[g] * per_layer;
@@ -946,7 +953,7 @@ static int plan_host_groups(taot_handle_t h, const int32_t* h_topk, int32_t* h_n
 // H2D copy of the routing table, the whole path on device staging buffers, D2H copy of the rewritten table (unless h_new is
 // null); `d` receives the device pointers.  Large tables go in layer groups on streams of their own, forked from and joined
 // back into the caller's: the copies of one group run under the kernels of another, and both copy engines at once (16
-// ranks, 24 layers, 12.6 MB each way: 718 -> 480 us; one after the other the copies alone take 460).
+// ranks, 24 layers, 12.6 MB each way: 716 -> 522 us; one after the other the copies alone take 460).
 static int plan_on_staging(taot_handle_t h, const int32_t* h_topk, int32_t* h_new, void* d_ws, void* stream, taot_outputs* d)
 {
     const taot_params& p = h->p;
@@ -968,7 +975,13 @@ static int plan_on_staging(taot_handle_t h, const int32_t* h_topk, int32_t* h_ne
     d->new_idx = reinterpret_cast<int32_t*>(at(d_ws, h->hoff_new));
     d->info = reinterpret_cast<int32_t*>(at(d_ws, h->hoff_info));
     int32_t* d_topk = reinterpret_cast<int32_t*>(at(d_ws, h->hoff_topk));
-    if (h->hgroups <= 1 || h->profiling) {
+    if (!h->profiling && h->hgroups > 1 && !host_groups_made(h)) {
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        TAOT_CUDA_OK(cudaStreamIsCapturing(st, &capture));
+        const int made = capture == cudaStreamCaptureStatusNone ? make_host_groups(h) : TAOT_OK;
+        if (made != TAOT_OK) return made;
+    }
+    if (h->profiling || !host_groups_made(h)) {
         TAOT_CUDA_OK(cudaMemcpyAsync(d_topk, h_topk, sizeof(int32_t) * NE, cudaMemcpyHostToDevice, st));
         const int rc = taot_plan(h, d_topk, d, at(d_ws, h->hoff_ws), stream);
         if (rc != TAOT_OK || !h_new) return rc;
@@ -1016,6 +1029,7 @@ int taot_plan_host(taot_handle_t h, const int32_t* h_topk, const taot_outputs* o
 int taot_host_block_layout(taot_handle_t h, size_t* offsets, size_t* bytes)
 {
     if (!h || !offsets || !bytes) return TAOT_ERR_NULL;
+    if (make_host_groups(h) != TAOT_OK) (void)cudaGetLastError();     // (the host call tries again)
     const size_t base = h->hoff_n;
     const size_t off[14] = {h->hoff_n, h->hoff_el, h->hoff_rl, h->hoff_ex, h->hoff_sp, h->hoff_plan, h->hoff_it,
                             h->hoff_err, h->hoff_se, h->hoff_st, h->hoff_X, h->hoff_rounds, 0, h->hoff_info};

@@ -85,10 +85,11 @@ struct taot_handle_s {
     cudaStream_t gstream[TAOT_MAX_GROUPS];     // [0] unused: group 0 runs on the caller's stream
     cudaEvent_t ev_fork, ev_hist[TAOT_MAX_GROUPS], ev_join[TAOT_MAX_GROUPS];
     // Layer groups of the host calls (tables of at least TAOT_HOST_GROUP_BYTES): views like the ones above, each on a stream
-    // of its own (gstream), so that copies in, kernels and copies out of different groups run side by side.
+    // of its own (gstream), so that copies in, kernels and copies out of different groups run side by side.  hgroups is set by
+    // taot_create, the rest when a host call is in sight.
     int32_t hgroups;
     taot_handle_s* hgroup[TAOT_MAX_GROUPS];
-    int32_t hgroup_l0[TAOT_MAX_GROUPS];
+    int32_t hgroup_l0[TAOT_MAX_GROUPS + 1];
     cudaStream_t bstream;                      // the one-byte copies of the groups' tables are made here, after all histograms
     cudaEvent_t ev_bytes[TAOT_MAX_GROUPS];     // group g's copy is there
 };

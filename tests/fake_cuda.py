@@ -54,6 +54,10 @@ class FakePlanner:
         at = lambda i: ctypes.c_void_p(i << 36)
         return self.so.taot_plan_host_block(self.handle, at(1), at(2), at(3), ctypes.c_void_p(DEVICE), self.stream)
 
+    def host_block_layout(self):
+        off, n = (ctypes.c_size_t * 14)(), ctypes.c_size_t()
+        return self.so.taot_host_block_layout(self.handle, off, ctypes.byref(n))
+
     def sinkhorn(self, B):
         at = lambda i: ctypes.c_void_p(DEVICE + (i << 34))
         return self.so.taot_sinkhorn(self.handle, at(1), at(2), ctypes.c_int32(B), at(3), at(4), at(5), at(6), at(7), self.stream)

@@ -334,3 +334,39 @@ def test_streaming_host_planner_keeps_steps_apart(groups):
     with pytest.raises(P.TaotError):
         sp.result(0)
     sp.close(); pl.close()
+
+
+@pytest.mark.parametrize("base,over,L", [("cfg2", dict(T=32768), 2), ("cfg2", {}, 5),
+                                         ("cfg2", dict(R=9, E=63, gpus_per_node=3, T=9 * 2049, k=7), 7)])
+def test_host_calls_in_layer_groups_equal_the_device_call_and_can_be_captured(base, over, L):
+    """Fewer layers than groups, groups whose tables start off a 16-byte boundary, and a host call inside a CUDA graph: captured
+    after an ordinary one (in groups) and before anything that makes the groups' streams (on one stream)."""
+    cfg = W.get_config(base).replace(L=L, **over)
+    assert 4 * cfg.L * cfg.T * cfg.k >= 2 << 20                # large enough to be split
+    topk = _routing(cfg)
+    pl = make_planner(cfg)
+    want = {k: cpu(v).copy() for k, v in pl.plan(topk).items()}
+    host = topk.cpu().pin_memory()
+    for grouped in (True, False):
+        hp = make_planner(cfg)
+        out = hp.alloc_host_block() if grouped else hp.alloc_host_outputs(tuple(want))
+        call = hp.plan_host_block if grouped else hp.plan_host
+        hp._host_ws = torch.empty(hp.host_ws_bytes, dtype=torch.uint8, device="cuda")
+        if grouped:
+            call(host, out)
+            torch.cuda.synchronize()
+            for key, val in want.items():
+                assert (out[key].numpy() == val).all(), key
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            call(host, out)
+        for _ in range(2):
+            for v in out.values():
+                v.zero_()
+            g.replay()
+            torch.cuda.synchronize()
+            for key, val in want.items():
+                assert (out[key].numpy() == val).all(), key
+        del g
+        hp.close()
+    pl.close()

@@ -46,6 +46,32 @@ def _streams_of(so, pl):
     return {e.stream for e in F.log(so) if e.kind in (F.LAUNCH, F.COPY)}
 
 
+def test_streams_of_host_calls_are_made_when_a_host_call_is_in_sight(so):
+    so.fake_reset()
+    pl = _host_planner(so)
+    assert not [e for e in F.log(so) if e.kind == F.STREAM_CREATE]
+    assert pl.plan() == 0 and not [e for e in F.log(so) if e.kind == F.STREAM_CREATE]
+    so.fake_reset()
+    so.fake_capturing(1)                             # captured before any other host call: nothing is made, all on one stream
+    assert _streams_of(so, pl) == {F.CALLER} and not [e for e in F.log(so) if e.kind in (F.STREAM_CREATE, F.EVENT_CREATE)]
+    so.fake_reset()
+    so.fake_fail(F.STREAM_CREATE, 2)
+    assert pl.plan_host_block() == -4 and not F.not_joined(F.log(so))
+    so.fake_reset()                                  # (what is there already is kept)
+    assert len(_streams_of(so, pl)) == 6
+    so.fake_reset()
+    so.fake_capturing(1)
+    assert len(_streams_of(so, pl)) == 6 and not [e for e in F.log(so) if e.kind in (F.STREAM_CREATE, F.EVENT_CREATE)]
+    pl.close()
+    pl = _host_planner(so)
+    so.fake_reset()
+    so.fake_fail(F.STREAM_CREATE, 0)
+    assert pl.host_block_layout() == 0 and pl.host_block_layout() == 0
+    so.fake_reset()
+    assert len(_streams_of(so, pl)) == 6 and not [e for e in F.log(so) if e.kind in (F.STREAM_CREATE, F.EVENT_CREATE)]
+    pl.close()
+
+
 @pytest.mark.parametrize("cap,L,want", [("1", 24, 1), ("3", 24, 3), (None, 24, 6), (None, 5, 5), ("9", 7, 6)])
 def test_the_cap_on_layer_groups_holds_for_host_calls(so, monkeypatch, cap, L, want):
     so.fake_reset()
