@@ -447,7 +447,11 @@ int taot_launch_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, in
             launched += nw + n;
             a.only_marked = nw + n > 0 ? 1 : 0;
         }
-        TAOT_CUDA_OK(taot_launch_chained(sinkhorn_kernel, nb, NT, smem, st, a));
+        // This kernel may release the one behind it before it has waited only with a kernel in front that has waited for the merge:
+        // the matching kernel, set up from there, reads loads that the merge wrote
+        SinkArgs last = a;
+        last.early = a.early && launched > 0;
+        TAOT_CUDA_OK(taot_launch_chained(sinkhorn_kernel, nb, NT, smem, st, last));
         launched += 1;
     }
     return launched;

@@ -21,7 +21,9 @@ struct SinkArgs {
     int32_t max_iters;
     float tol;
     int32_t check_every;
-    int32_t early;           // let the next kernel be set up from the start (it reads nothing this one writes before it has ended)
+    int32_t early;           // let the next kernel be set up from the start: it reads nothing this one writes before this one has
+                             // ended, but it does read what the kernels in front of the solve wrote, so either this kernel
+                             // releases it after its own wait or the kernel before this one did
     int32_t only_marked;     // generic kernel: solve only the problems the register-tile kernel handed back
     int32_t skip_solved;     // tile kernels: solve only the problems an earlier kernel of the chain handed back
     float* kt_global;        // [B][kcap_global] kernel-matrix scratch in global memory for problems too big for

@@ -41,15 +41,19 @@ static cudaError_t put(int kind, cudaStream_t st, long obj, long grid, const cha
     if (args && arg_bytes && strstr(e->name, arg_of)) memcpy(e->arg, args[0], arg_bytes);
     return cudaSuccess;
 }
-/* "sinkhorn_tile_kernel" out of a mangled name */
+/* "sinkhorn_tile_kernel" out of a mangled name: the identifier that ends in _kernel and whose length stands in front of it */
 static const char* short_name(const char* s, char* out, size_t n)
 {
     const char* end = strstr(s, "_kernel");
-    if (!end) { snprintf(out, n, "%s", s); return out; }
-    const char* b = end;
-    while (b > s && ((b[-1] >= 'a' && b[-1] <= 'z') || b[-1] == '_' || (b[-1] >= '0' && b[-1] <= '9'))) --b;
-    while (b < end && !(*b >= 'a' && *b <= 'z')) ++b;
-    snprintf(out, n, "%.*s", (int)(end + 7 - b), b);
+    snprintf(out, n, "%s", s);
+    if (!end) return out;
+    end += 7;
+    for (const char* b = end - 8; b > s; --b) {
+        const char* d = b;
+        while (d > s && d[-1] >= '0' && d[-1] <= '9') --d;
+        for (; d < b; ++d)
+            if (atol(d) == end - b && *d != '0') { snprintf(out, n, "%.*s", (int)(end - b), b); return out; }
+    }
     return out;
 }
 static const char* name_of(const void* f)

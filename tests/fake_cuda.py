@@ -33,6 +33,13 @@ def load(folder):
     return so
 
 
+class SinkArgs(ctypes.Structure):
+    """The argument of the Phase-1 kernels (sinkhorn_common.cuh)."""
+    _fields_ = [("pointers", ctypes.c_void_p * 8), ("R", ctypes.c_int32), ("kcap", ctypes.c_int32), ("inv_eps", ctypes.c_double),
+                ("eps0", ctypes.c_float), ("max_iters", ctypes.c_int32), ("tol", ctypes.c_float), ("check_every", ctypes.c_int32),
+                ("early", ctypes.c_int32), ("only_marked", ctypes.c_int32), ("skip_solved", ctypes.c_int32)]
+
+
 class FakePlanner:
     """A handle of the library over the fake runtime, with made-up device addresses."""
 

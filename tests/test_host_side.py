@@ -1,5 +1,8 @@
 """What the host code queues, on a CPU with a fake runtime: streams, joins, errors, the kernels that a call takes."""
+import ctypes
+
 import pytest
+import torch
 
 import fake_cuda as F
 import workloads as W
@@ -79,4 +82,28 @@ def test_the_cap_on_layer_groups_holds_for_host_calls(so, monkeypatch, cap, L, w
         monkeypatch.setenv("TAOT_PLAN_GROUPS", cap)
     pl = _host_planner(so, L)
     assert len(_streams_of(so, pl)) == want and not F.not_joined(F.log(so))
+    pl.close()
+
+
+def _rough(R, seed=1):
+    C = 1.0 + torch.rand((R, R), generator=torch.Generator().manual_seed(seed))
+    C.fill_diagonal_(0.0)
+    return C
+
+
+@pytest.mark.parametrize("R", [4, 32, 64, 100, 256])
+@pytest.mark.parametrize("general", [False, True])
+def test_a_plan_releases_the_matching_kernel_only_behind_the_merge(so, R, general):
+    """The matching kernel reads the merge's loads without waiting, so a kernel that releases it before its own wait needs another
+    one in front that has waited for the merge."""
+    so.fake_reset()
+    so.fake_keep_arg(b"sinkhorn_kernel", ctypes.sizeof(F.SinkArgs))
+    pl = F.FakePlanner(so, 3, R, 2 * R, 1, 2, 16 * R, _rough(R) if general else W.cost_matrix(R, 4, (0.0, 1.0, 8.0), None))
+    assert pl.plan() == 0
+    names = F.kernels(so)
+    launches = [e for e in F.log(so) if e.kind == F.LAUNCH]
+    at = names.index("sinkhorn_kernel")
+    args = F.SinkArgs.from_buffer_copy(bytes(launches[at].arg))
+    assert args.R == R and args.early == 1
+    assert names[at - 1] not in ("merge_kernel", "hist_chunk_kernel") and names[at + 1] == "match_kernel"
     pl.close()
