@@ -208,9 +208,9 @@ int taot_excess_spare(taot_handle_t h, const int32_t* d_rank_load, int32_t B, in
  *   d_plan [B,R,R] fp32 (fully overwritten), d_iters [B], d_row_err [B], d_info [B].
  * The iterates are carried so that neither M nor u, v can under- or overflow for any C/eps.
  * `ws` is needed only for R > 256 (the kernel matrix then lives in workspace; batches larger than
- * the handle's L are solved in slices of L).  Problems with |{s>0}| * |{d>0}| beyond the capacity
- * (R*R/4 for R > 128, which disjoint supply/demand ranks never exceed) get TAOT_INFO_SINKHORN_SIZE
- * and a zero plan.
+ * the handle's L are solved in slices of L).  Up to 256 ranks a problem whose |{s>0}| * |{d>0}| is beyond the
+ * capacity (R*R/4 for R > 128, which disjoint supply / demand ranks never exceed) and which has more supply ranks than
+ * the register tiles hold (128) gets TAOT_INFO_SINKHORN_SIZE and a zero plan; beyond 256 ranks every problem is solved.
  * Kernel choice (all give the same iterates up to fp32 rounding): ranks whose rows and columns of the cost agree form
  * classes (in a topology cost the nodes); with few enough of them (at most 32, or 512 in nodes and rail groups) a solve
  * runs on the classes beyond 256 ranks, and from 33 ranks on with a fixed iteration count (tol <= 0).  Otherwise a cost

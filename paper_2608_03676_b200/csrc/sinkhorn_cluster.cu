@@ -14,10 +14,9 @@
 // shared-memory kernel with the matrix in workspace, which holds anything.
 #include <cooperative_groups.h>
 
-#include "sinkhorn_common.cuh"
+#include "sinkhorn_generic.cuh"
 
 namespace cg = cooperative_groups;
-using namespace taot_sk;
 
 namespace {
 
@@ -370,33 +369,53 @@ constexpr int32_t kChained = 32;      // about as many as are resident at a time
 
 // One problem per cluster; in a chained launch few clusters walk the batch and solve what an earlier kernel left (a problem
 // left over has supply and demand, so none of the four CTAs writes iters[b] before all of them have met at a barrier, or
-// writes the mark that is there: the four always agree on what to skip).
+// writes the mark that is there: the four always agree on what to skip).  Mostly nothing is left: all marks of a cluster are
+// looked at together before the walk (one after the other they took 0.6 us each).
+// FINISH: nothing is launched behind; what the walk handed back is solved here, a CTA for each problem.
+template <bool FINISH>
 __global__ void __cluster_dims__(kCluster, 1, 1) __launch_bounds__(kNT, 1)
 sinkhorn_cluster_kernel(SinkArgs a, int32_t kcap, int32_t nprob)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     cg::cluster_group cluster = cg::this_cluster();
     taot_await();
+    if (a.skip_solved) {
+        bool left = false;
+        for (int64_t b = blockIdx.x / kCluster + (int64_t)threadIdx.x * (gridDim.x / kCluster); b < nprob; b += (int64_t)kNT * (gridDim.x / kCluster))
+            left = left || a.iters[b] == kHandBack;
+        if (!__syncthreads_or(left)) return;
+    }
     for (int64_t b = blockIdx.x / kCluster; b < nprob; b += gridDim.x / kCluster) {
         if (a.skip_solved && a.iters[b] != kHandBack) continue;
         cluster_problem(a, kcap, b, smem_raw, cluster);
         cluster.sync();
     }
+    if constexpr (FINISH) {
+        // (past the last barrier the marks are final; read where the first CTA's stores are, not from this SM's cache)
+        const int64_t step = gridDim.x / kCluster;
+        for (int64_t b = blockIdx.x / kCluster + (int64_t)cluster.block_rank() * step; b < nprob; b += kCluster * step) {
+            if (__ldcg(a.iters + b) != kHandBack) continue;
+            generic_problem(a, b, smem_raw);
+            __syncthreads();
+        }
+    }
 }
 
 }  // namespace
 
-int taot_launch_sinkhorn_cluster(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st)
+int taot_launch_sinkhorn_cluster(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st, bool finish = false)
 {
     const int R = h->p.R;
     const size_t state = (csmem_state_bytes(R) + 15) & ~(size_t)15;
     const size_t budget = 226 * 1024;                                     // the kernel also has a few static bytes
     if (state + 4096 > budget) return 0;                                 // no room for a slice: nothing launched
     const int32_t kcap = (int32_t)((budget - state) / sizeof(float));
-    const size_t smem = state + sizeof(float) * (size_t)kcap;
-    TAOT_CUDA_OK(cudaFuncSetAttribute(sinkhorn_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const size_t smem = state + sizeof(float) * (size_t)kcap;            // (more than generic_smem_bytes(R, kNT, 0), 60 R bytes)
     const int32_t clusters = a.skip_solved && B > kChained ? kChained : B;
-    sinkhorn_cluster_kernel<<<(unsigned)clusters * kCluster, kNT, smem, st>>>(a, kcap, B);
-    TAOT_CUDA_OK(cudaGetLastError());
+    const auto launch = [&](auto kernel) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        return e == cudaSuccess ? taot_launch_chained(kernel, (unsigned)clusters * kCluster, kNT, smem, st, a, kcap, B) : e;
+    };
+    TAOT_CUDA_OK(finish ? launch(sinkhorn_cluster_kernel<true>) : launch(sinkhorn_cluster_kernel<false>));
     return 1;
 }

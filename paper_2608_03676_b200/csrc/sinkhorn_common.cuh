@@ -28,6 +28,8 @@ struct SinkArgs {
     int32_t skip_solved;     // tile kernels: solve only the problems an earlier kernel of the chain handed back
     float* kt_global;        // [B][kcap_global] kernel-matrix scratch in global memory for problems too big for
     int64_t kcap_global;     // shared memory (floats per problem); null / 0 if the handle has none
+    int32_t plan_rows;       // generic kernel: a problem of at most this many supply ranks that fits in neither holds its matrix in
+                             // its own block of the plan
 };
 
 // exp(x) rounded to fp32 for an fp64 argument of either sign and any magnitude the solve meets: x = xh + xl with

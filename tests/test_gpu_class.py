@@ -75,3 +75,51 @@ def test_tree_batches_tolerance_and_costs_beyond_fp32(R, B, eps, iters, tol):
 
 def test_dense_cost_beyond_fp32():
     _solve(W.cost_matrix(64, 8, (0.0, 1.0, 12.0), None), 4, 0.012, 25)
+
+
+@pytest.mark.parametrize("R,node,B,iters,tol,both", [
+    (200, 8, 4, 30, 0.0, (1, 100)),           # up to 256 ranks: one rank with both, 100 x 200 (beyond the last kernel's shared memory)
+    (256, 8, 2, 300, 1e-6, (1, 100)),         # (the tier sums hand back)
+    (384, 8, 256, 30, 0.0, (1, 384, 200)),    # a batch that costs without classes solve as dense products
+    (384, 8, 3, 25, 1e-3, (1, 384, 200)),
+    (300, 4, 3, 40, 0.0, (300,)),
+    (512, 8, 14, 20, 0.0, (1, 512)),          # clusters of the tree kernel hand back
+    (1024, 8, 2, 12, 0.0, (1, 600))])
+def test_ranks_with_supply_and_demand_are_handed_back_and_solved(R, node, B, iters, tol, both):
+    """The class kernels take disjoint supports; problems with ranks in both (one, many, all) go to the kernels behind them,
+    whatever the size of their matrix, and leave their neighbours alone."""
+    import paper_2608_03676_b200 as P
+    C = W.cost_matrix(R, node, (0.0, 1.0, 6.0, 16.0), 4)
+    g = torch.Generator().manual_seed(R + B)
+    pl = P.Planner(L=B, R=R, E=R, K=1, k=1, T=R, e2r=torch.arange(R, dtype=torch.int32), C=C, eps=1.6, max_iters=iters, tol=tol)
+    ex, sp, s, d = (t.cpu() for t in pl.excess_spare(W.sweep_rank_loads(B, R, seed=5, device="cuda")))
+    for b, n in enumerate(both):              # problems 0, 1, ...: the first n ranks of an order of their own have both
+        p = torch.randperm(R, generator=g)[:n]
+        if n == 1:
+            s[b, p] += 100.0; d[b, p] += 50.0
+        else:
+            s[b].zero_(); d[b].zero_()
+            s[b, p] = torch.randint(1, 900, (n,), generator=g).float()
+            d[b, p] = torch.randint(1, 900, (n,), generator=g).float()
+            if R <= 256:
+                d[b] = torch.randint(1, 900, (R,), generator=g).float()
+        d[b] *= 1.01 * float(s[b].sum() / d[b].sum())
+    out = pl.sinkhorn(s.cuda(), d.cuda())
+    torch.cuda.synchronize()
+    info, it = cpu(out["info"]), cpu(out["iters"])
+    assert ((info & ~2) == 0).all() and (it >= 1).all()
+    for b in sorted({*range(len(both)), B - 1}):
+        check_sinkhorn_problem(s[b].numpy(), d[b].numpy(), C.numpy(), 1.6, cpu(out["plan"])[b], it[b], cpu(out["row_err"])[b], iters, tol)
+    pl.close()
+
+
+def test_more_supply_ranks_than_the_tiles_hold_are_flagged_up_to_256_ranks():
+    import paper_2608_03676_b200 as P
+    R = 200
+    pl = P.Planner(L=1, R=R, E=R, K=1, k=1, T=R, e2r=torch.arange(R, dtype=torch.int32), C=W.cost_matrix(R, 8, (0.0, 1.0, 6.0, 16.0), 4),
+                   eps=1.6, max_iters=10)
+    s = torch.ones((1, R), device="cuda"); d = torch.ones((1, R), device="cuda")
+    s[0, :60] = 0.0                           # 140 x 200
+    out = pl.sinkhorn(s, d)
+    assert int(out["info"][0]) & P.INFO_SINKHORN_SIZE and float(out["plan"].abs().max()) == 0.0
+    pl.close()

@@ -32,3 +32,21 @@ def test_wide_kernel_by_supply_ranks(R, rows, iters, tol, check_every):
         check_sinkhorn_problem(s[b].numpy(), d[b].numpy(), C.numpy(), eps, cpu(out["plan"])[b], cpu(out["iters"])[b],
                                cpu(out["row_err"])[b], iters, tol, check_every)
     pl.close()
+
+
+@pytest.mark.parametrize("R,n", [(512, 512), (300, 180)])
+def test_ranks_with_supply_and_demand_beyond_every_capacity(R, n):
+    """All ranks (or 180 of 300) with both: the matrix is larger than a quarter of R x R, which disjoint supports never exceed."""
+    import paper_2608_03676_b200 as P
+    g = torch.Generator().manual_seed(R)
+    C = 1.0 + 15.0 * torch.rand((R, R), generator=g)
+    C.fill_diagonal_(0.0)
+    s = torch.zeros((2, R)); d = torch.zeros((2, R))
+    s[0, :n] = torch.randint(1, 900, (n,), generator=g).float(); d[0, R - n:] = torch.randint(1, 900, (n,), generator=g).float()
+    s[1, :20] = 50.0; d[1, 20:] = 3.0
+    pl = P.Planner(L=2, R=R, E=R, K=1, k=1, T=R, e2r=torch.arange(R, dtype=torch.int32), C=C, eps=2.0, max_iters=66)
+    out = pl.sinkhorn(s.cuda(), d.cuda())
+    assert ((cpu(out["info"]) & ~16) == 0).all()
+    for b in range(2):
+        check_sinkhorn_problem(s[b].numpy(), d[b].numpy(), C.numpy(), 2.0, cpu(out["plan"])[b], cpu(out["iters"])[b], cpu(out["row_err"])[b], 66, 0.0)
+    pl.close()

@@ -107,3 +107,24 @@ def test_a_plan_releases_the_matching_kernel_only_behind_the_merge(so, R, genera
     assert args.R == R and args.early == 1
     assert names[at - 1] not in ("merge_kernel", "hist_chunk_kernel") and names[at + 1] == "match_kernel"
     pl.close()
+
+
+def _route(so, B, R, C, **kw):
+    """Kernels of one Phase-1 call, in order, each named once."""
+    so.fake_reset()
+    pl = F.FakePlanner(so, B, R, R, 1, 1, R, C, **kw)
+    so.fake_reset()
+    assert pl.sinkhorn(B) == 0
+    pl.close()
+    return list(dict.fromkeys(F.kernels(so)))
+
+
+@pytest.mark.parametrize("R,B,tol,want", [
+    (32, 3, 0.0, ["sinkhorn_tile_kernel", "sinkhorn_kernel", "sinkhorn_input_guard_kernel"]),
+    (64, 3, 1e-6, ["sinkhorn_tile_kernel", "sinkhorn_kernel", "sinkhorn_input_guard_kernel"]),
+    (64, 3, 0.0, ["sinkhorn_class_kernel", "sinkhorn_kernel"]),
+    (256, 300, 0.0, ["sinkhorn_class_kernel", "sinkhorn_kernel"]),
+    (384, 300, 0.0, ["sinkhorn_class_tree_kernel", "sinkhorn_cluster_kernel"]),
+    (1024, 3, 1e-6, ["sinkhorn_class_tree_kernel", "sinkhorn_cluster_kernel"])])
+def test_kernels_of_phase_1_on_a_cost_with_classes(so, R, B, tol, want):
+    assert _route(so, B, R, W.cost_matrix(R, 8, (0.0, 1.0, 6.0, 16.0), 4), tol=tol) == want
