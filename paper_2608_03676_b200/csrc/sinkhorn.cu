@@ -128,9 +128,10 @@ int taot_launch_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, in
                 if (ntc < 0) return ntc;
                 if (ntc > 0) { launched += ntc; continue; }
             }
-            // otherwise up to 512 ranks one CTA holds the compacted matrix in registers; what it hands back, and larger
-            // problems, go to four-CTA clusters that hold it in distributed shared memory; what those hand back (or
-            // everything, if no slice fits) to the kernel below with the matrix in workspace
+            // otherwise up to 512 ranks one CTA holds the compacted matrix in its registers and shared memory, whatever
+            // the number of supply ranks; what it hands back (supports that overlap), and larger problems, go to four-CTA
+            // clusters that hold it in distributed shared memory; what those hand back (or everything, if no slice fits) to
+            // the kernel below with the matrix in workspace
             a.skip_solved = 0;
             const int nw = taot_launch_sinkhorn_wide(h, a, nb, st);
             if (nw < 0) return nw;

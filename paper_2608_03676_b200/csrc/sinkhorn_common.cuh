@@ -49,7 +49,8 @@ constexpr float kSumHi = 1e30f;
 constexpr int kHandBack = -1;               // iters[b] value meaning "not solved here"
 
 // ordered compaction of {i < R : val[i] > 0} into list[], positions into pos[]; returns the count
-__device__ inline int compact_positive(const float* val, int R, int32_t* list, int32_t* pos, int32_t* wcnt)
+template <typename I>
+__device__ inline int compact_positive(const float* val, int R, I* list, I* pos, int32_t* wcnt)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = blockDim.x >> 5;
     int total = 0;
@@ -64,8 +65,8 @@ __device__ inline int compact_positive(const float* val, int R, int32_t* list, i
         if (i < R) pos[i] = -1;
         if (p) {
             const int q = off + __popc(m & ((1u << lane) - 1u));
-            list[q] = i;
-            pos[i] = q;
+            list[q] = (I)i;
+            pos[i] = (I)q;
         }
         for (int w = 0; w < NW; ++w) total += wcnt[w];
         __syncthreads();

@@ -1,6 +1,6 @@
-"""Phase 1 with a cost without structure at 257 to 512 ranks (the kernel matrix in the registers of one CTA): the edges of its
-row builds (16, 32 and 64 supply ranks, and one more, which goes to the kernels behind it), ragged rank counts, a fixed count
-and the stopping rule, against the oracle."""
+"""Phase 1 with a cost without structure at 257 to 512 ranks (the kernel matrix in the registers of one CTA, rows beyond 64 in
+its shared memory): the edges of its row builds (16, 32 and 64 supply ranks and one more; the largest products of supply and
+demand ranks; few demand ranks), ragged rank counts, a fixed count and the stopping rule, against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -10,7 +10,8 @@ from helpers import check_sinkhorn_problem, cpu
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("R,rows", [(257, (1, 16, 17, 32)), (288, (33, 64, 65, 2)), (300, (31, 63, 66, 15)), (512, (54, 64, 16, 200))])
+@pytest.mark.parametrize("R,rows", [(257, (1, 16, 17, 32)), (288, (33, 64, 65, 2)), (300, (31, 63, 66, 15)), (512, (54, 64, 16, 200)),
+                                    (257, (128, 250, 67, 256)), (301, (150, 185, 290, 68)), (512, (256, 288, 291, 285)), (511, (69, 448, 510, 130))])
 @pytest.mark.parametrize("iters,tol,check_every", [(70, 0.0, 1), (300, 1e-5, 1), (300, 1e-5, 7)])
 def test_wide_kernel_by_supply_ranks(R, rows, iters, tol, check_every):
     import paper_2608_03676_b200 as P
