@@ -216,11 +216,11 @@ int taot_excess_spare(taot_handle_t h, const int32_t* d_rank_load, int32_t B, in
  * runs on the classes beyond 256 ranks, and from 33 ranks on with a fixed iteration count (tol <= 0).  Otherwise a cost
  * that depends only on the tier of a rank pair (same node / same rail group / neither; see taot_tier_structure) at 256
  * ranks is summed tier by tier; up to 256 ranks the kernel matrix of a problem lives in registers or shared memory;
- * from 257 to 512 ranks (64 iterations and more) in the registers of one CTA.  A batch of at least 256 problems of more
- * than 512 ranks, or of fewer than 64 iterations, with a fixed iteration count and max(C)/eps <= 20 is solved as dense
+ * from 257 to 512 ranks in the registers and the shared memory of one CTA; beyond, in the shared memory of four.  A batch
+ * of at least 256 problems with a fixed iteration count, max(C)/eps <= 20 and a multiple of 128 ranks, either more than
+ * 512 of them or fewer than 64 iterations, is solved as dense
  * products [R,R] x [R,B] on the tensor cores (tcgen05, three TF32 products per term; the row error it reports is the
- * true row violation of the returned plan, a few 1e-6 of the total mass from accumulator truncation), anything else
- * beyond 256 ranks by four-CTA clusters.  Environment, read at taot_create / at the call: TAOT_NO_TENSOR_CORES (any value)
+ * true row violation of the returned plan, a few 1e-6 of the total mass from accumulator truncation).  Environment, read at taot_create / at the call: TAOT_NO_TENSOR_CORES (any value)
  * keeps the dense path off, TAOT_TC_TILE_N = 64 | 128 | 256 forces its tile width.
  * A problem whose s or d holds a NaN or an infinity gets TAOT_INFO_NONFINITE, a zero
  * plan and 0 iterations; the other problems of the batch are not affected.
@@ -353,8 +353,10 @@ int taot_report(taot_handle_t h, const int32_t* d_expert_load, const int32_t* d_
 
 /*
  * The hierarchy taot_create found in the cost matrix (Appendix A.1 builds W from node membership): if C depends
- * only on whether two ranks share a node, share a rail group of nodes, or neither, with block sizes that are recognised (ranks per node / per group: 8 / 32, 4 / 16, 4 / 32, 16 / 32; 256, 512 or 1024
- * ranks), *node and *group receive those sizes; otherwise both are 0 and the kernels that hold the kernel matrix run.
+ * only on whether two ranks share a node, share a rail group of nodes, or neither, with block sizes that are recognised
+ * (ranks per node / per group: 8 / 32, 4 / 16, 4 / 32, 16 / 32; 256, 512 or 1024 ranks), *node and *group receive those
+ * sizes; otherwise both are 0.  At 256 ranks it decides whether a solve is summed tier by tier; at 512 and 1024 it
+ * decides nothing (such a cost has classes, see taot_sinkhorn) and is only reported.
  */
 int taot_tier_structure(taot_handle_t h, int32_t* node, int32_t* group);
 

@@ -58,8 +58,6 @@ int taot_launch_sinkhorn_guard(taot_handle_t h, const float* d_s, const float* d
 // batch with a fixed iteration count (R > 32: below, the register tiles are as fast).  Inside taot_plan, and in tolerance mode,
 // Phase 1 stays on the tile and tier-sum kernels: the placement that follows decides exact ties (experts of one node's
 // ranks on one cold rank) by the last bits of the hint, so its kernel is part of the result.
-constexpr int kWideMinIters = 64;     // see taot_launch_sinkhorn_wide
-
 bool taot_sinkhorn_takes_classes(taot_handle_t h, bool from_loads)
 {
     const taot_params& p = h->p;
@@ -123,7 +121,7 @@ int taot_launch_sinkhorn(taot_handle_t h, const float* d_s, const float* d_d, in
         } else {
             // beyond 256 ranks.  A large batch with a short fixed count and a Gibbs kernel inside fp32 (or more than 512
             // ranks): the whole batch as dense products on the tensor cores (complete: nothing is handed on)
-            if (p.R > 512 || p.max_iters < kWideMinIters) {
+            if (p.R > 512 || p.max_iters < TAOT_WIDE_MIN_ITERS) {
                 const int ntc = taot_launch_sinkhorn_dense_tc(h, a, nb, d_tc, st);
                 if (ntc < 0) return ntc;
                 if (ntc > 0) { launched += ntc; continue; }

@@ -827,9 +827,8 @@ sinkhorn_wide_kernel(SinkArgs a, int64_t nprob, int32_t cap)
 
 // Launches the kernel for 257 to 512 ranks (returns 1), otherwise nothing (0).
 //
-// Against the dense tensor-core solve (sinkhorn_dense_tc.cu), which multiplies all R x R entries whatever the supports: that
-// one keeps the solves of fewer than kWideMinIters iterations it applies to (a few milliseconds at most; its cost does not
-// depend on how many ranks have supply, and its row error is measured on the plan itself), this one takes the long ones.
+// Against the dense tensor-core solve (sinkhorn_dense_tc.cu), which multiplies all R x R entries whatever the supports: see
+// TAOT_WIDE_MIN_ITERS.
 int taot_launch_sinkhorn_wide(taot_handle_t h, const SinkArgs& a, int32_t B, cudaStream_t st)
 {
     if (a.R <= 256 || a.R > kMaxR) return 0;

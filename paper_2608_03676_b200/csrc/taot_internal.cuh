@@ -16,6 +16,18 @@
 #define TAOT_MAX_TIERS 8                   // distinct bonus values the bit-set auction handles
 #define TAOT_MERGE_PARTS 8                 // CTAs that share the merge of one layer's chunk counts (256-rank tables)
 #define TAOT_HOST_GROUP_BYTES (2 << 20)    // routing table from which a host call is split into layer groups
+// Costs without structure at 257 to 512 ranks, large batches with a fixed count: from this many iterations on the kernel with the
+// matrix in one CTA (sinkhorn_wide.cu), below it the dense products on the tensor cores (sinkhorn_dense_tc.cu), whose time does
+// not depend on the supports.  512 ranks, 54 / 256 supply ranks against the dense products, ms:
+//   iterations       256 problems          1024 problems          4096 problems
+//       10        0.21 / 0.57 : 0.70     0.65 / 1.86 : 1.21      2.5 / 7.2 : 3.6
+//       40        0.25 / 0.75 : 1.93     0.77 / 2.50 : 2.43      3.0 / 9.8 : 5.9
+//       64        0.28 / 0.90 : 2.91     0.91 / 3.04 : 3.42      3.5 / 11.9 : 7.8
+//      500        1.01 / 3.64 : 20.8     3.46 / 12.6 : 21.3     13.8 / 50.2 : 41.7
+// So it is no line at which one becomes faster: with few supply ranks the one-CTA kernel always is.  From 64 iterations on it is
+// up to 1024 problems whatever the loads; below, the dense products are up to twice as fast where half of the ranks have
+// supply, and 1.4 to 8 times as slow where a tenth has.
+#define TAOT_WIDE_MIN_ITERS 64
 #define TAOT_MAX_GROUPS 6                  // layer groups taot_plan overlaps on internal streams
 
 struct taot_handle_s {

@@ -128,3 +128,15 @@ def _route(so, B, R, C, **kw):
     (1024, 3, 1e-6, ["sinkhorn_class_tree_kernel", "sinkhorn_cluster_kernel"])])
 def test_kernels_of_phase_1_on_a_cost_with_classes(so, R, B, tol, want):
     assert _route(so, B, R, W.cost_matrix(R, 8, (0.0, 1.0, 6.0, 16.0), 4), tol=tol) == want
+
+
+_WIDE = ["sinkhorn_wide_kernel", "sinkhorn_cluster_kernel", "sinkhorn_kernel", "sinkhorn_input_guard_kernel"]
+_DENSE = ["tc_prepare_kernel", "sinkhorn_tc_halfstep_kernel", "tc_finalize_kernel", "tc_report_kernel", "sinkhorn_input_guard_kernel"]
+
+
+@pytest.mark.parametrize("R,B,iters,tol,eps,want", [
+    (512, 300, 63, 0.0, 1.0, _DENSE), (512, 300, 64, 0.0, 1.0, _WIDE), (512, 255, 63, 0.0, 1.0, _WIDE), (512, 300, 63, 1e-6, 1.0, _WIDE),
+    (384, 300, 63, 0.0, 0.09, _WIDE), (300, 300, 63, 0.0, 1.0, _WIDE),             # C / eps beyond 20; no multiple of 128
+    (640, 300, 500, 0.0, 1.0, _DENSE), (640, 255, 500, 0.0, 1.0, _WIDE[1:])])
+def test_kernels_of_phase_1_on_a_cost_without_structure(so, R, B, iters, tol, eps, want):
+    assert _route(so, B, R, _rough(R), tol=tol, max_iters=iters, eps=eps) == want
