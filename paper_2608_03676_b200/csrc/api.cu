@@ -44,6 +44,12 @@ int upload(T** dst, const T* src, size_t count)
     return TAOT_OK;
 }
 
+// calls of a handle that may be solved as dense products on the tensor cores (taot_launch_sinkhorn; the cost decides further)
+bool dense_products_possible(const taot_params& p)
+{
+    return p.R > 256 && p.R % 128 == 0 && p.tol <= 0.0f && p.L >= 256 && (p.R > 512 || p.max_iters < TAOT_WIDE_MIN_ITERS);
+}
+
 void layout(taot_handle_t h)
 {
     const taot_params& p = h->p;
@@ -73,7 +79,7 @@ void layout(taot_handle_t h)
     h->off_dc = take(path * sizeof(int32_t) * LR * h->nc * ((size_t)p.E + (size_t)p.R * p.K + 1));
     h->off_wp = take(path * sizeof(uint16_t) * LR * h->nc * (TAOT_STREAM_THREADS / 32) * ((size_t)p.E + (size_t)p.R * p.K + 1));
     h->off_cyc = take(path * sizeof(long long) * (size_t)p.L * 16);
-    h->off_tc = take((p.R > 256 && p.R % 128 == 0) ? sizeof(float) * taot_sinkhorn_tc_ws_floats(p.R, p.L) : 0);
+    h->off_tc = take(dense_products_possible(p) ? sizeof(float) * taot_sinkhorn_tc_ws_floats(p.R, p.L) : 0);
     h->tb_ok = (path && p.E <= 256 && h->seg % 16 == 0) ? 1 : 0;
     h->off_tb = take(h->tb_ok ? (size_t)p.L * (size_t)p.T * p.k : 0);
     h->off_tbflag = take(path * sizeof(int32_t) * LR * h->nc);
@@ -310,11 +316,11 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
         for (int j = 0; j < R; ++j) acc += std::exp(-(double)h_C[(size_t)i * R + j] / (double)params->eps - mx);
         lse0[i] = mx + std::log(acc);
     }
-    // Gibbs kernel for the tensor-core solve (more than 256 ranks, no tier structure, exp(-C/eps) well inside fp32):
+    // Gibbs kernel for the tensor-core solve (where a call can take it; no classes, exp(-C/eps) well inside fp32):
     // M and its transpose, each split into two TF32-exact parts (high: low 13 mantissa bits cleared; low: the rest,
     // again with 13 bits cleared)
     std::vector<float> gibbs;
-    if (R > 256 && R % 128 == 0 && !classes.kind && !std::getenv("TAOT_NO_TENSOR_CORES")) {
+    if (dense_products_possible(h->p) && !classes.kind && !std::getenv("TAOT_NO_TENSOR_CORES")) {
         double worst = 0.0;
         for (size_t q = 0; q < (size_t)R * R; ++q) worst = std::max(worst, (double)h_C[q] / (double)params->eps);
         if (worst <= 20.0) {

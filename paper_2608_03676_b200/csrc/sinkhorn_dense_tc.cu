@@ -497,7 +497,8 @@ size_t taot_sinkhorn_tc_ws_floats(int32_t R, int32_t B)
 
 // The whole fixed-count solve of a batch on the tensor cores, or 0 launches if this call is not its case (the caller
 // then takes the other kernels): more than 256 ranks in multiples of 128, a handle whose Gibbs kernel fits fp32
-// (taot_create built it), no tolerance test, and a batch large enough to fill the GPU with tiles.
+// (taot_create built it, for handles whose calls can come here), no tolerance test, and a batch large enough to fill the GPU
+// with tiles.
 int taot_launch_sinkhorn_dense_tc(taot_handle_t h, const SinkArgs& a, int32_t B, float* ws_tc, cudaStream_t st)
 {
     if (!h->d_gibbs || !ws_tc || a.tol > 0.0f || a.R <= 256 || a.R % kTileM != 0 || B < 256 || B > h->p.L) return 0;

@@ -40,7 +40,7 @@ struct taot_handle_s {
     float* d_B;              // [R,R] topology preference (given or derived)
     double* d_rowlse0;       // [R]  LSE_j(-C_ij/eps) over all ranks j: the first u-update with v = 1
     float* d_gibbs;          // [4][R,R] exp(-C/eps) and its transpose, each as TF32-exact high and low parts (tensor-core
-                             // solve: more than 256 ranks, no tier structure, max C/eps <= 20), else null
+                             // solve: where a call can take it and max C/eps <= 20), else null
     int32_t* d_rank_off;     // [R+1] CSR of experts by home rank
     int32_t* d_rank_list;    // [E]
     uint32_t* d_tiermask;    // [ntiers][W][R hosts] bit r of word w set iff bonus(32w + r -> host) == tierval[t]; null if ntiers == 0

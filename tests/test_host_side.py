@@ -140,3 +140,12 @@ _DENSE = ["tc_prepare_kernel", "sinkhorn_tc_halfstep_kernel", "tc_finalize_kerne
     (640, 300, 500, 0.0, 1.0, _DENSE), (640, 255, 500, 0.0, 1.0, _WIDE[1:])])
 def test_kernels_of_phase_1_on_a_cost_without_structure(so, R, B, iters, tol, eps, want):
     assert _route(so, B, R, _rough(R), tol=tol, max_iters=iters, eps=eps) == want
+
+
+@pytest.mark.parametrize("R,L,iters,tol,made", [(512, 300, 63, 0.0, True), (640, 256, 500, 0.0, True), (512, 300, 64, 0.0, False),
+                                                (640, 255, 500, 0.0, False), (640, 256, 500, 1e-6, False), (512, 3, 10, 0.0, False)])
+def test_the_gibbs_kernel_is_made_only_for_handles_whose_calls_can_take_it(so, R, L, iters, tol, made):
+    so.fake_reset()
+    pl = F.FakePlanner(so, L, R, R, 1, 1, R, _rough(R), tol=tol, max_iters=iters)
+    assert (16 * R * R in [e.obj for e in F.log(so) if e.kind == F.DEVICE_ALLOC]) == made
+    pl.close()
