@@ -77,7 +77,8 @@ void layout(taot_handle_t h)
     h->off_t12 = take(path * sizeof(float) * (size_t)p.L * p.E * 2 * p.R);
     h->off_kt = take(sizeof(float) * (size_t)p.L * (size_t)h->kcap_global);
     h->off_dc = take(path * sizeof(int32_t) * LR * h->nc * ((size_t)p.E + (size_t)p.R * p.K + 1));
-    h->off_wp = take(path * sizeof(uint16_t) * LR * h->nc * (TAOT_STREAM_THREADS / 32) * ((size_t)p.E + (size_t)p.R * p.K + 1));
+    h->wp_ok = path && taot_dispatch_keeps_counts((int64_t)p.E + (int64_t)p.R * p.K + 1, h->seg) ? 1 : 0;
+    h->off_wp = take(h->wp_ok * sizeof(uint16_t) * LR * h->nc * (TAOT_STREAM_THREADS / 32) * ((size_t)p.E + (size_t)p.R * p.K + 1));
     h->off_cyc = take(path * sizeof(long long) * (size_t)p.L * 16);
     h->off_tc = take(dense_products_possible(p) ? sizeof(float) * taot_sinkhorn_tc_ws_floats(p.R, p.L) : 0);
     h->tb_ok = (path && p.E <= 256 && h->seg % 16 == 0) ? 1 : 0;

@@ -12,8 +12,8 @@
 //                            word per target and ranked by lane, so the order stays stable
 // 12 bytes of HBM traffic per entry (two reads of the table, one write of the positions), but what bounds it is random access
 // to shared memory: 32 lanes on 385 targets meet in the same bank 3.3 deep, and a step makes five such accesses beside the
-// count's one.  The count is made by warp, so that the scatter need not count its spans again: 64 ranks x 58 layers (1 GB)
-// 877 -> 757 us.  (One cluster per segment that reads the table once was built and made the same accesses in the same time:
+// count's one.  The count is made by warp, so that the scatter need not count its spans again where a chunk has entries
+// enough for its bins (taot_dispatch_keeps_counts): 64 ranks x 58 layers (1 GB) 877 -> 757 us.  (One cluster per segment that reads the table once was built and made the same accesses in the same time:
 // 0.83 to 1.05 ms at 64 ranks x 58 layers; finding the lanes by votes 1.05, by match 1.8 ms.)
 #include "taot_internal.cuh"
 
@@ -26,7 +26,7 @@ constexpr int kWarpSpan = TAOT_CHUNK / kWarps;
 struct DispatchArgs {
     const int32_t* idx;        // [L,T,k] rewritten routing table
     int32_t* dc;               // [L,R,NC,NB] chunk counts, then chunk bases
-    uint16_t* wp;              // [L,R,NC,kWarps,NB] entries of the bin in the spans of the chunk before this warp's
+    uint16_t* wp;              // [L,R,NC,kWarps,NB] entries of the bin in the spans of the chunk before this warp's, or null
     const int32_t* torder;     // [NB] bin at each sorted position
     const int32_t* tdest;      // [NB] destination rank of each bin (R for the undeliverable bin)
     int32_t* send_counts;      // [L,R,R]
@@ -51,25 +51,13 @@ __device__ __forceinline__ int bin_of(int32_t v, int NB) { return (unsigned)v < 
 
 __device__ __forceinline__ void count_add(uint32_t addr) { asm volatile("red.shared.add.u32 [%0], 1;" ::"r"(addr) : "memory"); }
 
-// Counts of a chunk by warp, each over its contiguous span, and from them the chunk's counts and the sums over the spans
-// before each warp's.  (At most 16384 entries before a span: 16 bits.)
-__global__ void __launch_bounds__(kThreads)
-dispatch_count_kernel(DispatchArgs a)
+// a warp's counts over its contiguous span of n entries
+__device__ __forceinline__ void count_span(const int32_t* src, int n, int32_t* counts, int NB, bool vec_ok)
 {
-    extern __shared__ int32_t wh[];            // [kWarps][NB]
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NB = a.NB;
-    const int64_t id = blockIdx.x;
-    int64_t goff; int32_t len;
-    chunk_span(a, id, goff, len);
-    for (int q = tid; q < kWarps * NB; q += kThreads) wh[q] = 0;
-    __syncthreads();
-    taot_await();
-    taot_release();
-    const int s0 = warp * kWarpSpan, n = min(len - s0, kWarpSpan);
-    const int32_t* src = a.idx + goff + s0;
-    const uint32_t mine = (uint32_t)__cvta_generic_to_shared(wh + warp * NB);
+    const int lane = threadIdx.x & 31;
+    const uint32_t mine = (uint32_t)__cvta_generic_to_shared(counts);
     int i = 0;
-    if (a.vec_ok && n == kWarpSpan) {
+    if (vec_ok && n == kWarpSpan) {
         const int4* src4 = reinterpret_cast<const int4*>(src) + lane;
 #pragma unroll 1
         for (int h = 0; h < kWarpSpan / 128; h += 8) {
@@ -87,8 +75,35 @@ dispatch_count_kernel(DispatchArgs a)
         i = kWarpSpan;
     }
     for (i += lane; i < n; i += 32) count_add(mine + 4u * (uint32_t)bin_of(__ldcs(src + i), NB));
+}
+
+// Counts of a chunk by warp, each over its contiguous span, and from them the chunk's counts and (a.wp) the sums over the spans
+// before each warp's.  (At most 16384 entries before a span: 16 bits.)
+__global__ void __launch_bounds__(kThreads)
+dispatch_count_kernel(DispatchArgs a)
+{
+    extern __shared__ int32_t wh[];            // [kWarps][NB]
+    const int tid = threadIdx.x, warp = tid >> 5, NB = a.NB;
+    const int64_t id = blockIdx.x;
+    int64_t goff; int32_t len;
+    chunk_span(a, id, goff, len);
+    for (int q = tid; q < kWarps * NB; q += kThreads) wh[q] = 0;
+    __syncthreads();
+    taot_await();
+    taot_release();
+    const int s0 = warp * kWarpSpan;
+    count_span(a.idx + goff + s0, min(len - s0, kWarpSpan), wh + warp * NB, NB, a.vec_ok);
     __syncthreads();
     int32_t* out = a.dc + id * NB;
+    if (!a.wp) {
+        for (int b = tid; b < NB; b += kThreads) {
+            int32_t run = 0;
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) run += wh[w * NB + b];
+            out[b] = run;
+        }
+        return;
+    }
     uint16_t* wp = a.wp + id * kWarps * NB;
     for (int b = tid; b < NB; b += kThreads) {
         int32_t run = 0;
@@ -160,7 +175,8 @@ dispatch_offsets_kernel(DispatchArgs a)
 
 // ALT: the mask words of consecutive ranking steps sit in alternating rows (one warp barrier fewer per step); otherwise one
 // row, for target counts whose three rows would not fit in shared memory.
-template <bool ALT>
+// PRE: where a warp's entries start comes from the counting pass (a.wp); otherwise the spans are counted again here.
+template <bool ALT, bool PRE>
 __global__ void __launch_bounds__(kThreads)
 dispatch_scatter_kernel(DispatchArgs a)
 {
@@ -173,9 +189,23 @@ dispatch_scatter_kernel(DispatchArgs a)
     const int s0 = warp * kWarpSpan, n = min(len - s0, kWarpSpan);
     const int32_t* src = a.idx + goff + s0;
     int32_t* dst = a.perm + goff + s0;
-    for (int q = kWarps * NB + tid; q < (ALT ? 3 : 2) * kWarps * NB; q += kThreads) wh[q] = 0;
+    for (int q = (PRE ? kWarps * NB : 0) + tid; q < (ALT ? 3 : 2) * kWarps * NB; q += kThreads) wh[q] = 0;
+    if constexpr (!PRE) __syncthreads();
     taot_await();
-    {
+    if constexpr (!PRE) {
+        count_span(src, n, wh + warp * NB, NB, a.vec_ok);
+        __syncthreads();
+        const int32_t* base = a.dc + id * (int64_t)NB;
+        for (int b = tid; b < NB; b += kThreads) {
+            int32_t run = base[b];
+#pragma unroll
+            for (int w = 0; w < kWarps; ++w) {
+                const int32_t t = wh[w * NB + b];
+                wh[w * NB + b] = run;
+                run += t;
+            }
+        }
+    } else {
         const int32_t* base = a.dc + id * (int64_t)NB;
         const uint16_t* wp = a.wp + id * kWarps * (int64_t)NB;
         for (int b = tid; b < NB; b += kThreads) {
@@ -245,7 +275,7 @@ int taot_launch_dispatch(taot_handle_t h, const int32_t* d_new_idx, int32_t* d_s
     DispatchArgs a;
     a.idx = d_new_idx;
     a.dc = reinterpret_cast<int32_t*>(static_cast<char*>(ws) + h->off_dc);
-    a.wp = reinterpret_cast<uint16_t*>(static_cast<char*>(ws) + h->off_wp);
+    a.wp = h->wp_ok ? reinterpret_cast<uint16_t*>(static_cast<char*>(ws) + h->off_wp) : nullptr;
     a.torder = h->d_torder; a.tdest = h->d_tdest;
     a.send_counts = d_send_counts; a.target_counts = d_target_counts; a.perm = d_perm; a.info = d_info;
     a.layer_elems = p.T * p.k; a.seg = h->seg; a.nc = h->nc; a.R = p.R; a.NB = p.E + p.R * p.K + 1;
@@ -255,12 +285,14 @@ int taot_launch_dispatch(taot_handle_t h, const int32_t* d_new_idx, int32_t* d_s
     const size_t sm2 = sizeof(int32_t) * (2 * (size_t)a.NB + p.R + 1);
     const bool alt = sizeof(int32_t) * 3 * (size_t)kWarps * a.NB <= 64 * 1024;
     const size_t sm3 = sizeof(int32_t) * (alt ? 3 : 2) * (size_t)kWarps * a.NB;
-    if (alt) TAOT_CUDA_OK(cudaFuncSetAttribute(dispatch_scatter_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3));
-    else TAOT_CUDA_OK(cudaFuncSetAttribute(dispatch_scatter_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3));
+    const auto scatter = [&](auto kernel) {
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm3);
+        return e == cudaSuccess ? taot_launch_chained(kernel, chunks, kThreads, sm3, st, a) : e;
+    };
     TAOT_CUDA_OK(cudaFuncSetAttribute(dispatch_count_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm1));
     TAOT_CUDA_OK(taot_launch_chained(dispatch_count_kernel, chunks, kThreads, sm1, st, a));
     TAOT_CUDA_OK(taot_launch_chained(dispatch_offsets_kernel, (unsigned)((int64_t)p.L * p.R), kThreads, sm2, st, a));
-    if (alt) TAOT_CUDA_OK(taot_launch_chained(dispatch_scatter_kernel<true>, chunks, kThreads, sm3, st, a));
-    else TAOT_CUDA_OK(taot_launch_chained(dispatch_scatter_kernel<false>, chunks, kThreads, sm3, st, a));
+    if (a.wp) TAOT_CUDA_OK(alt ? scatter(dispatch_scatter_kernel<true, true>) : scatter(dispatch_scatter_kernel<false, true>));
+    else TAOT_CUDA_OK(alt ? scatter(dispatch_scatter_kernel<true, false>) : scatter(dispatch_scatter_kernel<false, false>));
     return 3;
 }

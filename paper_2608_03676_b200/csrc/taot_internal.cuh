@@ -75,6 +75,7 @@ struct taot_handle_s {
     // workspace layout (byte offsets)
     size_t off_cc, off_excess, off_spare, off_s, off_d, off_nrem, off_t12, off_kt, off_dc, off_wp, off_cyc, off_tc;
     size_t off_tb, off_tbflag;   // one-byte copy of the routing table (see tb_ok) and one flag per chunk (a value that is no expert)
+    int32_t wp_ok;               // 1: dispatch keeps its counting pass's counts by warp for the scatter (off_wp)
     int32_t tb_ok;               // 1: the histogram pass also leaves the table as one byte per entry (E <= 256 experts,
                                  // segments of a multiple of 16 entries) for the reassignment to read instead of the table
     size_t ws_bytes;
@@ -141,6 +142,19 @@ int taot_launch_report(taot_handle_t h, const int32_t* d_expert_load, const int3
                        int32_t* d_spill, int32_t* d_load_after, int32_t* d_slot_moved, int32_t* d_slot_kind,
                        cudaStream_t st);
 
+// Whether the counting pass of dispatch leaves its counts by warp span, 16 bytes per bin and chunk, for the scatter, which otherwise
+// counts its spans again: not where a chunk has fewer entries than half the bins, and not where one scatter CTA fills an SM
+// (beyond 1816 bins: nothing hides those reads) unless a chunk has eight entries per bin.  Kept against counted again, us, by
+// entries per segment (layers x ranks chunks as in brackets):
+//     385 bins, 64 ranks     256: 56.9 : 57.1 [3840]     1024:  87 :  97 [3840]     16384: 51 : 59 [192]
+//    1281 bins, 256 ranks    256:  118 : 109  [2048]     1024: 143 : 158 [2048]     16384: 43 : 44 [256]
+//    2049 bins, 256 ranks    256:  212 : 169  [2048]     4096: 257 : 199 [1792]     16384: 56 : 55 [256]
+//    3073 bins, 256 ranks    256:  328 : 244  [2048]     4096: 386 : 298 [1792]     16384: 84 : 80 [256]
+static inline bool taot_dispatch_keeps_counts(int64_t bins, int64_t seg)
+{
+    const int64_t entries = seg < TAOT_CHUNK ? seg : TAOT_CHUNK;
+    return bins <= 1816 ? 2 * entries >= bins : entries >= 8 * bins;
+}
 int taot_launch_dispatch(taot_handle_t h, const int32_t* d_new_idx, int32_t* d_send_counts, int32_t* d_target_counts,
                          int32_t* d_perm, int32_t* d_info, void* ws, cudaStream_t st);
 

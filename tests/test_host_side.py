@@ -149,3 +149,16 @@ def test_the_gibbs_kernel_is_made_only_for_handles_whose_calls_can_take_it(so, R
     pl = F.FakePlanner(so, L, R, R, 1, 1, R, _rough(R), tol=tol, max_iters=iters)
     assert (16 * R * R in [e.obj for e in F.log(so) if e.kind == F.DEVICE_ALLOC]) == made
     pl.close()
+
+
+@pytest.mark.parametrize("R,E,K,seg,kept", [(256, 1024, 8, 16384, False), (256, 1024, 8, 300, False), (64, 256, 2, 192, False),
+                                            (64, 256, 2, 193, True), (128, 791, 8, 908, True), (128, 792, 8, 908, False), (128, 1023, 8, 16384, True)])
+def test_dispatch_workspace_follows_the_entries_of_a_chunk(so, R, E, K, seg, kept):
+    """Counts by warp take 16 bytes per bin and chunk; they are kept only where a chunk has entries enough for its bins."""
+    pl = F.FakePlanner(so, 2, R, E, K, 1, R * seg, W.cost_matrix(R, 8, (0.0, 1.0, 6.0, 16.0), 4), max_iters=10)
+    n = ctypes.c_size_t()
+    assert so.taot_workspace_bytes(pl.handle, ctypes.byref(n)) == 0
+    bins, S = E + R * K + 1, R * K
+    rest = 4 * 2 * R * (2 * E + 4 + bins + 2 * E + min(E, S) + 1) + 256 * 2 * R + 2 * R * seg + 4096 * 16       # everything else, generously
+    assert (n.value > 16 * bins * 2 * R) if kept else (n.value < rest)
+    pl.close()
