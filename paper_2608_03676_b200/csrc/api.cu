@@ -269,7 +269,8 @@ int taot_create(taot_handle_t* out, const taot_params* params, const int32_t* h_
     }
     h->nbid = (int32_t)bidlist.size();
     // a cost that depends only on "same node of 8 ranks / same rail group of 32 ranks / neither" lets the Sinkhorn
-    // sums be taken tier by tier (sinkhorn_tiered.cu)
+    // sums be taken tier by tier (sinkhorn_tiered.cu, 256 ranks; at 512 and 1024 only taot_tier_structure reports it: such a
+    // cost has classes)
     h->tier_ok = 0;
     if (R == 256 || R == 512 || R == 1024) {
         // The block sizes are read off the first row: a node is the run of ranks at rank 0's cheapest off-diagonal
@@ -960,7 +961,7 @@ static int plan_host_groups(taot_handle_t h, const int32_t* h_topk, int32_t* h_n
 // H2D copy of the routing table, the whole path on device staging buffers, D2H copy of the rewritten table (unless h_new is
 // null); `d` receives the device pointers.  Large tables go in layer groups on streams of their own, forked from and joined
 // back into the caller's: the copies of one group run under the kernels of another, and both copy engines at once (16
-// ranks, 24 layers, 12.6 MB each way: 716 -> 522 us; one after the other the copies alone take 460).
+// ranks, 24 layers, 12.6 MB each way: 716 -> 520 us; one after the other the copies alone take 460).
 static int plan_on_staging(taot_handle_t h, const int32_t* h_topk, int32_t* h_new, void* d_ws, void* stream, taot_outputs* d)
 {
     const taot_params& p = h->p;

@@ -14,7 +14,7 @@
 // Beyond 64 supply ranks (loads that are nearly even put half of the ranks above the mean) the warps that the columns leave idle
 // take further blocks of 64 rows, and the rows that are left sit in shared memory (wide_solve_tall): every problem whose supports
 // are disjoint fits one SM.  Bound there: the latency of four barriers and of one pass over shared memory per half-step, each
-// warp a chain of its own (7000 cycles an iteration at 256 x 256, 42 % of the issue slots, no bank conflicts).
+// warp a chain of its own (7000 cycles an iteration at 256 x 256, 42 % of the issue slots, hardly a bank conflict).
 //
 // Against 64-bit arithmetic (2-norm of the plan, 200 to 500 iterations, 70 to 288 supply ranks): 0.7 to 1.0e-7, the clusters 0.8
 // to 1.4e-7; with the column sums of the cap in fp32 it was up to 2.2e-7.
