@@ -1,14 +1,13 @@
 """The library's host code on a CPU: its object files linked with a stand-in for the CUDA runtime (fake_cuda.c) that writes down
 what is queued on which stream, runs nothing, and makes any chosen call fail."""
 import ctypes
-import glob
 import os
 import subprocess
 
 import torch
 
 from paper_2608_03676_b200.binding import TaotParams, _Outputs
-from paper_2608_03676_b200.build import OBJ, build
+from paper_2608_03676_b200.build import OBJ, SOURCES, build
 
 LAUNCH, RECORD, WAIT, COPY, SET, STREAM_CREATE, EVENT_CREATE, DEVICE_ALLOC = range(1, 9)
 CALLER = 0x77                                    # the stream that the caller passes
@@ -26,7 +25,7 @@ def load(folder):
     obj, lib = os.path.join(folder, "fake_cuda.o"), os.path.join(folder, "libtaot_fake.so")
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
     subprocess.run(["gcc", "-O1", "-fPIC", "-I", os.path.join(cuda, "include"), "-c", os.path.join(here, "fake_cuda.c"), "-o", obj], check=True)
-    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic", "-o", lib, obj] + sorted(glob.glob(os.path.join(OBJ, "*.o"))), check=True)
+    subprocess.run(["g++", "-shared", "-Wl,-Bsymbolic", "-o", lib, obj] + [os.path.join(OBJ, src.replace(".cu", ".o")) for src in SOURCES], check=True)
     so = ctypes.CDLL(lib)
     so.fake_entry.restype = ctypes.POINTER(Entry)
     so.fake_capturing.argtypes = [ctypes.c_int]
