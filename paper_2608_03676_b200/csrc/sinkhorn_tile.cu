@@ -3,7 +3,7 @@
 // that the build runs them in parallel.
 #include "sinkhorn_tile.cuh"
 
-int taot_launch_sinkhorn_tile_r32(const SinkArgs& a, int32_t B, int sm_count, cudaStream_t st);
+int taot_launch_sinkhorn_tile_r32(const SinkArgs& a, int32_t B, cudaStream_t st);
 int taot_launch_sinkhorn_tile_r32_batch(const SinkArgs& a, int32_t B, int sm_count, cudaStream_t st);
 int taot_launch_sinkhorn_tile_r64(const SinkArgs& a, int32_t B, int sm_count, cudaStream_t st);
 int taot_launch_sinkhorn_tile_r64_batch(const SinkArgs& a, int32_t B, int sm_count, cudaStream_t st);
@@ -18,7 +18,7 @@ int taot_launch_sinkhorn_tile(taot_handle_t h, const SinkArgs& a_in, int32_t B, 
     // a batch that fills the GPU several times over is bound by how many problems an SM holds, not by the latency of
     // one: it takes the register-capped builds
     const bool batch = B >= 4 * h->sm_count;
-    if (R <= 32) return batch ? taot_launch_sinkhorn_tile_r32_batch(a, B, h->sm_count, st) : taot_launch_sinkhorn_tile_r32(a, B, h->sm_count, st);
+    if (R <= 32) return batch ? taot_launch_sinkhorn_tile_r32_batch(a, B, h->sm_count, st) : taot_launch_sinkhorn_tile_r32(a, B, st);
     if (R <= 64) return batch ? taot_launch_sinkhorn_tile_r64_batch(a, B, h->sm_count, st) : taot_launch_sinkhorn_tile_r64(a, B, h->sm_count, st);
     int launched = 1;
     if (batch) {

@@ -2,7 +2,7 @@
 // REGISTERS.  Same arithmetic as the shared-memory kernel in sinkhorn.cu (absorbed potentials,
 // fp32 mat-vecs, fp64 folds), different data placement.  Two layouts:
 //
-// grid_solve (one warp per problem, up to 64 ranks): a 4 x 8 lane grid; lane (lr, lc) holds K~ for rows
+// grid_solve (one warp per problem, up to 64 ranks, batches that fill the GPU: sinkhorn_split.cuh has the few): a 4 x 8 lane grid; lane (lr, lc) holds K~ for rows
 //   ra*4 + lr and columns cg*8 + lc.  Row sums reduce over the 8 column lanes and column sums over the 4 row
 //   lanes by xor-butterflies, after which every lane of a group holds the same bits, so u~ and v~ are computed
 //   where they are needed and nothing is broadcast.  No barrier, no shared memory and (besides one rarely taken
