@@ -22,10 +22,11 @@
 // is the length of that dependent chain, so it has no branch but the loop's (a finished slot and an empty word leave it), and
 // the vote that ends the loop is taken while the next round's bids are on their way.
 //
-// Measured (B200): a round of one warp about 390 cycles, of several 650 and more (before, one thread per slot and two barriers:
-// 1000); matching stage at 64 ranks, 58 layers 174 -> 125 us, 256 ranks, 48 layers 1079 -> 980 us, 32 ranks 90 -> 75 us.  By
-// parts of the 390: the bid and its read-back 100, finding the won ranks 130 (reading them as one OR-ed word per 32 ranks
-// costs 160: reductions of different values into one word queue up), fetching what the rank holds 60, the updates 50.
+// Measured (B200), handles with at most four tiers and no equal scores (Lean, below; the others take Bidder): a round of one warp
+// about 310 cycles, of several 510 (Bidder 390 and 650 to 860; one thread per slot and two barriers before that: 1000).  A lone
+// warp takes three to five cycles per instruction, so what counts is their number; a reduction into shared memory takes two
+// cycles per lane that meets another in its bank, so arbiters and holdings are laid out against that.  Matching stage, 256 ranks,
+// 48 layers 967 -> 835 us, 32 ranks 67 -> 60 us, 64 ranks (where half the time is classes that move) 125 us as before.
 //
 // Equal scores.  Pairs whose fp32 scores are equal form a group and their candidates one set (the lowest rank wins, as in
 // a dense scan).  A group with two win counts of one tier (a price step below the scores' last bit) keeps a rank that was
@@ -54,7 +55,8 @@ __device__ __forceinline__ void bar_part(int nthreads) { asm volatile("bar.sync 
 
 // what the auction works on, in shared memory (nrem may be global)
 struct Tables {
-    uint32_t* arb;            // [2][R] best bid per rank, by parity of the round while there are several warps
+    uint32_t* arb;            // [2][R + W] best bid per rank, by parity of the round while there are several warps; a word's 32 begin a
+                              // bank further on than the word's before, since bids go to the lowest ranks of their words
     uint32_t* avail;          // [W][dmax] ranks still holding tokens of the expert in column col
     uint32_t* lvl;            // [W][S + 1] ranks by win count
     const uint32_t* list;     // [nbid] pairs, best score first: tier | win count << 8, bit 31: the next one scores the same
@@ -63,28 +65,28 @@ struct Tables {
     const uint32_t* tm;       // [ntiers][W][tms] tier masks, by class (by host, tms = R, if there is no room in shared memory)
     int32_t* tw_word;         // [ntiers][S] by class: the word that holds the whole tier, or -1
     uint32_t* tw_mask;        // [ntiers][S] that word's mask
+    const uint2* tw;          // [ntiers][S] (lean) both
     const int32_t* slot_e;    // [S]
-    int32_t* slot_a;          // [S] tokens a slot still collects
-    const uint16_t* nxt;      // [S] next slot of the class, 0xFFFF: none
+    int32_t* slot_a;          // [S + 1] tokens a slot still collects (S: 0)
+    const uint2* rec;         // [S + 1] (lean) next slot of the class and the tokens it collects
+    const uint16_t* nxt;      // [S + 1] next slot of the class, S: none (and S: S)
     const int32_t* dcol;      // [E] column of an expert
-    int32_t* nrem;            // [D][R] what each rank still holds of the expert in the column
+    int32_t* nrem;            // [D][RC] what each rank still holds of the expert in the column
     int32_t* X;               // [R][S] the plan of this layer (global)
     int32_t R, S, K, W, dmax, ntiers, tms;
-    uint32_t a_idle;          // shared address of this thread's word that nobody reads
-    int32_t* idle;            // the same in global memory
+    int32_t RC;               // odd in shared memory: bids for the same rank by different experts meet in no bank
+    int32_t* idle;            // a word in global memory that nobody reads
 };
 
-constexpr int kNoSlot = 0xFFFF;
 
-// A bidder: one class, its state in registers.  NT: tiers the build holds (the handle has at most as many); GROUPS: some pairs
-// have equal scores; NSM: nrem is in shared memory.
-// WM: most words of 32 ranks.
-template <int NT, bool GROUPS, bool NSM, int WM>
+// A bidder: one class, its state in registers, some pairs of which may have equal scores.  NT: tiers the build holds (the handle has
+// at most as many); WM: most words of 32 ranks.
+template <int NT, int WM>
 struct Bidder {
     const Tables& t;
     int c = 0;                // class
     int ci = 0;               // its column of tm
-    int s = kNoSlot;          // its lowest unfinished slot
+    int s;                    // its lowest unfinished slot (S: none)
     int col = 0;
     bool live = false;
     int32_t A = 0;            // tokens slot s still collects
@@ -100,7 +102,7 @@ struct Bidder {
     bool one = true;          // no other word to look at
     bool again = false;       // a group with two win counts of one tier: no word survives a round
 
-    __device__ __forceinline__ explicit Bidder(const Tables& tt) : t(tt), a_lv(smem_u32(tt.lvl))
+    __device__ __forceinline__ explicit Bidder(const Tables& tt) : t(tt), s(tt.S), a_lv(smem_u32(tt.lvl))
     {
 #pragma unroll
         for (int k = 0; k < NT; ++k) next[k] = 0xFFFFFFFFu;
@@ -137,7 +139,7 @@ struct Bidder {
             if (!one && pw + 1 < W) {
                 ++pw;
             } else {
-                if (et >= 0 && any == 0u && (!GROUPS || gend == 0)) set_next(et, 0xFFFFFFFFu);
+                if (et >= 0 && any == 0u && gend == 0) set_next(et, 0xFFFFFFFFu);
                 uint32_t best = next[0];
                 int bt = 0;
 #pragma unroll
@@ -152,8 +154,9 @@ struct Bidder {
                 one = wd >= 0;
                 pw = one ? wd : 0;
                 set_next(bt, after((uint32_t)bt, best & 0x7FFu));
-                if (GROUPS) { again = false; gend = 0; }
-                if (GROUPS && ((best >> 14) & 1u)) {     // equal scores: all pairs of the group at once, word by word
+                again = false;
+                gend = 0;
+                if ((best >> 14) & 1u) {     // equal scores: all pairs of the group at once, word by word
                     int g = (int)(best >> 16);
                     uint32_t seen = 1u << bt, pr;
                     do {
@@ -169,7 +172,7 @@ struct Bidder {
                 }
             }
             const uint32_t av = t.avail[pw * t.dmax + col];
-            if (!GROUPS || gend == 0) {
+            if (gend == 0) {
                 const uint32_t* lv = t.lvl + pw * LS + (ev & 0x7FFu);
                 const uint32_t* mp = one ? t.tw_mask + et * S + c : t.tm + (et * W + pw) * t.tms + ci;
                 const uint32_t h = *mp & av;
@@ -202,28 +205,23 @@ struct Bidder {
     }
 
     // ---- one round, in straight-line code for every lane: one without a bid sends a zero to some arbiter
-    uint32_t key = 0u, a_mine = 0u, a_cell = 0u, bitm = 0u;
+    uint32_t key = 0u, a_mine = 0u, bitm = 0u;
     int rank = 0;
     int32_t have = 0;
 
     // the bid: the lowest rank of the word.  rk = round << 13, a_arb: the round's arbiters
-    __device__ __forceinline__ void place(uint32_t rk, uint32_t a_arb, uint32_t a_col)
+    __device__ __forceinline__ void place(uint32_t rk, uint32_t a_arb)
     {
         const uint32_t c2 = A > 0 ? cw : 0u;            // (a finished slot waits for its class to move on)
         const int bit = c2 ? __ffs(c2) - 1 : 0;
-        if (GROUPS && c2 && gend) settle(bit);
-        const int word = GROUPS && pw < 0 ? 0 : pw;     // (a group that is walked anew stands before its first word)
+        if (c2 && gend) settle(bit);
+        const int word = pw < 0 ? 0 : pw;     // (a group that is walked anew stands before its first word)
         bitm = c2 & (0u - c2);
         rank = (word << 5) + bit;
         key = c2 ? rk | low : 0u;
-        a_mine = a_arb + ((uint32_t)rank << 2);
+        a_mine = a_arb + ((uint32_t)(rank + word) << 2);
         red_max_u32(a_mine, key);
-        if (NSM) {
-            a_cell = a_col + ((uint32_t)rank << 2);
-            have = (int32_t)lds_u32(a_cell);
-        } else {
-            have = c2 ? t.nrem[col * t.R + rank] : 0;
-        }
+        have = c2 ? t.nrem[col * t.RC + rank] : 0;
     }
 
     // Reads the round back.  The class that won its rank collects x = min(n, A); holdings, win count, price and plan follow.  The
@@ -237,7 +235,7 @@ struct Bidder {
         const uint32_t a_lane = a_arb + ((threadIdx.x & 31u) << 2);
 #pragma unroll
         for (int w = 0; w < WM; ++w) {
-            const uint32_t b = __ballot_sync(0xffffffffu, lds_u32(a_lane + 128u * w) >= rk);
+            const uint32_t b = __ballot_sync(0xffffffffu, lds_u32(a_lane + 132u * w) >= rk);
             gone = w == pw ? b : gone;
         }
         cw = again ? 0u : cw & ~gone;
@@ -249,8 +247,7 @@ struct Bidder {
         red_and_u32(a_lv, ~on);
         red_or_u32(a_lv + 4u, on);
         red_and_u32(smem_u32(t.avail + (rank >> 5) * t.dmax + col), ~off);
-        if (NSM) sts_u32(mine ? a_cell : t.a_idle, (uint32_t)rest);
-        else if (mine) t.nrem[col * t.R + rank] = rest;
+        if (mine) t.nrem[col * t.RC + rank] = rest;
         int32_t* const cell = mine ? t.X + (uint32_t)(rank * t.S + s) : t.idle;
         asm volatile("st.global.u32 [%0], %1;" ::"l"(cell), "r"(x) : "memory");
         A = mine ? A - x : A;
@@ -263,7 +260,7 @@ struct Bidder {
         if (live && A <= 0) {
             t.slot_a[s] = 0;
             s = t.nxt[s];
-            if (s == kNoSlot) {
+            if (s == t.S) {
                 live = false;
                 cw = 0u;
             } else {
@@ -272,7 +269,7 @@ struct Bidder {
             }
         }
         if (live && cw == 0u) {
-            if (GROUPS && again) pw = -1;
+            if (again) pw = -1;
             walk();
             live = cw != 0u;
         }
@@ -286,25 +283,24 @@ __device__ __forceinline__ uint32_t run_warp(B& b, uint32_t rd, uint32_t round_l
 {
     const Tables& t = b.t;
     const uint32_t a_arb = smem_u32(t.arb);
-    const uint32_t a_col = smem_u32(t.nrem + b.col * t.R);       // (used if nrem is in shared memory)
     while (rd <= round_limit) {
         __syncwarp();
         b.move_on();
         __syncwarp();
         if (!__any_sync(0xffffffffu, b.live)) break;
-        b.place(rd << 13, a_arb, a_col);          // (again, for most: that changes nothing)
+        b.place(rd << 13, a_arb);          // (again, for most: that changes nothing)
         bool stop;
         do {
             __syncwarp();
             b.collect(rd << 13, a_arb);
             ++rd;
             stop = b.must_move() || rd > round_limit;
-            b.place(rd << 13, a_arb, a_col);
+            b.place(rd << 13, a_arb);
             stop = __any_sync(0xffffffffu, stop);
         } while (!stop);
         last = rd - 1u;
     }
-    if (b.s != kNoSlot) t.slot_a[b.s] = b.A;      // what is left uncollected
+    if (b.s != t.S) t.slot_a[b.s] = b.A;      // what is left uncollected
     return last;
 }
 
@@ -324,13 +320,13 @@ __device__ __forceinline__ uint32_t run_block(B& b, const int NP, const int clas
 {
     const Tables& t = b.t;
     const int tid = threadIdx.x;
-    const uint32_t a_arb = smem_u32(t.arb), a_col = smem_u32(t.nrem + b.col * t.R);
+    const uint32_t a_arb = smem_u32(t.arb);
     const uint32_t a_ctl = smem_u32(ctl);
-    uint32_t rd = 1u, pass = 1u, apar = 4u * (uint32_t)t.R;      // round 1 takes the second set of arbiters
+    uint32_t rd = 1u, pass = 1u, apar = 4u * (uint32_t)(t.R + t.W);      // round 1 takes the second set of arbiters
     uint32_t dead0 = 0u, dead1 = 0u;
     bool died = false;
     while (rd <= round_limit) {
-        b.place(rd << 13, a_arb + apar, a_col);
+        b.place(rd << 13, a_arb + apar);
         const uint32_t a_ev = a_ctl + ((pass & 1u) << 2);
         if (b.must_move() || died) {
             if (died) red_add_u32(a_ctl + 8u + ((pass & 1u) << 2), 1u);
@@ -351,11 +347,264 @@ __device__ __forceinline__ uint32_t run_block(B& b, const int NP, const int clas
         }
         ++pass;
         if (b.collect(rd << 13, a_arb + apar)) sts_u32(a_ctl + 16u, rd);
-        apar ^= 4u * (uint32_t)t.R;
+        apar ^= 4u * (uint32_t)(t.R + t.W);
         ++rd;
     }
-    if (b.s != kNoSlot) t.slot_a[b.s] = b.A;
+    if (b.s != t.S) t.slot_a[b.s] = b.A;
     if (b.live && rd <= round_limit) ctl->hand[atomicAdd(&ctl->handed, 1u)] = ((uint32_t)b.c << 16) | (uint32_t)b.s;
+    return rd;
+}
+
+// ---- Handles with at most four tiers and no equal scores.
+//
+// The same rounds with fewer instructions: win counts and availability, which nobody reads but a class that walks, follow in one go
+// before the next walk; a finished slot makes way for the next of its class in place; the rounds are left only where a class's word
+// is empty or its last slot finished.  (Several classes per lane instead of several warps: 200 cycles a round for each, 1000 at
+// four; the loads of the next round ahead of the vote that ends the rounds: 60 cycles a round slower.)
+// NT: 2 or 4 tiers (walking goes through all of them: 32 ranks 67 -> 60 us with two); NSM: nrem is in shared memory; WM: most words
+// of 32 ranks.
+__device__ __forceinline__ void red_max_if(bool on, uint32_t addr, uint32_t v)
+{
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p red.shared.max.u32 [%0], %1; }" ::"r"(addr), "r"(v), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void sts_if(bool on, uint32_t addr, uint32_t v)
+{
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u32 [%0], %1; }" ::"r"(addr), "r"(v), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ void stg_if(bool on, int32_t* addr, int32_t v)
+{
+    asm volatile("{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.global.u32 [%0], %1; }" ::"l"(addr), "r"(v), "r"((uint32_t)on) : "memory");
+}
+__device__ __forceinline__ uint2 lds_u64(uint32_t addr)
+{
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
+    return v;
+}
+
+template <int NT, bool NSM, int WM>
+struct Lean {
+    const Tables& t;
+    const uint32_t a_arb, a_rec, a_slot, a_lvl, a_avail, a_ent, a_tw, S, LS, dmax;      // shared addresses of the tables
+    // what a round needs
+    bool act = false;         // the thread has a class that is not through
+    uint32_t cw = 0u;         // its candidates: ranks of word pw; 0 where there is no class
+    uint32_t A = 0u;          // tokens the slot in front still collects
+    uint32_t s = 0u, low = 0u;
+    uint32_t a_word;          // shared address of the word's arbiters
+    uint32_t cell = 0u;       // nrem: index (NSM: shared address) of the column's first rank of the word
+    uint32_t x0 = 0u;         // X: index of the word's first rank and the slot
+    uint32_t on = 0u, off = 0u;       // ranks of the word won by the class since the sets were last brought up to date; those now empty
+    // what a walk needs
+    uint32_t next[NT], ev = 0u;
+    uint32_t a_tw_c = 0u, a_av_c = 0u, cell_c = 0u;   // the class's and its column's places in the tables
+    uint32_t a_lv = 0u, a_av = 0u;                     // of the pair and word it rests on
+    int et = -1, pw = 0, c = 0;
+    bool one = true;
+
+    __device__ __forceinline__ explicit Lean(const Tables& tt)
+        : t(tt), a_arb(smem_u32(tt.arb)), a_rec(smem_u32(tt.rec)), a_slot(smem_u32(tt.slot_a)), a_lvl(smem_u32(tt.lvl)),
+          a_avail(smem_u32(tt.avail)), a_ent(smem_u32(tt.ent)), a_tw(smem_u32(tt.tw)), S((uint32_t)tt.S),
+          LS(4u * (uint32_t)tt.S + 4u), dmax(4u * (uint32_t)tt.dmax), a_word(a_arb)
+    {
+#pragma unroll
+        for (int k = 0; k < NT; ++k) next[k] = 0xFFFFFFFFu;
+        if (NSM) cell = smem_u32(tt.nrem);
+    }
+    __device__ __forceinline__ void start(int cc, int ss)
+    {
+        c = cc;
+        s = (uint32_t)ss;
+        low = 1023u - s;
+        const uint32_t col = (uint32_t)t.dcol[t.slot_e[ss]];
+        a_tw_c = a_tw + 8u * (uint32_t)cc;
+        a_av_c = a_avail + 4u * col;
+        cell_c = NSM ? smem_u32(t.nrem) + 4u * col * (uint32_t)t.RC : col * (uint32_t)t.RC;
+        A = lds_u32(a_slot + 4u * s);
+        act = A != 0u;
+#pragma unroll
+        for (int k = 0; k < NT; ++k) next[k] = k < t.ntiers ? lds_u32(a_ent + (uint32_t)k * LS) : 0xFFFFFFFFu;
+    }
+    // win counts and availability
+    __device__ __forceinline__ void settle()
+    {
+        if (on) {
+            red_and_u32(a_lv, ~on);
+            red_or_u32(a_lv + 4u, on);
+            if (off) red_and_u32(a_av, ~off);
+            on = off = 0u;
+        }
+    }
+    // to the next word with candidates; cw == 0: there is none, ever
+    __device__ __forceinline__ void walk()
+    {
+        int first = pw + 1;                           // first word to look at
+        uint32_t held = 1u, m = 0u;                   // held: members of the tier that hold tokens; only 0 matters
+#pragma unroll 1
+        for (;;) {
+            const uint32_t a_wins = a_lvl + 4u * (ev & 0x7FFu);
+            if (WM > 1 && et >= 0 && !one) {          // the tier's words from `first` on
+                const int ci = t.tms == t.S ? c : (int)(1023u - (low & 1023u)) / t.K;
+                const uint32_t* tm = t.tm + et * t.W * t.tms + ci;
+#pragma unroll
+                for (int w = WM - 1; w >= 0; --w) {
+                    if (w < t.W) {
+                        const uint32_t h = tm[w * t.tms] & lds_u32(a_av_c + (uint32_t)w * dmax);
+                        const uint32_t x = h & lds_u32(a_wins + (uint32_t)w * LS);
+                        held |= h;
+                        if (w >= first && x) { cw = x; pw = w; }
+                    }
+                }
+            } else if (first == 0) {
+                held = m & lds_u32(a_av_c + (uint32_t)pw * dmax);
+                cw = held & lds_u32(a_wins + (uint32_t)pw * LS);
+            }
+            if (cw) break;
+#pragma unroll
+            for (int k = 0; k < NT; ++k) next[k] = k == et && held == 0u ? 0xFFFFFFFFu : next[k];
+            uint32_t best = next[0];
+            et = 0;
+#pragma unroll
+            for (int k = 1; k < NT; ++k) {
+                et = next[k] < best ? k : et;
+                best = next[k] < best ? next[k] : best;
+            }
+            if (best == 0xFFFFFFFFu) return;
+            ev = best;
+            const uint32_t w = best & 0x7FFu;
+            const uint2 tw = lds_u64(a_tw_c + 8u * S * (uint32_t)et);
+            const uint32_t after = w < S ? lds_u32(a_ent + (uint32_t)et * LS + 4u * w + 4u) : 0xFFFFFFFFu;
+#pragma unroll
+            for (int k = 0; k < NT; ++k) next[k] = k == et ? after : next[k];
+            one = WM == 1 || (int)tw.x >= 0;
+            pw = WM > 1 && one ? (int)tw.x : 0;
+            m = tw.y;
+            first = 0;
+            held = 0u;
+        }
+        low = ((7u - ((ev >> 11) & 7u)) << 10) | (low & 1023u);
+        a_lv = a_lvl + 4u * (ev & 0x7FFu) + (uint32_t)pw * LS;
+        a_av = a_av_c + (uint32_t)pw * dmax;
+        a_word = a_arb + 132u * (uint32_t)pw;
+        cell = cell_c + (NSM ? 128u : 32u) * (uint32_t)pw;
+        x0 = 32u * (uint32_t)pw * S + s;
+    }
+    // a class without candidates, after settle() of all: on to its next word, or through
+    __device__ __forceinline__ void move_on()
+    {
+        if (A != 0u) walk();
+        act = cw != 0u;
+        if (!act && A != 0u) {
+            sts_u32(a_slot + 4u * s, A);              // (what is left uncollected)
+            A = 0u;
+        }
+    }
+
+    uint32_t bitm = 0u, bit = 0u, key = 0u, have = 0u, a_mine = 0u;
+
+    // the bid: the lowest rank of the word.  rk = round << 13, par: offset of the round's arbiters
+    __device__ __forceinline__ void place(uint32_t rk, uint32_t par)
+    {
+        bitm = cw & (0u - cw);
+        asm("bfind.u32 %0, %1;" : "=r"(bit) : "r"(bitm));           // (no candidates: -1, the word before, which is not used)
+        key = rk | low;
+        a_mine = a_word + par + 4u * bit;
+        red_max_if(cw != 0u, a_mine, key);
+        if (NSM) have = lds_u32(cell + 4u * bit);
+        else have = cw ? (uint32_t)t.nrem[cell + bit] : 0u;
+    }
+    // Reads the round back.  The class that won its rank collects x = min(n, A) > 0 (the rank holds tokens of the expert, its
+    // availability bit was set, and the slot still wants some).
+    __device__ __forceinline__ void collect(uint32_t rk, uint32_t par)
+    {
+        const uint32_t won = lds_u32(a_mine);
+        const uint2 then = lds_u64(a_rec + 8u * s);
+        const uint32_t a_lane = a_arb + par + ((threadIdx.x & 31u) << 2);
+        uint32_t g[WM];
+        // (beyond the last rank the loads run into other shared data: bits no candidate word has)
+#pragma unroll
+        for (int w = 0; w < WM; ++w) g[w] = lds_u32(a_lane + 132u * w);
+#pragma unroll
+        for (int w = 0; w < WM; ++w) g[w] = __ballot_sync(0xffffffffu, g[w] >= rk);
+#pragma unroll
+        for (int h = 1; h < WM; h <<= 1)
+#pragma unroll
+            for (int w = 0; w < WM; w += 2 * h) g[w] = pw & h ? g[w + h] : g[w];
+        const bool mine = (won == key) & (cw != 0u);
+        const uint32_t x = have < A ? have : A, rest = have - x;
+        on |= mine ? bitm : 0u;
+        off |= mine & (rest == 0u) ? bitm : 0u;
+        if (NSM) sts_if(mine, cell + 4u * bit, rest);
+        else stg_if(mine, t.nrem + (cell + bit), (int32_t)rest);
+        stg_if(mine, t.X + (x0 + bit * S), (int32_t)x);
+        A -= mine ? x : 0u;
+        const bool done = mine & (A == 0u);           // the next of the class (S, with nothing to collect, behind the last)
+        sts_if(done, a_slot + 4u * s, 0u);
+        const uint32_t step = done ? then.x - s : 0u;
+        s += step; low -= step; x0 += step;
+        A = done ? then.y : A;
+        cw = A != 0u ? cw & ~g[0] : 0u;
+    }
+};
+
+template <class B>
+__device__ __forceinline__ uint32_t run_warp_lean(B& b, uint32_t rd, uint32_t round_limit, uint32_t last)
+{
+    while (rd <= round_limit) {
+        __syncwarp();
+        b.settle();
+        __syncwarp();
+        if (b.act && b.cw == 0u) b.move_on();
+        __syncwarp();
+        if (!__any_sync(0xffffffffu, b.act)) break;
+        b.place(rd << 13, 0u);                        // (again, for most: that changes nothing)
+        do {
+            __syncwarp();
+            b.collect(rd << 13, 0u);
+            ++rd;
+            b.place(rd << 13, 0u);
+        } while (!__any_sync(0xffffffffu, (b.act & (b.cw == 0u)) | (rd > round_limit)));
+        last = rd - 1u;
+    }
+    if (b.act && b.A != 0u) b.t.slot_a[b.s] = (int32_t)b.A;
+    return last;
+}
+
+// More than 32 classes, a barrier a pass.  A pass in which some class has none but its next word or its end before it does only that
+// (and has one more).
+template <class B>
+__device__ __forceinline__ uint32_t run_block_lean(B& b, const int NP, const int classes, const uint32_t round_limit, Control* ctl)
+{
+    const uint32_t a_ctl = smem_u32(ctl), flip = 4u * (uint32_t)(b.t.R + b.t.W);
+    uint32_t rd = 1u, pass = 1u, par = flip;          // round 1 takes the second set of arbiters
+    bool moved = false;
+    while (rd <= round_limit) {
+        b.place(rd << 13, par);
+        const uint32_t a_ev = a_ctl + ((pass & 1u) << 2);
+        if (b.act && b.cw == 0u) sts_u32(a_ev, pass);
+        __syncwarp();
+        bar_part(NP);
+        if (moved && classes - (int)lds_u32(a_ctl + 8u) <= 32) break;         // (the same answer in every thread)
+        moved = lds_u32(a_ev) == pass;
+        ++pass;
+        if (moved) {
+            b.settle();
+            bar_part(NP);
+            if (b.act && b.cw == 0u) {
+                b.move_on();
+                if (!b.act) red_add_u32(a_ctl + 8u, 1u);
+            }
+            continue;
+        }
+        b.collect(rd << 13, par);
+        if (threadIdx.x == 0) sts_u32(a_ctl + 16u, rd);
+        par ^= flip;
+        ++rd;
+    }
+    if (b.act) {
+        b.t.slot_a[b.s] = (int32_t)b.A;
+        if (rd <= round_limit) ctl->hand[atomicAdd(&ctl->handed, 1u)] = ((uint32_t)b.c << 16) | b.s;
+    }
     return rd;
 }
 

@@ -83,6 +83,8 @@ __device__ __forceinline__ u64 warp_max_u64(u64 k)
     return k;
 }
 
+template <class T> struct Type { using type = T; };
+
 constexpr int kMaxW = 8;          // words of a rank bit set: R <= 256
 constexpr size_t kSmemBudget = 224 * 1024;   // dynamic shared memory the kernel plans with (227 KB per CTA less the static part)
 
@@ -121,7 +123,9 @@ match_kernel(MatchArgs a)
     // ---- carve shared memory
     u64* arb_e = reinterpret_cast<u64*>(smem_raw);            // [E]  Phase 2 arbitration per expert
     u64* arb_r = arb_e + E;                                    // [2][R]  Phase 3 arbitration per rank, ping-pong by round
-    int32_t* spill = reinterpret_cast<int32_t*>(arb_r + 2 * R); // [E]
+    uint2* rec_s = reinterpret_cast<uint2*>(arb_r + 2 * R);     // LEAN: [S+1] next slot of the class and its tokens
+    uint2* tw2 = rec_s + (LEAN && a.nbid ? S + 1 : 0);          // LEAN: [ntiers][S] word and mask of a tier that one word holds, by class
+    int32_t* spill = reinterpret_cast<int32_t*>(tw2 + (LEAN && a.nbid ? a.ntiers * S : 0)); // [E]
     int32_t* hot0 = spill + E;                                 // [E]  experts that spill at the start of Phase 2
     int32_t* hot_home = hot0 + E;                              // [E]  their home ranks
     int32_t* dcol = hot_home + E;                              // [E]  expert -> column of nrem, or -1
@@ -132,24 +136,23 @@ match_kernel(MatchArgs a)
     int32_t* wins = estar + R;                                 // [R]
     int32_t* slot_e = wins + R;                                // [S]
     int32_t* slot_a0 = slot_e + S;                             // [S]  planned tokens (Phase 2 result)
-    int32_t* slot_a = slot_a0 + S;                             // [S]  still to collect (Phase 3)
-    uint32_t* avail = reinterpret_cast<uint32_t*>(slot_a + S); // [W][dmax]  ranks still holding tokens of the expert (word-major: no bank conflicts across slots)
+    int32_t* slot_a = slot_a0 + S;                             // [S+1] still to collect (Phase 3)
+    uint32_t* avail = reinterpret_cast<uint32_t*>(slot_a + S + 1); // [W][dmax]  ranks still holding tokens of the expert (word-major: no bank conflicts across slots)
     uint32_t* lvl = avail + a.dmax * W;                        // [W][S+1]   ranks by win count (word-major)
     uint32_t* tm_s = lvl + (S + 1) * W;                                // [ntiers][W][S] tier masks by slot, if they fit
     uint32_t* bid_s = tm_s + (a.tm_in_smem ? a.ntiers * W * S : 0);    // [nbid] (tier, win count) pairs, best score first
     int32_t* tw_word = reinterpret_cast<int32_t*>(bid_s + a.nbid);     // [ntiers][S] word holding the whole tier for the class, or -1
-    uint32_t* tw_mask = reinterpret_cast<uint32_t*>(tw_word + (a.nbid ? a.ntiers * S : 0));   // [ntiers][S] that word's mask
-    uint32_t* ent_s = tw_mask + (a.nbid ? a.ntiers * S : 0);           // [nbid] the pairs by tier and win count
+    uint32_t* tw_mask = reinterpret_cast<uint32_t*>(tw_word + (!LEAN && a.nbid ? a.ntiers * S : 0));   // [ntiers][S] that word's mask (LEAN: both in tw2)
+    uint32_t* ent_s = tw_mask + (!LEAN && a.nbid ? a.ntiers * S : 0);           // [nbid] the pairs by tier and win count
     int32_t* key_s = reinterpret_cast<int32_t*>(ent_s + a.nbid);       // [S] class keys, then the classes' lists
     uint16_t* nxt_s = reinterpret_cast<uint16_t*>(key_s + (a.nbid ? S : 0));            // [S] next slot of the class
-    uint16_t* lead_s = nxt_s + (a.nbid ? S : 0);                       // [S] first slot of each class
+    uint16_t* lead_s = nxt_s + (a.nbid ? S + 2 : 0);                   // [S] first slot of each class
     const int RS = R | 1;
     float* bon_s = reinterpret_cast<float*>(lead_s + (a.nbid ? S : 0));                // dense scan, if it fits: [R][RS] bonus of rank r for host h at h * RS + r
     int32_t* nrem_s = reinterpret_cast<int32_t*>(bon_s + (a.bon_in_smem ? R * RS : 0)); // [dmax*R] if it fits
     __shared__ long long s_tot;
     __shared__ int s_cnt, s_any, s_ns;
     __shared__ taot_auction::Control ctl;
-    __shared__ uint32_t idle_s[32];
     __shared__ int s_wcnt[32];
 
     const int32_t* n = a.n + l * (int64_t)R * E;
@@ -157,6 +160,7 @@ match_kernel(MatchArgs a)
     const int32_t* rl = a.rank_load + l * R;
     const float* plan = a.plan + l * (int64_t)R * R;
     int32_t* nrem = a.nrem_in_smem ? nrem_s : a.nrem_g + l * (int64_t)a.dmax * R;
+    const int RC = a.nrem_in_smem ? RS : R;       // stride of its columns
     float* t12 = a.t12 + l * (int64_t)E * 2 * R;      // global scratch; replaced by shared memory below if the rows fit
 
     // Everything up to the flow hint itself follows from the loads, which are there before Phase 1 starts: in a plan (a.early)
@@ -587,7 +591,7 @@ match_kernel(MatchArgs a)
     for (int q = warp; q < D * W; q += NW) {
         const int col = q / W, w = q - col * W, r = 32 * w + lane;
         const int32_t v = r < R ? n[r * E + hot0[col]] : 0;
-        if (r < R) nrem[col * R + r] = v;
+        if (r < R) nrem[col * RC + r] = v;
         const unsigned word = __ballot_sync(0xffffffffu, v > 0);
         if (lane == 0) avail[w * a.dmax + col] = word;
     }
@@ -599,16 +603,16 @@ match_kernel(MatchArgs a)
     if (tiered && D > 0) {
         // ---- bit-set auction (auction.cuh): bidders are classes of slots that make the same bids
         namespace au = taot_auction;
-        uint32_t* const arb = reinterpret_cast<uint32_t*>(arb_r);       // [2][R]
-        for (int q = tid; q < 2 * R; q += NT) arb[q] = 0u;
+        uint32_t* const arb = reinterpret_cast<uint32_t*>(arb_r);       // [2][R + W]
+        for (int q = tid; q < 2 * (R + W); q += NT) arb[q] = 0u;
         // a live slot's class: expert and the way its host sees the ranks; the lowest slot leads, the others queue behind it
         const int s = tid;
         const bool slive = s < S && slot_e[s] >= 0 && slot_a[s] > 0;
         if (s < S) {
             key_s[s] = slive ? slot_e[s] * R + a.hostcls[s / K] : -1 - s;
-            nxt_s[s] = (uint16_t)au::kNoSlot;
+            nxt_s[s] = (uint16_t)S;
         }
-        if (tid == 0) { ctl.event[0] = ctl.event[1] = ctl.dead[0] = ctl.dead[1] = ctl.last = ctl.handed = 0u; }
+        if (tid == 0) { nxt_s[S] = (uint16_t)S; slot_a[S] = 0; ctl.event[0] = ctl.event[1] = ctl.dead[0] = ctl.dead[1] = ctl.last = ctl.handed = 0u; }
         __syncthreads();
         bool lead = slive;
         if (slive) {
@@ -627,6 +631,8 @@ match_kernel(MatchArgs a)
             for (int w = 0; w < NW; ++w) { const int cnt = s_wcnt[w]; if (w < warp) off += cnt; C += cnt; }
             if (lead) lead_s[off + __popc(lb & ((1u << lane) - 1u))] = (uint16_t)s;
         }
+        if constexpr (LEAN)
+            for (int q = tid; q <= S; q += NT) rec_s[q] = make_uint2(nxt_s[q], (uint32_t)slot_a[nxt_s[q]]);
         __syncthreads();
         // tier masks by class, and for each tier the word that holds all of it
         if (a.tm_in_smem) {
@@ -646,27 +652,31 @@ match_kernel(MatchArgs a)
                 const uint32_t mk = tm[(t * W + w) * tms + (a.tm_in_smem ? c : lead_s[c] / K)];
                 if (mk) { ++nz; wd = w; val = mk; }
             }
-            tw_word[t * S + c] = nz <= 1 ? wd : -1;
-            tw_mask[t * S + c] = val;
+            if constexpr (LEAN) {
+                tw2[t * S + c] = make_uint2(nz <= 1 ? (uint32_t)wd : 0xFFFFFFFFu, val);
+            } else {
+                tw_word[t * S + c] = nz <= 1 ? wd : -1;
+                tw_mask[t * S + c] = val;
+            }
         }
         __syncthreads();
         long long limit = cap;
         if (a.auction_max_rounds > 0 && a.auction_max_rounds < limit) limit = a.auction_max_rounds;
         const uint32_t round_limit = (uint32_t)limit;                   // at most R * S + S < 2^19
         if (timed) c_p3loop = clock64();
-        const au::Tables tab{arb, avail, lvl, bid_s, ent_s, tm, tw_word, tw_mask, slot_e, slot_a, nxt_s, dcol, nrem, Xl,
-                             R, S, K, W, a.dmax, a.ntiers, tms, au::smem_u32(idle_s + lane),
+        const au::Tables tab{arb, avail, lvl, bid_s, ent_s, tm, tw_word, tw_mask, tw2, slot_e, slot_a, rec_s, nxt_s, dcol, nrem, Xl,
+                             R, S, K, W, a.dmax, a.ntiers, tms, RC,
                              reinterpret_cast<int32_t*>(a.t12 + l * (int64_t)E * 2 * R)};       // (Phase 2's scratch)
         const int NP = ((C + 31) >> 5) << 5;
-        auto run = [&](auto bidder) {
-            using B = decltype(bidder);
+        auto run = [&](auto type, auto rounds_block, auto rounds_warp) {
+            using B = typename decltype(type)::type;
             uint32_t rd = 1u;
             if (C > 32) {
                 if (tid < NP) {
                     B b(tab);
                     if (tid < C) b.start(tid, lead_s[tid]);
                     __syncwarp();
-                    rd = au::run_block(b, NP, C, round_limit, &ctl);
+                    rd = rounds_block(b);
                 }
                 __syncthreads();
             }
@@ -679,14 +689,29 @@ match_kernel(MatchArgs a)
                     b.start(lane, lead_s[lane]);
                 }
                 __syncwarp();
-                const uint32_t last = au::run_warp(b, rd, round_limit, ctl.last);
+                const uint32_t last = rounds_warp(b, rd);
                 __syncwarp();
                 if (lane == 0) ctl.last = last;
             }
         };
-        if constexpr (!LEAN) run(au::Bidder<TAOT_MAX_TIERS, true, false, kMaxW>(tab));
-        else if (W <= 2) run(au::Bidder<4, false, NSM, 2>(tab));
-        else run(au::Bidder<4, false, NSM, kMaxW>(tab));
+        if constexpr (!LEAN) {
+            run(Type<au::Bidder<TAOT_MAX_TIERS, kMaxW>>{},
+                [&](auto& b) { return au::run_block(b, NP, C, round_limit, &ctl); },
+                [&](auto& b, uint32_t rd) { return au::run_warp(b, rd, round_limit, ctl.last); });
+        } else {
+            const auto lean = [&](auto tiers, auto words) {
+                run(Type<au::Lean<decltype(tiers)::value, NSM, decltype(words)::value>>{},
+                    [&](auto& b) { return au::run_block_lean(b, NP, C, round_limit, &ctl); },
+                    [&](auto& b, uint32_t rd) { return au::run_warp_lean(b, rd, round_limit, ctl.last); });
+            };
+            const auto lean_w = [&](auto tiers) {
+                if (W == 1) lean(tiers, std::integral_constant<int, 1>{});
+                else if (W == 2) lean(tiers, std::integral_constant<int, 2>{});
+                else lean(tiers, std::integral_constant<int, kMaxW>{});
+            };
+            if (a.ntiers <= 2) lean_w(std::integral_constant<int, 2>{});
+            else lean_w(std::integral_constant<int, 4>{});
+        }
         if (timed) c_p3end = clock64();
         __syncthreads();
         rounds3 = (int)ctl.last;                  // rounds in which somebody bid
@@ -713,7 +738,7 @@ match_kernel(MatchArgs a)
             own[p] = q < S && slot_e[q < S ? q : 0] >= 0;
             slot[p] = own[p] ? q : 0;
             host[p] = slot[p] / K;
-            coff[p] = own[p] ? dcol[slot_e[q]] * R : 0;
+            coff[p] = own[p] ? dcol[slot_e[q]] * RC : 0;
             boff[p] = host[p] * RS;
             r0[p] = (sub + slot[p]) % R;
         }
@@ -824,7 +849,7 @@ match_kernel(MatchArgs a)
 size_t match_smem_fixed(int R, int E, int K, int dmax, int W, int ntiers)
 {
     const size_t S = (size_t)R * K;
-    return sizeof(u64) * (E + 2 * (size_t)R) + sizeof(int32_t) * (4 * (size_t)E + 5 * (size_t)R + 3 * S) +
+    return sizeof(u64) * (E + 2 * (size_t)R) + sizeof(int32_t) * (4 * (size_t)E + 5 * (size_t)R + 3 * S + 1) +
            sizeof(uint32_t) * ((size_t)dmax * W + (S + 1) * W);
 }
 
@@ -853,10 +878,12 @@ int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expe
     a.eps0 = p.eps0; a.price_step = p.price_step; a.auction_max_rounds = p.auction_max_rounds;
     a.ablation = p.ablation;
     size_t smem = match_smem_fixed(p.R, p.E, p.K, a.dmax, a.W, a.ntiers);
-    const size_t lists = sizeof(uint32_t) * (2 * (size_t)h->nbid + 2 * (size_t)h->ntiers * p.R * p.K + 2 * (size_t)p.R * p.K);
+    const bool few_tiers = h->ntiers <= 4 && !h->bid_ties;
+    const size_t lists = sizeof(uint32_t) * (2 * (size_t)h->nbid + 2 * (size_t)h->ntiers * p.R * p.K + 2 * (size_t)p.R * p.K + 1 +
+                                             2 * ((size_t)p.R * p.K + 1));
     if (a.nbid > 0 && smem + lists > kSmemBudget) { a.nbid = 0; a.ntiers = 0; }      // (no room for the lists: the dense scan)
     if (a.nbid > 0) smem += lists;
-    const size_t nrem_bytes = sizeof(int32_t) * (size_t)a.dmax * p.R;
+    const size_t nrem_bytes = sizeof(int32_t) * (size_t)a.dmax * (p.R | 1);
     // the bonus matrix of the dense scan, where it fits beside the remaining counts
     const size_t bon_bytes = sizeof(float) * (size_t)p.R * (p.R | 1);
     a.bon_in_smem = (a.nbid == 0 && smem + bon_bytes + nrem_bytes <= kSmemBudget) ? 1 : 0;
@@ -886,7 +913,7 @@ int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expe
         TAOT_CUDA_OK(taot_launch_chained(kernel, p.L, NT, smem, st, a));
         return 1;
     };
-    const bool lean = a.nbid > 0 && a.ntiers <= 4 && !h->bid_ties, nsm = a.nrem_in_smem != 0;
+    const bool lean = a.nbid > 0 && few_tiers, nsm = a.nrem_in_smem != 0;
     auto build = [&](auto timed, auto maxt) -> int {
         constexpr bool TIMED = decltype(timed)::value;
         constexpr int MAXT = decltype(maxt)::value;
