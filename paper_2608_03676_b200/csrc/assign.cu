@@ -34,10 +34,14 @@
 
 namespace {
 
-constexpr int kThreads = TAOT_STREAM_THREADS;
-constexpr int kWarps = kThreads / 32;
-constexpr int kWarpSpan = TAOT_CHUNK / kWarps;           // entries one warp owns, contiguous: 2048
-constexpr int kIters = kWarpSpan / 128;                  // 16-byte accesses per lane: 16
+// NT threads share a chunk.  A table that fills the GPU takes 256, five CTAs per SM side by side; where all chunks are placed at
+// once anyway the stage lasts as long as its slowest chunk (the one of a hot rank), and 512 threads walk it in half the steps.
+template <int NT>
+struct Cta {
+    static constexpr int kThreads = NT, kWarps = NT / 32;
+    static constexpr int kWarpSpan = TAOT_CHUNK / kWarps;        // entries one warp owns, contiguous
+    static constexpr int kIters = kWarpSpan / 128;               // 16-byte accesses per lane
+};
 constexpr int kFewSplits = 4;                            // splits of a chunk that are applied as predicated overrides from registers
                                                          // (only up to 2: 16 ranks 158 -> 165 us a plan, 24 ranks 141 -> 149; up to 6: 32 ranks 114 -> 117)
 
@@ -115,9 +119,10 @@ __device__ __forceinline__ int4 unpack_bytes(const void* buf, int32_t pos)
     return make_int4((int)(w & 255u), (int)((w >> 8) & 255u), (int)((w >> 16) & 255u), (int)(w >> 24));
 }
 
-template <bool VEC, bool BYTES>
+template <bool VEC, bool BYTES, int NT>
 __device__ int32_t locate_split(const void* bufv, int32_t len, int eb, int rel, int* s_cntw, int* s_pos)
 {
+    constexpr int kWarpSpan = Cta<NT>::kWarpSpan, kIters = Cta<NT>::kIters;
     const int32_t* buf = static_cast<const int32_t*>(bufv);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int32_t wbase = warp * kWarpSpan + lane * 4;
@@ -181,12 +186,13 @@ __device__ int32_t locate_split(const void* bufv, int32_t len, int eb, int rel, 
 }
 
 // Rewrite one chunk: `buf` holds its entries (shared memory if staged, else global memory), `tab` its table and
-// `recs` its `ns` split records {expert, in-chunk ordinal of the split, target before, -} in shared memory; `scratch`: 4 words
-// per record.  Block-wide.
-template <bool VEC, bool BYTES>
+// `recs` its `ns` split records {expert, in-chunk ordinal of the split, target before, -} in shared memory; `scratch`: a word
+// per record and two warps.  Block-wide.
+template <bool VEC, bool BYTES, int NT>
 __device__ void rewrite_chunk(const AssignArgs& a, const void* bufv, int32_t* tab, int32_t* dst,
                               int32_t len, const int ns, int4* recs, int32_t* scratch, int* s_cntw, int* s_pos)
 {
+    constexpr int kThreads = NT, kWarps = Cta<NT>::kWarps, kWarpSpan = Cta<NT>::kWarpSpan, kIters = Cta<NT>::kIters;
     const int32_t* buf = static_cast<const int32_t*>(bufv);
     const int E = a.E;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -238,7 +244,7 @@ __device__ void rewrite_chunk(const AssignArgs& a, const void* bufv, int32_t* ta
                 const int4 rec = recs[k];
                 re[k] = rec.x;
                 rt[k] = rec.z;
-                rp[k] = locate_split<VEC, BYTES>(bufv, len, rec.x, rec.y, s_cntw, s_pos);
+                rp[k] = locate_split<VEC, BYTES, NT>(bufv, len, rec.x, rec.y, s_cntw, s_pos);
             }
         }
 #pragma unroll
@@ -287,7 +293,7 @@ __device__ void rewrite_chunk(const AssignArgs& a, const void* bufv, int32_t* ta
     // whole CTA and looked up by a walk over all records, the stage took 45 us at 32 ranks with one hot rank (51 MB of
     // routing); now 29 us.
     const int nrec = ns;
-    uint32_t* const count = reinterpret_cast<uint32_t*>(scratch);      // [kWarps / 2][nrec] two spans per word (at most 2048 each)
+    uint32_t* const count = reinterpret_cast<uint32_t*>(scratch);      // [kWarps / 2][nrec] two spans per word (at most 2048 entries each)
     for (int k = tid; k < nrec; k += kThreads) recs[k].w = tab[recs[k].x];          // target after the expert's last split
     for (int q = tid; q < kWarps / 2 * nrec; q += kThreads) count[q] = 0u;
     __syncthreads();
@@ -431,11 +437,11 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
 }
 
 // shared memory of one CTA after the staged chunk: table, this chunk's counts and starting ordinals per expert, the
-// entries of the source rank (slot, expert, ordinal interval), the split records
-__host__ __device__ inline size_t chunk_smem_words(int E, int S)
+// entries of the source rank (slot, expert, ordinal interval; later the counts of splits by warp), the split records
+inline size_t chunk_smem_words(int E, int S, int NT)
 {
     const size_t Ep = ((size_t)E + 3) & ~(size_t)3, Sp = ((size_t)S + 3) & ~(size_t)3;
-    return 3 * Ep + 4 * Sp + 4 * Sp;
+    return 3 * Ep + (NT / 64) * Sp + 4 * Sp;
 }
 
 // One CTA per chunk.  STAGE: the chunk is first copied to shared memory with bulk asynchronous copies; otherwise it
@@ -445,10 +451,11 @@ __host__ __device__ inline size_t chunk_smem_words(int E, int S)
 // chunk's last entry of that expert, and one split record per quota interval that ends inside the chunk.
 // BYTES (with STAGE): what is staged is the chunk as one byte per entry, left by the histogram pass -- a quarter of the
 // bytes; a chunk whose flag says it holds a value that is no expert is read from the table itself, without staging.
-template <bool VEC, bool STAGE, bool BYTES>
-__global__ void __launch_bounds__(kThreads)
+template <bool VEC, bool STAGE, bool BYTES, int NT>
+__global__ void __launch_bounds__(NT)
 assign_chunk_kernel(AssignArgs a)
 {
+    constexpr int kThreads = NT, kWarps = Cta<NT>::kWarps;
     extern __shared__ __align__(128) unsigned char shc[];
     const int E = a.E, S = a.R * a.K;
     const int Ep = (E + 3) & ~3, Sp = (S + 3) & ~3;
@@ -460,7 +467,7 @@ assign_chunk_kernel(AssignArgs a)
     int32_t* ent_e = ent_s + Sp;                         //     ... their experts ...
     int32_t* ent_lo = ent_e + Sp;                        //     ... and the ordinals [lo, hi) they take
     int32_t* ent_hi = ent_lo + Sp;
-    int4* recs = reinterpret_cast<int4*>(ent_hi + Sp);   // [S] split records of this chunk
+    int4* recs = reinterpret_cast<int4*>(ent_s + kWarps / 2 * Sp);   // [S] split records of this chunk
     __shared__ __align__(8) uint64_t bar;
     __shared__ int s_cntw[kWarps];
     __shared__ int s_wcnt[32];
@@ -521,8 +528,8 @@ assign_chunk_kernel(AssignArgs a)
             return;
         }
     }
-    if (BYTES && flagged) rewrite_chunk<VEC, false>(a, a.topk + goff, tab, a.out + goff, len, s_ns, recs, ent_s, s_cntw, &s_pos);
-    else rewrite_chunk<VEC, BYTES>(a, buf, tab, a.out + goff, len, s_ns, recs, ent_s, s_cntw, &s_pos);
+    if (BYTES && flagged) rewrite_chunk<VEC, false, NT>(a, a.topk + goff, tab, a.out + goff, len, s_ns, recs, ent_s, s_cntw, &s_pos);
+    else rewrite_chunk<VEC, BYTES, NT>(a, buf, tab, a.out + goff, len, s_ns, recs, ent_s, s_cntw, &s_pos);
 }
 
 }  // namespace
@@ -541,24 +548,29 @@ int taot_launch_assign(taot_handle_t h, const int32_t* d_topk, void* ws, const i
                        ((reinterpret_cast<uintptr_t>(d_new_idx) & 15) == 0) && (h->seg % 4 == 0);
     const int S = p.R * p.K;
     const unsigned blocks = (unsigned)((int64_t)p.L * p.R * h->nc);
-    const size_t words = chunk_smem_words(p.E, S);
+    // Up to four chunks per SM, 512 threads each.  Stage with 256 / 512 threads, us (with the 4 that its events cost): 16 ranks, 384 chunks
+    // 20.5 / 16.4, 640 chunks 24.6 / 22.5, 960 chunks 26.6 / 26.6; 32 ranks with one hot rank, 384 chunks 30.7 / 24.6, 1280 43.0 / 39.0,
+    // 1920 47.1 / 51.2; 64 ranks, 512 chunks 18.4 / 18.5, 1024 24.6 / 26.6; 24 ranks (no staging), 168 20.5 / 16.4, 720 26.6 / 28.7.
+    const bool wide = blocks <= 4u * (unsigned)h->sm_count;
     a.tb = nullptr; a.tbflag = nullptr;
+    const auto launch = [&](auto kernel, int nt, size_t staged) -> int {
+        const size_t smem = staged + sizeof(int32_t) * chunk_smem_words(p.E, S, nt);
+        TAOT_CUDA_OK(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        TAOT_CUDA_OK(taot_launch_chained(kernel, blocks, nt, smem, st, a));
+        return 1;
+    };
+    int n;
     if (vec_ok && h->tb_ok) {
         // the histogram pass that left the chunk counts also left the table as one byte per entry
         a.tb = reinterpret_cast<const uint8_t*>(w + h->off_tb);
         a.tbflag = reinterpret_cast<const int32_t*>(w + h->off_tbflag);
-        const size_t smem = (size_t)TAOT_CHUNK + sizeof(int32_t) * words;
-        TAOT_CUDA_OK(cudaFuncSetAttribute(assign_chunk_kernel<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        TAOT_CUDA_OK(taot_launch_chained(assign_chunk_kernel<true, true, true>, blocks, kThreads, smem, st, a));
+        n = wide ? launch(assign_chunk_kernel<true, true, true, 512>, 512, TAOT_CHUNK) : launch(assign_chunk_kernel<true, true, true, 256>, 256, TAOT_CHUNK);
     } else if (vec_ok) {
-        const size_t smem = (size_t)TAOT_CHUNK * 4 + sizeof(int32_t) * words;
-        TAOT_CUDA_OK(cudaFuncSetAttribute(assign_chunk_kernel<true, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        TAOT_CUDA_OK(taot_launch_chained(assign_chunk_kernel<true, true, false>, blocks, kThreads, smem, st, a));
+        n = wide ? launch(assign_chunk_kernel<true, true, false, 512>, 512, TAOT_CHUNK * 4) : launch(assign_chunk_kernel<true, true, false, 256>, 256, TAOT_CHUNK * 4);
     } else {
-        const size_t smem = sizeof(int32_t) * words;
-        TAOT_CUDA_OK(cudaFuncSetAttribute(assign_chunk_kernel<false, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        TAOT_CUDA_OK(taot_launch_chained(assign_chunk_kernel<false, false, false>, blocks, kThreads, smem, st, a));
+        n = wide ? launch(assign_chunk_kernel<false, false, false, 512>, 512, 0) : launch(assign_chunk_kernel<false, false, false, 256>, 256, 0);
     }
+    if (n < 0) return n;
     TAOT_CUDA_OK(cudaGetLastError());
     return 1;
 }
