@@ -116,9 +116,12 @@ __device__ void excess_spare_row(const int32_t* s_rl, int32_t R, long long* s_to
     const int tid = threadIdx.x;
     if (tid == 0) *s_tot = 0;
     __syncthreads();
-    long long part = 0;
-    for (int r = tid; r < R; r += blockDim.x) part += s_rl[r];
-    if (part) atomicAdd(reinterpret_cast<unsigned long long*>(s_tot), (unsigned long long)part);
+    // the total: by warp, in two halves of 16 bits, then an atomic per warp (64-bit ones on one word, a rank each, queue up)
+    for (int r0 = tid & ~31; r0 < R; r0 += blockDim.x) {
+        const int32_t v = r0 + (tid & 31) < R ? s_rl[r0 + (tid & 31)] : 0;
+        const long long part = (long long)__reduce_add_sync(0xffffffffu, v & 0xFFFF) + 65536ll * __reduce_add_sync(0xffffffffu, v >> 16);
+        if ((tid & 31) == 0 && part) atomicAdd(reinterpret_cast<unsigned long long*>(s_tot), (unsigned long long)part);
+    }
     __syncthreads();
     const long long m = *s_tot / R;
     for (int r = tid; r < R; r += blockDim.x) {
@@ -149,22 +152,56 @@ merge_kernel(const int32_t* __restrict__ cc, const int32_t* __restrict__ e2r, in
     int32_t* s_rl = sh + E;
     const int l = blockIdx.x / parts, part = blockIdx.x - l * parts, tid = threadIdx.x;
     for (int i = tid; i < E + R; i += blockDim.x) sh[i] = 0;
+    const uint32_t my_home = tid < E ? (uint32_t)e2r[tid] : 0u;      // (the map is no kernel's output; a caller-supplied one is there first)
     __syncthreads();
     taot_await();
     taot_release();
+    int bad = 0;
+    if (info_out)
+        for (int q = tid; q < R * nc; q += blockDim.x) bad |= chunk_bad[(int64_t)l * R * nc + q];
     const int32_t RE = R * E;                            // at most 256 x 1024
     const int32_t* ccl = cc + (int64_t)l * RE * nc;
     int32_t* nl = n + (int64_t)l * RE;
-    // (32-bit index arithmetic and several independent loads in flight per thread)
-    const int32_t i0 = (int32_t)((int64_t)RE * part / parts), i1 = (int32_t)((int64_t)RE * (part + 1) / parts);
+    const int r0 = R * part / parts, r1 = R * (part + 1) / parts;
+    if (E % 4 == 0 && ((reinterpret_cast<uintptr_t>(cc) | reinterpret_cast<uintptr_t>(n)) & 15) == 0) {
+        // a thread takes four experts of every G-th rank: 16-byte loads, four ranks and two chunks of them in flight, and its
+        // experts' loads in registers until the end (an element at a time with an atomic each: 64 ranks, 256 experts, 4 chunks a
+        // segment, 58 layers 26.6 us)
+        const int EQ = E >> 2, G = (int)blockDim.x / EQ, q = tid % EQ, g = tid / EQ;
+        const int4* src = reinterpret_cast<const int4*>(ccl) + q;
+        int4* dst = reinterpret_cast<int4*>(nl) + q;
+        int4 sum = make_int4(0, 0, 0, 0);
+        const auto add = [](int4& x, const int4 y) { x.x += y.x; x.y += y.y; x.z += y.z; x.w += y.w; };
+        for (int r = r0 + g; r < r1 && g < G; r += 4 * G) {
+            int4 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = make_int4(0, 0, 0, 0);
+#pragma unroll 2
+            for (int c = 0; c < nc; ++c) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (r + u * G < r1) add(v[u], __ldg(src + ((r + u * G) * nc + c) * EQ));
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (r + u * G < r1) dst[(r + u * G) * EQ] = v[u];
+                add(sum, v[u]);
+            }
+        }
+        if (sum.x) atomicAdd(s_el + 4 * q, sum.x);
+        if (sum.y) atomicAdd(s_el + 4 * q + 1, sum.y);
+        if (sum.z) atomicAdd(s_el + 4 * q + 2, sum.z);
+        if (sum.w) atomicAdd(s_el + 4 * q + 3, sum.w);
+    } else {
 #pragma unroll 4
-    for (int32_t idx = i0 + tid; idx < i1; idx += blockDim.x) {
-        const int32_t r = idx / E, e = idx - r * E;
-        const int32_t* p = ccl + r * nc * E + e;
-        int32_t v = 0;
-        for (int c = 0; c < nc; ++c) v += __ldg(p + c * E);
-        nl[idx] = v;
-        if (v) atomicAdd(s_el + e, v);
+        for (int32_t idx = r0 * E + tid; idx < r1 * E; idx += blockDim.x) {
+            const int32_t r = idx / E, e = idx - r * E;
+            const int32_t* p = ccl + r * nc * E + e;
+            int32_t v = 0;
+            for (int c = 0; c < nc; ++c) v += __ldg(p + c * E);
+            nl[idx] = v;
+            if (v) atomicAdd(s_el + e, v);
+        }
     }
     __syncthreads();
     if (parts > 1) {
@@ -186,8 +223,6 @@ merge_kernel(const int32_t* __restrict__ cc, const int32_t* __restrict__ e2r, in
         __syncthreads();
     }
     if (info_out) {
-        int bad = 0;
-        for (int q = tid; q < R * nc; q += blockDim.x) bad |= chunk_bad[(int64_t)l * R * nc + q];
         bad = __syncthreads_or(bad);
         if (tid == 0) info_out[l] = bad ? TAOT_INFO_BAD_INDEX : 0;
     }
@@ -196,7 +231,7 @@ merge_kernel(const int32_t* __restrict__ cc, const int32_t* __restrict__ e2r, in
         expert_load[(int64_t)l * E + e] = v;
         // a handle's map was validated on the host; a caller-supplied device map (the entry point without a handle)
         // was not: an expert whose home rank is out of range is left out of the rank loads and flagged
-        const uint32_t home = (uint32_t)e2r[e];
+        const uint32_t home = e == tid ? my_home : (uint32_t)e2r[e];
         if (home < (uint32_t)R) {
             if (v) atomicAdd(s_rl + home, v);
         } else if (info) {
