@@ -446,14 +446,13 @@ struct Lean {
             if (WM > 1 && et >= 0 && !one) {          // the tier's words from `first` on
                 const int ci = t.tms == t.S ? c : (int)(1023u - (low & 1023u)) / t.K;
                 const uint32_t* tm = t.tm + et * t.W * t.tms + ci;
-#pragma unroll
-                for (int w = WM - 1; w >= 0; --w) {
-                    if (w < t.W) {
-                        const uint32_t h = tm[w * t.tms] & lds_u32(a_av_c + (uint32_t)w * dmax);
-                        const uint32_t x = h & lds_u32(a_wins + (uint32_t)w * LS);
-                        held |= h;
-                        if (w >= first && x) { cw = x; pw = w; }
-                    }
+#pragma unroll 1
+                for (int w = first; w < t.W; ++w) {
+                    const uint32_t h = tm[w * t.tms] & lds_u32(a_av_c + (uint32_t)w * dmax);
+                    held |= h;
+                    cw = h & lds_u32(a_wins + (uint32_t)w * LS);
+                    pw = w;
+                    if (cw) break;
                 }
             } else if (first == 0) {
                 held = m & lds_u32(a_av_c + (uint32_t)pw * dmax);

@@ -123,9 +123,7 @@ match_kernel(MatchArgs a)
     // ---- carve shared memory
     u64* arb_e = reinterpret_cast<u64*>(smem_raw);            // [E]  Phase 2 arbitration per expert
     u64* arb_r = arb_e + E;                                    // [2][R]  Phase 3 arbitration per rank, ping-pong by round
-    uint2* rec_s = reinterpret_cast<uint2*>(arb_r + 2 * R);     // LEAN: [S+1] next slot of the class and its tokens
-    uint2* tw2 = rec_s + (LEAN && a.nbid ? S + 1 : 0);          // LEAN: [ntiers][S] word and mask of a tier that one word holds, by class
-    int32_t* spill = reinterpret_cast<int32_t*>(tw2 + (LEAN && a.nbid ? a.ntiers * S : 0)); // [E]
+    int32_t* spill = reinterpret_cast<int32_t*>(arb_r + 2 * R); // [E]
     int32_t* hot0 = spill + E;                                 // [E]  experts that spill at the start of Phase 2
     int32_t* hot_home = hot0 + E;                              // [E]  their home ranks
     int32_t* dcol = hot_home + E;                              // [E]  expert -> column of nrem, or -1
@@ -150,6 +148,9 @@ match_kernel(MatchArgs a)
     const int RS = R | 1;
     float* bon_s = reinterpret_cast<float*>(lead_s + (a.nbid ? S : 0));                // dense scan, if it fits: [R][RS] bonus of rank r for host h at h * RS + r
     int32_t* nrem_s = reinterpret_cast<int32_t*>(bon_s + (a.bon_in_smem ? R * RS : 0)); // [dmax*R] if it fits
+    // LEAN, Phase 3 only, behind the counts in the block that Phase 2 uses for its keys
+    uint2* rec_s = reinterpret_cast<uint2*>((reinterpret_cast<uintptr_t>(nrem_s + (a.nrem_in_smem ? a.dmax * (R | 1) : 0)) + 7) & ~(uintptr_t)7);   // [S+1] next slot of the class and its tokens
+    uint2* tw2 = rec_s + S + 1;                                // [ntiers][S] word and mask of a tier that one word holds, by class
     __shared__ long long s_tot;
     __shared__ int s_cnt, s_any, s_ns;
     __shared__ taot_auction::Control ctl;
@@ -707,6 +708,7 @@ match_kernel(MatchArgs a)
             const auto lean_w = [&](auto tiers) {
                 if (W == 1) lean(tiers, std::integral_constant<int, 1>{});
                 else if (W == 2) lean(tiers, std::integral_constant<int, 2>{});
+                else if (W <= 4) lean(tiers, std::integral_constant<int, 4>{});
                 else lean(tiers, std::integral_constant<int, kMaxW>{});
             };
             if (a.ntiers <= 2) lean_w(std::integral_constant<int, 2>{});
@@ -879,9 +881,11 @@ int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expe
     a.ablation = p.ablation;
     size_t smem = match_smem_fixed(p.R, p.E, p.K, a.dmax, a.W, a.ntiers);
     const bool few_tiers = h->ntiers <= 4 && !h->bid_ties;
-    const size_t lists = sizeof(uint32_t) * (2 * (size_t)h->nbid + 2 * (size_t)h->ntiers * p.R * p.K + 2 * (size_t)p.R * p.K + 1 +
-                                             2 * ((size_t)p.R * p.K + 1));
-    if (a.nbid > 0 && smem + lists > kSmemBudget) { a.nbid = 0; a.ntiers = 0; }      // (no room for the lists: the dense scan)
+    const size_t S = (size_t)p.R * p.K;
+    const size_t lists = sizeof(uint32_t) * (2 * (size_t)h->nbid + (few_tiers ? 0 : 2 * (size_t)h->ntiers * S) + 2 * S + 1);
+    // (few tiers: what only Phase 3 needs lies behind the counts, see below)
+    size_t lean_bytes = a.nbid > 0 && few_tiers ? sizeof(uint2) * (S + 1 + (size_t)h->ntiers * S) + 8 : 0;
+    if (a.nbid > 0 && smem + lists + lean_bytes > kSmemBudget) { a.nbid = 0; a.ntiers = 0; lean_bytes = 0; }      // (no room for the lists: the dense scan)
     if (a.nbid > 0) smem += lists;
     const size_t nrem_bytes = sizeof(int32_t) * (size_t)a.dmax * (p.R | 1);
     // the bonus matrix of the dense scan, where it fits beside the remaining counts
@@ -891,11 +895,11 @@ int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expe
     const size_t tm_bytes = sizeof(uint32_t) * (size_t)a.ntiers * a.W * p.R * p.K;
     a.tm_in_smem = (a.ntiers > 0 && smem + tm_bytes <= 96 * 1024) ? 1 : 0;
     if (a.tm_in_smem) smem += tm_bytes;
-    a.nrem_in_smem = (smem + nrem_bytes <= kSmemBudget) ? 1 : 0;
+    a.nrem_in_smem = (smem + nrem_bytes + lean_bytes <= kSmemBudget) ? 1 : 0;
     // one block for Phase 2 (per spilling expert R keys and 2 * R floats of round-invariant score rows) and then the
-    // remaining counts: as large as the counts need if those live in shared memory, and as much of what Phase 2 could
-    // use as there is room for
-    size_t big = a.nrem_in_smem ? nrem_bytes : 0;
+    // remaining counts and the lists of Phase 3: as large as those need, and as much of what Phase 2 could use as there is
+    // room for (a layer whose keys do not fit takes the full scan: 256 ranks, 1024 experts, 1024 slots 1.7 -> 2.1 ms with 8 KB less)
+    size_t big = (a.nrem_in_smem ? nrem_bytes : 0) + lean_bytes;
     const size_t want = sizeof(float) * ((size_t)p.R * ((size_t)p.E | 1) + 2 * (size_t)p.R * (size_t)p.E);
     const size_t room = kSmemBudget > smem ? kSmemBudget - smem : 0;
     if (big < want) big = want < room ? want : (room > big ? room : big);
