@@ -10,11 +10,12 @@
 // contraction), which keeps every integer decision reproducible bit for bit on a CPU.
 //
 // Phase 2: the two score terms that do not change between rounds (alpha*B and 0.1*alpha*T_norm)
-// are computed once per layer for the experts that spill, and the scores once per slot index; a
-// round re-forms the rows of the experts it served.  It is bound by that chain of rounds: up to 64
-// ranks one warp runs them (one or two ranks per lane, a rank scans again only if its best pair
-// changed), since the barriers of a CTA cost more than the scans (58 -> 50 k cycles at 32 ranks);
-// with more ranks a lane would hold four and its scans outweigh the barriers: several lanes per rank.
+// are computed once per layer for the experts that spill, and the scores once per slot index.  It is
+// bound by that chain of rounds.  A rank has several lanes and its state in their registers: they
+// re-form its entries of the experts served in the last round, and scan its row again only if its
+// best pair was among them; three barriers a round (one warp for up to 64 ranks: 87 -> 55 k cycles at
+// 64 ranks, 16 rounds; a fourth barrier and all rows scanned in every round beyond: matching stage of
+// 200 ranks with 600 slots 739 -> 688 us, 64 ranks 129 -> 123, 32 ranks 59.4 -> 57.3).
 //
 // In a plan the kernel is set up (loads, spills, score terms) while Phase 1 still runs and waits for
 // it where it first reads the hint: a plan of one 8-rank layer 69 -> 66 us, 32 ranks 141 -> 129 us,
@@ -307,7 +308,6 @@ match_kernel(MatchArgs a)
         const int32_t gain = se < sp ? se : sp;
         return ordered_bits(__fadd_rn(__fadd_rn((float)gain, t12[(int64_t)(2 * q) * R + r]), t12[(int64_t)(2 * q + 1) * R + r]));
     };
-    const bool small = R <= 64;                   // one warp runs the rounds, a rank or two per lane, without block barriers
     for (int kappa = 0; keyed && kappa < K; ++kappa) {
         // Between rounds a pair's score changes only when its expert was served (its spill shrank): a rank's spare
         // changes only when it is matched, and then it is out for this slot index.  So all keys are formed once per
@@ -318,190 +318,100 @@ match_kernel(MatchArgs a)
         uint32_t* arb_hi = reinterpret_cast<uint32_t*>(arb_e);
         uint32_t* arb_lo = arb_hi + E;
         int smax = 0;                              // largest spare of this slot index: a row changes only below it
-        for (int r = tid; r < R; r += NT) { matched[r] = 0; smax = spare[r] > smax ? spare[r] : smax; }
+        for (int r = tid; r < R; r += NT) { smax = spare[r] > smax ? spare[r] : smax; }
         for (int e = tid; e < E; e += NT) { arb_hi[e] = 0u; arb_lo[e] = 0xFFFFFFFFu; }
         smax = __reduce_max_sync(0xffffffffu, smax);
         if (tid == 0) s_cnt = 0;
         __syncthreads();
         if (lane == 0) atomicMax(&s_cnt, smax);
         if (my_r < R)
+#pragma unroll 4
             for (int q = my_q; q < nhot0; q += q_step) keyM[my_r * NHs + q] = pair_key(q, my_r, kappa);
         __syncthreads();
         const int32_t spare_cap = s_cnt;
         if (timed) c_build += clock64() - c_b0;
-        if (small) {
-            if (warp == 0) {
-                constexpr int RPL = 2;
-                int32_t sp[RPL];
-                uint32_t bk[RPL];                  // the rank's best candidate: key and position (0: none)
-                int bq[RPL];
-                bool open[RPL], scan[RPL];
-#pragma unroll
-                for (int k = 0; k < RPL; ++k) {
-                    const int r = lane + 32 * k;
-                    sp[k] = r < R ? spare[r] : 0;
-                    open[k] = sp[k] > 0; scan[k] = open[k];
-                    bk[k] = 0u; bq[k] = 0;
-                }
-                for (;;) {
-                    const long long c_s0 = timed ? clock64() : 0;
-                    // Steps 1-2: every unmatched cold rank takes its best candidate expert (ties: lowest position = lowest index); one
-                    // whose best pair did not change in the last round still has it, since keys only shrink
-#pragma unroll
-                    for (int k = 0; k < RPL; ++k) {
-                        if (scan[k]) {
-                            const uint32_t* row = keyM + (lane + 32 * k) * NHs;
-                            uint32_t best = 0u;
-                            int at = 0;
-#pragma unroll 8
-                            for (int q = 0; q < nhot0; ++q) {
-                                const uint32_t v = row[q];
-                                at = v > best ? q : at;
-                                best = v > best ? v : best;
-                            }
-                            bk[k] = best; bq[k] = at;
-                            open[k] = best != 0u;
-                            scan[k] = false;
-                        }
-                    }
-                    __syncwarp();
-                    bool bids = false;
-#pragma unroll
-                    for (int k = 0; k < RPL; ++k) bids = bids || open[k];
-                    if (!__any_sync(0xffffffffu, bids)) break;
-                    // Step 3: the best score any rank offers the expert, then among the ranks that offer it the lowest
-#pragma unroll
-                    for (int k = 0; k < RPL; ++k)
-                        if (open[k]) atomicMax(&arb_hi[bq[k]], bk[k]);
-                    __syncwarp();
-#pragma unroll
-                    for (int k = 0; k < RPL; ++k)
-                        if (open[k] && arb_hi[bq[k]] == bk[k]) atomicMin(&arb_lo[bq[k]], (uint32_t)(lane + 32 * k));
-                    __syncwarp();
-                    bool win[RPL];
-#pragma unroll
-                    for (int k = 0; k < RPL; ++k) win[k] = open[k] && arb_lo[bq[k]] == (uint32_t)(lane + 32 * k);
-                    __syncwarp();
-                    // Step 4: winners take min(spill, spare)
-#pragma unroll
-                    for (int k = 0; k < RPL; ++k) {
-                        if (win[k]) {
-                            const int r = lane + 32 * k, e = hot0[bq[k]];
-                            const int32_t se = spill[e], g = se < sp[k] ? se : sp[k];
-                            spill[e] = se - g;
-                            spare[r] = sp[k] - g;
-                            slot_e[r * K + kappa] = e;
-                            slot_a0[r * K + kappa] = g;
-                            arb_hi[bq[k]] = 0u;
-                            arb_lo[bq[k]] = 0xFFFFFFFFu;
-                            open[k] = false;
-                        }
-                    }
-                    __syncwarp();
-                    const long long c_s1 = timed ? clock64() : 0;
-                    if (timed) c_scan += c_s1 - c_s0;
-                    // the served experts' rows, each rank its own entry: it changes only where min(spill, spare) does
-#pragma unroll
-                    for (int k2 = 0; k2 < RPL; ++k2) {
-                        unsigned todo = __ballot_sync(0xffffffffu, win[k2]);
-                        while (todo) {
-                            const int q = __shfl_sync(0xffffffffu, bq[k2], __ffs(todo) - 1);
-                            todo &= todo - 1;
-                            const int32_t se = spill[hot0[q]];
-#pragma unroll
-                            for (int k = 0; k < RPL; ++k) {
-                                if (open[k] && se < sp[k]) {
-                                    const int r = lane + 32 * k;
-                                    uint32_t* cell = keyM + r * NHs + q;
-                                    if (*cell) {
-                                        *cell = se > 0 ? shrunk_key(q, r, se, sp[k]) : 0u;
-                                        if (q == bq[k]) scan[k] = true;
-                                    }
-                                }
-                            }
-                        }
-                    }
-                    __syncwarp();
-                    ++rounds2;
-                    if (timed) c_row += clock64() - c_s1;
-                }
-                if (lane == 0) s_any = rounds2;
-            }
-            __syncthreads();
-            rounds2 = s_any;
-            continue;
-        }
+        // QS adjacent lanes share a rank and its row of keys (QS * R <= NT: one pass covers every rank); the rank's state is in
+        // registers, the same in all of them.
+        const int r = tid >> qsh;
+        const bool lead = qs == 0;
+        const unsigned group = (QS == 32 ? 0xFFFFFFFFu : ((1u << QS) - 1u) << (lane & ~(QS - 1)));
+        uint32_t* const row = keyM + (r < R ? r : 0) * NHs;
+        const int32_t sp = r < R ? spare[r] : 0;
+        bool open = sp > 0, scan = open;
+        uint32_t bk = 0u;                          // the rank's best candidate: key and position (0: none)
+        int bq = 0, ns = 0;
         for (;;) {
             const long long c_s0 = timed ? clock64() : 0;
-            // Steps 1-2: every unmatched cold rank takes its best candidate expert (ties: lowest position = lowest index)
-            // (QS lanes per rank with QS * R <= NT: one pass covers every rank)
-            const int r = tid >> qsh;
-            uint32_t my_bk = 0u;                   // this thread's bid, if it is the lead lane of a bidding rank
-            int my_bq = -1;
-            {
-                u64 key = 0;
-                if (r < R && !matched[r] && spare[r] > 0) {
-                    const uint32_t* row = keyM + r * NHs;
-                    uint32_t bk = 0u;
-                    int bq = 0;
-#pragma unroll 4
-                    for (int q = qs; q < nhot0; q += QS) {      // ascending positions: a strict compare keeps the lowest
-                        const uint32_t k32 = row[q];
-                        if (k32 > bk) { bk = k32; bq = q; }
-                    }
-                    if (bk != 0u) key = ((u64)bk << 32) | (u64)(0xFFFFFFFFu - (uint32_t)bq);
-                }
-                for (int o = 1; o < QS; o <<= 1) {
-                    const u64 other = __shfl_xor_sync(0xffffffffu, key, o);
-                    key = other > key ? other : key;
-                }
-                if (qs == 0 && r < R && key != 0) {
-                    my_bk = (uint32_t)(key >> 32);
-                    my_bq = (int)(0xFFFFFFFFu - (uint32_t)key);
-                }
-            }
-            // Step 3, first half: the best score any rank offers the expert (native 32-bit shared-memory atomics; agreeing
-            // inside the warp first on the expert most lanes want was measured and cost more than the conflicts it saves)
-            if (my_bq >= 0) atomicMax(&arb_hi[my_bq], my_bk);
-            if (!__syncthreads_or(my_bq >= 0)) break;
-            if (tid == 0) s_ns = 0;
-            // Step 3, second half: among the ranks that offer it, the lowest
-            if (my_bq >= 0 && arb_hi[my_bq] == my_bk) atomicMin(&arb_lo[my_bq], (uint32_t)r);
-            __syncthreads();
-            const long long c_s1 = timed ? clock64() : 0;
-            if (timed) c_scan += c_s1 - c_s0;
-            // Step 4: winners take min(spill, spare), and put the arbitration entries back.  A row of keys changes only
-            // where min(spill, spare_r) does, i.e. for ranks with more spare than the expert now spills: rows whose
-            // expert still spills at least the largest spare of this slot index are left as they are.
-            if (my_bq >= 0 && arb_lo[my_bq] == (uint32_t)r) {
-                const int e = hot0[my_bq];
-                const int32_t se = spill[e], sp = spare[r], g = se < sp ? se : sp;
-                spill[e] = se - g;
-                spare[r] = sp - g;
-                matched[r] = 1;
-                slot_e[r * K + kappa] = e;
-                slot_a0[r * K + kappa] = g;
-                arb_hi[my_bq] = 0u;                // (a loser compares arb_lo with its own rank: the reset value is nobody's)
-                arb_lo[my_bq] = 0xFFFFFFFFu;
-                if (se - g < spare_cap) served[atomicAdd(&s_ns, 1)] = my_bq;
-            }
-            __syncthreads();
-            const long long c_s2 = timed ? clock64() : 0;
-            const int ns = s_ns;
+            // the served experts' entries of the row, which change only where min(spill, spare) does
             if (ns > 0) {                          // uniform over the CTA
-                if (my_r < R) {
-                    const int32_t sp = spare[my_r];
-                    for (int i = my_q; i < ns; i += q_step) {
+                bool hit = false;
+                if (open) {
+                    for (int i = qs; i < ns; i += QS) {
                         const int q = served[i];
                         const int32_t se = spill[hot0[q]];
-                        uint32_t* cell = keyM + my_r * NHs + q;
-                        if (se < sp && *cell) *cell = se > 0 ? shrunk_key(q, my_r, se, sp) : 0u;
+                        if (se < sp && row[q]) {
+                            row[q] = se > 0 ? shrunk_key(q, r, se, sp) : 0u;
+                            hit = hit || q == bq;
+                        }
                     }
                 }
-                __syncthreads();
+                scan = (__ballot_sync(0xffffffffu, hit) & group) != 0u;
+                __syncwarp();
             }
+            const long long c_s1 = timed ? clock64() : 0;
+            // Steps 1-2: every unmatched cold rank takes its best candidate expert (ties: lowest position = lowest index); one
+            // whose best pair did not change in the last round still has it, since keys only shrink
+            if (__any_sync(0xffffffffu, scan)) {
+                uint32_t best = 0u;
+                int at = 0;
+                if (open) {
+#pragma unroll 4
+                    for (int q = qs; q < nhot0; q += QS) {      // ascending positions: a strict compare keeps the lowest
+                        const uint32_t v = row[q];
+                        at = v > best ? q : at;
+                        best = v > best ? v : best;
+                    }
+                }
+                for (int o = 1; o < QS; o <<= 1) {
+                    const uint32_t v = __shfl_xor_sync(0xffffffffu, best, o);
+                    const int p = __shfl_xor_sync(0xffffffffu, at, o);
+                    const bool better = (v > best) | ((v == best) & (p < at));
+                    best = better ? v : best;
+                    at = better ? p : at;
+                }
+                bk = best; bq = at;
+                open = open && best != 0u;
+                scan = false;
+            }
+            // Step 3, first half: the best score any rank offers the expert
+            const bool bids = lead && open;
+            if (bids) atomicMax(&arb_hi[bq], bk);
+            if (!__syncthreads_or(bids)) break;
+            if (tid == 0) s_ns = 0;
+            // Step 3, second half: among the ranks that offer it, the lowest
+            if (bids && arb_hi[bq] == bk) atomicMin(&arb_lo[bq], (uint32_t)r);
+            __syncthreads();
+            const long long c_s2 = timed ? clock64() : 0;
+            // Step 4: winners take min(spill, spare), and put the arbitration entries back (a loser compares arb_lo with its own
+            // rank: the reset value is nobody's).  Rows whose expert still spills at least the largest spare of this slot index
+            // are left as they are.
+            const bool win = bids && arb_lo[bq] == (uint32_t)r;
+            if (win) {
+                const int e = hot0[bq];
+                const int32_t se = spill[e], g = se < sp ? se : sp;
+                spill[e] = se - g;
+                spare[r] = sp - g;
+                slot_e[r * K + kappa] = e;
+                slot_a0[r * K + kappa] = g;
+                arb_hi[bq] = 0u;
+                arb_lo[bq] = 0xFFFFFFFFu;
+                if (se - g < spare_cap) served[atomicAdd(&s_ns, 1)] = bq;
+            }
+            if (__ballot_sync(0xffffffffu, win) & group) open = false;
+            __syncthreads();
+            ns = s_ns;
             ++rounds2;
-            if (timed) { const long long c_s3 = clock64(); c_win += c_s2 - c_s1; c_row += c_s3 - c_s2; }
+            if (timed) { const long long c_s3 = clock64(); c_row += c_s1 - c_s0; c_scan += c_s2 - c_s1; c_win += c_s3 - c_s2; }
         }
         __syncthreads();
     }
