@@ -45,20 +45,21 @@ struct SplitSmem {
     alignas(16) float u[kSplitRows], e[kSplitGroup][kSplitRows];   // u~ and the rows' errors
     float st[kSplitRows], dd[RMAX], fg[RMAX];
     int32_t hot[kSplitRows], cold[RMAX];
+    int32_t fill;                          // what the other warps are to do: rebuild the tile, or go on behind the loop
     float err;                             // how the loop ended: row error of the iterate,
     int32_t status, t;                     // 1 solved, 0 handed back, and the iterate
 };
 
-// K~ (zero off the problem's block) by `nt` threads, a multiple of RMAX
+// K~ by `nt` threads, a multiple of RMAX: the first `rows` rows (all of them at first: zero off the problem's block)
 template <int RMAX>
-__device__ __forceinline__ void split_fill(const SinkArgs& a, SplitSmem<RMAX>& sm, int Hn, int Cn, int tid, int nt)
+__device__ __forceinline__ void split_fill(const SinkArgs& a, SplitSmem<RMAX>& sm, int Hn, int Cn, int rows, int tid, int nt)
 {
     const int j = tid & (RMAX - 1);
     const bool col = j < Cn;
     const double be = col ? sm.beta[j] : 0.0;
     const float* C = sm.C + (col ? sm.cold[j] : 0);
 #pragma unroll 4
-    for (int i = tid / RMAX; i < kSplitRows; i += nt / RMAX) {
+    for (int i = tid / RMAX; i < rows; i += nt / RMAX) {
         float v = 0.0f;
         if (i < Hn && col) {
             const double c = (double)C[sm.hot[i] * a.R] * a.inv_eps;
@@ -67,6 +68,9 @@ __device__ __forceinline__ void split_fill(const SinkArgs& a, SplitSmem<RMAX>& s
         sm.K[i * SplitSmem<RMAX>::KS + j] = v;
     }
 }
+
+template <int NT>
+__device__ __forceinline__ void split_sync() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); }
 
 // sum of the rows' errors in the grid's order
 template <int NRA>
@@ -86,7 +90,7 @@ __device__ __forceinline__ float split_error(const float* e)
 // Eight iterations at a time run without a branch on drift, tolerance or cap (a vote and a branch cost about 25 cycles); one look
 // at the end tells whether there was anything, and if there was the eight are taken back and done again one by one.  A row error
 // above the tolerance settles that the sum is; only if no row has one are the sums formed.
-template <int RMAX, int LR, int RPL, int NRA, int NCG, bool TOL>
+template <int RMAX, int NT, int LR, int RPL, int NRA, int NCG, bool TOL>
 __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& sm, const int Hn, const int Cn, const float tol_abs_f)
 {
     constexpr int CPL = RMAX / 32, RS = 32 / LR;       // RS: rows between a lane's
@@ -301,10 +305,10 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
                     if (col_ok[q]) sm.beta[lane + 32 * q] += log((double)vcol[q]);
                     sm.v[t & 1][lane + 32 * q] = vcol[q] = 1.0f;
                 }
-                __syncwarp();
-#pragma unroll 1
-                for (int q = 0; q < CPL; ++q) split_fill<RMAX>(a, sm, Hn, Cn, lane + 32 * q, RMAX);
-                __syncwarp();
+                if (lane == 0) sm.fill = 1;
+                split_sync<NT>();
+                split_fill<RMAX>(a, sm, Hn, Cn, Hn, lane, NT);
+                split_sync<NT>();
                 load_tile();
                 break;
             }
@@ -325,11 +329,10 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
     }
 }
 
-template <int RMAX, bool TOL>
+template <int RMAX, int NT, bool TOL>
 __device__ __forceinline__ void split_dispatch(const SinkArgs& a, SplitSmem<RMAX>& sm, int Hn, int Cn, float tol_abs_f)
 {
-    if (threadIdx.x >= 32) return;
-#define TAOT_SPLIT(LR, RPL, NRA, NCG) return split_loop<RMAX, LR, RPL, NRA, NCG, TOL>(a, sm, Hn, Cn, tol_abs_f)
+#define TAOT_SPLIT(LR, RPL, NRA, NCG) return split_loop<RMAX, NT, LR, RPL, NRA, NCG, TOL>(a, sm, Hn, Cn, tol_abs_f)
     if constexpr (RMAX == 32) {
 #define TAOT_SPLIT_ROWS(NCG)                           \
         if (Hn <= 4) TAOT_SPLIT(1, 1, 1, NCG);        \
@@ -486,9 +489,20 @@ sinkhorn_tile_kernel(SinkArgs a)
         }
         __syncthreads();
     }
-    split_fill<RMAX>(a, sm, Hn, Cn, tid, NT);
+    split_fill<RMAX>(a, sm, Hn, Cn, kSplitRows, tid, NT);
     __syncthreads();
-    split_dispatch<RMAX, TOL>(a, sm, Hn, Cn, (float)((double)a.tol * sum_st));
+    // one warp iterates; the others wait until a fold wants the tile rebuilt (64 ranks, 1000 iterations with a dozen folds: 2 us each
+    // by the one warp)
+    if (warp == 0) {
+        split_dispatch<RMAX, NT, TOL>(a, sm, Hn, Cn, (float)((double)a.tol * sum_st));
+        if (lane == 0) sm.fill = 0;
+        split_sync<NT>();
+    } else {
+        for (split_sync<NT>(); sm.fill; split_sync<NT>()) {
+            split_fill<RMAX>(a, sm, Hn, Cn, Hn, tid, NT);
+            split_sync<NT>();
+        }
+    }
     __syncthreads();
     taot_release();
     if (sm.status == 0) {
@@ -496,7 +510,7 @@ sinkhorn_tile_kernel(SinkArgs a)
         return;
     }
     // ---- T = diag(u) M diag(v) from the total potentials, then the column cap
-    split_fill<RMAX>(a, sm, Hn, Cn, tid, NT);
+    split_fill<RMAX>(a, sm, Hn, Cn, Hn, tid, NT);
     __syncthreads();
     if (tid < Cn) {
         float c0 = 0.0f, c1 = 0.0f, c2 = 0.0f, c3 = 0.0f;
