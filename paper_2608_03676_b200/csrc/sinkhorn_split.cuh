@@ -11,8 +11,9 @@
 // each more).  ns per iteration, grid -> here, with a tolerance: 8 ranks 137 -> 92, 16 162 -> 106, 32 175 -> 109, 64 253 -> 145;
 // fixed count: 119 -> 86, 125 -> 107, 140 -> 107, 188 -> 143.  What is left of the chain at 16 ranks: two exchanges 56, six loads
 // 48, two reciprocals with their products 46, chains and trees 32, the look at the end of a group 10, of 204 cycles.
-// (Two warps, 32 rows and 64 columns between them, behind named barriers: 150 ns at 64 ranks for a fixed count, 210 with a
-// tolerance; a branch in the loop that the compiler cannot prove uniform costs 25 to 50 cycles with the warp barrier behind it.)
+// More than 16 supply ranks (only beyond 32 ranks) take two warps and named barriers: there a lone warp would hold two rows a lane,
+// 193 ns an iteration against 165 (with up to 16 the two are as fast).  A branch in the loop that the compiler cannot prove
+// uniform costs 25 to 50 cycles with the warp barrier behind it.
 //
 // Set-up is spread over the CTA's warps: the cost matrix is in shared memory before the kernels in front have ended, and an
 // exponential of the first iteration and of K~ is one thread's work each (64 ranks: 27 -> 16 us for all but the iterations).
@@ -45,6 +46,7 @@ struct SplitSmem {
     alignas(16) float u[kSplitRows], e[kSplitGroup][kSplitRows];   // u~ and the rows' errors
     float st[kSplitRows], dd[RMAX], fg[RMAX];
     int32_t hot[kSplitRows], cold[RMAX];
+    uint32_t bits[2];                      // what the eight iterations met, by warp
     int32_t fill;                          // what the other warps are to do: rebuild the tile, or go on behind the loop
     float err;                             // how the loop ended: row error of the iterate,
     int32_t status, t;                     // 1 solved, 0 handed back, and the iterate
@@ -85,52 +87,56 @@ __device__ __forceinline__ float split_error(const float* e)
     return (s0 + s1) + (s2 + s3);
 }
 
-// The iterations, by one warp.  LR lanes hold RPL rows, a lane CPL columns; NRA: rows / 4, NCG: columns / 8.
+// The iterations, by NW warps.  LR lanes hold a row, a lane CPL columns; NRA: rows / 4, NCG: columns / 8.
 //
 // Eight iterations at a time run without a branch on drift, tolerance or cap (a vote and a branch cost about 25 cycles); one look
 // at the end tells whether there was anything, and if there was the eight are taken back and done again one by one.  A row error
 // above the tolerance settles that the sum is; only if no row has one are the sums formed.
-template <int RMAX, int NT, int LR, int RPL, int NRA, int NCG, bool TOL>
+template <int RMAX, int NT, int NW, int LR, int NRA, int NCG, bool TOL>
 __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& sm, const int Hn, const int Cn, const float tol_abs_f)
 {
-    constexpr int CPL = RMAX / 32, RS = 32 / LR;       // RS: rows between a lane's
+    constexpr int NL = 32 * NW, CPL = RMAX / NL;
     constexpr int Q = 2 / LR;                          // float4 of v~ per cg that a row's lane reads
     constexpr int KS = SplitSmem<RMAX>::KS;
-    const int lane = threadIdx.x;
-    const int row0 = lane / LR, half = lane & (LR - 1);
-    bool row_ok[RPL], col_ok[CPL];
+    const int lane = threadIdx.x;                      // (beyond 31 in the second warp)
+    const int row = lane / LR, half = lane & (LR - 1);
+    const auto sync = [&]() {
+        if (NW == 1) __syncwarp();
+        else asm volatile("bar.sync 2, %0;" ::"n"(NL) : "memory");
+    };
+    const auto any = [&](bool p) -> bool {
+        if (NW == 1) return __any_sync(kFull, p);
+        int r;
+        asm volatile("{ .reg .pred p, q; setp.ne.s32 p, %1, 0; barrier.cta.red.or.pred q, 3, %2, p; selp.s32 %0, 1, 0, q; }"
+                     : "=r"(r) : "r"((int)p), "n"(NL) : "memory");
+        return r != 0;
+    };
+    const bool row_ok = row < Hn;
+    bool col_ok[CPL];
     // Off the problem's block u~ and v~ are 0: no select (the compiler makes it a branch around the reciprocal, and the warp barrier
     // behind a branch another 25 cycles).  The sums there must not be 0, so the lane's own copy of K~ begins with a 1.
-    float st[RPL], dd[CPL];
-#pragma unroll
-    for (int k = 0; k < RPL; ++k) {
-        row_ok[k] = row0 + RS * k < Hn;
-        st[k] = row_ok[k] ? sm.st[row0 + RS * k] : 0.0f;
-    }
+    const float st = row_ok ? sm.st[row] : 0.0f;
+    float dd[CPL];
 #pragma unroll
     for (int q = 0; q < CPL; ++q) {
-        col_ok[q] = lane + 32 * q < Cn;
-        dd[q] = col_ok[q] ? sm.dd[lane + 32 * q] : 0.0f;
+        col_ok[q] = lane + NL * q < Cn;
+        dd[q] = col_ok[q] ? sm.dd[lane + NL * q] : 0.0f;
     }
     const uint32_t lo_bits = __float_as_uint(kDriftLo), span_bits = __float_as_uint(kDriftHi) - lo_bits;
     const auto drifted = [&](float x) { return (__float_as_uint(x) - lo_bits) > span_bits; };
     const auto in_range = [](float x) { return x > kSumLo && x < kSumHi; };
-    float4 Kr[RPL][NCG][Q], Kc[CPL][NRA];
+    float4 Kr[NCG][Q], Kc[CPL][NRA];
     const auto load_tile = [&]() {
 #pragma unroll
-        for (int k = 0; k < RPL; ++k) {
+        for (int cg = 0; cg < NCG; ++cg)
 #pragma unroll
-            for (int cg = 0; cg < NCG; ++cg)
-#pragma unroll
-                for (int q = 0; q < Q; ++q)
-                    Kr[k][cg][q] = *reinterpret_cast<const float4*>(&sm.K[(row0 + RS * k) * KS + cg * 8 + (half + q) * 4]);
-            if (!row_ok[k]) Kr[k][0][0].x = 1.0f;
-        }
+            for (int q = 0; q < Q; ++q) Kr[cg][q] = *reinterpret_cast<const float4*>(&sm.K[row * KS + cg * 8 + (half + q) * 4]);
+        if (!row_ok) Kr[0][0].x = 1.0f;
 #pragma unroll
         for (int q = 0; q < CPL; ++q) {
 #pragma unroll
             for (int ra = 0; ra < NRA; ++ra) {
-                const float* k = &sm.K[ra * 4 * KS + lane + 32 * q];
+                const float* k = &sm.K[ra * 4 * KS + lane + NL * q];
                 Kc[q][ra] = make_float4(k[0], k[KS], k[2 * KS], k[3 * KS]);
             }
             if (!col_ok[q]) Kc[q][0].x = 1.0f;
@@ -148,25 +154,18 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
         }
     };
     const auto tree = [](const float4 p) { return __fadd_rn(__fadd_rn(p.x, p.y), __fadd_rn(p.z, p.w)); };
-    float uo[RPL], un[RPL], r[RPL], vcol[CPL], cp[CPL];        // uo, vcol: iterate t in this lane's rows and columns
+    float uo = row_ok ? 1.0f : 0.0f, un = 0.0f, r = 1.0f, vcol[CPL], cp[CPL];       // uo, vcol: iterate t in this lane's row and columns
     const auto new_rows = [&](const float* v) {
         const float4* vb = reinterpret_cast<const float4*>(v) + half;
-        float4 p[RPL][Q];
+        float4 p[Q];
 #pragma unroll
         for (int cg = 0; cg < NCG; ++cg)
 #pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const float4 x = vb[cg * 2 + q];
-#pragma unroll
-                for (int k = 0; k < RPL; ++k) chain(p[k][q], Kr[k][cg][q], x, cg == 0);
-            }
-#pragma unroll
-        for (int k = 0; k < RPL; ++k) {
-            r[k] = tree(p[k][0]);
-            if constexpr (LR == 1) r[k] = __fadd_rn(r[k], tree(p[k][Q - 1]));
-            else r[k] = __fadd_rn(r[k], __shfl_xor_sync(kFull, r[k], 1));
-            un[k] = __fmul_rn(st[k], rcp_fast(r[k]));
-        }
+            for (int q = 0; q < Q; ++q) chain(p[q], Kr[cg][q], vb[cg * 2 + q], cg == 0);
+        r = tree(p[0]);
+        if constexpr (LR == 1) r = __fadd_rn(r, tree(p[Q - 1]));
+        else r = __fadd_rn(r, __shfl_xor_sync(kFull, r, 1));
+        un = __fmul_rn(st, rcp_fast(r));
     };
     const auto new_columns = [&](float* v) {
         float4 c[CPL];
@@ -180,43 +179,32 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
         for (int q = 0; q < CPL; ++q) {
             cp[q] = tree(c[q]);
             vcol[q] = __fmul_rn(dd[q], rcp_fast(cp[q]));
-            v[lane + 32 * q] = vcol[q];
+            v[lane + NL * q] = vcol[q];
         }
     };
-    // the new u~ and, with a tolerance, the errors of iterate t (a row's lanes hold the same); true: an error above the tolerance
+    // the new u~ and, with a tolerance, the row's error of iterate t (a row's lanes hold the same); true: it is above the tolerance
     const auto put_rows = [&](float* e) {
-        bool above = false;
-#pragma unroll
-        for (int k = 0; k < RPL; ++k) {
-            sm.u[row0 + RS * k] = un[k];
-            if (TOL) {
-                const float x = fabsf(fmaf(uo[k], r[k], -st[k]));
-                e[row0 + RS * k] = x;
-                above |= x > tol_abs_f;
-            }
-        }
-        return above;
+        sm.u[row] = un;
+        if (!TOL) return false;
+        const float x = fabsf(fmaf(uo, r, -st));
+        e[row] = x;
+        return x > tol_abs_f;
     };
     const auto any_drift = [&]() {
-        bool d = false;
-#pragma unroll
-        for (int k = 0; k < RPL; ++k) d |= row_ok[k] & drifted(uo[k]);
+        bool d = row_ok & drifted(uo);
 #pragma unroll
         for (int q = 0; q < CPL; ++q) d |= col_ok[q] & drifted(vcol[q]);
         return d;
     };
     load_tile();
 #pragma unroll
-    for (int k = 0; k < RPL; ++k) uo[k] = row_ok[k] ? 1.0f : 0.0f;
-#pragma unroll
     for (int q = 0; q < CPL; ++q) vcol[q] = 1.0f;
     int t = 1;
     for (;;) {
         const int t_end = t + kSplitGroup;
         if (t_end <= a.max_iters) {                    // (the last iterate is one of those below)
-            float u0[RPL], v0[CPL];
-#pragma unroll
-            for (int k = 0; k < RPL; ++k) u0[k] = uo[k];
+            const float u0 = uo;
+            float v0[CPL];
 #pragma unroll
             for (int q = 0; q < CPL; ++q) v0[q] = vcol[q];
             float* va = sm.v[t & 1];
@@ -227,17 +215,32 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
                 new_rows(g & 1 ? vb : va);
                 above[g] = put_rows(sm.e[g]);
                 odd |= any_drift();
-#pragma unroll
-                for (int k = 0; k < RPL; ++k) uo[k] = un[k];
-                __syncwarp();
+                uo = un;
+                sync();
                 new_columns(g & 1 ? va : vb);
-                __syncwarp();
+                if (NW == 1 || g < kSplitGroup - 1) sync();
             }
-            bool met = __any_sync(kFull, odd);
-            if (TOL) {
-                bool near = false;
+            bool met, near = false;
+            if (NW == 1) {
+                met = __any_sync(kFull, odd);
+                if (TOL) {
 #pragma unroll
-                for (int g = 0; g < kSplitGroup; ++g) near |= !__any_sync(kFull, above[g]);
+                    for (int g = 0; g < kSplitGroup; ++g) near |= !__any_sync(kFull, above[g]);
+                }
+            } else {
+                uint32_t bits = odd ? 1u << kSplitGroup : 0u;
+                if (TOL) {
+#pragma unroll
+                    for (int g = 0; g < kSplitGroup; ++g) bits |= above[g] ? 1u << g : 0u;
+                }
+                bits = __reduce_or_sync(kFull, bits);
+                if ((lane & 31) == 0) sm.bits[lane >> 5] = bits;
+                sync();
+                bits = sm.bits[0] | sm.bits[1];
+                met = (bits >> kSplitGroup) != 0u;
+                near = TOL && (~bits & ((1u << kSplitGroup) - 1u)) != 0u;
+            }
+            if (TOL) {
                 if (near) {
 #pragma unroll
                     for (int g = 0; g < kSplitGroup; ++g) met |= split_error<NRA>(sm.e[g]) <= tol_abs_f;
@@ -247,35 +250,27 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
                 t = t_end;
                 continue;
             }
-            __syncwarp();
+            sync();
+            uo = u0;
 #pragma unroll
-            for (int k = 0; k < RPL; ++k) uo[k] = u0[k];
-#pragma unroll
-            for (int q = 0; q < CPL; ++q) va[lane + 32 * q] = vcol[q] = v0[q];
-            __syncwarp();
+            for (int q = 0; q < CPL; ++q) va[lane + NL * q] = vcol[q] = v0[q];
+            sync();
         }
         // ---- one by one, until something has been seen to
-        float usave[RPL], rsave[RPL];
-#pragma unroll
-        for (int k = 0; k < RPL; ++k) usave[k] = rsave[k] = 1.0f;
+        float usave = 1.0f, rsave = 1.0f;
         bool odd_p = false, due = false;               // of the iterate before this one
         for (;; ++t) {
             new_rows(sm.v[t & 1]);                     // half-step 1: r = K~ v~, u' = s~ / r; r are the row sums of iterate t
             // what iteration t - 1 left to decide
             const bool stop = TOL && due && split_error<NRA>(sm.e[0]) <= tol_abs_f, last = t > a.max_iters;
             if (stop || last) {                        // iterate t - 1 is the result
-                bool bad = false;
-#pragma unroll
-                for (int k = 0; k < RPL; ++k) {
-                    bad |= row_ok[k] && !in_range(rsave[k]);
-                    if (!TOL) sm.e[0][row0 + RS * k] = row_ok[k] ? fabsf(fmaf(usave[k], rsave[k], -st[k])) : 0.0f;
-                    if (row_ok[k] && half == 0) sm.alpha[row0 + RS * k] += log((double)usave[k]);
-                }
+                const bool bad = any(row_ok && !in_range(rsave));
+                if (!TOL) sm.e[0][row] = row_ok ? fabsf(fmaf(usave, rsave, -st)) : 0.0f;
+                if (row_ok && half == 0) sm.alpha[row] += log((double)usave);
 #pragma unroll
                 for (int q = 0; q < CPL; ++q)
-                    if (col_ok[q]) sm.beta[lane + 32 * q] += log((double)sm.v[(t - 1) & 1][lane + 32 * q]);
-                bad = __any_sync(kFull, bad);
-                __syncwarp();
+                    if (col_ok[q]) sm.beta[lane + NL * q] += log((double)sm.v[(t - 1) & 1][lane + NL * q]);
+                sync();
                 if (lane == 0) {
                     sm.err = split_error<NRA>(sm.e[0]);
                     sm.status = bad ? 0 : 1;
@@ -286,24 +281,19 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
             if (odd_p) {
                 // u~, v~ merely drifted: fold them into the potentials and rebuild the tile; or a sum left the range in which
                 // fp32 products are trustworthy: hand the problem back
-                bool bad = false;
-#pragma unroll
-                for (int k = 0; k < RPL; ++k) bad |= row_ok[k] && !in_range(rsave[k]);
+                bool bad = row_ok && !in_range(rsave);
 #pragma unroll
                 for (int q = 0; q < CPL; ++q) bad |= col_ok[q] && !in_range(cp[q]);
-                if (__any_sync(kFull, bad)) {
+                if (any(bad)) {
                     if (lane == 0) sm.status = 0;
                     return;
                 }
-#pragma unroll
-                for (int k = 0; k < RPL; ++k) {
-                    if (row_ok[k] && half == 0) sm.alpha[row0 + RS * k] += log((double)uo[k]);
-                    uo[k] = row_ok[k] ? 1.0f : 0.0f;
-                }
+                if (row_ok && half == 0) sm.alpha[row] += log((double)uo);
+                uo = row_ok ? 1.0f : 0.0f;
 #pragma unroll
                 for (int q = 0; q < CPL; ++q) {
-                    if (col_ok[q]) sm.beta[lane + 32 * q] += log((double)vcol[q]);
-                    sm.v[t & 1][lane + 32 * q] = vcol[q] = 1.0f;
+                    if (col_ok[q]) sm.beta[lane + NL * q] += log((double)vcol[q]);
+                    sm.v[t & 1][lane + NL * q] = vcol[q] = 1.0f;
                 }
                 if (lane == 0) sm.fill = 1;
                 split_sync<NT>();
@@ -314,17 +304,12 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
             }
             if (t == t_end) break;
             due = t % a.check_every == 0;
-            odd_p = __any_sync(kFull, any_drift());
+            odd_p = any(any_drift());
             put_rows(sm.e[0]);                         // half-step 2: c = K~^T u', v' = d / c
-#pragma unroll
-            for (int k = 0; k < RPL; ++k) {
-                usave[k] = uo[k];
-                uo[k] = un[k];
-                rsave[k] = r[k];
-            }
-            __syncwarp();
+            usave = uo; uo = un; rsave = r;
+            sync();
             new_columns(sm.v[(t + 1) & 1]);
-            __syncwarp();
+            sync();
         }
     }
 }
@@ -332,7 +317,7 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
 template <int RMAX, int NT, bool TOL>
 __device__ __forceinline__ void split_dispatch(const SinkArgs& a, SplitSmem<RMAX>& sm, int Hn, int Cn, float tol_abs_f)
 {
-#define TAOT_SPLIT(LR, RPL, NRA, NCG) return split_loop<RMAX, NT, LR, RPL, NRA, NCG, TOL>(a, sm, Hn, Cn, tol_abs_f)
+#define TAOT_SPLIT(NW, LR, NRA, NCG) return split_loop<RMAX, NT, NW, LR, NRA, NCG, TOL>(a, sm, Hn, Cn, tol_abs_f)
     if constexpr (RMAX == 32) {
 #define TAOT_SPLIT_ROWS(NCG)                           \
         if (Hn <= 4) TAOT_SPLIT(1, 1, 1, NCG);        \
@@ -347,9 +332,9 @@ __device__ __forceinline__ void split_dispatch(const SinkArgs& a, SplitSmem<RMAX
 #undef TAOT_SPLIT_ROWS
     } else {
 #define TAOT_SPLIT_ROWS(NCG)                           \
-        if (Hn <= 8) TAOT_SPLIT(2, 1, 2, NCG);         \
-        if (Hn <= 12) TAOT_SPLIT(2, 1, 3, NCG);        \
-        if (Hn <= 16) TAOT_SPLIT(2, 1, 4, NCG);        \
+        if (Hn <= 8) TAOT_SPLIT(1, 2, 2, NCG);         \
+        if (Hn <= 12) TAOT_SPLIT(1, 2, 3, NCG);        \
+        if (Hn <= 16) TAOT_SPLIT(1, 2, 4, NCG);        \
         if (Hn <= 20) TAOT_SPLIT(2, 2, 5, NCG);        \
         if (Hn <= 24) TAOT_SPLIT(2, 2, 6, NCG);        \
         TAOT_SPLIT(2, 2, 8, NCG);
@@ -364,7 +349,7 @@ __device__ __forceinline__ void split_dispatch(const SinkArgs& a, SplitSmem<RMAX
 
 // one problem per CTA of NT threads (the name is that of the register-tile kernels it stands beside)
 template <int RMAX, int NT, bool TOL>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, RMAX == 32 ? 4 : 2)
 sinkhorn_tile_kernel(SinkArgs a)
 {
     __shared__ SplitSmem<RMAX> sm;
@@ -493,9 +478,9 @@ sinkhorn_tile_kernel(SinkArgs a)
     __syncthreads();
     // one warp iterates; the others wait until a fold wants the tile rebuilt (64 ranks, 1000 iterations with a dozen folds: 2 us each
     // by the one warp)
-    if (warp == 0) {
+    if (warp < (RMAX > 32 && Hn > 16 ? 2 : 1)) {
         split_dispatch<RMAX, NT, TOL>(a, sm, Hn, Cn, (float)((double)a.tol * sum_st));
-        if (lane == 0) sm.fill = 0;
+        if (tid == 0) sm.fill = 0;
         split_sync<NT>();
     } else {
         for (split_sync<NT>(); sm.fill; split_sync<NT>()) {
