@@ -28,8 +28,9 @@ int taot_launch_sinkhorn_tile(taot_handle_t h, const SinkArgs& a_in, int32_t B, 
         launched += n;
         a.skip_solved = 1;
     }
-    if (R <= 128) TAOT_CUDA_OK(taot_launch_chained(sinkhorn_tile_kernel<4, 4, 4, 8, 16, 1>, B, 128, 0, st, a, (int64_t)B));
-    else TAOT_CUDA_OK(taot_launch_chained(sinkhorn_tile_kernel<16, 8, 2, 4, 8, 1>, B, 512, 0, st, a, (int64_t)B));
+    const bool tol = a.tol > 0.0f;
+    if (R <= 128) TAOT_CUDA_OK(taot_launch_chained(tol ? sinkhorn_tile_kernel<4, 4, 4, 8, 16, 1, true> : sinkhorn_tile_kernel<4, 4, 4, 8, 16, 1, false>, B, 128, 0, st, a, (int64_t)B));
+    else TAOT_CUDA_OK(taot_launch_chained(tol ? sinkhorn_tile_kernel<16, 8, 2, 4, 8, 1, true> : sinkhorn_tile_kernel<16, 8, 2, 4, 8, 1, false>, B, 512, 0, st, a, (int64_t)B));
     TAOT_CUDA_OK(cudaGetLastError());
     return launched;
 }

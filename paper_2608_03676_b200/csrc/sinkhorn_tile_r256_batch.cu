@@ -6,7 +6,8 @@
 
 int taot_launch_sinkhorn_tile_r256_batch(const SinkArgs& a, int32_t B, cudaStream_t st)
 {
-    TAOT_CUDA_OK(taot_launch_chained(sinkhorn_tile_kernel<4, 8, 4, 8, 8, 1>, B, 128, 0, st, a, (int64_t)B));
+    if (a.tol > 0.0f) TAOT_CUDA_OK(taot_launch_chained(sinkhorn_tile_kernel<4, 8, 4, 8, 8, 1, true>, B, 128, 0, st, a, (int64_t)B));
+    else TAOT_CUDA_OK(taot_launch_chained(sinkhorn_tile_kernel<4, 8, 4, 8, 8, 1, false>, B, 128, 0, st, a, (int64_t)B));
     TAOT_CUDA_OK(cudaGetLastError());
     return 1;
 }
