@@ -275,7 +275,7 @@ def tiered_fma_per_iteration(R):
 
 def sinkhorn_chain_floor(out, cfg, lat):
     """Cycles of the dependent chain of ONE iteration of the kernel that solves this shape with few problems per
-    call, from the measured latencies: shuffle-reduction levels, the two scaling updates, and the multiply-add
+    call, from the measured latencies: reductions, exchanges, the two scaling updates, and the multiply-add
     chains in front of them.  None where no such model is kept (multi-warp tiles, clusters)."""
     ex = out["excess"].cpu().numpy(); sp = out["spare"].cpu().numpy()
     hn = int((ex > 0).sum(1).max()); cn = int((sp > 0).sum(1).max())
@@ -284,11 +284,12 @@ def sinkhorn_chain_floor(out, cfg, lat):
         # multiply-adds of the rank's own sum, the scaling update
         return 2 * (5 * lat["shuffle_level"] + 9 * lat["fma"] + lat["rcp_mul"]), "2 x (5 shuffle levels + 9 fma + rcp-mul)"
     if cfg.R <= 64:
-        # 4 x 8 lane grid: row sums over 8 column lanes (3 levels), column sums over 4 row lanes (2 levels); the
-        # lane-local multiply-add chains are as long as the tile is deep (rows in steps of 4, columns in steps of 8)
-        nra = max(1, -(-hn // 4)); ncg = max(2, -(-cn // 8))
-        return (5 * lat["shuffle_level"] + (nra + ncg) * lat["fma"] + 2 * lat["rcp_mul"],
-                f"5 shuffle levels + {nra + ncg} fma + 2 rcp-mul")
+        # a lane holds a row and a column: chains as deep as the columns in steps of 8 and the rows in steps of 4, trees of three and
+        # two additions (beyond 32 ranks one of them is a shuffle between the two lanes of a row), and u~, v~ handed over through
+        # shared memory, a store and the load behind it 28 cycles (measured; further loads of the same exchange not counted)
+        nra = max(1, -(-hn // 4)); ncg = max(1, -(-cn // 8)); adds = nra + ncg + (5 if cfg.R <= 32 else 4)
+        return (2 * 28.0 + adds * lat["fma"] + (0 if cfg.R <= 32 else lat["shuffle_level"]) + 2 * lat["rcp_mul"],
+                f"2 exchanges through shared memory + {adds} fma{'' if cfg.R <= 32 else ' + a shuffle level'} + 2 rcp-mul")
     return None, None
 
 
