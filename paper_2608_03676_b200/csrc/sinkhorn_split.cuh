@@ -105,7 +105,10 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
         else asm volatile("bar.sync 2, %0;" ::"n"(NL) : "memory");
     };
     const auto any = [&](bool p) -> bool {
-        if (NW == 1) return __any_sync(kFull, p);
+        if (NW == 1) {
+            __syncwarp();                              // (a vote orders no memory; the barrier below does)
+            return __any_sync(kFull, p);
+        }
         int r;
         asm volatile("{ .reg .pred p, q; setp.ne.s32 p, %1, 0; barrier.cta.red.or.pred q, 3, %2, p; selp.s32 %0, 1, 0, q; }"
                      : "=r"(r) : "r"((int)p), "n"(NL) : "memory");
@@ -244,6 +247,7 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
                 if (near) {
 #pragma unroll
                     for (int g = 0; g < kSplitGroup; ++g) met |= split_error<NRA>(sm.e[g]) <= tol_abs_f;
+                    sync();                            // every warp has the same sums before the next group writes over the errors
                 }
             }
             if (!met) {
@@ -302,7 +306,10 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
                 load_tile();
                 break;
             }
-            if (t == t_end) break;
+            if (t == t_end) {
+                if (TOL) sync();                       // (the errors that `stop` read, and the next group's)
+                break;
+            }
             due = t % a.check_every == 0;
             odd_p = any(any_drift());
             put_rows(sm.e[0]);                         // half-step 2: c = K~^T u', v' = d / c

@@ -1,0 +1,76 @@
+// One CTA of a kernel on a CPU, its threads as fibers, and a check of the order of their accesses to memory that they share.
+//
+// The kernel's source is compiled by g++ as it stands (PTX statements replaced, see cta.py) with -fsanitize=thread, which puts a call
+// before each load and store; those calls are answered in cta.cpp, not by a runtime of the compiler's.  Every thread has a vector
+// clock.  Barriers and __syncwarp() join the clocks of those that meet; votes and shuffles let their threads meet but order no
+// memory.  Two accesses to a 4-byte word, one of them a write, by threads neither of which has the other's behind it are a race,
+// whether or not they would meet in time.
+#pragma once
+#include <cuda_runtime.h>
+#include <math.h>
+#include <stdint.h>
+#include <string.h>
+
+namespace cta {
+
+extern int me, count;                    // the thread that runs, the threads of the CTA
+extern int block;
+
+// The `n` threads that come to (kind, id) meet; each brings a value and learns where all of them are, by thread of the CTA.
+const uint64_t* meet(int kind, int id, int n, uint64_t mine, bool orders);
+// Runs f by n threads.  Threads that come to no end (each waits for others) are given up.
+void launch(int b, int n, void (*f)());
+
+inline void bar(int id, int n) { meet(0, id, n, 0, true); }
+inline bool bar_or(int id, int n, bool p)                        // (by the first n threads)
+{
+    const uint64_t* v = meet(1, id, n, p, true);
+    bool r = false;
+    for (int t = 0; t < n; ++t) r |= v[t] != 0;
+    return r;
+}
+inline const uint64_t* warp(uint64_t mine, bool orders = false) { return meet(2, me / 32, 32, mine, orders) + me / 32 * 32; }
+
+struct Now { const int* p; operator unsigned() const { return (unsigned)*p; } };
+struct Index { Now x; };
+
+}  // namespace cta
+
+// ---- the device's names
+#undef __shared__
+#define __shared__ static
+#define __launch_bounds__(...)
+const cta::Index threadIdx{{&cta::me}}, blockIdx{{&cta::block}}, blockDim{{&cta::count}};
+
+inline void __syncthreads() { cta::bar(0, cta::count); }
+inline int __syncthreads_or(int p) { return cta::bar_or(0, cta::count, p != 0); }
+inline void __syncwarp(unsigned = ~0u) { cta::warp(0, true); }
+template <class T>
+T __shfl_xor_sync(unsigned, T v, int o)
+{
+    uint64_t x = 0;
+    memcpy(&x, &v, sizeof v);
+    x = cta::warp(x)[cta::me % 32 ^ o];
+    memcpy(&v, &x, sizeof v);
+    return v;
+}
+inline unsigned __ballot_sync(unsigned, bool p)
+{
+    const uint64_t* v = cta::warp(p);
+    unsigned r = 0u;
+    for (int k = 0; k < 32; ++k) r |= (unsigned)v[k] << k;
+    return r;
+}
+inline bool __any_sync(unsigned m, bool p) { return __ballot_sync(m, p) != 0u; }
+inline unsigned __reduce_or_sync(unsigned, unsigned x)
+{
+    const uint64_t* v = cta::warp(x);
+    unsigned r = 0u;
+    for (int k = 0; k < 32; ++k) r |= (unsigned)v[k];
+    return r;
+}
+inline int __popc(unsigned x) { return __builtin_popcount(x); }
+inline float __fmul_rn(float a, float b) { return a * b; }
+inline float __fadd_rn(float a, float b) { return a + b; }
+inline uint32_t __float_as_uint(float x) { uint32_t r; memcpy(&r, &x, 4); return r; }
+inline int atomicOr(int* p, int v) { const int old = *p; *p |= v; return old; }

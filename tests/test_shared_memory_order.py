@@ -1,0 +1,64 @@
+"""Every pair of accesses to shared memory that depend on each other has a wait between them, whatever the speed of the warps: the
+Phase-1 kernel of few problems, run on a CPU thread by thread with vector clocks (cta.h), at one and two warps, one and two ranks a
+lane, ends on every iteration of a group of eight, iterations looked at one by one, folds and hand-backs; its results against the
+oracle's."""
+import ctypes
+
+import numpy as np
+import pytest
+
+import cta
+import oracle as O
+
+
+@pytest.fixture(scope="module")
+def so(tmp_path_factory):
+    return cta.load(str(tmp_path_factory.mktemp("cta")), "cta_split.cpp", ["sinkhorn_split.cuh", "sinkhorn_common.cuh", "taot_internal.cuh"])
+
+
+def test_a_vote_orders_no_memory_and_a_barrier_does(so):
+    so.cta_reset()
+    so.cta_exchange(1)
+    assert so.cta_races() == 0 and so.cta_stuck() == 0
+    so.cta_exchange(0)
+    assert so.cta_races() > 0
+    so.cta_reset()
+
+
+@pytest.mark.parametrize("R,hot,cold,threads", [(8, 3, 5, 128), (24, 9, 15, 128), (32, 20, 32, 128), (48, 16, 32, 128), (48, 16, 32, 64),
+                                                (40, 18, 40, 128), (64, 20, 44, 128), (64, 31, 33, 128), (64, 20, 44, 64), (64, 40, 24, 128)])
+@pytest.mark.parametrize("iters,tol,check_every", [(25, 0.0, 1), (120, 1e-3, 1), (120, 1e-3, 3), (30, 1e-9, 1),
+                                                   (200, 3.5e-8, 8)])       # near what fp32 sums leave: met, and missed where it is asked
+@pytest.mark.parametrize("eps", [0.05, 2.0])             # 0.05: folds
+def test_no_unordered_accesses(so, R, hot, cold, threads, iters, tol, check_every, eps):
+    g = np.random.default_rng(R + hot + iters)
+    B = 1
+    C = (1.0 + 7.0 * g.random((R, R))).astype(np.float32)
+    np.fill_diagonal(C, 0.0)
+    s = np.zeros((B, R), np.float32)
+    d = np.zeros((B, R), np.float32)
+    for b in range(B):
+        s[b, g.permutation(R)[:hot]] = g.integers(1, 4000, hot)
+        free = np.flatnonzero(s[b] == 0) if hot + cold <= R else np.arange(R)
+        d[b, free[:cold]] = g.integers(1, 900, cold)
+        d[b] *= s[b].sum() / d[b].sum()
+    x = -C.astype(np.float64) / eps
+    lse0 = np.log(np.exp(x - x.max(1, keepdims=True)).sum(1)) + x.max(1)
+    plan = np.full((B, R, R), np.nan, np.float32)
+    its, err, info = np.full(B, -9, np.int32), np.zeros(B, np.float32), np.zeros(B, np.int32)
+    at = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    so.cta_reset()
+    so.cta_sinkhorn(B, R, threads, at(s), at(d), at(C), at(lse0), ctypes.c_double(1.0 / np.float64(np.float32(eps))), iters, ctypes.c_float(tol),
+                    check_every, at(plan), at(its), at(err), at(info))
+    assert so.cta_races() == 0, so.cta_first().decode()
+    assert so.cta_stuck() == 0
+    for b in range(B):
+        if hot > 32:
+            assert its[b] == -1
+            continue
+        if its[b] == -1:                                 # handed back: a sum out of fp32's comfortable range
+            assert eps == 0.05
+            continue
+        want = O.sinkhorn(s[b], d[b], C, eps, int(its[b]), 0.0, 1, 1e-8)["plan"]
+        floor = 1e-7 * s[b].sum() / (R * R)
+        assert (np.abs(plan[b] - want) <= 1e-4 * np.maximum(want, floor)).all()
