@@ -62,7 +62,7 @@ struct Tables {
     const uint32_t* list;     // [nbid] pairs, best score first: tier | win count << 8, bit 31: the next one scores the same
     const uint32_t* ent;      // [ntiers][S + 1] the same by pair: list position << 16 | tie << 14 | class << 11 | win count,
                               // class = tiers that score strictly higher at this win count (orders the bids of a rank)
-    const uint32_t* tm;       // [ntiers][W][tms] tier masks, by class (by host, tms = R, if there is no room in shared memory)
+    const uint32_t* tm;       // [ntiers][W][tms] tier masks: by class, or by host if there is no room in shared memory
     int32_t* tw_word;         // [ntiers][S] by class: the word that holds the whole tier, or -1
     uint32_t* tw_mask;        // [ntiers][S] that word's mask
     const uint2* tw;          // [ntiers][S] (lean) both
@@ -74,6 +74,7 @@ struct Tables {
     int32_t* nrem;            // [D][RC] what each rank still holds of the expert in the column
     int32_t* X;               // [R][S] the plan of this layer (global)
     int32_t R, S, K, W, dmax, ntiers, tms;
+    bool by_class;            // how tm goes (with a slot per rank both strides are the same)
     int32_t RC;               // odd in shared memory: bids for the same rank by different experts meet in no bank
     int32_t* idle;            // a word in global memory that nobody reads
 };
@@ -111,7 +112,7 @@ struct Bidder {
     __device__ __forceinline__ void start(int cc, int ss)
     {
         c = cc; s = ss;
-        ci = t.tms == t.S ? cc : ss / t.K;
+        ci = t.by_class ? cc : ss / t.K;
         live = true;
         col = t.dcol[t.slot_e[ss]];
         A = t.slot_a[ss];
@@ -444,7 +445,7 @@ struct Lean {
         for (;;) {
             const uint32_t a_wins = a_lvl + 4u * (ev & 0x7FFu);
             if (WM > 1 && et >= 0 && !one) {          // the tier's words from `first` on
-                const int ci = t.tms == t.S ? c : (int)(1023u - (low & 1023u)) / t.K;
+                const int ci = t.by_class ? c : (int)(1023u - (low & 1023u)) / t.K;
                 const uint32_t* tm = t.tm + et * t.W * t.tms + ci;
 #pragma unroll 1
                 for (int w = first; w < t.W; ++w) {

@@ -576,7 +576,7 @@ match_kernel(MatchArgs a)
         const uint32_t round_limit = (uint32_t)limit;                   // at most R * S + S < 2^19
         if (timed) c_p3loop = clock64();
         const au::Tables tab{arb, avail, lvl, bid_s, ent_s, tm, tw_word, tw_mask, tw2, slot_e, slot_a, rec_s, nxt_s, dcol, nrem, Xl,
-                             R, S, K, W, a.dmax, a.ntiers, tms, RC,
+                             R, S, K, W, a.dmax, a.ntiers, tms, a.tm_in_smem != 0, RC,
                              reinterpret_cast<int32_t*>(a.t12 + l * (int64_t)E * 2 * R)};       // (Phase 2's scratch)
         const int NP = ((C + 31) >> 5) << 5;
         auto run = [&](auto type, auto rounds_block, auto rounds_warp) {

@@ -1,6 +1,7 @@
 """Phase 3 on classes of slots: one warp and several, the hand-over between them, word edges of the rank sets, remaining counts
 in and out of shared memory, and pairs of equal score, against the oracle."""
 import pytest
+import torch
 
 import oracle as O
 import workloads as W
@@ -36,4 +37,36 @@ def test_auction_bit_exact(name, step, cap):
         assert (out["X"][l] == a["X"]).all()
         assert out["rounds"][l].tolist() == [m["inner_rounds"], a["rounds"]]
         assert bool(out["info"][l] & 8) == (a["residual"] > 0)
+    pl.close()
+
+
+def _nested(R, levels):
+    """Ranks in nested groups: the cost is that of the smallest group that holds both."""
+    at = torch.arange(R)
+    C = torch.full((R, R), 2.0 ** len(levels))
+    for i, size in reversed(list(enumerate(levels))):
+        C[(at[:, None] // size) == (at[None, :] // size)] = 2.0 ** i
+    return C.fill_diagonal_(0.0)
+
+
+@pytest.mark.parametrize("levels,E", [((8, 16, 32, 64, 128), 128), ((8, 32, 64, 128), 256), ((4, 8, 16, 32, 64, 128), 100),
+                                      ((2, 4, 8, 16, 32, 64, 128), 250), ((8, 64, 128), 1024)])
+@pytest.mark.parametrize("step", [0.1, 0.125])
+def test_one_slot_per_rank_with_tier_masks_in_global_memory(levels, E, step):
+    """As many slots as ranks: the tier masks that find no room in shared memory go by host and not by class."""
+    import paper_2608_03676_b200 as P
+    R, L, k = 256, 2, 4
+    C = _nested(R, levels)
+    e2r = (torch.arange(E) * R // E).int()
+    cfg = BASE.replace(L=L, R=R, E=E, K=1, k=k, T=R * 300)
+    g = torch.Generator().manual_seed(E + len(levels))
+    topk = torch.stack([torch.multinomial((1.0 + torch.randperm(E, generator=g)) ** -1.2, cfg.T * k, replacement=True, generator=g).view(cfg.T, k) for _ in range(L)]).int()
+    pl = P.Planner(L=L, R=R, E=E, K=1, k=k, T=cfg.T, e2r=e2r, C=C, eps=0.5, max_iters=40, tol=0.0, price_step=step)
+    out = {q: cpu(v) for q, v in pl.plan(topk.cuda()).items()}
+    B = O.default_preference(C.numpy())
+    for l in range(L):
+        m, a = oracle_schedule_layer(cfg, e2r.numpy(), B, out["n"][l], out["expert_load"][l], out["rank_load"][l], out["plan"][l], price_step=step)
+        assert (out["slot_expert"][l].ravel() == m["slot_expert"]).all()
+        assert (out["X"][l] == a["X"]).all()
+        assert out["rounds"][l].tolist() == [m["inner_rounds"], a["rounds"]]
     pl.close()
