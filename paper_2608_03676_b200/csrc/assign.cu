@@ -109,9 +109,6 @@ __device__ int build_entries(const int32_t* Xrow, const int32_t* se, int S, int 
     return m;
 }
 
-// Flat position, inside the chunk held at `buf`, of the entry of expert eb whose in-chunk ordinal is rel
-// (entries of eb before it belong to the slot whose quota ends there).  Block-wide: warp w owns entries
-// [w*2048, (w+1)*2048); per-warp counts, then ballots in the one warp that holds the entry.
 // four entries at pos (a multiple of 4) of a chunk held as one byte per entry
 __device__ __forceinline__ int4 unpack_bytes(const void* buf, int32_t pos)
 {
@@ -119,6 +116,10 @@ __device__ __forceinline__ int4 unpack_bytes(const void* buf, int32_t pos)
     return make_int4((int)(w & 255u), (int)((w >> 8) & 255u), (int)((w >> 16) & 255u), (int)(w >> 24));
 }
 
+// Flat position, inside the chunk held at `buf`, of the entry of expert eb whose in-chunk ordinal is rel
+// (entries of eb before it belong to the slot whose quota ends there).  Block-wide: warp w owns entries
+// [w * kWarpSpan, (w + 1) * kWarpSpan); per-warp counts, then ballots in the one warp that holds the entry.  s_pos: calls one after the other take
+// different words in turn, since a warp may still be reading the last call's when another is in the next one.
 template <bool VEC, bool BYTES, int NT>
 __device__ int32_t locate_split(const void* bufv, int32_t len, int eb, int rel, int* s_cntw, int* s_pos)
 {
@@ -244,7 +245,7 @@ __device__ void rewrite_chunk(const AssignArgs& a, const void* bufv, int32_t* ta
                 const int4 rec = recs[k];
                 re[k] = rec.x;
                 rt[k] = rec.z;
-                rp[k] = locate_split<VEC, BYTES, NT>(bufv, len, rec.x, rec.y, s_cntw, s_pos);
+                rp[k] = locate_split<VEC, BYTES, NT>(bufv, len, rec.x, rec.y, s_cntw, s_pos + (k & 1));
             }
         }
 #pragma unroll
@@ -355,6 +356,7 @@ __device__ void rewrite_chunk(const AssignArgs& a, const void* bufv, int32_t* ta
             running += tot;
         }
         at = __reduce_min_sync(0xffffffffu, at);
+        __syncwarp();                                      // (all lanes have read the ordinal)
         if (lane == 0) recs[k].y = at;                     // from here on y is the position
     }
     __syncthreads();
@@ -471,7 +473,7 @@ assign_chunk_kernel(AssignArgs a)
     __shared__ __align__(8) uint64_t bar;
     __shared__ int s_cntw[kWarps];
     __shared__ int s_wcnt[32];
-    __shared__ int s_pos;
+    __shared__ int s_pos[2];
     __shared__ int s_ns;
     const int tid = threadIdx.x;
     const int64_t id = blockIdx.x;
@@ -528,8 +530,8 @@ assign_chunk_kernel(AssignArgs a)
             return;
         }
     }
-    if (BYTES && flagged) rewrite_chunk<VEC, false, NT>(a, a.topk + goff, tab, a.out + goff, len, s_ns, recs, ent_s, s_cntw, &s_pos);
-    else rewrite_chunk<VEC, BYTES, NT>(a, buf, tab, a.out + goff, len, s_ns, recs, ent_s, s_cntw, &s_pos);
+    if (BYTES && flagged) rewrite_chunk<VEC, false, NT>(a, a.topk + goff, tab, a.out + goff, len, s_ns, recs, ent_s, s_cntw, s_pos);
+    else rewrite_chunk<VEC, BYTES, NT>(a, buf, tab, a.out + goff, len, s_ns, recs, ent_s, s_cntw, s_pos);
 }
 
 }  // namespace

@@ -13,6 +13,7 @@
 namespace cta {
 
 int me, count, block;
+alignas(1024) unsigned char dynamic[227 * 1024];
 
 namespace {
 
@@ -29,7 +30,9 @@ struct Meeting {
     uint64_t round = 0;                  // how often it has taken place
     uint64_t value[2][kMax];             // what they brought, by parity of the round
 };
-struct Word { int writer = -1; uint32_t at = 0; std::vector<uint32_t> read; };      // last write, and last read by thread
+struct At { int thread; uint32_t clock; };
+struct Word { At write = {-1, 0}; std::vector<At> read, atomic; };      // the last write, reads and atomic operations since
+enum Kind { kRead, kWrite, kAtomic };
 
 char* stacks = static_cast<char*>(aligned_alloc(4096, kMax * kStack));
 std::vector<Thread> threads;
@@ -50,27 +53,41 @@ void run()
     for (;;) yield();
 }
 
-void access(uintptr_t p, size_t bytes, bool write)
+void access(uintptr_t p, size_t bytes, Kind kind)
 {
     if (me >= count || p - (uintptr_t)stacks < kMax * kStack) return;       // between launches; a thread's own
     const std::vector<uint32_t>& clock = threads[me].clock;
+    const auto unordered = [&](const At& x) { return x.thread >= 0 && x.thread != me && x.clock > clock[x.thread]; };
     for (uintptr_t w = p / 4; w <= (p + bytes - 1) / 4; ++w) {
         Word& x = words[w];
-        if (x.read.empty()) x.read.assign(count, 0u);
-        int by = x.writer >= 0 && x.writer != me && x.at > clock[x.writer] ? x.writer : -1;
-        if (write && by >= 0 && by / 32 == me / 32) by = -1;     // (one store instruction of a warp: one of its threads performs the write)
-        const bool written = by >= 0;
-        for (int t = 0; write && by < 0 && t < count; ++t)
-            if (t != me && x.read[t] > clock[t]) by = t;
-        if (by >= 0 && races++ == 0)
-            snprintf(first, sizeof first, "thread %d %s a word that thread %d %s, and no wait lies between", me, write ? "writes" : "reads", by,
-                     written ? "writes" : "reads");
-        if (write) { x.writer = me; x.at = clock[me]; }
-        else x.read[me] = clock[me];
+        const char* other = nullptr;
+        int by = -1;
+        // (one store instruction of a warp: one of its threads performs the write)
+        if (unordered(x.write) && !(kind == kWrite && x.write.thread / 32 == me / 32)) { by = x.write.thread; other = "writes"; }
+        if (kind != kRead)
+            for (const At& r : x.read) if (unordered(r)) { by = r.thread; other = "reads"; }
+        if (kind != kAtomic)
+            for (const At& r : x.atomic) if (unordered(r)) { by = r.thread; other = "updates"; }
+        if (other && races++ == 0)
+            snprintf(first, sizeof first, "thread %d %s a word that thread %d %s, and no wait lies between", me,
+                     kind == kRead ? "reads" : (kind == kWrite ? "writes" : "updates"), by, other);
+        if (kind == kWrite) {
+            x.write = {me, clock[me]};
+            x.read.clear();
+            x.atomic.clear();
+            continue;
+        }
+        std::vector<At>& seen = kind == kRead ? x.read : x.atomic;
+        size_t q = 0;
+        while (q < seen.size() && seen[q].thread != me) ++q;
+        if (q < seen.size()) seen[q].clock = clock[me];
+        else seen.push_back({me, clock[me]});
     }
 }
 
 }  // namespace
+
+void atomic(const void* p) { access((uintptr_t)p, 4, kAtomic); }
 
 const uint64_t* meet(int kind, int id, int n, uint64_t mine, bool orders)
 {
@@ -102,6 +119,7 @@ void launch(int b, int n, void (*f)())
     threads.assign(n, Thread());
     meetings.clear();
     words.clear();
+    memset(dynamic, 0xa5, sizeof dynamic);
     for (int t = 0; t < n; ++t) {
         Thread& x = threads[t];
         x.clock.assign(n, 0u);
@@ -134,17 +152,17 @@ void cta_reset() { cta::races = cta::stuck = 0; cta::first[0] = 0; }
 
 // what the compiler calls before an access
 #define CTA_HOOK(N)                                                            \
-    void __tsan_read##N(void* p) { cta::access((uintptr_t)p, N, false); }      \
-    void __tsan_write##N(void* p) { cta::access((uintptr_t)p, N, true); }      \
-    void __tsan_unaligned_read##N(void* p) { cta::access((uintptr_t)p, N, false); }  \
-    void __tsan_unaligned_write##N(void* p) { cta::access((uintptr_t)p, N, true); }
+    void __tsan_read##N(void* p) { cta::access((uintptr_t)p, N, cta::kRead); }      \
+    void __tsan_write##N(void* p) { cta::access((uintptr_t)p, N, cta::kWrite); }      \
+    void __tsan_unaligned_read##N(void* p) { cta::access((uintptr_t)p, N, cta::kRead); }  \
+    void __tsan_unaligned_write##N(void* p) { cta::access((uintptr_t)p, N, cta::kWrite); }
 CTA_HOOK(1)
 CTA_HOOK(2)
 CTA_HOOK(4)
 CTA_HOOK(8)
 CTA_HOOK(16)
-void __tsan_read_range(void* p, size_t n) { cta::access((uintptr_t)p, n, false); }
-void __tsan_write_range(void* p, size_t n) { cta::access((uintptr_t)p, n, true); }
+void __tsan_read_range(void* p, size_t n) { cta::access((uintptr_t)p, n, cta::kRead); }
+void __tsan_write_range(void* p, size_t n) { cta::access((uintptr_t)p, n, cta::kWrite); }
 void __tsan_func_entry(void*) {}
 void __tsan_func_exit() {}
 void __tsan_init() {}

@@ -9,15 +9,19 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <stdlib.h>
 #include <string.h>
 
 namespace cta {
 
 extern int me, count;                    // the thread that runs, the threads of the CTA
 extern int block;
+extern unsigned char dynamic[];          // shared memory whose size the launch gives
 
 // The `n` threads that come to (kind, id) meet; each brings a value and learns where all of them are, by thread of the CTA.
 const uint64_t* meet(int kind, int id, int n, uint64_t mine, bool orders);
+// An atomic operation on a word: in no race with others of its kind.
+void atomic(const void* p);
 // Runs f by n threads.  Threads that come to no end (each waits for others) are given up.
 void launch(int b, int n, void (*f)());
 
@@ -69,8 +73,32 @@ inline unsigned __reduce_or_sync(unsigned, unsigned x)
     for (int k = 0; k < 32; ++k) r |= (unsigned)v[k];
     return r;
 }
+inline int __reduce_min_sync(unsigned, int x)
+{
+    const uint64_t* v = cta::warp((uint32_t)x);
+    int r = (int)v[0];
+    for (int k = 1; k < 32; ++k) r = (int)v[k] < r ? (int)v[k] : r;
+    return r;
+}
+inline unsigned __vcmpeq4(unsigned a, unsigned b)
+{
+    unsigned r = 0u;
+    for (int k = 0; k < 32; k += 8) r |= (a >> k & 255u) == (b >> k & 255u) ? 255u << k : 0u;
+    return r;
+}
+inline uint32_t __cvta_generic_to_shared(const void* p) { return (uint32_t)(uintptr_t)p; }
 inline int __popc(unsigned x) { return __builtin_popcount(x); }
 inline float __fmul_rn(float a, float b) { return a * b; }
 inline float __fadd_rn(float a, float b) { return a + b; }
 inline uint32_t __float_as_uint(float x) { uint32_t r; memcpy(&r, &x, 4); return r; }
-inline int atomicOr(int* p, int v) { const int old = *p; *p |= v; return old; }
+#define CTA_ATOMIC(NAME, NEW)                                                          \
+    template <class T, class U>                                                        \
+    __attribute__((no_sanitize("thread"))) T NAME(T* p, U v)                           \
+    {                                                                                  \
+        cta::atomic(p);                                                                \
+        const T old = *p;                                                              \
+        *p = NEW;                                                                      \
+        return old;                                                                    \
+    }
+CTA_ATOMIC(atomicOr, old | (T)v)
+CTA_ATOMIC(atomicAdd, old + (T)v)

@@ -1,7 +1,7 @@
-"""Every pair of accesses to shared memory that depend on each other has a wait between them, whatever the speed of the warps: the
-Phase-1 kernel of few problems, run on a CPU thread by thread with vector clocks (cta.h), at one and two warps, one and two ranks a
-lane, ends on every iteration of a group of eight, iterations looked at one by one, folds and hand-backs; its results against the
-oracle's."""
+"""Every pair of accesses to shared memory that depend on each other has a wait between them, whatever the speed of the warps.  Kernels
+run on a CPU thread by thread with vector clocks (cta.h), their results against the oracle's: the Phase-1 kernel of few problems at one
+and two warps, one and two ranks a lane, ends on every iteration of a group of eight, iterations looked at one by one, folds and
+hand-backs; the reassignment of chunks with no split, with splits located one by one and with splits located together."""
 import ctypes
 
 import numpy as np
@@ -62,3 +62,32 @@ def test_no_unordered_accesses(so, R, hot, cold, threads, iters, tol, check_ever
         want = O.sinkhorn(s[b], d[b], C, eps, int(its[b]), 0.0, 1, 1e-8)["plan"]
         floor = 1e-7 * s[b].sum() / (R * R)
         assert (np.abs(plan[b] - want) <= 1e-4 * np.maximum(want, floor)).all()
+
+
+@pytest.fixture(scope="module")
+def assign(tmp_path_factory):
+    return cta.load(str(tmp_path_factory.mktemp("cta")), "cta_assign.cpp", ["assign.cu", "taot_internal.cuh"])
+
+
+@pytest.mark.parametrize("fed", [0, 1, 2, 4, 5, 14])     # slots a rank feeds; up to four splits of a chunk are located one by one
+@pytest.mark.parametrize("seg,vec", [(900, 1), (1037, 0)])
+@pytest.mark.parametrize("threads", [256, 512])
+def test_reassignment_of_a_chunk(assign, fed, seg, vec, threads):
+    R, E, K, chunk = 2, 5, 8, 16384
+    S, nc = R * K, -(-seg // chunk)
+    g = np.random.default_rng(fed + seg)
+    topk = g.integers(0, E, (1, R, seg)).astype(np.int32)
+    cc = np.zeros((1, R, nc, E), np.int32)
+    X = np.zeros((1, R, S), np.int32)
+    slots = g.integers(0, E, S).astype(np.int32)
+    for r in range(R):
+        for c in range(nc):
+            cc[0, r, c] = np.bincount(topk[0, r, c * chunk:(c + 1) * chunk], minlength=E)
+        X[0, r, g.permutation(S)[:fed]] = g.integers(1, seg // (E * 6), fed)
+    out, info = np.full_like(topk, -7), np.zeros(1, np.int32)
+    at = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    assign.cta_reset()
+    assign.cta_assign(1, R, E, K, ctypes.c_long(R * seg), ctypes.c_long(seg), nc, vec, threads, at(topk), at(cc), at(slots), at(X), at(out), at(info))
+    assert assign.cta_races() == 0, assign.cta_first().decode()
+    assert assign.cta_stuck() == 0
+    assert (out.ravel() == O.assign(topk.reshape(R * seg, 1), R, E, K, slots, X[0]).ravel()).all()
