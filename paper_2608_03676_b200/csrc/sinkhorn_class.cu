@@ -508,8 +508,9 @@ sinkhorn_class_kernel(ClassArgs k, int64_t nprob)
                 auto fold = [&]() {
 #pragma unroll
                     for (int i = 0; i < VPL; ++i) {
-                        if (S[i] > 0.0) m.al[slot0 + i] += log_factor(u[i]);
-                        if (D[i] > 0.0) m.be[slot0 + i] += log_factor(v[i]);
+                        // (the lanes that hold copies of a class hold the same factors; one of them adds)
+                        if (counts && S[i] > 0.0) m.al[slot0 + i] += log_factor(u[i]);
+                        if (counts && D[i] > 0.0) m.be[slot0 + i] += log_factor(v[i]);
                         u[i] = 1.0f; v[i] = 1.0f;
                     }
                     rebuild();

@@ -12,7 +12,7 @@
 
 namespace cta {
 
-int me, count, block;
+int me, count, block, blocks;
 alignas(1024) unsigned char dynamic[227 * 1024];
 
 namespace {

@@ -15,7 +15,7 @@
 namespace cta {
 
 extern int me, count;                    // the thread that runs, the threads of the CTA
-extern int block;
+extern int block, blocks;                // its place in the grid, the CTAs of the grid
 extern unsigned char dynamic[];          // shared memory whose size the launch gives
 
 // The `n` threads that come to (kind, id) meet; each brings a value and learns where all of them are, by thread of the CTA.
@@ -35,6 +35,16 @@ inline bool bar_or(int id, int n, bool p)                        // (by the firs
 }
 inline const uint64_t* warp(uint64_t mine, bool orders = false) { return meet(2, me / 32, 32, mine, orders) + me / 32 * 32; }
 
+// two floats in a 64-bit register
+inline float low(uint64_t x) { float f; memcpy(&f, &x, 4); return f; }
+inline float high(uint64_t x) { x >>= 32; float f; memcpy(&f, &x, 4); return f; }
+inline uint64_t pack(float a, float b) { uint32_t l, h; memcpy(&l, &a, 4); memcpy(&h, &b, 4); return (uint64_t)h << 32 | l; }
+// not a number, if one of them is
+inline float least(float a, float b) { return a != a || a < b ? a : b; }
+inline float largest(float a, float b) { return a != a || a > b ? a : b; }
+inline float least(float a, float b, float c) { return least(least(a, b), c); }
+inline float largest(float a, float b, float c) { return largest(largest(a, b), c); }
+
 struct Now { const int* p; operator unsigned() const { return (unsigned)*p; } };
 struct Index { Now x; };
 
@@ -44,7 +54,7 @@ struct Index { Now x; };
 #undef __shared__
 #define __shared__ static
 #define __launch_bounds__(...)
-const cta::Index threadIdx{{&cta::me}}, blockIdx{{&cta::block}}, blockDim{{&cta::count}};
+const cta::Index threadIdx{{&cta::me}}, blockIdx{{&cta::block}}, blockDim{{&cta::count}}, gridDim{{&cta::blocks}};
 
 inline void __syncthreads() { cta::bar(0, cta::count); }
 inline int __syncthreads_or(int p) { return cta::bar_or(0, cta::count, p != 0); }
@@ -65,7 +75,24 @@ inline unsigned __ballot_sync(unsigned, bool p)
     for (int k = 0; k < 32; ++k) r |= (unsigned)v[k] << k;
     return r;
 }
+template <class T>
+T __shfl_sync(unsigned, T v, int lane)
+{
+    uint64_t x = 0;
+    memcpy(&x, &v, sizeof v);
+    x = cta::warp(x)[lane & 31];
+    memcpy(&v, &x, sizeof v);
+    return v;
+}
+inline unsigned __reduce_add_sync(unsigned, unsigned x)
+{
+    const uint64_t* v = cta::warp(x);
+    unsigned r = 0u;
+    for (int k = 0; k < 32; ++k) r += (unsigned)v[k];
+    return r;
+}
 inline bool __any_sync(unsigned m, bool p) { return __ballot_sync(m, p) != 0u; }
+inline bool __all_sync(unsigned m, bool p) { return __ballot_sync(m, p) == ~0u; }
 inline unsigned __reduce_or_sync(unsigned, unsigned x)
 {
     const uint64_t* v = cta::warp(x);
@@ -88,9 +115,12 @@ inline unsigned __vcmpeq4(unsigned a, unsigned b)
 }
 inline uint32_t __cvta_generic_to_shared(const void* p) { return (uint32_t)(uintptr_t)p; }
 inline int __popc(unsigned x) { return __builtin_popcount(x); }
+inline int __ffs(int x) { return __builtin_ffs(x); }
 inline float __fmul_rn(float a, float b) { return a * b; }
 inline float __fadd_rn(float a, float b) { return a + b; }
 inline uint32_t __float_as_uint(float x) { uint32_t r; memcpy(&r, &x, 4); return r; }
+inline int __float_as_int(float x) { return (int)__float_as_uint(x); }
+inline float __int_as_float(int x) { float r; memcpy(&r, &x, 4); return r; }
 #define CTA_ATOMIC(NAME, NEW)                                                          \
     template <class T, class U>                                                        \
     __attribute__((no_sanitize("thread"))) T NAME(T* p, U v)                           \

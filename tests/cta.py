@@ -7,25 +7,47 @@ import subprocess
 from paper_2608_03676_b200.build import CSRC, ROOT
 
 HERE = os.path.dirname(os.path.abspath(__file__))
-#: what a PTX statement stands for, by its instruction
+#: what a PTX statement stands for, by how it begins; {0}, {1}, ... are its operands
 PTX = {
-    "rcp.approx.ftz.f32": "y = 1.0f / x;",
-    "bar.sync 1,": "cta::bar(1, NT);",
-    "bar.sync 2,": "cta::bar(2, NL);",
-    "barrier.cta.red.or.pred": "r = cta::bar_or(3, NL, p);",
+    "rcp.approx.ftz.f32": "{0} = 1.0f / ({1});",
+    "min.NaN.f32": "{0} = cta::least({operands});",
+    "max.NaN.f32": "{0} = cta::largest({operands});",
+    "mul.rn.f32x2": "{0} = cta::pack(cta::low({1}) * cta::low({2}), cta::high({1}) * cta::high({2}));",
+    "add.rn.f32x2 %0, %0": "{0} = cta::pack(cta::low({0}) + cta::low({1}), cta::high({0}) + cta::high({1}));",
+    "fma.rn.f32x2 %0, %1, %2, %0": "{0} = cta::pack(fmaf(cta::low({1}), cta::low({2}), cta::low({0})), fmaf(cta::high({1}), cta::high({2}), cta::high({0})));",
+    "mov.b64 {": "{{ {0} = cta::low({2}); {1} = cta::high({2}); }}",
+    "mov.b64 %0": "{0} = cta::pack({1}, {2});",
+    "bar.sync 1,": "cta::bar(1, {0});",
+    "bar.sync 2,": "cta::bar(2, {0});",
+    "{ .reg .pred p, q; setp.ne.s32 p, %1, 0; barrier.cta.red.or.pred q, 3, %2": "{0} = cta::bar_or(3, {2}, {1});",
     "griddepcontrol": ";",
-    "st.global.cs.v4.s32": "*p = v;",
-    "mbarrier": "abort();",               # (bulk copies: the builds without them are the ones that run here)
-    "createpolicy": "abort();",
+    "st.global.cs.v4.s32": "*({0}) = make_int4({1}, {2}, {3}, {4});",
+    # bulk copies and clusters: the builds without them are the ones that run here
+    "mbarrier": "abort();", "{\\n\\t.reg .pred p;\\n\\tmbarrier": "abort();", "fence.mbarrier": "abort();", "cp.async.bulk": "abort();",
+    "createpolicy": "abort();", "barrier.cluster": "abort();", "mapa": "abort();", "ld.shared::cluster": "abort();",
 }
+
+
+def operands(text):
+    """The expressions of `"constraint"(expression)`, in order."""
+    found = []
+    for m in re.finditer(r'"[=+]?[a-z]"\s*\(', text):
+        end, depth = m.end(), 1
+        while depth:
+            depth += {"(": 1, ")": -1}.get(text[end], 0)
+            end += 1
+        found.append(text[m.end():end - 1])
+    return found
 
 
 def without_ptx(text):
     def one(m):
-        found = [c for ptx, c in PTX.items() if ptx in m.group(0)]
+        ptx = re.match(r'\s*"([^"]*)"', m.group(1)).group(1)
+        found = [c for begin, c in PTX.items() if ptx.startswith(begin)]
         assert len(found) == 1, m.group(0)
-        return found[0]
-    text = re.sub(r"\basm\s*(?:volatile)?\s*\(.*?\);", one, text, flags=re.S)
+        ops = operands(m.group(1))
+        return found[0].format(*ops, operands=", ".join(ops))
+    text = re.sub(r"\basm\s*(?:volatile)?\s*\((.*?)\);", one, text, flags=re.S)
     return re.sub(r"extern __shared__ (?:__align__\(\d+\) )?([\w ]+) (\w+)\[\];", r"\1* \2 = reinterpret_cast<\1*>(cta::dynamic);", text)
 
 

@@ -1,7 +1,7 @@
 """Every pair of accesses to shared memory that depend on each other has a wait between them, whatever the speed of the warps.  Kernels
 run on a CPU thread by thread with vector clocks (cta.h), their results against the oracle's: the Phase-1 kernel of few problems at one
 and two warps, one and two ranks a lane, ends on every iteration of a group of eight, iterations looked at one by one, folds and
-hand-backs; the reassignment of chunks with no split, with splits located one by one and with splits located together."""
+hand-backs; the one on classes of ranks where several lanes hold copies of a class; the reassignment of chunks with no split, with splits located one by one and with splits located together."""
 import ctypes
 
 import numpy as np
@@ -25,43 +25,80 @@ def test_a_vote_orders_no_memory_and_a_barrier_does(so):
     so.cta_reset()
 
 
-@pytest.mark.parametrize("R,hot,cold,threads", [(8, 3, 5, 128), (24, 9, 15, 128), (32, 20, 32, 128), (48, 16, 32, 128), (48, 16, 32, 64),
-                                                (40, 18, 40, 128), (64, 20, 44, 128), (64, 31, 33, 128), (64, 20, 44, 64), (64, 40, 24, 128)])
-@pytest.mark.parametrize("iters,tol,check_every", [(25, 0.0, 1), (120, 1e-3, 1), (120, 1e-3, 3), (30, 1e-9, 1),
-                                                   (200, 3.5e-8, 8)])       # near what fp32 sums leave: met, and missed where it is asked
-@pytest.mark.parametrize("eps", [0.05, 2.0])             # 0.05: folds
-def test_no_unordered_accesses(so, R, hot, cold, threads, iters, tol, check_every, eps):
-    g = np.random.default_rng(R + hot + iters)
-    B = 1
-    C = (1.0 + 7.0 * g.random((R, R))).astype(np.float32)
-    np.fill_diagonal(C, 0.0)
-    s = np.zeros((B, R), np.float32)
-    d = np.zeros((B, R), np.float32)
-    for b in range(B):
-        s[b, g.permutation(R)[:hot]] = g.integers(1, 4000, hot)
-        free = np.flatnonzero(s[b] == 0) if hot + cold <= R else np.arange(R)
-        d[b, free[:cold]] = g.integers(1, 900, cold)
-        d[b] *= s[b].sum() / d[b].sum()
+def _loads(g, R, hot, cold):
+    s, d = np.zeros((1, R), np.float32), np.zeros((1, R), np.float32)
+    s[0, g.permutation(R)[:hot]] = g.integers(1, 4000, hot)
+    free = np.flatnonzero(s[0] == 0) if hot + cold <= R else np.arange(R)
+    d[0, free[:cold]] = g.integers(1, 900, cold)
+    d *= s.sum() / d.sum()
+    return s, d
+
+
+def _solve(run, R, s, d, C, eps):
+    """run(*pointers of s, d, C, the rows' log-sum-exp, 1 / eps, plan, iterations, row error, status) -> plan, iterations"""
+    B = len(s)
     x = -C.astype(np.float64) / eps
     lse0 = np.log(np.exp(x - x.max(1, keepdims=True)).sum(1)) + x.max(1)
     plan = np.full((B, R, R), np.nan, np.float32)
     its, err, info = np.full(B, -9, np.int32), np.zeros(B, np.float32), np.zeros(B, np.int32)
     at = lambda a: a.ctypes.data_as(ctypes.c_void_p)
+    run((at(s), at(d), at(C), at(lse0), ctypes.c_double(1.0 / np.float64(np.float32(eps)))), (at(plan), at(its), at(err), at(info)))
+    return plan, its
+
+
+def _check_plan(plan, s, d, C, eps, its):
+    want = O.sinkhorn(s, d, C, eps, int(its), 0.0, 1, 1e-8)["plan"]
+    assert (np.abs(plan - want) <= 1e-4 * np.maximum(want, 1e-7 * s.sum() / s.size ** 2)).all()
+
+
+@pytest.mark.parametrize("R,hot,cold,threads", [(8, 3, 5, 128), (24, 9, 15, 128), (32, 20, 32, 128), (48, 16, 32, 128), (48, 16, 32, 64),
+                                                (40, 18, 40, 128), (64, 20, 44, 128), (64, 31, 33, 128), (64, 20, 44, 64), (64, 40, 24, 128)])
+@pytest.mark.parametrize("iters,tol,check_every", [(25, 0.0, 1), (120, 1e-3, 1), (120, 1e-3, 3), (30, 1e-9, 1),
+                                                   (200, 3.5e-8, 8)])       # near what fp32 sums leave: met, and missed where it is asked
+@pytest.mark.parametrize("eps", [0.05, 2.0])             # 0.05: folds
+def test_few_problems(so, R, hot, cold, threads, iters, tol, check_every, eps):
+    g = np.random.default_rng(R + hot + iters)
+    C = (1.0 + 7.0 * g.random((R, R))).astype(np.float32)
+    np.fill_diagonal(C, 0.0)
+    s, d = _loads(g, R, hot, cold)
     so.cta_reset()
-    so.cta_sinkhorn(B, R, threads, at(s), at(d), at(C), at(lse0), ctypes.c_double(1.0 / np.float64(np.float32(eps))), iters, ctypes.c_float(tol),
-                    check_every, at(plan), at(its), at(err), at(info))
+    plan, its = _solve(lambda i, o: so.cta_sinkhorn(1, R, threads, *i, iters, ctypes.c_float(tol), check_every, *o), R, s, d, C, eps)
     assert so.cta_races() == 0, so.cta_first().decode()
     assert so.cta_stuck() == 0
+    if hot > 32:
+        assert its[0] == -1
+    elif its[0] == -1:                                   # handed back: a sum out of fp32's comfortable range
+        assert eps == 0.05
+    else:
+        _check_plan(plan[0], s[0], d[0], C, eps, its[0])
+
+
+@pytest.fixture(scope="module")
+def classes(tmp_path_factory):
+    return cta.load(str(tmp_path_factory.mktemp("cta")), "cta_class.cpp", ["sinkhorn_class.cu", "sinkhorn_class.h", "sinkhorn_common.cuh", "taot_internal.cuh"])
+
+
+@pytest.mark.parametrize("R,node,nc", [(64, 8, 8), (64, 32, 2)])
+@pytest.mark.parametrize("B,share", [(1, 0), (5, 1)])
+@pytest.mark.parametrize("iters,tol", [(60, 0.0), (200, 1e-6)])
+@pytest.mark.parametrize("eps", [0.05, 2.0])             # 0.05: folds
+def test_classes_of_ranks(classes, R, node, nc, B, share, iters, tol, eps):
+    g = np.random.default_rng(R + node + B)
+    at = np.arange(R) // node
+    C = np.where(at[:, None] == at[None, :], 1.0, np.where(at[:, None] // 4 == at[None, :] // 4, 6.0, 16.0)).astype(np.float32)
+    np.fill_diagonal(C, 0.0)
+    loads = [_loads(g, R, 10 + b, 40 - b) for b in range(B)]
+    s, d = (np.concatenate(x) for x in zip(*loads))
+    classes.cta_reset()
+
+    def run(i, o):
+        assert classes.cta_classes(B, R, share, *i, iters, ctypes.c_float(tol), *o) == nc
+    plan, its = _solve(run, R, s, d, C, eps)
+    assert classes.cta_races() == 0, classes.cta_first().decode()
+    assert classes.cta_stuck() == 0
     for b in range(B):
-        if hot > 32:
-            assert its[b] == -1
-            continue
-        if its[b] == -1:                                 # handed back: a sum out of fp32's comfortable range
-            assert eps == 0.05
-            continue
-        want = O.sinkhorn(s[b], d[b], C, eps, int(its[b]), 0.0, 1, 1e-8)["plan"]
-        floor = 1e-7 * s[b].sum() / (R * R)
-        assert (np.abs(plan[b] - want) <= 1e-4 * np.maximum(want, floor)).all()
+        assert its[b] > 0
+        _check_plan(plan[b], s[b], d[b], C, eps, its[b])
 
 
 @pytest.fixture(scope="module")
