@@ -93,6 +93,7 @@ inline unsigned __reduce_add_sync(unsigned, unsigned x)
 }
 inline bool __any_sync(unsigned m, bool p) { return __ballot_sync(m, p) != 0u; }
 inline bool __all_sync(unsigned m, bool p) { return __ballot_sync(m, p) == ~0u; }
+inline int min(int a, int b) { return a < b ? a : b; }
 inline unsigned __reduce_or_sync(unsigned, unsigned x)
 {
     const uint64_t* v = cta::warp(x);

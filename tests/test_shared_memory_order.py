@@ -1,7 +1,7 @@
 """Every pair of accesses to shared memory that depend on each other has a wait between them, whatever the speed of the warps.  Kernels
 run on a CPU thread by thread with vector clocks (cta.h), their results against the oracle's: the Phase-1 kernel of few problems at one
 and two warps, one and two ranks a lane, ends on every iteration of a group of eight, iterations looked at one by one, folds and
-hand-backs; the one on classes of ranks where several lanes hold copies of a class; the reassignment of chunks with no split, with splits located one by one and with splits located together."""
+hand-backs; the one of batches of up to 32 ranks; the one on classes of ranks where several lanes hold copies of a class; the reassignment of chunks with no split, with splits located one by one and with splits located together."""
 import ctypes
 
 import numpy as np
@@ -68,6 +68,29 @@ def test_few_problems(so, R, hot, cold, threads, iters, tol, check_every, eps):
     if hot > 32:
         assert its[0] == -1
     elif its[0] == -1:                                   # handed back: a sum out of fp32's comfortable range
+        assert eps == 0.05
+    else:
+        _check_plan(plan[0], s[0], d[0], C, eps, its[0])
+
+
+@pytest.fixture(scope="module")
+def tile(tmp_path_factory):
+    return cta.load(str(tmp_path_factory.mktemp("cta")), "cta_tile.cpp", ["sinkhorn_tile.cuh", "sinkhorn_common.cuh", "taot_internal.cuh"])
+
+
+@pytest.mark.parametrize("R,hot,cold", [(8, 3, 5), (24, 9, 15), (32, 20, 12), (32, 15, 17)])
+@pytest.mark.parametrize("iters,tol,check_every", [(40, 0.0, 1), (120, 1e-3, 1), (120, 1e-3, 3)])
+@pytest.mark.parametrize("eps", [0.05, 2.0])             # 0.05: folds
+def test_batches_of_problems(tile, R, hot, cold, iters, tol, check_every, eps):
+    g = np.random.default_rng(R + hot + iters)
+    C = (1.0 + 7.0 * g.random((R, R))).astype(np.float32)
+    np.fill_diagonal(C, 0.0)
+    s, d = _loads(g, R, hot, cold)
+    tile.cta_reset()
+    plan, its = _solve(lambda i, o: tile.cta_sinkhorn(1, R, *i, iters, ctypes.c_float(tol), check_every, *o), R, s, d, C, eps)
+    assert tile.cta_races() == 0, tile.cta_first().decode()
+    assert tile.cta_stuck() == 0
+    if its[0] == -1:
         assert eps == 0.05
     else:
         _check_plan(plan[0], s[0], d[0], C, eps, its[0])
