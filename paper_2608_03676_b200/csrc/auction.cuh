@@ -296,6 +296,7 @@ __device__ __forceinline__ uint32_t run_warp(B& b, uint32_t rd, uint32_t round_l
             b.collect(rd << 13, a_arb);
             ++rd;
             stop = b.must_move() || rd > round_limit;
+            __syncwarp();                  // the arbiters have been read
             b.place(rd << 13, a_arb);
             stop = __any_sync(0xffffffffu, stop);
         } while (!stop);
@@ -562,6 +563,7 @@ __device__ __forceinline__ uint32_t run_warp_lean(B& b, uint32_t rd, uint32_t ro
             __syncwarp();
             b.collect(rd << 13, 0u);
             ++rd;
+            __syncwarp();                             // the arbiters have been read
             b.place(rd << 13, 0u);
         } while (!__any_sync(0xffffffffu, (b.act & (b.cw == 0u)) | (rd > round_limit)));
         last = rd - 1u;

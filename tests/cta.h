@@ -35,6 +35,9 @@ inline bool bar_or(int id, int n, bool p)                        // (by the firs
 }
 inline const uint64_t* warp(uint64_t mine, bool orders = false) { return meet(2, me / 32, 32, mine, orders) + me / 32 * 32; }
 
+// the address that __cvta_generic_to_shared() gave for a place in `dynamic`
+inline void* shared(uint32_t a) { return dynamic + (uint32_t)(a - (uint32_t)(uintptr_t)dynamic); }
+
 // two floats in a 64-bit register
 inline float low(uint64_t x) { float f; memcpy(&f, &x, 4); return f; }
 inline float high(uint64_t x) { x >>= 32; float f; memcpy(&f, &x, 4); return f; }
@@ -133,3 +136,5 @@ inline float __int_as_float(int x) { float r; memcpy(&r, &x, 4); return r; }
     }
 CTA_ATOMIC(atomicOr, old | (T)v)
 CTA_ATOMIC(atomicAdd, old + (T)v)
+CTA_ATOMIC(atomicAnd, old & (T)v)
+CTA_ATOMIC(atomicMax, old > (T)v ? old : (T)v)

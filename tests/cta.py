@@ -22,6 +22,18 @@ PTX = {
     "{ .reg .pred p, q; setp.ne.s32 p, %1, 0; barrier.cta.red.or.pred q, 3, %2": "{0} = cta::bar_or(3, {2}, {1});",
     "griddepcontrol": ";",
     "st.global.cs.v4.s32": "*({0}) = make_int4({1}, {2}, {3}, {4});",
+    "st.global.u32": "*({0}) = {1};",
+    "ld.shared.u32": "{0} = *static_cast<uint32_t*>(cta::shared({1}));",
+    "ld.shared.v2.u32": "{{ const uint2 q = *static_cast<uint2*>(cta::shared({2})); {0} = q.x; {1} = q.y; }}",
+    "st.shared.u32": "*static_cast<uint32_t*>(cta::shared({0})) = {1};",
+    "red.shared.max.u32": "atomicMax(static_cast<uint32_t*>(cta::shared({0})), {1});",
+    "red.shared.and.b32": "atomicAnd(static_cast<uint32_t*>(cta::shared({0})), {1});",
+    "red.shared.or.b32": "atomicOr(static_cast<uint32_t*>(cta::shared({0})), {1});",
+    "red.shared.add.u32": "atomicAdd(static_cast<uint32_t*>(cta::shared({0})), {1});",
+    "{ .reg .pred p; setp.ne.u32 p, %2, 0; @p red.shared.max.u32": "if ({2}) atomicMax(static_cast<uint32_t*>(cta::shared({0})), {1});",
+    "{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.shared.u32": "if ({2}) *static_cast<uint32_t*>(cta::shared({0})) = {1};",
+    "{ .reg .pred p; setp.ne.u32 p, %2, 0; @p st.global.u32": "if ({2}) *({0}) = {1};",
+    "bfind.u32": "{0} = ({1}) ? 31u - (uint32_t)__builtin_clz({1}) : ~0u;",
     # bulk copies and clusters: the builds without them are the ones that run here
     "mbarrier": "abort();", "{\\n\\t.reg .pred p;\\n\\tmbarrier": "abort();", "fence.mbarrier": "abort();", "cp.async.bulk": "abort();",
     "createpolicy": "abort();", "barrier.cluster": "abort();", "mapa": "abort();", "ld.shared::cluster": "abort();",

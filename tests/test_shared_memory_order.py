@@ -1,7 +1,7 @@
 """Every pair of accesses to shared memory that depend on each other has a wait between them, whatever the speed of the warps.  Kernels
 run on a CPU thread by thread with vector clocks (cta.h), their results against the oracle's: the Phase-1 kernel of few problems at one
 and two warps, one and two ranks a lane, ends on every iteration of a group of eight, iterations looked at one by one, folds and
-hand-backs; the one of batches of up to 32 ranks; the one on classes of ranks where several lanes hold copies of a class; the reassignment of chunks with no split, with splits located one by one and with splits located together."""
+hand-backs; the one of batches of up to 32 ranks; the one on classes of ranks where several lanes hold copies of a class; the rounds of the auction in one warp; the reassignment of chunks with no split, with splits located one by one and with splits located together."""
 import ctypes
 
 import numpy as np
@@ -151,3 +151,75 @@ def test_reassignment_of_a_chunk(assign, fed, seg, vec, threads):
     assert assign.cta_races() == 0, assign.cta_first().decode()
     assert assign.cta_stuck() == 0
     assert (out.ravel() == O.assign(topk.reshape(R * seg, 1), R, E, K, slots, X[0]).ravel()).all()
+
+
+@pytest.fixture(scope="module")
+def auction(tmp_path_factory):
+    return cta.load(str(tmp_path_factory.mktemp("cta")), "cta_auction.cpp", ["auction.cuh", "taot_internal.cuh"])
+
+
+@pytest.mark.parametrize("R,D", [(32, 6), (64, 4)])      # one word of ranks and two; at most 32 classes
+@pytest.mark.parametrize("lean,far,step", [(1, 12.0, 0.1), (0, 12.0, 0.1), (0, 2.0, 0.125)])     # the last: equal scores
+@pytest.mark.parametrize("seed", [0, 1])
+def test_auction_in_one_warp(auction, R, D, lean, far, step, seed):
+    K, W, node = 2, R // 32, 8
+    S = R * K
+    g = np.random.default_rng(seed)
+    at = np.arange(R) // node
+    C = np.where(at[:, None] == at[None, :], 1.0, far).astype(np.float32)
+    np.fill_diagonal(C, 0.0)
+    B = O.default_preference(C)
+    B3 = np.where(np.eye(R, dtype=bool), np.float32(1), B)                       # [rank, host]
+    n = (g.integers(0, 60, (R, D)) * (g.random((R, D)) < 0.7)).astype(np.int32)
+    slot_e = np.concatenate([g.permutation(D)[:K] for _ in range(R)]).astype(np.int32)
+    tokens = (g.integers(1, 200, S) * (g.random(S) < 0.7)).astype(np.int32)
+    # the (tier, win count) pairs, best score first
+    tiers = np.unique(B3)[::-1].astype(np.float32)
+    pairs = sorted(((t, w) for t in range(len(tiers)) for w in range(S + 1)),
+                   key=lambda p: -(tiers[p[0]] - np.float32(step) * np.float32(p[1])))
+    score = [tiers[t] - np.float32(step) * np.float32(w) for t, w in pairs]
+    lst, ent = np.zeros(len(pairs), np.uint32), np.zeros((len(tiers), S + 1), np.uint32)
+    for i, (t, w) in enumerate(pairs):
+        tie = i + 1 < len(pairs) and score[i + 1] == score[i]
+        above = len({float(tiers[q] - np.float32(step) * np.float32(w)) for q in range(t)} - {float(score[i])})
+        lst[i] = w << 8 | t | (tie << 31)
+        ent[t, w] = i << 16 | tie << 14 | above << 11 | w
+    assert lean == 0 or not (lst >> 31).any()
+    # classes: live slots of an expert on hosts of a node
+    lead, nxt, of = [], np.full(S + 1, S, np.uint16), {}
+    for s in range(S):
+        if tokens[s]:
+            key = (slot_e[s], at[s // K])
+            if key in of:
+                nxt[of[key]] = s
+            else:
+                lead.append(s)
+            of[key] = s
+    assert 16 < len(lead) <= 32
+    a = np.append(tokens, 0).astype(np.int32)
+    rec = np.stack([nxt.astype(np.uint32), a[nxt].astype(np.uint32)], 1)
+    bits = lambda m: np.packbits(m.reshape(W, 32), axis=1, bitorder="little").view(np.uint32).ravel()
+    avail = np.stack([bits(n[:, e] > 0) for e in range(D)], 1).astype(np.uint32)             # [W][D]
+    lvl = np.zeros((W, S + 1), np.uint32)
+    lvl[:, 0] = 0xFFFFFFFF
+    tm, tw = np.zeros((len(tiers), W, S), np.uint32), np.zeros((len(tiers), S, 2), np.uint32)
+    for t, value in enumerate(tiers):
+        for c, s in enumerate(lead):
+            tm[t, :, c] = bits(B3[:, s // K] == value)
+            words = np.flatnonzero(tm[t, :, c])
+            tw[t, c] = (words[-1] if len(words) else 0, tm[t, words[-1], c] if len(words) else 0)
+            if len(words) > 1:
+                tw[t, c, 0] = 0xFFFFFFFF
+    nrem = np.zeros((D, R | 1), np.int32)
+    nrem[:, :R] = n.T
+    arrays = [np.ascontiguousarray(x) for x in (avail, lvl, lst, ent, tm, tw, slot_e, a, rec, nxt, np.arange(D, dtype=np.int32), nrem, np.array(lead, np.int32))]
+    X, left, rounds = np.zeros((R, S), np.int32), np.zeros(S + 1, np.int32), np.zeros(1, np.int32)
+    ptr = lambda x: x.ctypes.data_as(ctypes.c_void_p)
+    auction.cta_reset()
+    auction.cta_auction(lean, ptr(np.array([R, S, K, W, D, len(tiers), len(lead)], np.int32)), (ctypes.c_void_p * len(arrays))(*[x.ctypes.data for x in arrays]),
+                        ptr(X), ptr(left), ptr(rounds))
+    assert auction.cta_races() == 0, auction.cta_first().decode()
+    assert auction.cta_stuck() == 0
+    want = O.auction(R, D, K, n, np.where(tokens > 0, slot_e, -1), tokens, B, price_step=step)
+    assert (X == want["X"]).all() and rounds[0] == want["rounds"]
+    assert (left[:S] == np.where(tokens > 0, tokens - want["X"].sum(0), 0)).all()
