@@ -321,6 +321,11 @@ __device__ __forceinline__ void split_loop(const SinkArgs& a, SplitSmem<RMAX>& s
     }
 }
 
+// The smallest build that holds the problem.  What the finer steps are worth, ns an iteration with the step : with the next larger build
+// (8 problems, 2048 iterations, with a tolerance as without):
+//   32 ranks  12 rows  102 : 105 (7 columns), 110 : 113 (20)             24 columns  107 : 118 (7 or 8 rows), 113 : 124 (14)
+//   64 ranks  12 rows  127 : 132 (30 columns), 133 : 138 (46)            56 columns  132 : 138 (7 rows), 144 : 148 (14)
+//             20 rows  133 : 147 (30), 141 : 154 (46)   24 rows  137 : 147 (30), 143 : 154 (42)
 template <int RMAX, int NT, bool TOL>
 __device__ __forceinline__ void split_dispatch(const SinkArgs& a, SplitSmem<RMAX>& sm, int Hn, int Cn, float tol_abs_f)
 {
