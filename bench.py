@@ -286,10 +286,10 @@ def sinkhorn_chain_floor(out, cfg, lat):
     if cfg.R <= 64:
         # a lane holds a row and a column: chains as deep as the columns in steps of 8 and the rows in steps of 4, trees of three and
         # two additions (beyond 32 ranks one of them is a shuffle between the two lanes of a row), and u~, v~ handed over through
-        # shared memory, a store and the load behind it 28 cycles (measured; further loads of the same exchange not counted)
+        # shared memory, each time at least one load that is waited for (the store in front of it and further loads not counted)
         nra = max(1, -(-hn // 4)); ncg = max(1, -(-cn // 8)); adds = nra + ncg + (5 if cfg.R <= 32 else 4)
-        return (2 * 28.0 + adds * lat["fma"] + (0 if cfg.R <= 32 else lat["shuffle_level"]) + 2 * lat["rcp_mul"],
-                f"2 exchanges through shared memory + {adds} fma{'' if cfg.R <= 32 else ' + a shuffle level'} + 2 rcp-mul")
+        return (2 * lat["shared_load"] + adds * lat["fma"] + (0 if cfg.R <= 32 else lat["shuffle_level"]) + 2 * lat["rcp_mul"],
+                f"2 shared loads + {adds} fma{'' if cfg.R <= 32 else ' + a shuffle level'} + 2 rcp-mul")
     return None, None
 
 
@@ -345,7 +345,8 @@ def roofline_for(stage, ms, cfg, out, peaks, sm_count, match_cyc=None):
                                achieved_ns_per_iteration=ach_ns, frac=floor_ns / ach_ns, iterations=its, model=model,
                                cycles=peaks["latency_cycles"],
                                note="achieved = stage time / iterations of the slowest problem (set-up and "
-                                    "write-out included); floor from taot_measure_latencies at the maximum SM clock")
+                                    "write-out included); floor from taot_measure_latencies (a shared load: "
+                                    "taot_measure_round_latencies) at the maximum SM clock")
         d = dict(kernel="sinkhorn_tiered_mw_kernel" if tiered else "sinkhorn_tile_kernel", bound="alu", achieved=a,
                     peak=fp32_peak, unit="TFLOP/s",
                     frac=a / fp32_peak, traffic=None,
@@ -385,21 +386,20 @@ def roofline_for(stage, ms, cfg, out, peaks, sm_count, match_cyc=None):
                  "and on one warp after that")
         rl = peaks.get("round_latency_cycles")
         if rl and r3 > 0:
-            # One auction round as a dependent chain: the probe (two independent shared-memory loads, AND, find-first-set,
-            # rank index), the arbitration (atomicMax, barrier, read-back: measured as a unit), the winner's update
-            # (load of its holding, subtract, store) and the closing barrier; six dependent integer operations at the
-            # latency of a multiply-add stand for the ALU steps in between.
+            # One auction round as a dependent chain: the bid, a maximum into the rank's arbiter, a barrier and the read-back
+            # (measured as a unit), then the won rank leaves the word of candidates and the next bid is formed: six dependent
+            # integer operations at the latency of a multiply-add (the vote that gathers the won ranks is not counted).
             fma = (peaks.get("latency_cycles") or {}).get("fma", 4.0)
-            floor_cyc = 2 * rl["shared_load"] + rl["arbitration"] + rl["barrier"] + 6 * fma
+            floor_cyc = rl["arbitration"] + 6 * fma
             share3 = c[12] / c[5]
             ach_ns = ms * 1e6 * share3 / r3
             floor_ns = floor_cyc / (peaks["sm_max_mhz"] * 1e-3)
             d["latency"] = dict(bound="dependent chain of one auction round", floor_ns_per_round=floor_ns,
                                 achieved_ns_per_round=ach_ns, frac=floor_ns / ach_ns, rounds=r3, cycles=rl,
-                                model="2 shared loads + (atomicMax, barrier, read-back) + barrier + 6 integer operations",
+                                model="(atomicMax, barrier, read-back) + 6 integer operations",
                                 note="achieved = stage time x the Phase-3 share of the slowest layer's cycles / its "
-                                     "rounds; floor from taot_measure_round_latencies (eight warps, one CTA per SM) at "
-                                     "the maximum SM clock")
+                                     "rounds; floor from taot_measure_round_latencies (eight warps, one CTA per SM; "
+                                     "rounds of at most 32 classes have one warp and a warp barrier) at the maximum SM clock")
     return d
 
 
@@ -531,6 +531,7 @@ def run_ours(args):
     peaks.update(P.measure_alu_peaks())              # FP32-FMA and ex2 ceilings of this GPU, measured once, untimed
     peaks["latency_cycles"] = P.measure_latencies() # dependent-operation latencies, for the chain floor of the Sinkhorn stage
     peaks["round_latency_cycles"] = P.measure_round_latencies()   # the operations an auction round is a chain of
+    peaks["latency_cycles"]["shared_load"] = peaks["round_latency_cycles"]["shared_load"]
     props = torch.cuda.get_device_properties(local)
     topk = W.routing_topk(cfg, device="cuda")
     pl = build_planner(cfg)
