@@ -815,6 +815,10 @@ int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expe
     if (big < want) big = want < room ? want : (room > big ? room : big);
     a.big_floats = (int32_t)(big / 4);
     smem += big;
+    // a round of the auction reads the arbiters of all words of its build, and on behind the last rank's: that has to be there for a
+    // handful of ranks and experts too
+    const size_t reach = sizeof(u64) * (size_t)p.E + sizeof(uint32_t) * ((size_t)p.R + a.W + 33 * (kMaxW - 1) + 32);
+    if (smem < reach) smem = reach;
     if (smem > 227 * 1024) return TAOT_ERR_UNSUPPORTED;
     const int need = p.R * p.K;
     // two threads per slot: Phase 2 splits each rank's scan over more lanes, and the extra warps cost less than that saves

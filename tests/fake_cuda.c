@@ -8,6 +8,7 @@
 #include <string.h>
 
 enum { LAUNCH = 1, RECORD, WAIT, COPY, SET, STREAM_CREATE, EVENT_CREATE, DEVICE_ALLOC };
+/* obj: the event, or a launch's dynamic shared memory in bytes */
 typedef struct { int kind; long stream, obj, grid; char name[96]; unsigned char arg[256]; } entry;
 enum { MAX_LOG = 20000, MAX_KERNELS = 512 };
 static entry log_[MAX_LOG];
@@ -91,12 +92,12 @@ cudaError_t __cudaPopCallConfiguration(dim3* grid, dim3* block, size_t* smem, vo
 }
 cudaError_t cudaLaunchKernel(const void* f, dim3 grid, dim3 block, void** args, size_t smem, cudaStream_t st)
 {
-    (void)block; (void)smem;
-    return put(LAUNCH, st, 0, (long)grid.x * grid.y * grid.z, name_of(f), args);
+    (void)block;
+    return put(LAUNCH, st, (long)smem, (long)grid.x * grid.y * grid.z, name_of(f), args);
 }
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void** args)
 {
-    return put(LAUNCH, c->stream, 0, (long)c->gridDim.x * c->gridDim.y * c->gridDim.z, name_of(f), args);
+    return put(LAUNCH, c->stream, (long)c->dynamicSmemBytes, (long)c->gridDim.x * c->gridDim.y * c->gridDim.z, name_of(f), args);
 }
 cudaError_t cudaFuncSetAttribute(const void* f, enum cudaFuncAttribute a, int v) { (void)f; (void)a; (void)v; return cudaSuccess; }
 cudaError_t cudaGetLastError(void) { cudaError_t e = last_error; last_error = cudaSuccess; return e; }

@@ -17,6 +17,8 @@ SHAPES = {
     "many_classes": BASE.replace(R=120, E=480, K=3, T=120 * 700, gpus_per_node=4),       # more than 128 classes
     "counts_in_global_memory": BASE.replace(R=200, E=400, K=2, T=200 * 400),
     "eight_words_four_tiers": BASE.replace(R=256, E=256, K=2, T=256 * 300, tiers=(0.0, 1.0, 3.0, 9.0), nodes_per_group=4),
+    "a_few_ranks": BASE.replace(R=2, E=6, K=1, T=2 * 999, k=2, gpus_per_node=1, tiers=(0.0, 1.0, 10.0)),
+    "a_few_ranks_equal_scores": BASE.replace(R=4, E=8, K=2, T=4 * 999, k=2, gpus_per_node=2, tiers=(0.0, 1.0, 10.0)),
     "equal_scores": BASE.replace(R=48, E=192, K=2, T=48 * 600, tiers=(0.0, 1.0, 2.0)),   # bonus 1 and 0.5, step 0.125
 }
 

@@ -162,3 +162,16 @@ def test_dispatch_workspace_follows_the_entries_of_a_chunk(so, R, E, K, seg, kep
     rest = 4 * 2 * R * (2 * E + 4 + bins + 2 * E + min(E, S) + 1) + 256 * 2 * R + 2 * R * seg + 4096 * 16       # everything else, generously
     assert (n.value > 16 * bins * 2 * R) if kept else (n.value < rest)
     pl.close()
+
+
+@pytest.mark.parametrize("far", [2.0, 8.0, 10.0])        # 10: with the price step of 0.1 some scores are equal
+@pytest.mark.parametrize("R,E,K", [(2, 2, 1), (2, 5, 3), (3, 3, 1), (4, 4, 2), (8, 8, 1), (11, 2, 1), (16, 16, 1)])
+def test_a_round_of_the_auction_reads_inside_its_shared_memory(so, R, E, K, far):
+    """The arbiters [2][R + words of 32 ranks] lie behind 8 bytes an expert; a round of the general build reads those of eight words,
+    33 apart, by 32 lanes, of either half."""
+    so.fake_reset()
+    pl = F.FakePlanner(so, 1, R, E, K, 1, R * 16, W.cost_matrix(R, 2, (0.0, 1.0, far), None))
+    assert pl.plan() == 0
+    smem = [e.obj for e in F.log(so) if e.kind == F.LAUNCH and e.name == b"match_kernel"]
+    assert len(smem) == 1 and smem[0] >= 8 * E + 4 * (R + 1) + 4 * (7 * 33 + 32)
+    pl.close()
