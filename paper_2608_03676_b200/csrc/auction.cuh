@@ -53,6 +53,8 @@ __device__ __forceinline__ void red_add_u32(uint32_t addr, uint32_t v) { asm vol
 // barrier over the first `nthreads` threads of the CTA (a multiple of 32): the warps that hold classes
 __device__ __forceinline__ void bar_part(int nthreads) { asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory"); }
 
+constexpr int kMaxWords = 8;  // words of 32 ranks of a rank set: R <= 256
+
 // what the auction works on, in shared memory (nrem may be global)
 struct Tables {
     uint32_t* arb;            // [2][R + W] best bid per rank, by parity of the round while there are several warps; a word's 32 begin a
@@ -63,9 +65,7 @@ struct Tables {
     const uint32_t* ent;      // [ntiers][S + 1] the same by pair: list position << 16 | tie << 14 | class << 11 | win count,
                               // class = tiers that score strictly higher at this win count (orders the bids of a rank)
     const uint32_t* tm;       // [ntiers][W][tms] tier masks: by class, or by host if there is no room in shared memory
-    int32_t* tw_word;         // [ntiers][S] by class: the word that holds the whole tier, or -1
-    uint32_t* tw_mask;        // [ntiers][S] that word's mask
-    const uint2* tw;          // [ntiers][S] (lean) both
+    const uint2* tw;          // [ntiers][S] by class: the word that holds the whole tier (-1: no one does) and its mask there
     const int32_t* slot_e;    // [S]
     int32_t* slot_a;          // [S + 1] tokens a slot still collects (S: 0)
     const uint2* rec;         // [S + 1] (lean) next slot of the class and the tokens it collects
@@ -80,10 +80,9 @@ struct Tables {
 };
 
 
-// A bidder: one class, its state in registers, some pairs of which may have equal scores.  NT: tiers the build holds (the handle has
-// at most as many); WM: most words of 32 ranks.
-template <int NT, int WM>
+// A bidder: one class, its state in registers, some pairs of which may have equal scores.
 struct Bidder {
+    static constexpr int NT = TAOT_MAX_TIERS, WM = kMaxWords;
     const Tables& t;
     int c = 0;                // class
     int ci = 0;               // its column of tm
@@ -135,6 +134,7 @@ struct Bidder {
     __device__ __forceinline__ void walk()
     {
         const int S = t.S, W = t.W, LS = t.S + 1;
+        uint32_t m_tw = 0u;                       // the tier's mask, if one word holds all of it
 #pragma unroll 1
         for (;;) {
             if (!one && pw + 1 < W) {
@@ -149,11 +149,12 @@ struct Bidder {
                     best = next[k] < best ? next[k] : best;
                 }
                 if (best == 0xFFFFFFFFu) { cw = 0u; return; }
-                const int wd = t.tw_word[bt * S + c];
+                const uint2 tw = t.tw[bt * S + c];
                 et = bt; ev = best;
                 any = 0u;
-                one = wd >= 0;
-                pw = one ? wd : 0;
+                one = (int)tw.x >= 0;
+                pw = one ? (int)tw.x : 0;
+                m_tw = tw.y;
                 set_next(bt, after((uint32_t)bt, best & 0x7FFu));
                 again = false;
                 gend = 0;
@@ -175,8 +176,7 @@ struct Bidder {
             const uint32_t av = t.avail[pw * t.dmax + col];
             if (gend == 0) {
                 const uint32_t* lv = t.lvl + pw * LS + (ev & 0x7FFu);
-                const uint32_t* mp = one ? t.tw_mask + et * S + c : t.tm + (et * W + pw) * t.tms + ci;
-                const uint32_t h = *mp & av;
+                const uint32_t h = (one ? m_tw : t.tm[(et * W + pw) * t.tms + ci]) & av;
                 any |= h;
                 cw = h & *lv;
                 a_lv = smem_u32(lv);

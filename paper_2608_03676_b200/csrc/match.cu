@@ -86,7 +86,6 @@ __device__ __forceinline__ u64 warp_max_u64(u64 k)
 
 template <class T> struct Type { using type = T; };
 
-constexpr int kMaxW = 8;          // words of a rank bit set: R <= 256
 constexpr size_t kSmemBudget = 224 * 1024;   // dynamic shared memory the kernel plans with (227 KB per CTA less the static part)
 
 // Arbitration "best bidder per target" for one warp's worth of bids.  Many bidders often pick the
@@ -124,7 +123,8 @@ match_kernel(MatchArgs a)
     // ---- carve shared memory
     u64* arb_e = reinterpret_cast<u64*>(smem_raw);            // [E]  Phase 2 arbitration per expert
     u64* arb_r = arb_e + E;                                    // [2][R]  Phase 3 arbitration per rank, ping-pong by round
-    int32_t* spill = reinterpret_cast<int32_t*>(arb_r + 2 * R); // [E]
+    uint2* tw_s = reinterpret_cast<uint2*>(arb_r + 2 * R);     // [ntiers][S] word and mask of a tier that one word holds, by class (LEAN: elsewhere)
+    int32_t* spill = reinterpret_cast<int32_t*>(tw_s + (!LEAN && a.nbid ? a.ntiers * S : 0)); // [E]
     int32_t* hot0 = spill + E;                                 // [E]  experts that spill at the start of Phase 2
     int32_t* hot_home = hot0 + E;                              // [E]  their home ranks
     int32_t* dcol = hot_home + E;                              // [E]  expert -> column of nrem, or -1
@@ -140,9 +140,7 @@ match_kernel(MatchArgs a)
     uint32_t* lvl = avail + a.dmax * W;                        // [W][S+1]   ranks by win count (word-major)
     uint32_t* tm_s = lvl + (S + 1) * W;                                // [ntiers][W][S] tier masks by slot, if they fit
     uint32_t* bid_s = tm_s + (a.tm_in_smem ? a.ntiers * W * S : 0);    // [nbid] (tier, win count) pairs, best score first
-    int32_t* tw_word = reinterpret_cast<int32_t*>(bid_s + a.nbid);     // [ntiers][S] word holding the whole tier for the class, or -1
-    uint32_t* tw_mask = reinterpret_cast<uint32_t*>(tw_word + (!LEAN && a.nbid ? a.ntiers * S : 0));   // [ntiers][S] that word's mask (LEAN: both in tw2)
-    uint32_t* ent_s = tw_mask + (!LEAN && a.nbid ? a.ntiers * S : 0);           // [nbid] the pairs by tier and win count
+    uint32_t* ent_s = bid_s + a.nbid;                                  // [nbid] the pairs by tier and win count
     int32_t* key_s = reinterpret_cast<int32_t*>(ent_s + a.nbid);       // [S] class keys, then the classes' lists
     uint16_t* nxt_s = reinterpret_cast<uint16_t*>(key_s + (a.nbid ? S : 0));            // [S] next slot of the class
     uint16_t* lead_s = nxt_s + (a.nbid ? S + 2 : 0);                   // [S] first slot of each class
@@ -151,7 +149,7 @@ match_kernel(MatchArgs a)
     int32_t* nrem_s = reinterpret_cast<int32_t*>(bon_s + (a.bon_in_smem ? R * RS : 0)); // [dmax*R] if it fits
     // LEAN, Phase 3 only, behind the counts in the block that Phase 2 uses for its keys
     uint2* rec_s = reinterpret_cast<uint2*>((reinterpret_cast<uintptr_t>(nrem_s + (a.nrem_in_smem ? a.dmax * (R | 1) : 0)) + 7) & ~(uintptr_t)7);   // [S+1] next slot of the class and its tokens
-    uint2* tw2 = rec_s + S + 1;                                // [ntiers][S] word and mask of a tier that one word holds, by class
+    uint2* const tw = LEAN ? rec_s + S + 1 : tw_s;
     __shared__ long long s_tot;
     __shared__ int s_cnt, s_any, s_ns;
     __shared__ taot_auction::Control ctl;
@@ -563,19 +561,14 @@ match_kernel(MatchArgs a)
                 const uint32_t mk = tm[(t * W + w) * tms + (a.tm_in_smem ? c : lead_s[c] / K)];
                 if (mk) { ++nz; wd = w; val = mk; }
             }
-            if constexpr (LEAN) {
-                tw2[t * S + c] = make_uint2(nz <= 1 ? (uint32_t)wd : 0xFFFFFFFFu, val);
-            } else {
-                tw_word[t * S + c] = nz <= 1 ? wd : -1;
-                tw_mask[t * S + c] = val;
-            }
+            tw[t * S + c] = make_uint2(nz <= 1 ? (uint32_t)wd : 0xFFFFFFFFu, val);
         }
         __syncthreads();
         long long limit = cap;
         if (a.auction_max_rounds > 0 && a.auction_max_rounds < limit) limit = a.auction_max_rounds;
         const uint32_t round_limit = (uint32_t)limit;                   // at most R * S + S < 2^19
         if (timed) c_p3loop = clock64();
-        const au::Tables tab{arb, avail, lvl, bid_s, ent_s, tm, tw_word, tw_mask, tw2, slot_e, slot_a, rec_s, nxt_s, dcol, nrem, Xl,
+        const au::Tables tab{arb, avail, lvl, bid_s, ent_s, tm, tw, slot_e, slot_a, rec_s, nxt_s, dcol, nrem, Xl,
                              R, S, K, W, a.dmax, a.ntiers, tms, a.tm_in_smem != 0, RC,
                              reinterpret_cast<int32_t*>(a.t12 + l * (int64_t)E * 2 * R)};       // (Phase 2's scratch)
         const int NP = ((C + 31) >> 5) << 5;
@@ -606,7 +599,7 @@ match_kernel(MatchArgs a)
             }
         };
         if constexpr (!LEAN) {
-            run(Type<au::Bidder<TAOT_MAX_TIERS, kMaxW>>{},
+            run(Type<au::Bidder>{},
                 [&](auto& b) { return au::run_block(b, NP, C, round_limit, &ctl); },
                 [&](auto& b, uint32_t rd) { return au::run_warp(b, rd, round_limit, ctl.last); });
         } else {
@@ -619,7 +612,7 @@ match_kernel(MatchArgs a)
                 if (W == 1) lean(tiers, std::integral_constant<int, 1>{});
                 else if (W == 2) lean(tiers, std::integral_constant<int, 2>{});
                 else if (W <= 4) lean(tiers, std::integral_constant<int, 4>{});
-                else lean(tiers, std::integral_constant<int, kMaxW>{});
+                else lean(tiers, std::integral_constant<int, au::kMaxWords>{});
             };
             if (a.ntiers <= 2) lean_w(std::integral_constant<int, 2>{});
             else lean_w(std::integral_constant<int, 4>{});
@@ -758,7 +751,7 @@ match_kernel(MatchArgs a)
     }
 }
 
-size_t match_smem_fixed(int R, int E, int K, int dmax, int W, int ntiers)
+size_t match_smem_fixed(int R, int E, int K, int dmax, int W)
 {
     const size_t S = (size_t)R * K;
     return sizeof(u64) * (E + 2 * (size_t)R) + sizeof(int32_t) * (4 * (size_t)E + 5 * (size_t)R + 3 * S + 1) +
@@ -785,11 +778,11 @@ int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expe
     a.R = p.R; a.E = p.E; a.K = p.K;
     a.dmax = p.E < p.R * p.K ? p.E : p.R * p.K;
     a.W = (p.R + 31) / 32;
-    a.nbid = (h->ntiers > 0 && h->nbid > 0 && a.W <= kMaxW && p.R * p.K <= 1024) ? h->nbid : 0;
+    a.nbid = (h->ntiers > 0 && h->nbid > 0 && a.W <= taot_auction::kMaxWords && p.R * p.K <= 1024) ? h->nbid : 0;
     a.ntiers = a.nbid > 0 ? h->ntiers : 0;
     a.eps0 = p.eps0; a.price_step = p.price_step; a.auction_max_rounds = p.auction_max_rounds;
     a.ablation = p.ablation;
-    size_t smem = match_smem_fixed(p.R, p.E, p.K, a.dmax, a.W, a.ntiers);
+    size_t smem = match_smem_fixed(p.R, p.E, p.K, a.dmax, a.W);
     const bool few_tiers = h->ntiers <= 4 && !h->bid_ties;
     const size_t S = (size_t)p.R * p.K;
     const size_t lists = sizeof(uint32_t) * (2 * (size_t)h->nbid + (few_tiers ? 0 : 2 * (size_t)h->ntiers * S) + 2 * S + 1);
@@ -817,7 +810,7 @@ int taot_launch_match(taot_handle_t h, const int32_t* d_n, const int32_t* d_expe
     smem += big;
     // a round of the auction reads the arbiters of all words of its build, and on behind the last rank's: that has to be there for a
     // handful of ranks and experts too
-    const size_t reach = sizeof(u64) * (size_t)p.E + sizeof(uint32_t) * ((size_t)p.R + a.W + 33 * (kMaxW - 1) + 32);
+    const size_t reach = sizeof(u64) * (size_t)p.E + sizeof(uint32_t) * ((size_t)p.R + a.W + 33 * (taot_auction::kMaxWords - 1) + 32);
     if (smem < reach) smem = reach;
     if (smem > 227 * 1024) return TAOT_ERR_UNSUPPORTED;
     const int need = p.R * p.K;

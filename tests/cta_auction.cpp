@@ -31,7 +31,7 @@ void kernel()
     Tables t;
     const size_t pairs = (size_t)n.ntiers * (n.S + 1), cols = n.R | 1;
     t.R = n.R; t.S = n.S; t.K = n.K; t.W = n.W; t.dmax = n.dmax; t.ntiers = n.ntiers; t.tms = n.S; t.by_class = true; t.RC = (int32_t)cols;
-    t.arb = place<uint32_t>(at, nullptr, 2 * (n.R + n.W));
+    t.arb = place<uint32_t>(at, nullptr, 2 * (n.R + n.W) + 33 * kMaxWords);      // (a round reads on behind the last rank's)
     for (int i = cta::me; i < 2 * (n.R + n.W); i += cta::count) t.arb[i] = 0u;
     t.avail = place(at, avail, (size_t)n.W * n.dmax);
     t.lvl = place(at, lvl, (size_t)n.W * (n.S + 1));
@@ -39,9 +39,6 @@ void kernel()
     t.ent = place(at, ent, pairs);
     t.tm = place(at, tm, (size_t)n.ntiers * n.W * n.S);
     t.tw = reinterpret_cast<uint2*>(place(at, tw, 2 * (size_t)n.ntiers * n.S));
-    t.tw_word = place<int32_t>(at, nullptr, (size_t)n.ntiers * n.S);
-    t.tw_mask = place<uint32_t>(at, nullptr, (size_t)n.ntiers * n.S);
-    for (int i = cta::me; i < n.ntiers * n.S; i += cta::count) { t.tw_word[i] = (int32_t)tw[2 * i]; t.tw_mask[i] = tw[2 * i + 1]; }
     t.slot_e = place(at, slot_e, n.S);
     t.slot_a = place(at, slot_a, n.S + 1);
     t.rec = reinterpret_cast<uint2*>(place(at, rec, 2 * (size_t)(n.S + 1)));
@@ -72,5 +69,5 @@ extern "C" void cta_auction(int lean, const Sizes* sizes, const void* const* in,
     next(avail); next(lvl); next(list); next(ent); next(tm); next(tw); next(slot_e); next(slot_a); next(rec); next(nxt); next(dcol); next(nrem); next(lead);
     X = plan; left = slots_left; last = rounds;
     if (lean) cta::launch(0, 32, [] { kernel<Lean<4, true, 2>, true>(); });
-    else cta::launch(0, 32, [] { kernel<Bidder<8, 2>, false>(); });
+    else cta::launch(0, 32, [] { kernel<Bidder, false>(); });
 }
