@@ -1,4 +1,4 @@
-"""Phase 1 of few problems of at most 64 ranks (rows and columns in one warp's registers): the edges of its builds (multiples of
+"""Phase 1 of few problems of at most 64 ranks (rows and columns in the registers of one or two warps): the edges of its builds (multiples of
 four supply ranks, of eight demand ranks, and one more), ends on every iteration of a group of eight, folds, hand-backs, unaligned
 blocks.  The sums are those of the lane grid that large batches take, so a batch of the same problems gives the same bits; and the
 oracle."""
