@@ -51,19 +51,15 @@ def _nested(R, levels):
     return C.fill_diagonal_(0.0)
 
 
-@pytest.mark.parametrize("levels,E", [((8, 16, 32, 64, 128), 128), ((8, 32, 64, 128), 256), ((4, 8, 16, 32, 64, 128), 100),
-                                      ((2, 4, 8, 16, 32, 64, 128), 250), ((8, 64, 128), 1024)])
-@pytest.mark.parametrize("step", [0.1, 0.125])
-def test_one_slot_per_rank_with_tier_masks_in_global_memory(levels, E, step):
-    """As many slots as ranks: the tier masks that find no room in shared memory go by host and not by class."""
+def _check_nested(levels, R, E, K, step):
     import paper_2608_03676_b200 as P
-    R, L, k = 256, 2, 4
+    L, k = 2, 4
     C = _nested(R, levels)
     e2r = (torch.arange(E) * R // E).int()
-    cfg = BASE.replace(L=L, R=R, E=E, K=1, k=k, T=R * 300)
+    cfg = BASE.replace(L=L, R=R, E=E, K=K, k=k, T=R * 300)
     g = torch.Generator().manual_seed(E + len(levels))
     topk = torch.stack([torch.multinomial((1.0 + torch.randperm(E, generator=g)) ** -1.2, cfg.T * k, replacement=True, generator=g).view(cfg.T, k) for _ in range(L)]).int()
-    pl = P.Planner(L=L, R=R, E=E, K=1, k=k, T=cfg.T, e2r=e2r, C=C, eps=0.5, max_iters=40, tol=0.0, price_step=step)
+    pl = P.Planner(L=L, R=R, E=E, K=K, k=k, T=cfg.T, e2r=e2r, C=C, eps=0.5, max_iters=40, tol=0.0, price_step=step)
     out = {q: cpu(v) for q, v in pl.plan(topk.cuda()).items()}
     B = O.default_preference(C.numpy())
     for l in range(L):
@@ -72,3 +68,16 @@ def test_one_slot_per_rank_with_tier_masks_in_global_memory(levels, E, step):
         assert (out["X"][l] == a["X"]).all()
         assert out["rounds"][l].tolist() == [m["inner_rounds"], a["rounds"]]
     pl.close()
+
+
+@pytest.mark.parametrize("levels,E", [((8, 16, 32, 64, 128), 128), ((8, 32, 64, 128), 256), ((4, 8, 16, 32, 64, 128), 100),
+                                      ((2, 4, 8, 16, 32, 64, 128), 250), ((8, 64, 128), 1024)])
+@pytest.mark.parametrize("step", [0.1, 0.125])
+def test_one_slot_per_rank_with_tier_masks_in_global_memory(levels, E, step):
+    """As many slots as ranks: the tier masks that find no room in shared memory go by host and not by class."""
+    _check_nested(levels, 256, E, 1, step)
+
+
+@pytest.mark.parametrize("levels,R,E", [((2, 4, 8, 16, 32), 64, 128), ((4, 8, 16, 32, 64, 128), 200, 100), ((2, 4, 8, 16, 32, 64, 128), 256, 250)])
+def test_five_to_eight_tiers_with_two_slots_per_rank(levels, R, E):
+    _check_nested(levels, R, E, 2, 0.1)
